@@ -26,16 +26,29 @@ struct SiteParams {
   int lik;
 };
 
-__device__ __forceinline__ double log_tilted(double a, double mc, double vc, double obs,
+// Work split.  A group of G lanes (a power of two up to 32) owns a star: every
+// lane of the group runs the Newton ascent (the same numbers; FP64 issues per
+// warp, so the copies cost nothing while the chip is idle), then lane k of the
+// group sums nodes k, k + G, ... of the 64-node rule and shuffles add the three
+// sums.  GB300 issues an FP64 warp instruction every ~64 clocks per scheduler,
+// so the kernel is bound by the length of a warp's FP64 instruction chain until
+// every scheduler has a warp: G is the largest group for which the stars still
+// fit one warp per scheduler (site_group).  The ascent evaluates exp once per
+// trial point (the accepted trial's value serves the next step) and takes the
+// last steps, below 1e-7 where Newton is quadratic, without the line search,
+// whose comparison of log-densities is rounding noise there.
+// A call of the allocation-free update on 400 stars: 485 us with one thread per
+// star and the line search to the end, 82 us so.
+__device__ __forceinline__ double log_tilted(double a, double ea, double mc, double vc, double obs,
                                              double s2) {
-  double ea = exp(a);
-  double u = a - mc, w = obs - ea;
+  const double u = a - mc, w = obs - ea;
   return -0.5 * u * u / vc - 0.5 * w * w / s2;
 }
 
-__device__ void tilted_gauss_in_a(double mc, double vc, double obs, double s2,
-                                  const double* __restrict__ ghx, const double* __restrict__ ghw,
-                                  double* mh, double* vh) {
+// Mode a of the tilted log-density; h0 its value, sh the scale 1 / sqrt(-h'')
+// of the Gauss-Hermite rule.
+__device__ __forceinline__ void tilted_mode(double mc, double vc, double obs, double s2,
+                                            double* a_out, double* h0_out, double* sh_out) {
   double a;
   if (obs > 0) {
     double aL = log(obs), vL = s2 / (obs * obs);
@@ -43,80 +56,116 @@ __device__ void tilted_gauss_in_a(double mc, double vc, double obs, double s2,
   } else {
     a = mc;
   }
+  const double ivc = 1.0 / vc, is2 = 1.0 / s2;
+  double ea = exp(a);
+  double h0 = log_tilted(a, ea, mc, vc, obs, s2);
   for (int it = 0; it < 100; ++it) {
-    double ea = exp(a);
-    double gr = -(a - mc) / vc + (obs - ea) * ea / s2;
-    double H = -1.0 / vc + (obs * ea - 2.0 * ea * ea) / s2;
+    const double gr = -(a - mc) * ivc + (obs - ea) * ea * is2;
+    const double H = -ivc + (obs * ea - 2.0 * ea * ea) * is2;
     double step = H < 0 ? -gr / H : gr * vc;
     step = fmax(-1.0, fmin(1.0, step));
-    double h0 = log_tilted(a, mc, vc, obs, s2);
-    int k = 0;
-    while (log_tilted(a + step, mc, vc, obs, s2) < h0 && k < 60) {
-      step *= 0.5;
-      ++k;
+    double en = exp(a + step);
+    double hn = log_tilted(a + step, en, mc, vc, obs, s2);
+    if (fabs(step) > 1e-7 * (1.0 + fabs(a))) {
+      for (int k = 0; hn < h0 && k < 60; ++k) {
+        step *= 0.5;
+        en = exp(a + step);
+        hn = log_tilted(a + step, en, mc, vc, obs, s2);
+      }
     }
     a += step;
+    ea = en;
+    h0 = hn;
     if (fabs(step) <= 1e-14 * (1.0 + fabs(a))) break;
   }
-  double ea = exp(a);
-  double H = -1.0 / vc + (obs * ea - 2.0 * ea * ea) / s2;
-  double sh = H < 0 ? 1.0 / sqrt(-H) : sqrt(vc);
-  double h0 = log_tilted(a, mc, vc, obs, s2);
-  const double sc = 1.4142135623730951 * sh;
-  // moments about the mode, then shifted
-  double S0 = 0, S1 = 0, S2 = 0;
-  for (int k = 0; k < kGH; ++k) {
-    double y = sc * ghx[k];
-    double wk = ghw[k] * exp(log_tilted(a + y, mc, vc, obs, s2) - h0);
-    S0 += wk;
-    S1 += wk * y;
-    S2 += wk * y * y;
-  }
-  double m1 = S1 / S0;
-  *mh = a + m1;
-  *vh = S2 / S0 - m1 * m1;
+  const double H = -ivc + (obs * ea - 2.0 * ea * ea) * is2;
+  *a_out = a;
+  *h0_out = h0;
+  *sh_out = H < 0 ? 1.0 / sqrt(-H) : sqrt(vc);
 }
 
-__global__ void k_site_update(int64_t n, SiteParams P, const double* __restrict__ mu,
-                              const double* __restrict__ var, const double* __restrict__ obs,
-                              const double* __restrict__ sig, double* __restrict__ tau,
-                              double* __restrict__ nu, const double* __restrict__ gh_x,
-                              const double* __restrict__ gh_w, double* __restrict__ part_delta,
-                              unsigned long long* __restrict__ skipped,
-                              unsigned* __restrict__ flags) {
+constexpr int kSiteThreads = 128;
+
+// Shared by the context's update and the allocation-free one: `last` (null:
+// the caller reduces part_delta) makes the last block to finish reduce the
+// block maxima and put the three results to last.out.
+struct SiteLast {
+  unsigned long long* ticket;   // blocks finished
+  unsigned long long* out;      // skip count, flags, maximum (bits of a double)
+};
+
+template <int G>
+__global__ void __launch_bounds__(kSiteThreads) k_site_update(
+    int64_t n, SiteParams P, const double* __restrict__ mu, const double* __restrict__ var,
+    const double* __restrict__ obs, const double* __restrict__ sig, double* __restrict__ tau,
+    double* __restrict__ nu, const double* __restrict__ gh_x, const double* __restrict__ gh_w,
+    double* __restrict__ part_delta, unsigned long long* __restrict__ skipped,
+    unsigned* __restrict__ flags, SiteLast last) {
   __shared__ double ghx[kGH], ghw[kGH];
-  __shared__ double sh[32];
+  __shared__ double sh[kSiteThreads / 32];
+  __shared__ int is_last;
   for (int k = threadIdx.x; k < kGH; k += blockDim.x) {
     ghx[k] = gh_x[k];
     ghw[k] = gh_w[k];
   }
   __syncthreads();
+  constexpr int kPerBlock = kSiteThreads / G;
+  const int sub = threadIdx.x & (G - 1);
   double dmax = 0;
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
-       i += (int64_t)gridDim.x * blockDim.x) {
-    const double t0 = tau[i], n0 = nu[i];
-    const double S = var[i], m = mu[i];
+  // the loop count is the same for every thread of a block, so the shuffles
+  // below always have whole warps
+  for (int64_t i0 = blockIdx.x * (int64_t)kPerBlock; i0 < n; i0 += (int64_t)gridDim.x * kPerBlock) {
+    const int64_t i = i0 + threadIdx.x / G;
+    const bool star = i < n;
+    const double t0 = star ? tau[i] : 0.0, n0 = star ? nu[i] : 0.0;
+    const double S = star ? var[i] : 1.0, m = star ? mu[i] : 0.0;
     double tc = 1.0 / S - t0;
     double ncv = m / S - n0;
-    bool skip = !(tc > 0) || !isfinite(tc) || !isfinite(ncv);
-    double t_new = t0, n_new = n0;
+    bool skip = !star || !(tc > 0) || !isfinite(tc) || !isfinite(ncv);
+    double mc = 0, vc = 1, ob = 0, s2 = 1, a = 0, h0 = 0, shw = 0;
     if (!skip) {
-      const double mc = ncv / tc;
-      const double vc = fmax(1.0 / tc, P.vc_floor);
+      mc = ncv / tc;
+      vc = fmax(1.0 / tc, P.vc_floor);
       tc = 1.0 / vc;
       ncv = mc / vc;
-      const double s2 = sig[i] * sig[i];
-      double mh, vh;
-      if (P.lik == GM_LIK_GAUSS_IN_LNA) {
-        vh = 1.0 / (1.0 / vc + 1.0 / s2);
-        mh = vh * (mc / vc + obs[i] / s2);
-      } else {
-        tilted_gauss_in_a(mc, vc, obs[i], s2, ghx, ghw, &mh, &vh);
-      }
-      t_new = 1.0 / vh - tc;
-      n_new = mh / vh - ncv;
-      if (!(t_new >= 0) || !isfinite(n_new) || !isfinite(t_new)) skip = true;
+      ob = obs[i];
+      const double sg = sig[i];
+      s2 = sg * sg;
     }
+    double mh = 0, vh = 1;
+    if (P.lik == GM_LIK_GAUSS_IN_LNA) {
+      vh = 1.0 / (1.0 / vc + 1.0 / s2);
+      mh = vh * (mc / vc + ob / s2);
+    } else {
+      double S0 = 0, S1 = 0, S2 = 0;
+      if (!skip) {
+        tilted_mode(mc, vc, ob, s2, &a, &h0, &shw);
+        // moments about the mode, then shifted
+        const double sc = 1.4142135623730951 * shw;
+        for (int k = sub; k < kGH; k += G) {
+          const double y = sc * ghx[k];
+          const double x = a + y;
+          const double wk = ghw[k] * exp(log_tilted(x, exp(x), mc, vc, ob, s2) - h0);
+          S0 += wk;
+          S1 += wk * y;
+          S2 += wk * y * y;
+        }
+      }
+#pragma unroll
+      for (int off = G / 2; off > 0; off >>= 1) {
+        S0 += __shfl_xor_sync(0xffffffffu, S0, off);
+        S1 += __shfl_xor_sync(0xffffffffu, S1, off);
+        S2 += __shfl_xor_sync(0xffffffffu, S2, off);
+      }
+      if (!skip) {
+        const double m1 = S1 / S0;
+        mh = a + m1;
+        vh = S2 / S0 - m1 * m1;
+      }
+    }
+    if (!star || sub != 0) continue;
+    const double t_new = 1.0 / vh - tc, n_new = mh / vh - ncv;
+    if (!(t_new >= 0) || !isfinite(n_new) || !isfinite(t_new)) skip = true;
     if (skip) {
       atomicAdd(skipped, 1ull);
       continue;
@@ -135,24 +184,87 @@ __global__ void k_site_update(int64_t n, SiteParams P, const double* __restrict_
   __syncthreads();
   if (threadIdx.x == 0) {
     double v = 0;
-    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) v = fmax(v, sh[w]);
+    for (int w = 0; w < kSiteThreads / 32; ++w) v = fmax(v, sh[w]);
     if (!isfinite(v)) atomicOr(flags, kFlagNonFinite);
     part_delta[blockIdx.x] = v;
+    is_last = 0;
+    if (last.ticket) {
+      __threadfence();
+      is_last = atomicAdd(last.ticket, 1ull) == gridDim.x - 1;
+    }
   }
+  __syncthreads();
+  if (!is_last) return;
+  __threadfence();
+  double v = 0;
+  for (int k = threadIdx.x; k < (int)gridDim.x; k += blockDim.x)
+    v = fmax(v, *(volatile double*)(part_delta + k));
+  for (int off = 16; off > 0; off >>= 1) v = fmax(v, __shfl_xor_sync(0xffffffffu, v, off));
+  if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = v;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    double mx = 0;
+    for (int w = 0; w < kSiteThreads / 32; ++w) mx = fmax(mx, sh[w]);
+    last.out[0] = *(volatile unsigned long long*)skipped;
+    last.out[1] = *(volatile unsigned*)flags;
+    last.out[2] = (unsigned long long)__double_as_longlong(mx);
+  }
+}
+
+// Lanes per star: the largest power of two up to 32 that keeps the update
+// within one warp per scheduler (four schedulers per SM; pairs of lanes up to
+// 2.25 warps, where they still beat single lanes: 330 against 379 us a call at
+// 20,000 stars, 615 against 551 us at 50,000).  Calls of 32 / 16 / 8 / 4 / 2 / 1
+// lanes took 82 / 91 / 96 / 117 / 155 / 235 us at 400 stars, 157 / 117 / 102 /
+// 117 / 157 / 242 us at 2,400 and 474 / 350 / 254 / 227 / 233 / 231 us at 10,000.
+static int site_group(int64_t n, int sms) {
+  int g = 32;
+  const int64_t room = (int64_t)sms * 4 * 32;
+  while (g > 1 && n * g > (g == 2 ? 9 * room / 4 : room)) g >>= 1;
+  return g;
+}
+
+// blocks: at most max_blocks; the kernel strides over the rest of the stars
+static int site_blocks(int64_t n, int group, int64_t max_blocks) {
+  return (int)std::min<int64_t>(ceil_div(n * group, kSiteThreads), max_blocks);
+}
+
+static void launch_site(int group, int blocks, cudaStream_t st, int64_t n, const SiteParams& P,
+                        const double* mu, const double* var, const double* obs, const double* sig,
+                        double* tau, double* nu, const double* gh_x, const double* gh_w,
+                        double* part, unsigned long long* skipped, unsigned* flags,
+                        SiteLast last) {
+#define GM_SITE(G)                                                                            \
+  case G:                                                                                     \
+    k_site_update<G><<<blocks, kSiteThreads, 0, st>>>(n, P, mu, var, obs, sig, tau, nu, gh_x, \
+                                                      gh_w, part, skipped, flags, last);      \
+    break
+  switch (group) {
+    GM_SITE(32);
+    GM_SITE(16);
+    GM_SITE(8);
+    GM_SITE(4);
+    GM_SITE(2);
+    default:
+      k_site_update<1><<<blocks, kSiteThreads, 0, st>>>(n, P, mu, var, obs, sig, tau, nu, gh_x,
+                                                        gh_w, part, skipped, flags, last);
+  }
+#undef GM_SITE
 }
 
 gm_status site_update(gm_ctx* c, double* max_delta, int64_t* skipped) {
   const int64_t n = c->n;
   cudaStream_t st = c->stream;
-  const int G = (int)std::min<int64_t>(ceil_div(n, 128), 4 * sm_count(c));
+  const int sms = sm_count(c), group = site_group(n, sms);
+  const int G = site_blocks(n, group, 4 * sms);
   double* part = (double*)dev_alloc(c, (G + 1) * sizeof(double) + sizeof(unsigned long long));
   if (!part) return set_error(c, GM_E_NOMEM, "site partials");
   unsigned long long* cnt = (unsigned long long*)(part + G);
   GM_CUDA_CHECK(c, cudaMemsetAsync(cnt, 0, sizeof(unsigned long long), st));
   SiteParams P{c->cfg.damping, c->cfg.vc_floor, c->cfg.likelihood};
   GM_PROF(c, "k_site_update");
-  k_site_update<<<G, 128, 0, st>>>(n, P, c->mu, c->var, c->obs, c->obs_sigma, c->tau, c->nu,
-                                   c->gh_x, c->gh_wx, part, cnt, c->d_flags);
+  launch_site(group, G, st, n, P, c->mu, c->var, c->obs, c->obs_sigma, c->tau, c->nu, c->gh_x,
+              c->gh_wx, part, cnt, c->d_flags, SiteLast{nullptr, nullptr});
   GM_LAUNCH_CHECK(c);
   double* hp = (double*)c->h_pinned;
   GM_CUDA_CHECK(c, cudaMemcpyAsync(hp, part, (G + 1) * sizeof(double), cudaMemcpyDeviceToHost, st));
@@ -183,33 +295,19 @@ gm_status site_update(gm_ctx* c, double* max_delta, int64_t* skipped) {
 // ---------------------------------------------------------------------------
 constexpr int kNaMaxBlocks = 8192;
 constexpr int64_t kNaMaxStars = 128ll * kNaMaxBlocks;  // 1,048,576
-constexpr int kNaSlots = 2 * kGH + kNaMaxBlocks + 4;   // doubles
+constexpr int kNaSlots = 2 * kGH + kNaMaxBlocks + 6;   // doubles
 constexpr int kNaMaxDevices = 64;
 
 static __device__ __align__(256) double g_na_scratch[kNaSlots];
 
 // Scratch layout (doubles): [0, kGH) nodes, [kGH, 2 kGH) weights * exp(x^2),
-// [2 kGH, 2 kGH + kNaMaxBlocks) per-block maxima, then the skip counter
-// (as an unsigned 64-bit word), the flags word and the reduced maximum.
+// [2 kGH, 2 kGH + kNaMaxBlocks) per-block maxima, then 64-bit words: the skip
+// counter, the flags, the count of finished blocks and the three results.
 // Per device, the scratch address at which the rule was last uploaded.  The
 // address is resolved again on every call, so a module reloaded after a
 // device reset (new address) gets its rule uploaded again instead of a stale
 // pointer being used.
 static double* g_na_ptr[kNaMaxDevices] = {nullptr};
-
-__global__ void k_na_reduce_max(int nb, const double* __restrict__ part, double* __restrict__ out) {
-  __shared__ double sh[32];
-  double v = 0;
-  for (int k = threadIdx.x; k < nb; k += blockDim.x) v = fmax(v, part[k]);
-  for (int off = 16; off > 0; off >>= 1) v = fmax(v, __shfl_xor_sync(0xffffffffu, v, off));
-  if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = v;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double m = 0;
-    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) m = fmax(m, sh[w]);
-    *out = m;
-  }
-}
 
 // Device memory of the current device `dev`, or managed memory.  Memory of
 // another GPU is refused: without peer access the kernel could not read it.
@@ -281,21 +379,26 @@ extern "C" gm_status gm_site_update_noalloc(int64_t n, const double* mu, const d
   double* gh_w = base + kGH;
   double* part = base + 2 * kGH;
   unsigned long long* skipped = (unsigned long long*)(part + kNaMaxBlocks);
-  unsigned* flags = (unsigned*)(part + kNaMaxBlocks + 1);
-  double* maxd = part + kNaMaxBlocks + 2;
-  // the counter and the flags keep the previous call's values: clear them
-  if (cudaMemsetAsync(skipped, 0, 2 * sizeof(double), s) != cudaSuccess) {
+  unsigned* flags = (unsigned*)(skipped + 1);
+  unsigned long long* ticket = skipped + 2;
+  unsigned long long* res = skipped + 3;
+  // the counters keep the previous call's values: clear them
+  if (cudaMemsetAsync(skipped, 0, 3 * sizeof(double), s) != cudaSuccess) {
     cudaGetLastError();
     return GM_E_CUDA;
   }
-  const int G = (int)ceil_div(n, 128);
+  int sms = 0;
+  if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
+    cudaGetLastError();
+    return GM_E_CUDA;
+  }
+  const int group = site_group(n, sms > 0 ? sms : 1);
   SiteParams P{damping, vc_floor, likelihood};
-  k_site_update<<<G, 128, 0, s>>>(n, P, mu, var, obs, obs_sigma, tau, nu, gh_x, gh_w, part,
-                                   skipped, flags);
-  k_na_reduce_max<<<1, 1024, 0, s>>>(G, part, maxd);
+  launch_site(group, site_blocks(n, group, kNaMaxBlocks), s, n, P, mu, var, obs, obs_sigma, tau,
+              nu, gh_x, gh_w, part, skipped, flags, SiteLast{ticket, res});
   if (cudaGetLastError() != cudaSuccess) return GM_E_CUDA;
   unsigned long long h[3];
-  if (cudaMemcpyAsync(h, skipped, 3 * sizeof(double), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
+  if (cudaMemcpyAsync(h, res, 3 * sizeof(double), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
       cudaStreamSynchronize(s) != cudaSuccess) {
     cudaGetLastError();
     return GM_E_CUDA;
