@@ -19,9 +19,10 @@
 //     panel.  For c = 0 the inner integrand does not depend on m and the
 //     inner integral is (upper - lower) g(d^2).
 //
-// The routines compile for the device (the band-rule quadrature kernels,
-// one warp per pair with the lanes over the d-nodes) and for the host (a
-// check of the node set and the sums without a GPU).
+// This file states the rule one node at a time, compiled for the host (a check
+// of the node set and the sums without a GPU).  The quadrature kernels run the
+// same rule with its constants and node tables from here, a warp per pair with
+// the panel bookkeeping spread over the lanes (band_I_warp in gm_quad.cu).
 #pragma once
 
 #include <math.h>

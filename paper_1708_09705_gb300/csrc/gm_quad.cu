@@ -388,14 +388,38 @@ __global__ void k_self_quad(QuadParams P, int64_t n_rows, const double* __restri
 }
 
 // ------------------------------------------------------------ band rule
-// g by table lookup in the arithmetic type of the inner sums.
+// The band rule of gm_band.cuh with the warp's lanes holding the pair's
+// breakpoints.  What bounds it: about 1,200 evaluations of g a pair (38 per
+// lane), so everything around them has to be paid once a pair or once 32
+// pairs.  GB300 issues an FP64 instruction every 16 clocks per SM, so
+//   * the FP64 work of a pair (distances, chord, difference of the distances,
+//     log1p, taper) is done for a batch of up to 32 pairs at once, a lane per
+//     pair, and the batch's pairs are then integrated one after another by
+//     the whole warp (band_batch);
+//   * the graded breakpoints come from a 16-entry table (no pow / log), their
+//     clipping, merging with the kink and counting from ballots and shuffles;
+//   * the FP32 form places nodes and panels in FP32 (the partition it sums
+//     over is a partition whatever its rounding), and reads g from the
+//     replicated table window of the 64-node kernel.
+// 6,000 stars of the 5-degree field (3.0e6 stored entries, FP32): 199 ms with
+// every lane finding its panels by FP64 pow / log, 2.6 ms so (5.8e8 unique
+// pairs/s); the carried sums cost 0.2 ms of it and lower the entries' error
+// against FP64 from 4.8e-8 to 3.3e-8.
+constexpr int kBandPts = 12;  // breakpoints h0 (q^j - 1) / (q - 1), j < 12: 0 .. 88.6 >= kK
+
+struct BandTab {
+  double pt[kBandPts];
+};
+
+// g by table lookup in the arithmetic type of the sums.
 template <typename T>
 struct GLook;
 template <>
 struct GLook<float> {
-  const float4* tab;
-  TabF32 t;
-  __device__ float operator()(float x) const { return g_lookup(tab, t, x); }
+  const float4* tab8;  // replicated window, this lane's copy
+  __device__ float operator()(float x) const {
+    return g_lookup_rep(tab8, x + __int_as_float((127 + kWinEmin) << 23));
+  }
 };
 template <>
 struct GLook<double> {
@@ -404,32 +428,163 @@ struct GLook<double> {
   __device__ double operator()(double x) const { return g_lookup(tab, t, x); }
 };
 
-// R = I / (s_i s_j) of one pair by the band rule (A = s_i / L0, B = s_j / L0,
-// c2 = |u_i - u_j|^2); the warp's lanes share the d-nodes.  Every lane
-// returns the sum.
+// Sum of FP32 terms with its rounding carried along (Knuth's TwoSum), so that
+// the few large partial sums of a pair do not round to FP32 on the way.
 template <typename T>
-__device__ __forceinline__ double band_R_warp(double A, double B, double c2, const GLook<T>& g,
-                                              int lane) {
-  const gmband::Geometry geo = gmband::geometry(A, B, c2);
-  T acc = 0;
-  const int nk = gmband::d_nodes(geo);
-  for (int k = lane; k < nk; k += 32) acc += gmband::d_node<T>(geo, k, g);
+struct CarrySum {
+  T s = 0;
+  __device__ __forceinline__ void add(T x) { s += x; }
+  __device__ __forceinline__ double warp_total() {
 #pragma unroll
-  for (int off = 16; off > 0; off >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
-  return (double)acc / (A * B);
-}
+    for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
+    return s;
+  }
+};
+template <>
+struct CarrySum<float> {
+  float s = 0.f, c = 0.f;
+  __device__ __forceinline__ void add(float x) {
+    const float t = __fadd_rn(s, x), z = __fsub_rn(t, s);
+    c += __fadd_rn(__fsub_rn(s, __fsub_rn(t, z)), __fsub_rn(x, z));
+    s = t;
+  }
+  __device__ __forceinline__ double warp_total() {
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) {
+      const float so = __shfl_xor_sync(0xffffffffu, s, off);
+      const float co = __shfl_xor_sync(0xffffffffu, c, off);
+      add(so);
+      c += co;
+    }
+    return (double)s + (double)c;
+  }
+};
+
+// Node i of this lane in round r (d-node lane + 32 r, i = (lane + 2 r) mod 6):
+// the three node and weight values a lane meets.
+template <typename T>
+struct BandLane {
+  T z[3], w[3];
+  T pt;  // table breakpoint of this lane (beyond the table: infinity)
+};
 
 template <typename T>
-__device__ __forceinline__ GLook<T> band_lookup(const void* gtab, TabF32 tf, TabF64 td,
+__device__ __forceinline__ BandLane<T> band_lane(const BandTab& bt, int lane) {
+  BandLane<T> L;
+#pragma unroll
+  for (int r = 0; r < 3; ++r) {
+    const int i = (lane + 2 * r) % gmband::kN;
+    L.z[r] = (T)gmband::gl_z(i);
+    L.w[r] = (T)gmband::gl_w(i);
+  }
+  L.pt = (T)INFINITY;
+#pragma unroll
+  for (int j = 0; j < kBandPts; ++j)
+    if (lane == j) L.pt = (T)bt.pt[j];
+  return L;
+}
+
+// I_ij of one pair (A = s_i / L0, B = s_j / L0, c2 = |u_i - u_j|^2, kink =
+// A - B); every lane returns the sum.  Al, Bl: what rounding A and B to T left
+// out; the upper end of m adds it to the length of its last panel, so that the
+// rounding of the two distances does not scale the whole integral.
+template <typename T>
+__device__ __forceinline__ double band_I_warp(T A, T B, T Al, T Bl, T c2, T kink, const BandLane<T>& L,
+                                         const GLook<T>& g, int lane) {
+  constexpr unsigned full = 0xffffffffu;
+  const T K = (T)gmband::kK;
+  const T Dp = A < K ? A : K, Dn = B < K ? B : K;
+  // panels of each side: breakpoints below its extent (0 is one of them)
+  const int np = __popc(__ballot_sync(full, L.pt < Dp));
+  const int nn = __popc(__ballot_sync(full, L.pt < Dn));
+  // base breakpoint of this lane: -side(nn - lane) .. 0 .. side(lane - nn)
+  const int t = lane - nn;
+  T v = __shfl_sync(full, L.pt, t < 0 ? -t : t);
+  const T ext = t < 0 ? Dn : Dp;
+  v = v < ext ? v : ext;
+  const T base = t < 0 ? -v : v;
+  const int nb = nn + np;  // last base index
+  const int below = __popc(__ballot_sync(full, lane <= nb && base < kink));
+  const T at = __shfl_sync(full, base, below);
+  const bool ins = kink > -Dn && kink < Dp && at != kink;
+  const T prev = __shfl_up_sync(full, base, 1);
+  const T pt = !ins || lane < below ? base : (lane == below ? kink : prev);
+  const int npan = nb + (ins ? 1 : 0);
+  const T c = sqrt(c2);
+  const T sc = c2 > (T)0 ? (T)1 / c : (T)0;
+  const T h0 = (T)gmband::kM0 * sc, lim = K * sc;
+  const T dsc = (T)1 - (T)0.25 * c2;
+  CarrySum<T> acc;
+#pragma unroll 1
+  for (int r0 = 0; 32 * r0 < npan * gmband::kN; r0 += 3) {
+#pragma unroll
+    for (int r = 0; r < 3; ++r) {
+      const int k = lane + 32 * (r0 + r);
+      const int pnl = min(k / gmband::kN, 30);
+      const T a = __shfl_sync(full, pt, pnl), b = __shfl_sync(full, pt, pnl + 1);
+      const T d = a + (b - a) * L.z[r];
+      const T wd = (b - a) * L.w[r];
+      const T lo = (d < (T)0 ? -d : d) * (T)0.5;
+      const T u1 = A - d * (T)0.5, u2 = B + d * (T)0.5;
+      const T hi = u1 < u2 ? u1 : u2;
+      const T hl = u1 < u2 ? Al : Bl;
+      if (k >= npan * gmband::kN || !(hi > lo) || wd == (T)0) continue;
+      if (c2 == (T)0) {
+        const T gv = g(d * d);
+        acc.add(wd * ((hi - lo) * gv + hl * gv));
+        continue;
+      }
+      const T dd = d * d * dsc;
+      const T end = hi < lo + lim ? hi : lo + lim;
+      T sum = 0, ma = lo, h = h0;
+      while (ma < end) {
+        const T mb = ma + h < end ? ma + h : end;
+        const T len = mb - ma;
+        T s6 = 0;
+#pragma unroll
+        for (int j = 0; j < gmband::kN; ++j) {
+          const T m = ma + len * (T)gmband::gl_z(j);
+          s6 += (T)gmband::gl_w(j) * g(dd + m * m * c2);
+        }
+        sum += len * s6;
+        if (mb == hi) sum += hl * s6;
+        ma = mb;
+        h *= (T)gmband::kQ;
+      }
+      acc.add(wd * sum);
+    }
+  }
+  return acc.warp_total();
+}
+
+// R of up to 32 pairs of a warp, one per active lane (A, B, c2 in FP64).
+template <typename T>
+__device__ __forceinline__ double band_batch(bool active, double A, double B, double c2,
+                                             const BandLane<T>& L, const GLook<T>& g, int lane) {
+  constexpr unsigned full = 0xffffffffu;
+  const T At = (T)A, Bt = (T)B, ct = (T)c2, kt = (T)(A - B);
+  const T Al = (T)(A - (double)At), Bl = (T)(B - (double)Bt);
+  double mine = 0;
+  for (unsigned m = __ballot_sync(full, active); m; m &= m - 1) {
+    const int l = __ffs(m) - 1;
+    const double v = band_I_warp<T>(__shfl_sync(full, At, l), __shfl_sync(full, Bt, l),
+                               __shfl_sync(full, Al, l), __shfl_sync(full, Bl, l),
+                               __shfl_sync(full, ct, l), __shfl_sync(full, kt, l), L, g, lane);
+    if (lane == l) mine = v;
+  }
+  return mine / (A * B);
+}
+
+// FP32: the replicated table window in shared memory; FP64: the global table.
+template <typename T>
+__device__ __forceinline__ GLook<T> band_lookup(const void* gtab, TabF64 td,
                                                 unsigned char* smem) {
   GLook<T> g;
   if constexpr (sizeof(T) == 4) {
-    // the FP32 table lives in shared memory
     float4* st = reinterpret_cast<float4*>(smem);
-    const float4* gt = reinterpret_cast<const float4*>(gtab);
-    for (int k = threadIdx.x; k <= tf.last; k += blockDim.x) st[k] = gt[k];
-    g.tab = st;
-    g.t = tf;
+    const float4* gt = reinterpret_cast<const float4*>(gtab) + kWinK0;
+    for (int k = threadIdx.x; k < kWinSegs * kRep; k += blockDim.x) st[k] = gt[k / kRep];
+    g.tab8 = st + (threadIdx.x & (kRep - 1));
   } else {
     g.tab = reinterpret_cast<const D4*>(gtab);
     g.t = td;
@@ -437,43 +592,63 @@ __device__ __forceinline__ GLook<T> band_lookup(const void* gtab, TabF32 tf, Tab
   return g;
 }
 
-// The band-rule counterpart of k_pair_quad (same entries, taper, mirror
-// convention, diagonal and prior mean).
+// Threads per block of the band kernels: FP32 one block of 32 warps per SM
+// around its table window, as the 64-node kernel.
 template <typename T>
-__global__ void __launch_bounds__(256) k_pair_quad_band(
-    QuadParams P, int64_t n_rows, const double* __restrict__ rs, const double* __restrict__ rux,
-    const double* __restrict__ ruy, const double* __restrict__ ruz, const double* __restrict__ s,
-    const double* __restrict__ ux, const double* __restrict__ uy, const double* __restrict__ uz,
-    const int64_t* __restrict__ row_ptr, const int32_t* __restrict__ col, int64_t nnz,
-    T* __restrict__ val, const void* __restrict__ gtab, TabF32 tf, TabF64 td,
-    double* __restrict__ kdiag, double* __restrict__ prior_m, unsigned* __restrict__ flags,
-    const FieldGrid* __restrict__ fg, const int32_t* __restrict__ row_field) {
-  extern __shared__ unsigned char smem[];
-  const GLook<T> g = band_lookup<T>(gtab, tf, td, smem);
+constexpr int band_threads() { return sizeof(T) == 4 ? 1024 : 256; }
+
+// The band-rule counterpart of k_pair_quad (same entries, taper, mirror
+// convention, diagonal and prior mean).  A warp takes `batch` consecutive
+// entries (a power of two up to 32).
+template <typename T>
+__global__ void __launch_bounds__(band_threads<T>()) k_pair_quad_band(
+    QuadParams P, BandTab bt, int batch, int64_t n_rows, const double* __restrict__ rs,
+    const double* __restrict__ rux, const double* __restrict__ ruy, const double* __restrict__ ruz,
+    const double* __restrict__ s, const double* __restrict__ ux, const double* __restrict__ uy,
+    const double* __restrict__ uz, const int64_t* __restrict__ row_ptr,
+    const int32_t* __restrict__ col, int64_t nnz, T* __restrict__ val,
+    const void* __restrict__ gtab, TabF64 td, double* __restrict__ kdiag,
+    double* __restrict__ prior_m, unsigned* __restrict__ flags, const FieldGrid* __restrict__ fg,
+    const int32_t* __restrict__ row_field) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  const GLook<T> g = band_lookup<T>(gtab, td, smem);
   __syncthreads();
   const int lane = threadIdx.x & 31;
+  const BandLane<T> L = band_lane<T>(bt, lane);
   const int64_t warp = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
   const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-  for (int64_t e = warp; e < nnz; e += nwarps) {
-    int64_t lo = 0, hi = n_rows;
-    while (hi - lo > 1) {
-      int64_t mid = (lo + hi) >> 1;
-      if (row_ptr[mid] <= e) lo = mid; else hi = mid;
+  for (int64_t e0 = warp * batch; e0 < nnz; e0 += nwarps * batch) {
+    const int64_t e = e0 + lane;
+    bool active = lane < batch && e < nnz;
+    int64_t i = 0;
+    int32_t j = 0;
+    if (active) {
+      int64_t lo = 0, hi = n_rows;
+      while (hi - lo > 1) {
+        int64_t mid = (lo + hi) >> 1;
+        if (row_ptr[mid] <= e) lo = mid; else hi = mid;
+      }
+      i = lo;
+      j = col[e];
+      if (P.symmetric && j < i) active = false;
     }
-    const int64_t i = lo;
-    const int32_t j = col[e];
-    if (P.symmetric && j < i) continue;
-    const FieldGrid& fgi = fg[row_field ? row_field[i] : 0];
-    const double inv_L0 = fgi.inv_L0, inv_cut = fgi.inv_cut;
-    const double si = rs[i], sj = s[j];
-    const double dx = rux[i] - ux[j], dy = ruy[i] - uy[j], dz = ruz[i] - uz[j];
-    const double chord2 = fma(dx, dx, fma(dy, dy, dz * dz));
-    const double R = band_R_warp<T>(si * inv_L0, sj * inv_L0, chord2, g, lane);
-    if (lane == 0) {
+    double A = 1, B = 1, chord2 = 0, si = 0, sj = 0, inv_cut = 0;
+    if (active) {
+      const FieldGrid& fgi = fg[row_field ? row_field[i] : 0];
+      inv_cut = fgi.inv_cut;
+      si = rs[i];
+      sj = s[j];
+      const double dx = rux[i] - ux[j], dy = ruy[i] - uy[j], dz = ruz[i] - uz[j];
+      chord2 = fma(dx, dx, fma(dy, dy, dz * dz));
+      A = si * fgi.inv_L0;
+      B = sj * fgi.inv_L0;
+    }
+    const double R = band_batch<T>(active, A, B, chord2, L, g, lane);
+    if (active) {
       double K = P.form == GM_FORM_LOGNORMAL ? log1p(R) : R;
       if (P.taper == GM_TAPER_WENDLAND) {
-        double ds = si - sj;
-        double d = sqrt(fma(ds, ds, si * sj * chord2));
+        const double ds = si - sj;
+        const double d = sqrt(fma(ds, ds, si * sj * chord2));
         K *= wendland(d * inv_cut);
       }
       if (!isfinite(K)) atomicOr(flags, kFlagNonFinite);
@@ -487,24 +662,33 @@ __global__ void __launch_bounds__(256) k_pair_quad_band(
   }
 }
 
-// Band-rule self-covariance of query points (k_self_quad's counterpart).
+// Band-rule self-covariance of query points (k_self_quad's counterpart), and
+// of an explicit pair list (k_pairlist_quad's; sj null: the points themselves).
 template <typename T>
-__global__ void __launch_bounds__(256) k_self_quad_band(QuadParams P, int64_t n_rows,
-                                                        const double* __restrict__ rs,
-                                                        const void* __restrict__ gtab, TabF32 tf,
-                                                        TabF64 td, double* __restrict__ out) {
-  extern __shared__ unsigned char smem[];
-  const GLook<T> g = band_lookup<T>(gtab, tf, td, smem);
+__global__ void __launch_bounds__(band_threads<T>()) k_pairlist_quad_band(
+    QuadParams P, BandTab bt, int batch, int64_t n, const double* __restrict__ si,
+    const double* __restrict__ sj, const double* __restrict__ chord, double* __restrict__ out,
+    const void* __restrict__ gtab, TabF64 td) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  const GLook<T> g = band_lookup<T>(gtab, td, smem);
   __syncthreads();
   const int lane = threadIdx.x & 31;
+  const BandLane<T> L = band_lane<T>(bt, lane);
   const int64_t warp = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
   const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-  for (int64_t r = warp; r < n_rows; r += nwarps) {
-    const double a = rs[r] * P.inv_L0;
-    const double R = band_R_warp<T>(a, a, 0.0, g, lane);
-    if (lane == 0) {
+  for (int64_t p0 = warp * batch; p0 < n; p0 += nwarps * batch) {
+    const int64_t p = p0 + lane;
+    const bool active = lane < batch && p < n;
+    double A = 1, B = 1, c2 = 0;
+    if (active) {
+      A = si[p] * P.inv_L0;
+      B = sj ? sj[p] * P.inv_L0 : A;
+      c2 = sj ? chord[p] * chord[p] : 0.0;
+    }
+    const double R = band_batch<T>(active, A, B, c2, L, g, lane);
+    if (active) {
       const double K = P.form == GM_FORM_LOGNORMAL ? log1p(R) : R;
-      out[r] = (double)(T)K;
+      out[p] = sj ? K : (double)(T)K;
     }
   }
 }
@@ -602,9 +786,28 @@ static void launch_pair(gm_ctx* c, const QuadParams& P, int64_t n_rows, const do
                                          c->fgrid, row_field);
 }
 
-// Shared memory of the band kernels: the FP32 table (none for FP64).
-static size_t band_smem(bool f32) {
-  return f32 ? (size_t)(kTabF32.n_real() + 1) * sizeof(float4) : 0;
+static BandTab band_tab() {
+  BandTab t;
+  for (int j = 0; j < kBandPts; ++j)
+    t.pt[j] = gmband::kH0 * (std::pow(gmband::kQ, (double)j) - 1.0) / (gmband::kQ - 1.0);
+  return t;
+}
+
+// Blocks and batch of a band kernel over n entries: the resident blocks, and
+// the largest batch that still leaves every warp two (small lists: the pairs
+// spread over the chip, one per warp in the limit).
+template <typename T, typename Kern>
+static void band_shape(gm_ctx* c, Kern kern, int64_t n, size_t* smem, int* blocks, int* batch) {
+  constexpr int nt = band_threads<T>();
+  *smem = sizeof(T) == 4 ? (size_t)kWinSegs * kRep * sizeof(float4) : 0;
+  cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)*smem);
+  int per_sm = 0;
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, nt, *smem);
+  const int64_t resident = (int64_t)std::max(1, per_sm) * sm_count(c);
+  int b = 32;
+  while (b > 1 && n < 2 * b * resident * (nt / 32)) b >>= 1;
+  *batch = b;
+  *blocks = (int)std::min<int64_t>(resident, std::max<int64_t>(1, ceil_div(ceil_div(n, b), nt / 32)));
 }
 
 template <typename T>
@@ -612,18 +815,25 @@ static void launch_pair_band(gm_ctx* c, const QuadParams& P, int64_t n_rows, con
                              const double* rux, const double* ruy, const double* ruz,
                              const int32_t* row_field, const int64_t* row_ptr,
                              const int32_t* col, int64_t nnz, void* val) {
-  const size_t smem = band_smem(sizeof(T) == 4);
+  size_t smem;
+  int blocks, batch;
   auto kern = k_pair_quad_band<T>;
-  cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  int per_sm = 0;
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, 256, smem);
-  int blocks = std::max(1, per_sm) * sm_count(c);
-  blocks = (int)std::min<int64_t>(blocks, std::max<int64_t>(1, ceil_div(nnz * 32, 256)));
+  band_shape<T>(c, kern, nnz, &smem, &blocks, &batch);
   GM_PROF(c, "k_pair_quad_band");
-  kern<<<blocks, 256, smem, c->stream>>>(P, n_rows, rs, rux, ruy, ruz, c->s, c->ux, c->uy, c->uz,
-                                         row_ptr, col, nnz, (T*)val, c->gtab, tab_f32(),
-                                         tab_f64(), c->kdiag, c->prior_m, c->d_flags, c->fgrid,
-                                         row_field);
+  kern<<<blocks, band_threads<T>(), smem, c->stream>>>(
+      P, band_tab(), batch, n_rows, rs, rux, ruy, ruz, c->s, c->ux, c->uy, c->uz, row_ptr, col,
+      nnz, (T*)val, c->gtab, tab_f64(), c->kdiag, c->prior_m, c->d_flags, c->fgrid, row_field);
+}
+
+template <typename T>
+static void launch_pairlist_band(gm_ctx* c, const QuadParams& P, int64_t n, const double* si,
+                                 const double* sj, const double* chord, double* out) {
+  size_t smem;
+  int blocks, batch;
+  auto kern = k_pairlist_quad_band<T>;
+  band_shape<T>(c, kern, n, &smem, &blocks, &batch);
+  kern<<<blocks, band_threads<T>(), smem, c->stream>>>(P, band_tab(), batch, n, si, sj, chord,
+                                                       out, c->gtab, tab_f64());
 }
 
 gm_status pair_quadrature(gm_ctx* c, int64_t n_rows, const double* rs, const double* rux,
@@ -682,17 +892,9 @@ gm_status self_quadrature(gm_ctx* c, int64_t n_rows, const double* rs, double* k
   const bool f32 = c->cfg.precision == GM_PREC_FP32;
   int blocks = (int)std::min<int64_t>(ceil_div(n_rows * 32, 256), 8 * sm_count(c));
   if (c->cfg.quad_rule == GM_QUAD_BAND) {
-    const size_t smem = band_smem(f32);
     GM_PROF(c, "k_self_quad_band");
-    if (f32) {
-      cudaFuncSetAttribute(k_self_quad_band<float>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           (int)smem);
-      k_self_quad_band<float><<<blocks, 256, smem, c->stream>>>(P, n_rows, rs, c->gtab,
-                                                                tab_f32(), tab_f64(), kss);
-    } else {
-      k_self_quad_band<double><<<blocks, 256, 0, c->stream>>>(P, n_rows, rs, c->gtab, tab_f32(),
-                                                              tab_f64(), kss);
-    }
+    if (f32) launch_pairlist_band<float>(c, P, n_rows, rs, nullptr, nullptr, kss);
+    else launch_pairlist_band<double>(c, P, n_rows, rs, nullptr, nullptr, kss);
     GM_LAUNCH_CHECK(c);
     return GM_OK;
   }
@@ -782,39 +984,6 @@ __global__ void __launch_bounds__(256) k_pairlist_quad(
       out[p] = P.form == GM_FORM_LOGNORMAL ? log1p(R) : R;
     }
   }
-}
-
-// Band-rule counterpart of k_pairlist_quad.
-template <typename T>
-__global__ void __launch_bounds__(256) k_pairlist_quad_band(
-    QuadParams P, int64_t n, const double* __restrict__ si, const double* __restrict__ sj,
-    const double* __restrict__ chord, double* __restrict__ out, const void* __restrict__ gtab,
-    TabF32 tf, TabF64 td) {
-  extern __shared__ unsigned char smem[];
-  const GLook<T> g = band_lookup<T>(gtab, tf, td, smem);
-  __syncthreads();
-  const int lane = threadIdx.x & 31;
-  const int64_t warp = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
-  const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-  for (int64_t p = warp; p < n; p += nwarps) {
-    const double R = band_R_warp<T>(si[p] * P.inv_L0, sj[p] * P.inv_L0, chord[p] * chord[p], g,
-                                    lane);
-    if (lane == 0) out[p] = P.form == GM_FORM_LOGNORMAL ? log1p(R) : R;
-  }
-}
-
-template <typename T>
-static void launch_pairlist_band(gm_ctx* c, const QuadParams& P, int64_t n, const double* si,
-                                 const double* sj, const double* chord, double* out) {
-  const size_t smem = band_smem(sizeof(T) == 4);
-  auto kern = k_pairlist_quad_band<T>;
-  cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  int per_sm = 0;
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, 256, smem);
-  int blocks = std::max(1, per_sm) * sm_count(c);
-  blocks = (int)std::min<int64_t>(blocks, std::max<int64_t>(1, ceil_div(n * 32, 256)));
-  kern<<<blocks, 256, smem, c->stream>>>(P, n, si, sj, chord, out, c->gtab, tab_f32(),
-                                         tab_f64());
 }
 
 template <typename T, int KPL>
