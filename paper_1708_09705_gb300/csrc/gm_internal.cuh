@@ -144,6 +144,7 @@ struct gm_ctx {
   double* gh_wx = nullptr;     // weights * exp(x^2)
   double* phi_pts = nullptr;   // phi at table points (hyperparameter-free)
   void* gtab = nullptr;        // cubic coefficients of g (float4 / double4)
+  void* gtab_df = nullptr;     // FP64 contexts: the same cubics in pairs of floats
   double gtab_sigma2 = -1;
   int gtab_form = -1;
 

@@ -24,7 +24,6 @@
 #include <algorithm>
 #include <cmath>
 #include <cstring>
-#include <type_traits>
 #include <vector>
 
 #include "gm_band.cuh"
@@ -192,42 +191,35 @@ struct QuadParams {
   int symmetric;
 };
 
-// One warp per CSR entry (i, j): lanes own the nodes q' of sightline j,
-// loop over the nodes q of sightline i, and the warp sums the products.
+// FP32 form.  One warp per CSR entry (i, j): lanes own the nodes q' of sightline
+// j, loop over the nodes q of sightline i, and the warp sums the products.
 // In symmetric mode entries with j < i are left for k_mirror.
-// Threads per block of the pair kernel: the FP32 form runs one block of 32
-// warps per SM around its replicated table (at most 64 registers a thread).
-template <typename T, int KPL>
-constexpr int pair_threads() { return sizeof(T) == 4 ? (KPL <= 2 ? 1024 : 512) : 256; }
+// One block of 32 warps per SM around the replicated table (at most 64
+// registers a thread).
+template <int KPL>
+constexpr int pair_threads() { return KPL <= 2 ? 1024 : 512; }
 
-template <typename T, int KPL>
-__global__ void __launch_bounds__(pair_threads<T, KPL>()) k_pair_quad(
+template <int KPL>
+__global__ void __launch_bounds__(pair_threads<KPL>()) k_pair_quad(
     QuadParams P, int64_t n_rows, const double* __restrict__ rs, const double* __restrict__ rux,
     const double* __restrict__ ruy, const double* __restrict__ ruz, const double* __restrict__ s,
     const double* __restrict__ ux, const double* __restrict__ uy, const double* __restrict__ uz,
     const int64_t* __restrict__ row_ptr, const int32_t* __restrict__ col, int64_t nnz,
-    T* __restrict__ val, const double* __restrict__ gl_zeta, const double* __restrict__ gl_w,
-    const void* __restrict__ gtab, TabF32 tf, TabF64 td, double* __restrict__ kdiag,
-    double* __restrict__ prior_m, unsigned* __restrict__ flags, const FieldGrid* __restrict__ fg,
+    float* __restrict__ val, const double* __restrict__ gl_zeta, const double* __restrict__ gl_w,
+    const float4* __restrict__ gtab, double* __restrict__ kdiag, double* __restrict__ prior_m,
+    unsigned* __restrict__ flags, const FieldGrid* __restrict__ fg,
     const int32_t* __restrict__ row_field) {
-  extern __shared__ unsigned char smem[];
-  typedef typename std::conditional<sizeof(T) == 4, float4, D4>::type T4;
-  T* zq = reinterpret_cast<T*>(smem);
-  T* wq = zq + kMaxNodes;
-  const T4* tab;
+  extern __shared__ __align__(16) unsigned char smem[];
+  float* zq = reinterpret_cast<float*>(smem);
+  float* wq = zq + kMaxNodes;
   const int lane = threadIdx.x & 31;
-  if (sizeof(T) == 4) {
-    // the FP32 table window lives in shared memory, kRep copies per segment
-    float4* st = reinterpret_cast<float4*>(smem + 2 * kMaxNodes * sizeof(T));
-    const float4* gt = reinterpret_cast<const float4*>(gtab) + kWinK0;
-    for (int k = threadIdx.x; k < kWinSegs * kRep; k += blockDim.x) st[k] = gt[k / kRep];
-    tab = reinterpret_cast<const T4*>(st + (lane & (kRep - 1)));
-  } else {
-    tab = reinterpret_cast<const T4*>(gtab);
-  }
+  // the table window lives in shared memory, kRep copies per segment
+  float4* st = reinterpret_cast<float4*>(smem + 2 * kMaxNodes * sizeof(float));
+  for (int k = threadIdx.x; k < kWinSegs * kRep; k += blockDim.x) st[k] = gtab[kWinK0 + k / kRep];
+  const float4* tab = st + (lane & (kRep - 1));
   for (int q = threadIdx.x; q < P.Q; q += blockDim.x) {
-    zq[q] = (T)gl_zeta[q];
-    wq[q] = (T)gl_w[q];
+    zq[q] = (float)gl_zeta[q];
+    wq[q] = (float)gl_w[q];
   }
   __syncthreads();
 
@@ -248,67 +240,45 @@ __global__ void __launch_bounds__(pair_threads<T, KPL>()) k_pair_quad(
     const double si = rs[i], sj = s[j];
     const double dx = rux[i] - ux[j], dy = ruy[i] - uy[j], dz = ruz[i] - uz[j];
     const double chord2 = fma(dx, dx, fma(dy, dy, dz * dz));
-    const T a = (T)(si * inv_L0), b = (T)(sj * inv_L0), c2 = (T)chord2;
+    const float a = (float)(si * inv_L0), b = (float)(sj * inv_L0), c2 = (float)chord2;
     // this lane's nodes on sightline j
-    T tp[KPL], ctp[KPL], wp[KPL];
+    float tp[KPL], ctp[KPL], wp[KPL];
 #pragma unroll
     for (int k = 0; k < KPL; ++k) {
       int q = lane + 32 * k;
       bool ok = q < P.Q;
-      tp[k] = ok ? b * zq[q] : (T)0;
+      tp[k] = ok ? b * zq[q] : 0.f;
       ctp[k] = c2 * tp[k];
-      wp[k] = ok ? wq[q] : (T)0;
+      wp[k] = ok ? wq[q] : 0.f;
     }
-    T acc = 0;
+    float acc = 0;
     for (int q = 0; q < P.Q; ++q) {
-      const T t = a * zq[q];
-      T inner = 0;
+      const float t = a * zq[q];
+      float inner = 0;
 #pragma unroll
       for (int k = 0; k < KPL; ++k) {
-        T d = t - tp[k];
-        T gv;
-        if (sizeof(T) == 4) {
-          // x >= 2^kWinEmin by construction: the window's floor is added
-          const float x = fmaf((float)d, (float)d,
-                               fmaf((float)t, (float)ctp[k], __int_as_float((127 + kWinEmin) << 23)));
-          gv = (T)g_lookup_rep(reinterpret_cast<const float4*>(tab), x);
-        } else {
-          const T x = d * d + t * ctp[k];
-          gv = (T)g_lookup(reinterpret_cast<const D4*>(tab), td, (double)x);
-        }
-        inner += wp[k] * gv;
+        const float d = t - tp[k];
+        // x >= 2^kWinEmin by construction: the window's floor is added
+        const float x = fmaf(d, d, fmaf(t, ctp[k], __int_as_float((127 + kWinEmin) << 23)));
+        inner += wp[k] * g_lookup_rep(tab, x);
       }
       acc += wq[q] * inner;
     }
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
     if (lane == 0) {
-      T K;
-      if (sizeof(T) == 4) {
-        // FP32 form: the entry's own arithmetic in FP32 too (GB300's FP64
-        // pipe is narrow; per-pair FP64 work, not the node sum, bounded this
-        // kernel): log1p and the taper to ~1e-7 relative
-        const float R = (float)acc;
-        float Kf = P.form == GM_FORM_LOGNORMAL ? log1pf(R) : R;
-        if (P.taper == GM_TAPER_WENDLAND) {
-          // the difference of the distances in FP64: it cancels, and the
-          // taper near the cutoff amplifies its error
-          const float ds = (float)(si - sj);
-          const float d = sqrtf(fmaf(ds, ds, (float)si * (float)sj * (float)c2));
-          Kf *= wendland_f(d * (float)inv_cut);
-        }
-        K = (T)Kf;
-      } else {
-        const double R = (double)acc;
-        double Kd = P.form == GM_FORM_LOGNORMAL ? log1p(R) : R;
-        if (P.taper == GM_TAPER_WENDLAND) {
-          const double ds = si - sj;
-          const double d = sqrt(fma(ds, ds, si * sj * chord2));
-          Kd *= wendland(d * inv_cut);
-        }
-        K = (T)Kd;
+      // the entry's own arithmetic in FP32 too (GB300's FP64 pipe is narrow;
+      // per-pair FP64 work, not the node sum, bounded this kernel): log1p and
+      // the taper to ~1e-7 relative
+      float K = P.form == GM_FORM_LOGNORMAL ? log1pf(acc) : acc;
+      if (P.taper == GM_TAPER_WENDLAND) {
+        // the difference of the distances in FP64: it cancels, and the
+        // taper near the cutoff amplifies its error
+        const float ds = (float)(si - sj);
+        const float d = sqrtf(fmaf(ds, ds, (float)si * (float)sj * c2));
+        K *= wendland_f(d * (float)inv_cut);
       }
-      if (!isfinite((double)K)) atomicOr(flags, kFlagNonFinite);
+      if (!isfinite(K)) atomicOr(flags, kFlagNonFinite);
       val[e] = K;
       if (P.symmetric && j == i) {
         kdiag[i] = (double)K;
@@ -341,48 +311,41 @@ __global__ void k_mirror(int64_t n, const int64_t* __restrict__ row_ptr,
   }
 }
 
-// Self-covariance k_qq of query points (FP64, same rule as the diagonal).
-template <typename T, int KPL>
+// Self-covariance k_qq of query points (FP32 form, same rule as the diagonal).
+template <int KPL>
 __global__ void k_self_quad(QuadParams P, int64_t n_rows, const double* __restrict__ rs,
                             const double* __restrict__ gl_zeta, const double* __restrict__ gl_w,
-                            const void* __restrict__ gtab, TabF32 tf, TabF64 td,
-                            double* __restrict__ out) {
+                            const void* __restrict__ gtab, TabF32 tf, double* __restrict__ out) {
   const int lane = threadIdx.x & 31;
   const int64_t warp = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
   const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
   for (int64_t r = warp; r < n_rows; r += nwarps) {
-    const T a = (T)(rs[r] * P.inv_L0);
-    T tp[KPL], wp[KPL];
+    const float a = (float)(rs[r] * P.inv_L0);
+    float tp[KPL], wp[KPL];
 #pragma unroll
     for (int k = 0; k < KPL; ++k) {
       int q = lane + 32 * k;
       bool ok = q < P.Q;
-      tp[k] = ok ? a * (T)gl_zeta[q] : (T)0;
-      wp[k] = ok ? (T)gl_w[q] : (T)0;
+      tp[k] = ok ? a * (float)gl_zeta[q] : 0.f;
+      wp[k] = ok ? (float)gl_w[q] : 0.f;
     }
-    T acc = 0;
+    float acc = 0;
     for (int q = 0; q < P.Q; ++q) {
-      const T t = a * (T)gl_zeta[q];
-      T inner = 0;
+      const float t = a * (float)gl_zeta[q];
+      float inner = 0;
 #pragma unroll
       for (int k = 0; k < KPL; ++k) {
-        T d = t - tp[k];
-        T x = d * d;
-        T gv;
-        if (sizeof(T) == 4)
-          gv = (T)g_lookup(reinterpret_cast<const float4*>(gtab), tf, (float)x);
-        else
-          gv = (T)g_lookup(reinterpret_cast<const D4*>(gtab), td, (double)x);
-        inner += wp[k] * gv;
+        const float d = t - tp[k];
+        inner += wp[k] * g_lookup(reinterpret_cast<const float4*>(gtab), tf, d * d);
       }
-      acc += (T)gl_w[q] * inner;
+      acc += (float)gl_w[q] * inner;
     }
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
     if (lane == 0) {
       double R = (double)acc;
       double K = P.form == GM_FORM_LOGNORMAL ? log1p(R) : R;
-      out[r] = (double)(T)K;
+      out[r] = (double)(float)K;
     }
   }
 }
@@ -557,64 +520,276 @@ __device__ __forceinline__ double band_I_warp(T A, T B, T Al, T Bl, T c2, T kink
   return acc.warp_total();
 }
 
-// R of up to 32 pairs of a warp, one per active lane (A, B, c2 in FP64).
+// Node rules.  A rule integrates up to 32 pairs of a warp, one per active lane
+// (A = s_i / L0, B = s_j / L0 and c2 in FP64): the warp takes the active lanes'
+// pairs one after another.  Val is the type of the stored entries.
 template <typename T>
-__device__ __forceinline__ double band_batch(bool active, double A, double B, double c2,
-                                             const BandLane<T>& L, const GLook<T>& g, int lane) {
-  constexpr unsigned full = 0xffffffffu;
-  const T At = (T)A, Bt = (T)B, ct = (T)c2, kt = (T)(A - B);
-  const T Al = (T)(A - (double)At), Bl = (T)(B - (double)Bt);
-  double mine = 0;
-  for (unsigned m = __ballot_sync(full, active); m; m &= m - 1) {
-    const int l = __ffs(m) - 1;
-    const double v = band_I_warp<T>(__shfl_sync(full, At, l), __shfl_sync(full, Bt, l),
-                               __shfl_sync(full, Al, l), __shfl_sync(full, Bl, l),
-                               __shfl_sync(full, ct, l), __shfl_sync(full, kt, l), L, g, lane);
-    if (lane == l) mine = v;
-  }
-  return mine / (A * B);
-}
-
-// FP32: the replicated table window in shared memory; FP64: the global table.
-template <typename T>
-__device__ __forceinline__ GLook<T> band_lookup(const void* gtab, TabF64 td,
-                                                unsigned char* smem) {
+struct BandRule {
+  typedef T Val;
+  struct Par {
+    BandTab bt;
+    const void* gtab;
+    TabF64 td;
+  };
+  // FP32: one block of 32 warps per SM around the replicated table window
+  static constexpr int kThreads = sizeof(T) == 4 ? 1024 : 256;
   GLook<T> g;
-  if constexpr (sizeof(T) == 4) {
-    float4* st = reinterpret_cast<float4*>(smem);
-    const float4* gt = reinterpret_cast<const float4*>(gtab) + kWinK0;
-    for (int k = threadIdx.x; k < kWinSegs * kRep; k += blockDim.x) st[k] = gt[k / kRep];
-    g.tab8 = st + (threadIdx.x & (kRep - 1));
-  } else {
-    g.tab = reinterpret_cast<const D4*>(gtab);
-    g.t = td;
+  BandLane<T> L;
+  int lane;
+
+  static size_t smem() { return sizeof(T) == 4 ? (size_t)kWinSegs * kRep * sizeof(float4) : 0; }
+  __device__ __forceinline__ BandRule(const Par& P, unsigned char* sm) {
+    lane = threadIdx.x & 31;
+    if constexpr (sizeof(T) == 4) {
+      float4* st = reinterpret_cast<float4*>(sm);
+      const float4* gt = reinterpret_cast<const float4*>(P.gtab) + kWinK0;
+      for (int k = threadIdx.x; k < kWinSegs * kRep; k += blockDim.x) st[k] = gt[k / kRep];
+      g.tab8 = st + (threadIdx.x & (kRep - 1));
+    } else {
+      g.tab = reinterpret_cast<const D4*>(P.gtab);
+      g.t = P.td;
+    }
+    L = band_lane<T>(P.bt, lane);
+    __syncthreads();
   }
-  return g;
+  __device__ __forceinline__ double R(bool active, double A, double B, double c2) const {
+    constexpr unsigned full = 0xffffffffu;
+    const T At = (T)A, Bt = (T)B, ct = (T)c2, kt = (T)(A - B);
+    const T Al = (T)(A - (double)At), Bl = (T)(B - (double)Bt);
+    double mine = 0;
+    for (unsigned m = __ballot_sync(full, active); m; m &= m - 1) {
+      const int l = __ffs(m) - 1;
+      const double v = band_I_warp<T>(__shfl_sync(full, At, l), __shfl_sync(full, Bt, l),
+                                      __shfl_sync(full, Al, l), __shfl_sync(full, Bl, l),
+                                      __shfl_sync(full, ct, l), __shfl_sync(full, kt, l), L, g, lane);
+      if (lane == l) mine = v;
+    }
+    return mine / (A * B);
+  }
+};
+
+// ------------------------------------------------------------ FP64 node sums
+// The Q-node rule of FP64 contexts on the FP32 units.  GB300 runs 64 FP32
+// instructions in the time of one FP64 instruction, and a node pair takes ten
+// of the latter; so the separation, the table cubic and the node sums are
+// carried as unevaluated sums of two floats (Dekker 1971, Knuth's TwoSum; 48
+// bits), about 70 FP32 instructions.  The table is the cubic of the FP64 table
+// re-expanded about the middle of each segment, leading coefficients in two
+// floats; its error (2e-12 of g(0)) stays the rule's largest.  It covers
+// 2^kDfEmin <= x < 2^11 in shared memory; smaller separations (nodes that
+// coincide: the diagonal) use the FP64 table.
+// PIC workload at 6,000 stars (cross-covariances of 4,140 points): 152 ms with
+// FP64 instructions, 19.2 ms so; entries differ by 1e-13 (against FP64 Bessel
+// functions both are 1.3e-10 off, on the diagonal).
+struct F2 {
+  float h, l;
+};
+__device__ __forceinline__ F2 f2_of(double x) {
+  F2 r;
+  r.h = (float)x;
+  r.l = (float)(x - (double)r.h);
+  return r;
+}
+__device__ __forceinline__ F2 f2_fast(float a, float b) {  // |a| >= |b|
+  const float s = __fadd_rn(a, b);
+  return {s, __fsub_rn(b, __fsub_rn(s, a))};
+}
+__device__ __forceinline__ F2 f2_sum(float a, float b) {
+  const float s = __fadd_rn(a, b), z = __fsub_rn(s, a);
+  return {s, __fadd_rn(__fsub_rn(a, __fsub_rn(s, z)), __fsub_rn(b, z))};
+}
+__device__ __forceinline__ F2 f2_mul(F2 a, F2 b) {
+  const float p = __fmul_rn(a.h, b.h);
+  const float e = __fmaf_rn(a.l, b.h, __fmaf_rn(a.h, b.l, __fmaf_rn(a.h, b.h, -p)));
+  return f2_fast(p, e);
+}
+// acc += a b (both low parts kept, not renormalised)
+__device__ __forceinline__ void f2_fma(F2& acc, F2 a, F2 b) {
+  const float p = __fmul_rn(a.h, b.h);
+  const float e = __fmaf_rn(a.l, b.h, __fmaf_rn(a.h, b.l, __fmaf_rn(a.h, b.h, -p)));
+  const F2 s = f2_sum(acc.h, p);
+  acc.h = s.h;
+  acc.l = __fadd_rn(acc.l, __fadd_rn(s.l, e));
 }
 
-// Threads per block of the band kernels: FP32 one block of 32 warps per SM
-// around its table window, as the 64-node kernel.
-template <typename T>
-constexpr int band_threads() { return sizeof(T) == 4 ? 1024 : 256; }
+constexpr int kDfEmin = -20;
+constexpr int kDfSegs = (kTabF64.emax - kDfEmin) << kTabF64.m;  // 3,968: 93 KB
+constexpr int kDfShift = 23 - kTabF64.m;
+constexpr int kDfBase = (127 + kDfEmin) << kTabF64.m;
 
-// The band-rule counterpart of k_pair_quad (same entries, taper, mirror
-// convention, diagonal and prior mean).  A warp takes `batch` consecutive
-// entries (a power of two up to 32).
-template <typename T>
-__global__ void __launch_bounds__(band_threads<T>()) k_pair_quad_band(
-    QuadParams P, BandTab bt, int batch, int64_t n_rows, const double* __restrict__ rs,
+// coefficients of v = (x - x_mid) / H in [-1/2, 1/2): c0 and c1 as two floats
+// (tab4), c2 and c3 as one (tab2)
+__global__ void k_gtab_df(const D4* __restrict__ tab, float4* __restrict__ tab4,
+                          float2* __restrict__ tab2) {
+  for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < kDfSegs; k += gridDim.x * blockDim.x) {
+    const D4 d = tab[k + ((kDfEmin - kTabF64.emin) << kTabF64.m)];
+    const double H = ldexp(1.0 / (double)(1 << kTabF64.m), kDfEmin + (k >> kTabF64.m));
+    const double c1 = d.y * H, c2 = d.z * H * H, c3 = d.w * H * H * H;  // of (x - x_lo) / H
+    const F2 a0 = f2_of(d.x + 0.5 * (c1 + 0.5 * (c2 + 0.5 * c3)));
+    const F2 a1 = f2_of(c1 + c2 + 0.75 * c3);
+    tab4[k] = make_float4(a0.h, a0.l, a1.h, a1.l);
+    tab2[k] = make_float2((float)(c2 + 1.5 * c3), (float)c3);
+  }
+}
+
+template <int KPL>
+struct DfRule {
+  typedef double Val;
+  struct Par {
+    const double* gl_zeta;
+    const double* gl_w;
+    const D4* gtab;
+    TabF64 td;
+    const float4* tab4;
+    const float2* tab2;
+    int Q;
+  };
+  static constexpr int kThreads = 512;
+  static constexpr int kWarps = kThreads / 32;
+  const float4* t4;
+  const float2* t2;
+  const float4* zw;   // nodes and weights (zh, zl, wh, wl), shared memory
+  float2* tq;         // this warp's nodes on sightline i
+  const D4* gtab;
+  TabF64 td;
+  int lane, Q;
+
+  static size_t smem() {
+    return kDfSegs * (sizeof(float4) + sizeof(float2)) + kMaxNodes * sizeof(float4) +
+           kWarps * 32 * KPL * sizeof(float2);
+  }
+  __device__ __forceinline__ DfRule(const Par& P, unsigned char* sm)
+      : gtab(P.gtab), td(P.td), Q(P.Q) {
+    lane = threadIdx.x & 31;
+    float4* a = reinterpret_cast<float4*>(sm);
+    float4* z = a + kDfSegs;
+    float2* b = reinterpret_cast<float2*>(z + kMaxNodes);
+    tq = b + kDfSegs + (threadIdx.x >> 5) * 32 * KPL;
+    for (int k = threadIdx.x; k < kDfSegs; k += blockDim.x) {
+      a[k] = P.tab4[k];
+      b[k] = P.tab2[k];
+    }
+    for (int q = threadIdx.x; q < Q; q += blockDim.x) {
+      const F2 x = f2_of(P.gl_zeta[q]), w = f2_of(P.gl_w[q]);
+      z[q] = make_float4(x.h, x.l, w.h, w.l);
+    }
+    t4 = a;
+    t2 = b;
+    zw = z;
+    __syncthreads();
+  }
+
+  // g at x = xh + xl
+  __device__ __forceinline__ F2 g(float xh, float xl) const {
+    const int bits = __float_as_int(xh);
+    const int k = (bits >> kDfShift) - kDfBase;
+    if ((unsigned)k >= (unsigned)kDfSegs) {
+      // below the window (coinciding nodes) or beyond the table (zero)
+      if (k >= 0) return {0.f, 0.f};
+      return f2_of(g_lookup(gtab, td, (double)xh + (double)xl));
+    }
+    const float4 c = t4[k];
+    const float2 d = t2[k];
+    // v: the mantissa bits below the segment index, and xl in segment widths
+    const float vh = __int_as_float(((bits << kTabF64.m) & 0x007fffff) | 0x3f800000) - 1.5f;
+    const float vl =
+        xl * __int_as_float(((254 + kTabF64.m) << 23) - (bits & 0x7f800000));
+    const float s = __fmaf_rn(vh, d.y, d.x);
+    const F2 t = f2_fast(c.z, __fmul_rn(vh, s));
+    const float tl = __fmaf_rn(vl, s, __fadd_rn(t.l, c.w));
+    const float p = __fmul_rn(vh, t.h);
+    const float e = __fmaf_rn(vl, t.h, __fmaf_rn(vh, tl, __fmaf_rn(vh, t.h, -p)));
+    const F2 r = f2_fast(c.x, p);
+    return {r.h, __fadd_rn(r.l, __fadd_rn(e, c.y))};
+  }
+
+  // sum over the nodes of both sightlines
+  __device__ __forceinline__ double pair(F2 A, F2 B, F2 c2) const {
+    F2 tp[KPL], ct[KPL], acc[KPL];
+    __syncwarp();
+#pragma unroll
+    for (int k = 0; k < KPL; ++k) {
+      const int q = lane + 32 * k;
+      const float4 z = q < Q ? zw[q] : make_float4(0.f, 0.f, 0.f, 0.f);
+      const F2 zn = {z.x, z.y};
+      tp[k] = f2_mul(B, zn);
+      ct[k] = f2_mul(c2, tp[k]);
+      acc[k] = {0.f, 0.f};
+      const F2 t = f2_mul(A, zn);
+      tq[q] = make_float2(t.h, t.l);
+    }
+    __syncwarp();
+#pragma unroll 1
+    for (int q = 0; q < Q; ++q) {
+      const float2 t = tq[q];
+      const float4 z = zw[q];
+      const F2 w = {z.z, z.w};
+#pragma unroll
+      for (int k = 0; k < KPL; ++k) {
+        const F2 d = f2_sum(t.x, -tp[k].h);
+        const float dl = __fadd_rn(d.l, __fsub_rn(t.y, tp[k].l));
+        const float p = __fmul_rn(d.h, d.h);
+        const float pe = __fmaf_rn(2.f * d.h, dl, __fmaf_rn(d.h, d.h, -p));
+        const float c = __fmul_rn(t.x, ct[k].h);
+        const float ce = __fmaf_rn(t.y, ct[k].h,
+                                   __fmaf_rn(t.x, ct[k].l, __fmaf_rn(t.x, ct[k].h, -c)));
+        const F2 x = f2_sum(p, c);
+        f2_fma(acc[k], w, g(x.h, __fadd_rn(x.l, __fadd_rn(pe, ce))));
+      }
+    }
+    F2 tot = {0.f, 0.f};
+#pragma unroll
+    for (int k = 0; k < KPL; ++k) {
+      const int q = lane + 32 * k;
+      const float4 z = q < Q ? zw[q] : make_float4(0.f, 0.f, 0.f, 0.f);
+      f2_fma(tot, acc[k], F2{z.z, z.w});
+    }
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) {
+      const float oh = __shfl_xor_sync(0xffffffffu, tot.h, off);
+      const float ol = __shfl_xor_sync(0xffffffffu, tot.l, off);
+      const F2 r = f2_sum(tot.h, oh);
+      tot.h = r.h;
+      tot.l = __fadd_rn(__fadd_rn(tot.l, ol), r.l);
+    }
+    return (double)tot.h + (double)tot.l;
+  }
+
+  __device__ __forceinline__ double R(bool active, double A, double B, double c2) const {
+    constexpr unsigned full = 0xffffffffu;
+    const F2 a = f2_of(A), b = f2_of(B), c = f2_of(c2);
+    double mine = 0;
+    for (unsigned m = __ballot_sync(full, active); m; m &= m - 1) {
+      const int l = __ffs(m) - 1;
+      const F2 al = {__shfl_sync(full, a.h, l), __shfl_sync(full, a.l, l)};
+      const F2 bl = {__shfl_sync(full, b.h, l), __shfl_sync(full, b.l, l)};
+      const F2 cl = {__shfl_sync(full, c.h, l), __shfl_sync(full, c.l, l)};
+      const double v = pair(al, bl, cl);
+      if (lane == l) mine = v;
+    }
+    return mine;
+  }
+};
+
+// ------------------------------------------------------------ entries
+// Entries (i, j) of a CSR by a node rule, with the taper; in symmetric mode
+// entries with j < i are left for k_mirror, and the diagonal gives K_ii and
+// the prior mean.  A warp takes `batch` consecutive entries (a power of two up
+// to 32): the FP64 part of a pair (distances, chord, log1p, taper) runs a lane
+// per pair, the node sums a warp per pair.
+template <typename Rule>
+__global__ void __launch_bounds__(Rule::kThreads) k_pair_entries(
+    QuadParams P, typename Rule::Par rp, int batch, int64_t n_rows, const double* __restrict__ rs,
     const double* __restrict__ rux, const double* __restrict__ ruy, const double* __restrict__ ruz,
     const double* __restrict__ s, const double* __restrict__ ux, const double* __restrict__ uy,
     const double* __restrict__ uz, const int64_t* __restrict__ row_ptr,
-    const int32_t* __restrict__ col, int64_t nnz, T* __restrict__ val,
-    const void* __restrict__ gtab, TabF64 td, double* __restrict__ kdiag,
-    double* __restrict__ prior_m, unsigned* __restrict__ flags, const FieldGrid* __restrict__ fg,
-    const int32_t* __restrict__ row_field) {
+    const int32_t* __restrict__ col, int64_t nnz, typename Rule::Val* __restrict__ val,
+    double* __restrict__ kdiag, double* __restrict__ prior_m, unsigned* __restrict__ flags,
+    const FieldGrid* __restrict__ fg, const int32_t* __restrict__ row_field) {
+  typedef typename Rule::Val T;
   extern __shared__ __align__(16) unsigned char smem[];
-  const GLook<T> g = band_lookup<T>(gtab, td, smem);
-  __syncthreads();
+  const Rule rule(rp, smem);
   const int lane = threadIdx.x & 31;
-  const BandLane<T> L = band_lane<T>(bt, lane);
   const int64_t warp = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
   const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
   for (int64_t e0 = warp * batch; e0 < nnz; e0 += nwarps * batch) {
@@ -643,7 +818,7 @@ __global__ void __launch_bounds__(band_threads<T>()) k_pair_quad_band(
       A = si * fgi.inv_L0;
       B = sj * fgi.inv_L0;
     }
-    const double R = band_batch<T>(active, A, B, chord2, L, g, lane);
+    const double R = rule.R(active, A, B, chord2);
     if (active) {
       double K = P.form == GM_FORM_LOGNORMAL ? log1p(R) : R;
       if (P.taper == GM_TAPER_WENDLAND) {
@@ -662,18 +837,16 @@ __global__ void __launch_bounds__(band_threads<T>()) k_pair_quad_band(
   }
 }
 
-// Band-rule self-covariance of query points (k_self_quad's counterpart), and
-// of an explicit pair list (k_pairlist_quad's; sj null: the points themselves).
-template <typename T>
-__global__ void __launch_bounds__(band_threads<T>()) k_pairlist_quad_band(
-    QuadParams P, BandTab bt, int batch, int64_t n, const double* __restrict__ si,
-    const double* __restrict__ sj, const double* __restrict__ chord, double* __restrict__ out,
-    const void* __restrict__ gtab, TabF64 td) {
+// An explicit list of pair geometries (distances si, sj in pc, chord |u_i -
+// u_j|): K = log1p(R) (or R) without the taper; sj null: the self-covariance of
+// the points si, at the precision of the stored entries.
+template <typename Rule>
+__global__ void __launch_bounds__(Rule::kThreads) k_pair_list(
+    QuadParams P, typename Rule::Par rp, int batch, int64_t n, const double* __restrict__ si,
+    const double* __restrict__ sj, const double* __restrict__ chord, double* __restrict__ out) {
   extern __shared__ __align__(16) unsigned char smem[];
-  const GLook<T> g = band_lookup<T>(gtab, td, smem);
-  __syncthreads();
+  const Rule rule(rp, smem);
   const int lane = threadIdx.x & 31;
-  const BandLane<T> L = band_lane<T>(bt, lane);
   const int64_t warp = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
   const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
   for (int64_t p0 = warp * batch; p0 < n; p0 += nwarps * batch) {
@@ -685,10 +858,10 @@ __global__ void __launch_bounds__(band_threads<T>()) k_pairlist_quad_band(
       B = sj ? sj[p] * P.inv_L0 : A;
       c2 = sj ? chord[p] * chord[p] : 0.0;
     }
-    const double R = band_batch<T>(active, A, B, c2, L, g, lane);
+    const double R = rule.R(active, A, B, c2);
     if (active) {
       const double K = P.form == GM_FORM_LOGNORMAL ? log1p(R) : R;
-      out[p] = sj ? K : (double)(T)K;
+      out[p] = sj ? K : (double)(typename Rule::Val)K;
     }
   }
 }
@@ -726,6 +899,10 @@ gm_status phi_points_init(gm_ctx* c) {
   size_t tb = (size_t)(g.n_real() + 1) * (c->cfg.precision == GM_PREC_FP32 ? 16 : 32);
   c->gtab = dev_alloc(c, tb);
   if (!c->phi_pts || !c->gtab) return set_error(c, GM_E_NOMEM, "phi table");
+  if (c->cfg.precision != GM_PREC_FP32) {
+    c->gtab_df = dev_alloc(c, kDfSegs * (sizeof(float4) + sizeof(float2)));
+    if (!c->gtab_df) return set_error(c, GM_E_NOMEM, "phi table");
+  }
   const double cnorm = std::pow(2.0, 2.0 / 3.0) / std::tgamma(1.0 / 3.0);
   int blocks = (int)std::min<int64_t>(ceil_div(g.n_pts(), 128), 4 * sm_count(c));
   GM_PROF(c, "k_phi_points");
@@ -747,6 +924,13 @@ gm_status gtab_update(gm_ctx* c) {
     k_gtab<D4><<<blocks, 256, 0, c->stream>>>(g, c->phi_pts, c->cfg.sigma2, c->cfg.form, 0,
                                                    (D4*)c->gtab);
   GM_LAUNCH_CHECK(c);
+  if (c->cfg.precision != GM_PREC_FP32) {
+    float4* t4 = (float4*)c->gtab_df;
+    GM_PROF(c, "k_gtab_df");
+    k_gtab_df<<<(kDfSegs + 255) / 256, 256, 0, c->stream>>>((const D4*)c->gtab, t4,
+                                                            (float2*)(t4 + kDfSegs));
+    GM_LAUNCH_CHECK(c);
+  }
   c->gtab_sigma2 = c->cfg.sigma2;
   c->gtab_form = c->cfg.form;
   return GM_OK;
@@ -765,15 +949,14 @@ static QuadParams quad_params(const gm_ctx* c, bool symmetric) {
   return P;
 }
 
-template <typename T, int KPL>
+template <int KPL>
 static void launch_pair(gm_ctx* c, const QuadParams& P, int64_t n_rows, const double* rs,
                         const double* rux, const double* ruy, const double* ruz,
                         const int32_t* row_field, const int64_t* row_ptr, const int32_t* col,
                         int64_t nnz, void* val) {
-  size_t smem = 2 * kMaxNodes * sizeof(T);
-  if (sizeof(T) == 4) smem += (size_t)kWinSegs * kRep * sizeof(float4);
-  constexpr int nt = pair_threads<T, KPL>();
-  auto kern = k_pair_quad<T, KPL>;
+  const size_t smem = 2 * kMaxNodes * sizeof(float) + (size_t)kWinSegs * kRep * sizeof(float4);
+  constexpr int nt = pair_threads<KPL>();
+  auto kern = k_pair_quad<KPL>;
   cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   int per_sm = 0;
   cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, nt, smem);
@@ -781,9 +964,9 @@ static void launch_pair(gm_ctx* c, const QuadParams& P, int64_t n_rows, const do
   blocks = (int)std::min<int64_t>(blocks, std::max<int64_t>(1, ceil_div(nnz * 32, nt)));
   GM_PROF(c, "k_pair_quad");
   kern<<<blocks, nt, smem, c->stream>>>(P, n_rows, rs, rux, ruy, ruz, c->s, c->ux, c->uy, c->uz,
-                                         row_ptr, col, nnz, (T*)val, c->gl_zeta, c->gl_w, c->gtab,
-                                         tab_f32(), tab_f64(), c->kdiag, c->prior_m, c->d_flags,
-                                         c->fgrid, row_field);
+                                        row_ptr, col, nnz, (float*)val, c->gl_zeta, c->gl_w,
+                                        (const float4*)c->gtab, c->kdiag, c->prior_m, c->d_flags,
+                                        c->fgrid, row_field);
 }
 
 static BandTab band_tab() {
@@ -793,16 +976,15 @@ static BandTab band_tab() {
   return t;
 }
 
-// Blocks and batch of a band kernel over n entries: the resident blocks, and
+// Blocks and batch of a rule's kernel over n entries: the resident blocks, and
 // the largest batch that still leaves every warp two (small lists: the pairs
 // spread over the chip, one per warp in the limit).
-template <typename T, typename Kern>
-static void band_shape(gm_ctx* c, Kern kern, int64_t n, size_t* smem, int* blocks, int* batch) {
-  constexpr int nt = band_threads<T>();
-  *smem = sizeof(T) == 4 ? (size_t)kWinSegs * kRep * sizeof(float4) : 0;
-  cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)*smem);
+template <typename Rule, typename Kern>
+static void rule_shape(gm_ctx* c, Kern kern, int64_t n, int* blocks, int* batch) {
+  constexpr int nt = Rule::kThreads;
+  cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Rule::smem());
   int per_sm = 0;
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, nt, *smem);
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, nt, Rule::smem());
   const int64_t resident = (int64_t)std::max(1, per_sm) * sm_count(c);
   int b = 32;
   while (b > 1 && n < 2 * b * resident * (nt / 32)) b >>= 1;
@@ -810,30 +992,41 @@ static void band_shape(gm_ctx* c, Kern kern, int64_t n, size_t* smem, int* block
   *blocks = (int)std::min<int64_t>(resident, std::max<int64_t>(1, ceil_div(ceil_div(n, b), nt / 32)));
 }
 
-template <typename T>
-static void launch_pair_band(gm_ctx* c, const QuadParams& P, int64_t n_rows, const double* rs,
-                             const double* rux, const double* ruy, const double* ruz,
-                             const int32_t* row_field, const int64_t* row_ptr,
-                             const int32_t* col, int64_t nnz, void* val) {
-  size_t smem;
+template <typename Rule>
+static void launch_entries(gm_ctx* c, const QuadParams& P, const typename Rule::Par& rp,
+                           int64_t n_rows, const double* rs, const double* rux, const double* ruy,
+                           const double* ruz, const int32_t* row_field, const int64_t* row_ptr,
+                           const int32_t* col, int64_t nnz, void* val, const char* name) {
   int blocks, batch;
-  auto kern = k_pair_quad_band<T>;
-  band_shape<T>(c, kern, nnz, &smem, &blocks, &batch);
-  GM_PROF(c, "k_pair_quad_band");
-  kern<<<blocks, band_threads<T>(), smem, c->stream>>>(
-      P, band_tab(), batch, n_rows, rs, rux, ruy, ruz, c->s, c->ux, c->uy, c->uz, row_ptr, col,
-      nnz, (T*)val, c->gtab, tab_f64(), c->kdiag, c->prior_m, c->d_flags, c->fgrid, row_field);
+  auto kern = k_pair_entries<Rule>;
+  rule_shape<Rule>(c, kern, nnz, &blocks, &batch);
+  GM_PROF(c, name);
+  kern<<<blocks, Rule::kThreads, Rule::smem(), c->stream>>>(
+      P, rp, batch, n_rows, rs, rux, ruy, ruz, c->s, c->ux, c->uy, c->uz, row_ptr, col, nnz,
+      (typename Rule::Val*)val, c->kdiag, c->prior_m, c->d_flags, c->fgrid, row_field);
+}
+
+template <typename Rule>
+static void launch_list(gm_ctx* c, const QuadParams& P, const typename Rule::Par& rp, int64_t n,
+                        const double* si, const double* sj, const double* chord, double* out,
+                        const char* name) {
+  int blocks, batch;
+  auto kern = k_pair_list<Rule>;
+  rule_shape<Rule>(c, kern, n, &blocks, &batch);
+  GM_PROF(c, name);
+  kern<<<blocks, Rule::kThreads, Rule::smem(), c->stream>>>(P, rp, batch, n, si, sj, chord, out);
 }
 
 template <typename T>
-static void launch_pairlist_band(gm_ctx* c, const QuadParams& P, int64_t n, const double* si,
-                                 const double* sj, const double* chord, double* out) {
-  size_t smem;
-  int blocks, batch;
-  auto kern = k_pairlist_quad_band<T>;
-  band_shape<T>(c, kern, n, &smem, &blocks, &batch);
-  kern<<<blocks, band_threads<T>(), smem, c->stream>>>(P, band_tab(), batch, n, si, sj, chord,
-                                                       out, c->gtab, tab_f64());
+static typename BandRule<T>::Par band_par(const gm_ctx* c) {
+  return {band_tab(), c->gtab, tab_f64()};
+}
+
+template <int KPL>
+static typename DfRule<KPL>::Par df_par(const gm_ctx* c) {
+  const float4* t4 = (const float4*)c->gtab_df;
+  return {c->gl_zeta, c->gl_w, (const D4*)c->gtab, tab_f64(), t4, (const float2*)(t4 + kDfSegs),
+          c->cfg.n_nodes};
 }
 
 gm_status pair_quadrature(gm_ctx* c, int64_t n_rows, const double* rs, const double* rux,
@@ -846,19 +1039,22 @@ gm_status pair_quadrature(gm_ctx* c, int64_t n_rows, const double* rs, const dou
   QuadParams P = quad_params(c, symmetric);
   const int Q = c->cfg.n_nodes;
   const bool f32 = c->cfg.precision == GM_PREC_FP32;
+#define GM_ENTRIES(RULE, PAR, NAME) \
+  launch_entries<RULE>(c, P, PAR, n_rows, rs, rux, ruy, ruz, row_field, row_ptr, col, nnz, val, NAME)
   if (c->cfg.quad_rule == GM_QUAD_BAND) {
-    if (f32) launch_pair_band<float>(c, P, n_rows, rs, rux, ruy, ruz, row_field, row_ptr, col, nnz, val);
-    else launch_pair_band<double>(c, P, n_rows, rs, rux, ruy, ruz, row_field, row_ptr, col, nnz, val);
+    if (f32) GM_ENTRIES(BandRule<float>, band_par<float>(c), "k_pair_quad_band");
+    else GM_ENTRIES(BandRule<double>, band_par<double>(c), "k_pair_quad_band");
   } else if (Q <= 32) {
-    if (f32) launch_pair<float, 1>(c, P, n_rows, rs, rux, ruy, ruz, row_field, row_ptr, col, nnz, val);
-    else launch_pair<double, 1>(c, P, n_rows, rs, rux, ruy, ruz, row_field, row_ptr, col, nnz, val);
+    if (f32) launch_pair<1>(c, P, n_rows, rs, rux, ruy, ruz, row_field, row_ptr, col, nnz, val);
+    else GM_ENTRIES(DfRule<1>, df_par<1>(c), "k_pair_quad");
   } else if (Q <= 64) {
-    if (f32) launch_pair<float, 2>(c, P, n_rows, rs, rux, ruy, ruz, row_field, row_ptr, col, nnz, val);
-    else launch_pair<double, 2>(c, P, n_rows, rs, rux, ruy, ruz, row_field, row_ptr, col, nnz, val);
+    if (f32) launch_pair<2>(c, P, n_rows, rs, rux, ruy, ruz, row_field, row_ptr, col, nnz, val);
+    else GM_ENTRIES(DfRule<2>, df_par<2>(c), "k_pair_quad");
   } else {
-    if (f32) launch_pair<float, 4>(c, P, n_rows, rs, rux, ruy, ruz, row_field, row_ptr, col, nnz, val);
-    else launch_pair<double, 4>(c, P, n_rows, rs, rux, ruy, ruz, row_field, row_ptr, col, nnz, val);
+    if (f32) launch_pair<4>(c, P, n_rows, rs, rux, ruy, ruz, row_field, row_ptr, col, nnz, val);
+    else GM_ENTRIES(DfRule<4>, df_par<4>(c), "k_pair_quad");
   }
+#undef GM_ENTRIES
   GM_LAUNCH_CHECK(c);
   if (symmetric) {
     int blocks = (int)std::min<int64_t>(ceil_div(nnz, 256), 16 * sm_count(c));
@@ -891,25 +1087,30 @@ gm_status self_quadrature(gm_ctx* c, int64_t n_rows, const double* rs, double* k
   const int Q = c->cfg.n_nodes;
   const bool f32 = c->cfg.precision == GM_PREC_FP32;
   int blocks = (int)std::min<int64_t>(ceil_div(n_rows * 32, 256), 8 * sm_count(c));
+#define GM_SELF32(K)                                                                      \
+  k_self_quad<K><<<blocks, 256, 0, c->stream>>>(P, n_rows, rs, c->gl_zeta, c->gl_w, c->gtab, \
+                                                tab_f32(), kss)
+#define GM_SELF64(K) \
+  launch_list<DfRule<K>>(c, P, df_par<K>(c), n_rows, rs, nullptr, nullptr, kss, "k_self_quad")
   if (c->cfg.quad_rule == GM_QUAD_BAND) {
-    GM_PROF(c, "k_self_quad_band");
-    if (f32) launch_pairlist_band<float>(c, P, n_rows, rs, nullptr, nullptr, kss);
-    else launch_pairlist_band<double>(c, P, n_rows, rs, nullptr, nullptr, kss);
-    GM_LAUNCH_CHECK(c);
-    return GM_OK;
-  }
-#define GM_SELF(T, K)                                                                     \
-  k_self_quad<T, K><<<blocks, 256, 0, c->stream>>>(P, n_rows, rs, c->gl_zeta, c->gl_w, \
-                                                    c->gtab, tab_f32(), tab_f64(), kss)
-  GM_PROF(c, "k_self_quad");
-  if (Q <= 32) {
-    if (f32) GM_SELF(float, 1); else GM_SELF(double, 1);
-  } else if (Q <= 64) {
-    if (f32) GM_SELF(float, 2); else GM_SELF(double, 2);
+    if (f32)
+      launch_list<BandRule<float>>(c, P, band_par<float>(c), n_rows, rs, nullptr, nullptr, kss,
+                                   "k_self_quad_band");
+    else
+      launch_list<BandRule<double>>(c, P, band_par<double>(c), n_rows, rs, nullptr, nullptr, kss,
+                                    "k_self_quad_band");
+  } else if (f32) {
+    GM_PROF(c, "k_self_quad");
+    if (Q <= 32) GM_SELF32(1);
+    else if (Q <= 64) GM_SELF32(2);
+    else GM_SELF32(4);
   } else {
-    if (f32) GM_SELF(float, 4); else GM_SELF(double, 4);
+    if (Q <= 32) GM_SELF64(1);
+    else if (Q <= 64) GM_SELF64(2);
+    else GM_SELF64(4);
   }
-#undef GM_SELF
+#undef GM_SELF32
+#undef GM_SELF64
   GM_LAUNCH_CHECK(c);
   return GM_OK;
 }
@@ -920,60 +1121,47 @@ namespace gm {
 
 // Sightline quadrature for an explicit list of pair geometries (distances
 // si, sj in pc, chord |u_i - u_j|): K = log1p(R) (or R) without the taper.
-// Same rule and kernel table as the covariance assembly; one warp per pair.
-template <typename T, int KPL>
+// FP32 form; same rule and kernel table as the covariance assembly; one warp
+// per pair.
+template <int KPL>
 __global__ void __launch_bounds__(256) k_pairlist_quad(
     QuadParams P, int64_t n, const double* __restrict__ si, const double* __restrict__ sj,
     const double* __restrict__ chord, double* __restrict__ out,
     const double* __restrict__ gl_zeta, const double* __restrict__ gl_w,
-    const void* __restrict__ gtab, TabF32 tf, TabF64 td) {
-  extern __shared__ unsigned char smem[];
-  typedef typename std::conditional<sizeof(T) == 4, float4, D4>::type T4;
-  T* zq = reinterpret_cast<T*>(smem);
-  T* wq = zq + kMaxNodes;
-  const T4* tab;
-  if (sizeof(T) == 4) {
-    float4* st = reinterpret_cast<float4*>(smem + 2 * kMaxNodes * sizeof(T));
-    const float4* gt = reinterpret_cast<const float4*>(gtab);
-    for (int k = threadIdx.x; k <= tf.last; k += blockDim.x) st[k] = gt[k];
-    tab = reinterpret_cast<const T4*>(st);
-  } else {
-    tab = reinterpret_cast<const T4*>(gtab);
-  }
+    const float4* __restrict__ gtab, TabF32 tf) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  float* zq = reinterpret_cast<float*>(smem);
+  float* wq = zq + kMaxNodes;
+  float4* tab = reinterpret_cast<float4*>(smem + 2 * kMaxNodes * sizeof(float));
+  for (int k = threadIdx.x; k <= tf.last; k += blockDim.x) tab[k] = gtab[k];
   for (int q = threadIdx.x; q < P.Q; q += blockDim.x) {
-    zq[q] = (T)gl_zeta[q];
-    wq[q] = (T)gl_w[q];
+    zq[q] = (float)gl_zeta[q];
+    wq[q] = (float)gl_w[q];
   }
   __syncthreads();
   const int lane = threadIdx.x & 31;
   const int64_t warp = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
   const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
   for (int64_t p = warp; p < n; p += nwarps) {
-    const T a = (T)(si[p] * P.inv_L0), b = (T)(sj[p] * P.inv_L0);
-    const T c2 = (T)(chord[p] * chord[p]);
-    T tp[KPL], ctp[KPL], wp[KPL];
+    const float a = (float)(si[p] * P.inv_L0), b = (float)(sj[p] * P.inv_L0);
+    const float c2 = (float)(chord[p] * chord[p]);
+    float tp[KPL], ctp[KPL], wp[KPL];
 #pragma unroll
     for (int k = 0; k < KPL; ++k) {
       int q = lane + 32 * k;
       bool ok = q < P.Q;
-      tp[k] = ok ? b * zq[q] : (T)0;
+      tp[k] = ok ? b * zq[q] : 0.f;
       ctp[k] = c2 * tp[k];
-      wp[k] = ok ? wq[q] : (T)0;
+      wp[k] = ok ? wq[q] : 0.f;
     }
-    T acc = 0;
+    float acc = 0;
     for (int q = 0; q < P.Q; ++q) {
-      const T t = a * zq[q];
-      T inner = 0;
+      const float t = a * zq[q];
+      float inner = 0;
 #pragma unroll
       for (int k = 0; k < KPL; ++k) {
-        T d = t - tp[k];
-        T x = d * d + t * ctp[k];
-        T gv;
-        if (sizeof(T) == 4)
-          gv = (T)g_lookup(reinterpret_cast<const float4*>(tab), tf, (float)x);
-        else
-          gv = (T)g_lookup(reinterpret_cast<const D4*>(tab), td, (double)x);
-        inner += wp[k] * gv;
+        const float d = t - tp[k];
+        inner += wp[k] * g_lookup(tab, tf, d * d + t * ctp[k]);
       }
       acc += wq[q] * inner;
     }
@@ -986,19 +1174,19 @@ __global__ void __launch_bounds__(256) k_pairlist_quad(
   }
 }
 
-template <typename T, int KPL>
+template <int KPL>
 static void launch_pairlist(gm_ctx* c, const QuadParams& P, int64_t n, const double* si,
                             const double* sj, const double* chord, double* out) {
-  size_t smem = 2 * kMaxNodes * sizeof(T);
-  if (sizeof(T) == 4) smem += (size_t)(kTabF32.n_real() + 1) * sizeof(float4);
-  auto kern = k_pairlist_quad<T, KPL>;
+  const size_t smem = 2 * kMaxNodes * sizeof(float) + (size_t)(kTabF32.n_real() + 1) * sizeof(float4);
+  auto kern = k_pairlist_quad<KPL>;
   cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   int per_sm = 0;
   cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, 256, smem);
   int blocks = std::max(1, per_sm) * sm_count(c);
   blocks = (int)std::min<int64_t>(blocks, std::max<int64_t>(1, ceil_div(n * 32, 256)));
-  kern<<<blocks, 256, smem, c->stream>>>(P, n, si, sj, chord, out, c->gl_zeta, c->gl_w, c->gtab,
-                                         tab_f32(), tab_f64());
+  GM_PROF(c, "k_pairlist_quad");
+  kern<<<blocks, 256, smem, c->stream>>>(P, n, si, sj, chord, out, c->gl_zeta, c->gl_w,
+                                         (const float4*)c->gtab, tab_f32());
 }
 
 gm_status pairlist_quadrature(gm_ctx* c, int64_t n, const double* si, const double* sj,
@@ -1009,24 +1197,21 @@ gm_status pairlist_quadrature(gm_ctx* c, int64_t n, const double* si, const doub
   QuadParams P = quad_params(c, false);
   const int Q = c->cfg.n_nodes;
   const bool f32 = c->cfg.precision == GM_PREC_FP32;
+#define GM_LIST(RULE, PAR, NAME) launch_list<RULE>(c, P, PAR, n, si, sj, chord, out, NAME)
   if (c->cfg.quad_rule == GM_QUAD_BAND) {
-    GM_PROF(c, "k_pairlist_quad_band");
-    if (f32) launch_pairlist_band<float>(c, P, n, si, sj, chord, out);
-    else launch_pairlist_band<double>(c, P, n, si, sj, chord, out);
-    GM_LAUNCH_CHECK(c);
-    return GM_OK;
-  }
-  GM_PROF(c, "k_pairlist_quad");
-  if (Q <= 32) {
-    if (f32) launch_pairlist<float, 1>(c, P, n, si, sj, chord, out);
-    else launch_pairlist<double, 1>(c, P, n, si, sj, chord, out);
+    if (f32) GM_LIST(BandRule<float>, band_par<float>(c), "k_pairlist_quad_band");
+    else GM_LIST(BandRule<double>, band_par<double>(c), "k_pairlist_quad_band");
+  } else if (Q <= 32) {
+    if (f32) launch_pairlist<1>(c, P, n, si, sj, chord, out);
+    else GM_LIST(DfRule<1>, df_par<1>(c), "k_pairlist_quad");
   } else if (Q <= 64) {
-    if (f32) launch_pairlist<float, 2>(c, P, n, si, sj, chord, out);
-    else launch_pairlist<double, 2>(c, P, n, si, sj, chord, out);
+    if (f32) launch_pairlist<2>(c, P, n, si, sj, chord, out);
+    else GM_LIST(DfRule<2>, df_par<2>(c), "k_pairlist_quad");
   } else {
-    if (f32) launch_pairlist<float, 4>(c, P, n, si, sj, chord, out);
-    else launch_pairlist<double, 4>(c, P, n, si, sj, chord, out);
+    if (f32) launch_pairlist<4>(c, P, n, si, sj, chord, out);
+    else GM_LIST(DfRule<4>, df_par<4>(c), "k_pairlist_quad");
   }
+#undef GM_LIST
   GM_LAUNCH_CHECK(c);
   return GM_OK;
 }
