@@ -84,6 +84,55 @@ __device__ __forceinline__ void tilted_mode(double mc, double vc, double obs, do
   *sh_out = H < 0 ? 1.0 / sqrt(-H) : sqrt(vc);
 }
 
+// The same moments with the line search to the last step and the node sums in
+// order: what FP32 contexts run (a single lane a star).  Their mean solve stops
+// at cg_tol of a residual that a few stars with large site precisions dominate,
+// so the last bit of a site can move a posterior mean by 1e-4; and the update is
+// 0.2 % of an FP32 sweep, so it keeps its roundings there.
+__device__ __forceinline__ void tilted_in_order(double mc, double vc, double obs, double s2,
+                                                const double* __restrict__ ghx,
+                                                const double* __restrict__ ghw, double* mh,
+                                                double* vh) {
+  double a;
+  if (obs > 0) {
+    double aL = log(obs), vL = s2 / (obs * obs);
+    a = (mc / vc + aL / vL) / (1.0 / vc + 1.0 / vL);
+  } else {
+    a = mc;
+  }
+  for (int it = 0; it < 100; ++it) {
+    double ea = exp(a);
+    double gr = -(a - mc) / vc + (obs - ea) * ea / s2;
+    double H = -1.0 / vc + (obs * ea - 2.0 * ea * ea) / s2;
+    double step = H < 0 ? -gr / H : gr * vc;
+    step = fmax(-1.0, fmin(1.0, step));
+    double h0 = log_tilted(a, ea, mc, vc, obs, s2);
+    int k = 0;
+    while (log_tilted(a + step, exp(a + step), mc, vc, obs, s2) < h0 && k < 60) {
+      step *= 0.5;
+      ++k;
+    }
+    a += step;
+    if (fabs(step) <= 1e-14 * (1.0 + fabs(a))) break;
+  }
+  double ea = exp(a);
+  double H = -1.0 / vc + (obs * ea - 2.0 * ea * ea) / s2;
+  double sh = H < 0 ? 1.0 / sqrt(-H) : sqrt(vc);
+  double h0 = log_tilted(a, ea, mc, vc, obs, s2);
+  const double sc = 1.4142135623730951 * sh;
+  double S0 = 0, S1 = 0, S2 = 0;
+  for (int k = 0; k < kGH; ++k) {
+    double y = sc * ghx[k];
+    double wk = ghw[k] * exp(log_tilted(a + y, exp(a + y), mc, vc, obs, s2) - h0);
+    S0 += wk;
+    S1 += wk * y;
+    S2 += wk * y * y;
+  }
+  double m1 = S1 / S0;
+  *mh = a + m1;
+  *vh = S2 / S0 - m1 * m1;
+}
+
 constexpr int kSiteThreads = 128;
 
 // Shared by the context's update and the allocation-free one: `last` (null:
@@ -94,7 +143,7 @@ struct SiteLast {
   unsigned long long* out;      // skip count, flags, maximum (bits of a double)
 };
 
-template <int G>
+template <int G, bool IN_ORDER>
 __global__ void __launch_bounds__(kSiteThreads) k_site_update(
     int64_t n, SiteParams P, const double* __restrict__ mu, const double* __restrict__ var,
     const double* __restrict__ obs, const double* __restrict__ sig, double* __restrict__ tau,
@@ -136,6 +185,8 @@ __global__ void __launch_bounds__(kSiteThreads) k_site_update(
     if (P.lik == GM_LIK_GAUSS_IN_LNA) {
       vh = 1.0 / (1.0 / vc + 1.0 / s2);
       mh = vh * (mc / vc + ob / s2);
+    } else if (IN_ORDER) {
+      if (!skip) tilted_in_order(mc, vc, ob, s2, ghx, ghw, &mh, &vh);
     } else {
       double S0 = 0, S1 = 0, S2 = 0;
       if (!skip) {
@@ -229,6 +280,7 @@ static int site_blocks(int64_t n, int group, int64_t max_blocks) {
   return (int)std::min<int64_t>(ceil_div(n * group, kSiteThreads), max_blocks);
 }
 
+// group 0: the in-order update
 static void launch_site(int group, int blocks, cudaStream_t st, int64_t n, const SiteParams& P,
                         const double* mu, const double* var, const double* obs, const double* sig,
                         double* tau, double* nu, const double* gh_x, const double* gh_w,
@@ -236,8 +288,8 @@ static void launch_site(int group, int blocks, cudaStream_t st, int64_t n, const
                         SiteLast last) {
 #define GM_SITE(G)                                                                            \
   case G:                                                                                     \
-    k_site_update<G><<<blocks, kSiteThreads, 0, st>>>(n, P, mu, var, obs, sig, tau, nu, gh_x, \
-                                                      gh_w, part, skipped, flags, last);      \
+    k_site_update<G, false><<<blocks, kSiteThreads, 0, st>>>(                                 \
+        n, P, mu, var, obs, sig, tau, nu, gh_x, gh_w, part, skipped, flags, last);            \
     break
   switch (group) {
     GM_SITE(32);
@@ -245,9 +297,11 @@ static void launch_site(int group, int blocks, cudaStream_t st, int64_t n, const
     GM_SITE(8);
     GM_SITE(4);
     GM_SITE(2);
+    GM_SITE(1);
     default:
-      k_site_update<1><<<blocks, kSiteThreads, 0, st>>>(n, P, mu, var, obs, sig, tau, nu, gh_x,
-                                                        gh_w, part, skipped, flags, last);
+      k_site_update<1, true><<<blocks, kSiteThreads, 0, st>>>(n, P, mu, var, obs, sig, tau, nu,
+                                                              gh_x, gh_w, part, skipped, flags,
+                                                              last);
   }
 #undef GM_SITE
 }
@@ -255,8 +309,9 @@ static void launch_site(int group, int blocks, cudaStream_t st, int64_t n, const
 gm_status site_update(gm_ctx* c, double* max_delta, int64_t* skipped) {
   const int64_t n = c->n;
   cudaStream_t st = c->stream;
-  const int sms = sm_count(c), group = site_group(n, sms);
-  const int G = site_blocks(n, group, 4 * sms);
+  const int sms = sm_count(c);
+  const int group = c->cfg.precision == GM_PREC_FP32 ? 0 : site_group(n, sms);
+  const int G = site_blocks(n, std::max(group, 1), 4 * sms);
   double* part = (double*)dev_alloc(c, (G + 1) * sizeof(double) + sizeof(unsigned long long));
   if (!part) return set_error(c, GM_E_NOMEM, "site partials");
   unsigned long long* cnt = (unsigned long long*)(part + G);
