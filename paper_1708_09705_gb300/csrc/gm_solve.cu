@@ -18,6 +18,7 @@
 #include <vector>
 
 #include "gm_internal.cuh"
+#include "gm_tcgen05.cuh"
 
 namespace gm {
 
@@ -64,14 +65,41 @@ __device__ __forceinline__ double block_sum(double v, double* sh) {
   return t;
 }
 
-// Sum of a partials array, same fixed order in every block.
-__device__ __forceinline__ double sum_partials(const double* __restrict__ part, int n, double* sh) {
-  double v = 0;
-  for (int k = threadIdx.x; k < n; k += blockDim.x) v += part[k];
-  double t = block_sum(v, sh);
-  if (threadIdx.x == 0) sh[32] = t;
+// Two block sums with one pass of shuffles and barriers.
+__device__ __forceinline__ double2 block_sum2(double a, double b, double* sh) {
+  a = warp_sum(a);
+  b = warp_sum(b);
+  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  if (lane == 0) {
+    sh[w] = a;
+    sh[16 + w] = b;
+  }
   __syncthreads();
-  double r = sh[32];
+  double2 t = make_double2(0.0, 0.0);
+  if (w == 0) {
+    const bool in = lane < (int)(blockDim.x >> 5);
+    t.x = warp_sum(in ? sh[lane] : 0.0);
+    t.y = warp_sum(in ? sh[16 + lane] : 0.0);
+  }
+  __syncthreads();
+  return t;
+}
+
+// Sums of two partials arrays, same fixed order in every block.
+__device__ __forceinline__ double2 sum_partials2(const double* __restrict__ p,
+                                                 const double* __restrict__ q, int n, double* sh) {
+  double a = 0, b = 0;
+  for (int k = threadIdx.x; k < n; k += blockDim.x) {
+    a += p[k];
+    b += q[k];
+  }
+  const double2 t = block_sum2(a, b, sh);
+  if (threadIdx.x == 0) {
+    sh[32] = t.x;
+    sh[33] = t.y;
+  }
+  __syncthreads();
+  const double2 r = make_double2(sh[32], sh[33]);
   __syncthreads();
   return r;
 }
@@ -216,8 +244,8 @@ __global__ void __launch_bounds__(kBT) k_cg_update1(int64_t n, int it, const TV*
   __shared__ double sh[40];
   const int G = gridDim.x;
   const int prev = (it & 1) ? 1 : 2, next = (it & 1) ? 2 : 1;
-  double pq = sum_partials(part, G, sh);
-  double rzp = sum_partials(part + prev * G, G, sh);
+  const double2 sums = sum_partials2(part, part + prev * G, G, sh);
+  const double pq = sums.x, rzp = sums.y;
   double alpha = 0;
   if (rzp > 0) {
     if (pq > 0) alpha = rzp / pq;
@@ -233,11 +261,10 @@ __global__ void __launch_bounds__(kBT) k_cg_update1(int64_t n, int it, const TV*
     rz += (double)ri * (double)(minv[i] * ri);
     rr += (double)ri * (double)ri;
   }
-  double t1 = block_sum(rz, sh);
-  double t2 = block_sum(rr, sh);
+  const double2 t = block_sum2(rz, rr, sh);
   if (threadIdx.x == 0) {
-    part[next * G + blockIdx.x] = t1;
-    part[3 * G + blockIdx.x] = t2;
+    part[next * G + blockIdx.x] = t.x;
+    part[3 * G + blockIdx.x] = t.y;
   }
 }
 
@@ -251,8 +278,8 @@ __global__ void __launch_bounds__(kBT) k_cg_update2(int64_t n, int it, const TV*
   __shared__ double sh[40];
   const int G = gridDim.x;
   const int prev = (it & 1) ? 1 : 2, next = (it & 1) ? 2 : 1;
-  double rzp = sum_partials(part + prev * G, G, sh);
-  double rzn = sum_partials(part + next * G, G, sh);
+  const double2 sums = sum_partials2(part + prev * G, part + next * G, G, sh);
+  const double rzp = sums.x, rzn = sums.y;
   const TV beta = (TV)(rzp > 0 ? rzn / rzp : 0.0);
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
        i += (int64_t)G * blockDim.x) {
@@ -582,60 +609,80 @@ __global__ void __launch_bounds__(kBT) k_panel_spmm(int64_t n, int R,
 // 2 rz_prev, 3 rz_new, 4 bb, 5 rr.  mode 0: after init (rz_prev, bb);
 // mode 1: after spmm (alpha); mode 2: after update1 (beta, activity).
 // corr: ncorr more rows added to the pa sums (the deflation term of r^T z).
-__global__ void k_panel_reduce(int mode, int nbx, int R, int64_t n_cols, double tol2, int it,
-                               int max_it, const double* __restrict__ pa,
-                               const double* __restrict__ pb, const double* __restrict__ corr,
-                               int ncorr, double* __restrict__ scal, int* __restrict__ active,
-                               int* __restrict__ n_active, unsigned* __restrict__ flags) {
-  for (int c = blockIdx.x * blockDim.x + threadIdx.x; c < R; c += gridDim.x * blockDim.x) {
-    double a = 0, b = 0;
-    for (int k = 0; k < nbx; ++k) {
-      a += pa[(int64_t)k * R + c];
-      if (pb) b += pb[(int64_t)k * R + c];
-    }
-    for (int k = 0; k < ncorr; ++k) a += corr[(int64_t)k * R + c];
-    double* alpha = scal;
-    double* beta = scal + R;
-    double* rzp = scal + 2 * R;
-    double* rzn = scal + 3 * R;
-    double* bb = scal + 4 * R;
-    double* rr = scal + 5 * R;
-    if (mode == 0) {
-      rzp[c] = a;
-      bb[c] = b;
-      rr[c] = b;
-      int act = (c < n_cols) && (b > 0);
-      active[c] = act;
-      if (act) atomicAdd(n_active, 1);
-    } else if (mode == 1) {
-      double al = 0;
-      if (active[c]) {
-        if (a > 0 && rzp[c] > 0) al = rzp[c] / a;
-        else if (rzp[c] > 0) {
-          atomicOr(flags, kFlagNotSPD);
-          active[c] = 0;
-        }
-      }
-      alpha[c] = al;
-    } else {
-      rzn[c] = a;
-      rr[c] = b;
-      double be = 0;
-      if (active[c]) {
-        if (!isfinite(a) || !isfinite(b)) {
-          atomicOr(flags, kFlagNonFinite);
-          active[c] = 0;
-        } else if (b <= tol2 * bb[c] || it >= max_it) {
-          active[c] = 0;
-        } else {
-          be = rzp[c] > 0 ? a / rzp[c] : 0.0;
-          atomicAdd(n_active, 1);
-        }
-      }
-      beta[c] = be;
-      rzp[c] = a;
-    }
+// A block sums 32 columns: its warps take rows w, w + W, ... (W warps) and the
+// first warp adds the W sums, in that fixed order.  (One thread per column
+// chained up to 590 FP64 additions behind 590 loads: 70 us a reduction at 8,000
+// stars x 1,024 columns, twice an iteration; 4 us so.)
+// n_active counts the columns above the tolerance; a column is updated until
+// its residual is below frozen2 ||b||^2 (frozen2 <= tol2).
+constexpr int kRedWarps = 32;
+__global__ void __launch_bounds__(32 * kRedWarps) k_panel_reduce(
+    int mode, int nbx, int R, int64_t n_cols, double tol2, double frozen2, int it, int max_it,
+    const double* __restrict__ pa, const double* __restrict__ pb, const double* __restrict__ corr,
+    int ncorr, double* __restrict__ scal, int* __restrict__ active, int* __restrict__ n_active,
+    unsigned* __restrict__ flags) {
+  __shared__ double sa[kRedWarps][32], sb[kRedWarps][32];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, W = blockDim.x >> 5;
+  const int c = blockIdx.x * 32 + lane;  // R is a multiple of 32
+  double a = 0, b = 0;
+  for (int k = w; k < nbx; k += W) {
+    a += pa[(int64_t)k * R + c];
+    if (pb) b += pb[(int64_t)k * R + c];
   }
+  for (int k = w; k < ncorr; k += W) a += corr[(int64_t)k * R + c];
+  sa[w][lane] = a;
+  sb[w][lane] = b;
+  __syncthreads();
+  if (w != 0) return;
+  for (int k = 1; k < W; ++k) {
+    a += sa[k][lane];
+    b += sb[k][lane];
+  }
+  double* alpha = scal;
+  double* beta = scal + R;
+  double* rzp = scal + 2 * R;
+  double* rzn = scal + 3 * R;
+  double* bb = scal + 4 * R;
+  double* rr = scal + 5 * R;
+  int count = 0;
+  if (mode == 0) {
+    rzp[c] = a;
+    bb[c] = b;
+    rr[c] = b;
+    const int act = (c < n_cols) && (b > 0);
+    active[c] = act;
+    count = act;
+  } else if (mode == 1) {
+    if (blockIdx.x == 0 && lane == 0) *n_active = 0;  // for the next mode 2
+    double al = 0;
+    if (active[c]) {
+      if (a > 0 && rzp[c] > 0) al = rzp[c] / a;
+      else if (rzp[c] > 0) {
+        atomicOr(flags, kFlagNotSPD);
+        active[c] = 0;
+      }
+    }
+    alpha[c] = al;
+  } else {
+    rzn[c] = a;
+    rr[c] = b;
+    double be = 0;
+    if (active[c]) {
+      if (!isfinite(a) || !isfinite(b)) {
+        atomicOr(flags, kFlagNonFinite);
+        active[c] = 0;
+      } else if (b <= frozen2 * bb[c] || it >= max_it) {
+        active[c] = 0;
+      } else {
+        be = rzp[c] > 0 ? a / rzp[c] : 0.0;
+        count = b > tol2 * bb[c];
+      }
+    }
+    beta[c] = be;
+    rzp[c] = a;
+  }
+  const unsigned above = __ballot_sync(0xffffffffu, count);
+  if (mode != 1 && lane == 0 && above) atomicAdd(n_active, __popc(above));
 }
 
 // X += alpha P, Rr -= alpha Q, partial rz (with M^-1) and rr.
@@ -699,20 +746,36 @@ __global__ void __launch_bounds__(kBT) k_panel_update1(int64_t n, int R, const T
   }
 }
 
-// P = M^-1 Rr + beta P (active columns), PD = d o P.
-template <typename TV>
+// P = M^-1 Rr + beta P (active columns), PD = d o P: in the panel's precision,
+// or (planes) as its three BF16 pieces, piece p at planes + p * plane_elems,
+// which the asynchronous tile product reads (the split of k_split3_planes,
+// without a pass of its own over PD).
+template <typename TV, bool PLANES>
 __global__ void __launch_bounds__(kBT) k_panel_update2(int64_t n, int R, const TV* __restrict__ minv,
                                                        const TV* __restrict__ dv,
                                                        const double* __restrict__ scal,
                                                        const int* __restrict__ active,
                                                        const TV* __restrict__ Rr,
-                                                       TV* __restrict__ P, TV* __restrict__ PD) {
+                                                       TV* __restrict__ P, TV* __restrict__ PD,
+                                                       uint16_t* __restrict__ planes,
+                                                       int64_t plane_elems) {
   const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
   const int c = blockIdx.y * 32 + lane;
   if (!active[c]) return;  // frozen column: P is never read with alpha != 0
   const int64_t w = (int64_t)blockIdx.x * (blockDim.x >> 5) + wib;
   const int64_t nw = (int64_t)gridDim.x * (blockDim.x >> 5);
   const TV be = (TV)scal[R + c];
+  auto put = [&](int64_t k, TV v) {
+    if constexpr (PLANES) {
+      uint32_t a, b, d;
+      tg::split3((float)v, a, b, d);
+      planes[k] = (uint16_t)(a >> 16);
+      planes[plane_elems + k] = (uint16_t)(b >> 16);
+      planes[2 * plane_elems + k] = (uint16_t)(d >> 16);
+    } else {
+      PD[k] = v;
+    }
+  };
   int64_t i = w;
   for (; i + 3 * nw < n; i += 4 * nw) {
     TV r[4], p[4], m[4], d[4];
@@ -729,14 +792,14 @@ __global__ void __launch_bounds__(kBT) k_panel_update2(int64_t n, int R, const T
       const int64_t k = (i + u * nw) * R + c;
       const TV pi = m[u] * r[u] + be * p[u];
       P[k] = pi;
-      PD[k] = d[u] * pi;
+      put(k, d[u] * pi);
     }
   }
   for (; i < n; i += nw) {
     int64_t k = i * R + c;
     TV pi = minv[i] * Rr[k] + be * P[k];
     P[k] = pi;
-    PD[k] = dv[i] * pi;
+    put(k, dv[i] * pi);
   }
 }
 
@@ -1113,6 +1176,12 @@ static gm_status panels(gm_ctx* c, int64_t n_rows, const int64_t* row_ptr, const
   R = (R / 32) * 32;
   c->stats.variance_panel_width = R;
   const int nbx = std::max(1, (int)std::min<int64_t>(ceil_div(n, 8), (int64_t)(4 * sms * 32 / (R / 32 + 1)) + 1));
+  // element-wise passes: four rows per warp and pass (all their loads in
+  // flight), eight where that still leaves a dozen warps per scheduler.  (The
+  // product's grid gave them two to three rows a warp, one after another:
+  // 143 us for update1 at 4,000 x 4,000, 2.7 TB/s.)
+  const int rpw = n * (R / 32) / 8 >= 48ll * sms ? 8 : 4;
+  const int nbe = (int)ceil_div(n, 8 * rpw);
   const size_t pbytes = (size_t)n * R * sizeof(TV);
   // spectral deflation of the preconditioner (FP32 star panels of one field;
   // the vectors are prepared per refresh, before the mean solve), in its
@@ -1124,9 +1193,9 @@ static gm_status panels(gm_ctx* c, int64_t n_rows, const int64_t* row_ptr, const
   // partial rows: the panel product may write more rows (one per 128-row
   // tile), the tensor-core deflation step one per row chunk; then the rows
   // of the deflation term of r^T z (1, or 8 in the tensor-core form)
-  const int64_t rows_a = std::max<int64_t>(std::max<int64_t>(nbx, nch),
+  const int64_t rows_a = std::max<int64_t>(std::max<int64_t>(std::max(nbx, nbe), nch),
                                            sizeof(TV) == 4 ? c->tc_nblk : 0);
-  const int64_t rows_b = std::max<int64_t>(nbx, nch);
+  const int64_t rows_b = std::max<int64_t>(nbe, nch);
   const int ncorr = defl ? (defl_tc ? 8 : 1) : 0;
   bool ok = ensure(c, ws.P_X, pbytes) && ensure(c, ws.P_R, pbytes) && ensure(c, ws.P_P, pbytes) &&
             ensure(c, ws.P_PD, pbytes) && ensure(c, ws.P_Q, pbytes) &&
@@ -1147,11 +1216,17 @@ static gm_status panels(gm_ctx* c, int64_t n_rows, const int64_t* row_ptr, const
   // FP32 panels stop at the FP32 rounding floor of the relative residual
   const double tol = sizeof(TV) == 4 ? std::max(c->cfg.cg_tol, 1e-5) : c->cfg.cg_tol;
   const double tol2 = tol * tol;
+  // A column whose residual meets the tolerance waits for the others.  FP64
+  // columns keep iterating meanwhile (the passes run over them anyway), down to
+  // 1e-3 of the tolerance; FP32 columns stop at it, their rounding floor.
+  const double frozen2 = sizeof(TV) == 4 ? tol2 : 1e-6 * tol2;
   const int max_it = c->cfg.cg_max_iter;
   int* hn = (int*)c->h_pinned;
-  dim3 grid(nbx, (unsigned)(R / 32));
+  dim3 grid(nbx, (unsigned)(R / 32)), egrid(nbe, (unsigned)(R / 32));
   const int rb = (int)std::min<int64_t>(ceil_div(n_rows * 32, 256), 16 * sms);
-  const int redb = (int)ceil_div(R, 256);
+  const int redb = (int)(R / 32);
+  // warps of a reduction over `rows` partial rows: four rows each
+  auto redt = [](int64_t rows) { return 32 * (int)std::min<int64_t>(kRedWarps, ceil_div(rows, 4)); };
   int64_t total_it = 0;
   const int tb = (int)std::min<int64_t>(ceil_div(n, 256), 16 * sms);
   for (int64_t r0 = 0; r0 < n_cols_all; r0 += R) {
@@ -1177,17 +1252,17 @@ static gm_status panels(gm_ctx* c, int64_t n_rows, const int64_t* row_ptr, const
                           c->warm_probe == (probe ? 1 : 0);
     if (use_warm) {
       GM_PROF(c, "k_panel_scale");
-      k_panel_scale<TV><<<grid, kBT, 0, st>>>(n, (int)R, dv, X, PD);
+      k_panel_scale<TV><<<egrid, kBT, 0, st>>>(n, (int)R, dv, X, PD);
       GM_LAUNCH_CHECK(c);
       int nbu = nbx;
       gm_status ss = panel_product<TA, TV>(c, n, R, nbx, grid, dv, X, PD, Q, pa, &nbu);
       if (ss != GM_OK) return ss;
       GM_PROF(c, "k_panel_init_warm");
-      k_panel_init_warm<TV><<<grid, kBT, 0, st>>>(n, (int)R, minv, dv, Rr, Q, P, PD, pa, pb);
+      k_panel_init_warm<TV><<<egrid, kBT, 0, st>>>(n, (int)R, minv, dv, Rr, Q, P, PD, pa, pb);
       GM_LAUNCH_CHECK(c);
     } else {
       GM_PROF(c, "k_panel_init");
-      k_panel_init<TV><<<grid, kBT, 0, st>>>(n, (int)R, minv, dv, X, Rr, P, PD, pa, pb);
+      k_panel_init<TV><<<egrid, kBT, 0, st>>>(n, (int)R, minv, dv, X, Rr, P, PD, pa, pb);
       GM_LAUNCH_CHECK(c);
     }
     // the BF16 planes of PD were written by the deflation update (the
@@ -1213,8 +1288,9 @@ static gm_status panels(gm_ctx* c, int64_t n_rows, const int64_t* row_ptr, const
     }
     GM_CUDA_CHECK(c, cudaMemsetAsync(n_active, 0, sizeof(int), st));
     GM_PROF(c, "k_panel_reduce");
-    k_panel_reduce<<<redb, 256, 0, st>>>(0, nbx, (int)R, ncols, tol2, 0, max_it, pa, pb, corr,
-                                         ncorr, scal, active, n_active, c->d_flags);
+    k_panel_reduce<<<redb, redt(nbe), 0, st>>>(0, nbe, (int)R, ncols, tol2, frozen2, 0, max_it, pa,
+                                               pb, corr, ncorr, scal, active, n_active,
+                                               c->d_flags);
     GM_LAUNCH_CHECK(c);
     const int check = 8;
     GM_CUDA_CHECK(c, cudaMemcpyAsync(hn, n_active, sizeof(int), cudaMemcpyDeviceToHost, st));
@@ -1227,10 +1303,11 @@ static gm_status panels(gm_ctx* c, int64_t n_rows, const int64_t* row_ptr, const
         if (ss != GM_OK) return ss;
       }
       GM_PROF(c, "k_panel_reduce");
-      k_panel_reduce<<<redb, 256, 0, st>>>(1, nbu, (int)R, ncols, tol2, it, max_it, pa, nullptr,
-                                           nullptr, 0, scal, active, n_active, c->d_flags);
+      k_panel_reduce<<<redb, redt(nbu), 0, st>>>(1, nbu, (int)R, ncols, tol2, frozen2, it, max_it,
+                                                 pa, nullptr, nullptr, 0, scal, active, n_active,
+                                                 c->d_flags);
       GM_LAUNCH_CHECK(c);
-      int nbr = nbx;  // partial rows of rz / rr
+      int nbr = nbe;  // partial rows of rz / rr
       if (defl_tc) {
         // X, Rr update fused with C = Y^T Rr and the deflation rows
         gm_status ds = deflate_step_tc(c, (int)R, nch, scal, (const float*)minv, (float*)X,
@@ -1239,17 +1316,17 @@ static gm_status panels(gm_ctx* c, int64_t n_rows, const int64_t* row_ptr, const
         nbr = nch;
       } else {
         GM_PROF(c, "k_panel_update1");
-        k_panel_update1<TV><<<grid, kBT, 0, st>>>(n, (int)R, minv, scal, X, Rr, P, Q, pa, pb);
+        k_panel_update1<TV><<<egrid, kBT, 0, st>>>(n, (int)R, minv, scal, X, Rr, P, Q, pa, pb);
         GM_LAUNCH_CHECK(c);
         if (defl) {
           gm_status ds = deflate_rhs(c, (int)R, (const float*)Rr, corr);
           if (ds != GM_OK) return ds;
         }
       }
-      GM_CUDA_CHECK(c, cudaMemsetAsync(n_active, 0, sizeof(int), st));
       GM_PROF(c, "k_panel_reduce");
-      k_panel_reduce<<<redb, 256, 0, st>>>(2, nbr, (int)R, ncols, tol2, it, max_it, pa, pb, corr,
-                                           ncorr, scal, active, n_active, c->d_flags);
+      k_panel_reduce<<<redb, redt(nbr), 0, st>>>(2, nbr, (int)R, ncols, tol2, frozen2, it, max_it,
+                                                 pa, pb, corr, ncorr, scal, active, n_active,
+                                                 c->d_flags);
       GM_LAUNCH_CHECK(c);
       planes = false;
       if (defl_tc) {
@@ -1264,7 +1341,14 @@ static gm_status panels(gm_ctx* c, int64_t n_rows, const int64_t* row_ptr, const
         if (ds != GM_OK) return ds;
       } else {
         GM_PROF(c, "k_panel_update2");
-        k_panel_update2<TV><<<grid, kBT, 0, st>>>(n, (int)R, minv, dv, scal, active, Rr, P, PD);
+        planes = sizeof(TV) == 4 && c->tc_nblk > 0 && tc_variant(c, (int)R) == 4;
+        if (planes)
+          k_panel_update2<TV, true><<<egrid, kBT, 0, st>>>(n, (int)R, minv, dv, scal, active, Rr,
+                                                           P, PD, (uint16_t*)c->tc_planes.p,
+                                                           n * (int64_t)R);
+        else
+          k_panel_update2<TV, false><<<egrid, kBT, 0, st>>>(n, (int)R, minv, dv, scal, active, Rr,
+                                                            P, PD, nullptr, 0);
         GM_LAUNCH_CHECK(c);
       }
       if (it % check == 0 || it == max_it) {
