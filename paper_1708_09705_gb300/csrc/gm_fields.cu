@@ -22,10 +22,15 @@
 #include <vector>
 
 #include "gm_internal.cuh"
+#include "gm_tcgen05.cuh"
 
 namespace gm {
 
-constexpr int kSeg = 256;  // rows per element-wise work item
+// Rows per element-wise work item.  256 rows, one after another, left 16 fields
+// of a thousand stars on 520 warps and their element-wise passes at 75 us each;
+// 64 rows, four loads of each array in flight, keep the chip busy at the same
+// number of partial rows per thousand stars as warps that share a column.
+constexpr int kSeg = 64;
 constexpr int kTileF = 32;
 
 struct PackField {
@@ -121,10 +126,38 @@ __global__ void k_pk_rhs_probe(int64_t n, const int32_t* __restrict__ field_of,
   }
 }
 
+// The same with a warp per row, for colourings at least 2 x cutoff apart: a
+// row's neighbours then have distinct colours, so every entry is written once
+// (added to zero: the same bits; see the single-panel solver).
+__global__ void k_pk_rhs_probe_w(int64_t n, const int32_t* __restrict__ field_of,
+                                 const PackField* __restrict__ pf,
+                                 const int64_t* __restrict__ row_ptr,
+                                 const int32_t* __restrict__ col, const float* __restrict__ val,
+                                 const float* __restrict__ dv, const double* __restrict__ tau,
+                                 const double* __restrict__ kd, const int32_t* __restrict__ pcol,
+                                 float* __restrict__ Rr) {
+  const int lane = threadIdx.x & 31;
+  const int64_t warp = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
+  const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
+  for (int64_t j = warp; j < n; j += nw) {
+    const PackField F = pf[field_of[j]];
+    float* row = Rr + F.P + (j - F.row0) * F.W;
+    const float dj = dv[j];
+    for (int64_t e = row_ptr[j] + lane; e < row_ptr[j + 1]; e += 32) {
+      const int32_t r = col[e];
+      if (tau[r] * kd[r] >= 1.0) continue;
+      atomicAdd(row + pcol[r], dj * val[e]);
+    }
+    if (lane == 0 && tau[j] * kd[j] >= 1.0) atomicAdd(row + pcol[j], 1.f);
+  }
+}
+
 enum { kPkInit = 0, kPkPQ = 1, kPkUpd1 = 2, kPkUpd2 = 3 };
 
 // Element-wise pass over (field, column chunk, row segment) items; one warp
-// per item, lane = column.  Partials pa/pb at PO_f + s W_f + c.
+// per item, lane = column.  Partials pa/pb at PO_f + s W_f + c.  planes (the
+// direction update only, null: none): the three BF16 pieces of PD for the
+// asynchronous tile product instead of PD, piece p at planes + p * plane_elems.
 template <int MODE>
 __global__ void k_pk_elem(int64_t n_items, const int4* __restrict__ items,
                           const PackField* __restrict__ pf, const float* __restrict__ minv,
@@ -132,7 +165,8 @@ __global__ void k_pk_elem(int64_t n_items, const int4* __restrict__ items,
                           int64_t tcols, const int* __restrict__ active, float* __restrict__ X,
                           float* __restrict__ Rr, float* __restrict__ P, float* __restrict__ PD,
                           const float* __restrict__ Q, double* __restrict__ pa,
-                          double* __restrict__ pb) {
+                          double* __restrict__ pb, uint16_t* __restrict__ planes,
+                          int64_t plane_elems) {
   const int lane = threadIdx.x & 31;
   const int64_t warp = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
   const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
@@ -146,28 +180,53 @@ __global__ void k_pk_elem(int64_t n_items, const int4* __restrict__ items,
     if (MODE == kPkUpd2 && !active[gid]) continue;
     const float alpha = MODE == kPkUpd1 ? (float)scal[gid] : 0.f;
     const float beta = MODE == kPkUpd2 ? (float)scal[tcols + gid] : 0.f;
-    for (int64_t i = i0; i < i1; ++i) {
-      const int64_t k = F.P + i * F.W + c;
-      const int64_t r = F.row0 + i;
-      if (MODE == kPkInit) {
-        const float ri = Rr[k], zi = minv[r] * ri;
-        X[k] = 0.f;
-        P[k] = zi;
-        PD[k] = dv[r] * zi;
-        s1.add(ri * zi);
-        s2.add(ri * ri);
-      } else if (MODE == kPkPQ) {
-        s1.add(P[k] * Q[k]);
-      } else if (MODE == kPkUpd1) {
-        X[k] += alpha * P[k];
-        const float ri = Rr[k] - alpha * Q[k];
-        Rr[k] = ri;
-        s1.add(ri * (minv[r] * ri));
-        s2.add(ri * ri);
-      } else {
-        const float pi = minv[r] * Rr[k] + beta * P[k];
-        P[k] = pi;
-        PD[k] = dv[r] * pi;
+    constexpr int U = 4;  // rows in flight
+    for (int64_t ib = i0; ib < i1; ib += U) {
+      float r[U], p[U], q[U], x[U], mi[U], di[U];
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const int64_t i = min(ib + u, i1 - 1);
+        const int64_t k = F.P + i * F.W + c;
+        if (MODE != kPkPQ) r[u] = Rr[k];
+        if (MODE != kPkInit) p[u] = P[k];
+        if (MODE == kPkPQ || MODE == kPkUpd1) q[u] = Q[k];
+        if (MODE == kPkUpd1) x[u] = X[k];
+        if (MODE != kPkPQ) mi[u] = minv[F.row0 + i];
+        if (MODE == kPkInit || MODE == kPkUpd2) di[u] = dv[F.row0 + i];
+      }
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        if (ib + u >= i1) break;
+        const int64_t k = F.P + (ib + u) * F.W + c;
+        if (MODE == kPkInit) {
+          const float zi = mi[u] * r[u];
+          X[k] = 0.f;
+          P[k] = zi;
+          PD[k] = di[u] * zi;
+          s1.add(r[u] * zi);
+          s2.add(r[u] * r[u]);
+        } else if (MODE == kPkPQ) {
+          s1.add(p[u] * q[u]);
+        } else if (MODE == kPkUpd1) {
+          X[k] = x[u] + alpha * p[u];
+          const float ri = r[u] - alpha * q[u];
+          Rr[k] = ri;
+          s1.add(ri * (mi[u] * ri));
+          s2.add(ri * ri);
+        } else {
+          const float pi = mi[u] * r[u] + beta * p[u];
+          P[k] = pi;
+          const float v = di[u] * pi;
+          if (planes) {
+            uint32_t a, b, d;
+            tg::split3(v, a, b, d);
+            planes[k] = (uint16_t)(a >> 16);
+            planes[plane_elems + k] = (uint16_t)(b >> 16);
+            planes[2 * plane_elems + k] = (uint16_t)(d >> 16);
+          } else {
+            PD[k] = v;
+          }
+        }
       }
     }
     if (MODE != kPkUpd2) {
@@ -179,66 +238,82 @@ __global__ void k_pk_elem(int64_t n_items, const int4* __restrict__ items,
 }
 
 // Per-column sums of the partials of its field's segments, and the CG
-// scalars (scal layout: alpha, beta, rz_prev, rz_new, bb, rr; each tcols).
-__global__ void k_pk_reduce(int mode, int64_t tcols, int n_fields, const int64_t* __restrict__ wptr,
-                            const PackField* __restrict__ pf, double tol2,
-                            const double* __restrict__ pa, const double* __restrict__ pb,
-                            double* __restrict__ scal, int* __restrict__ active,
-                            int* __restrict__ n_active, unsigned* __restrict__ flags) {
-  for (int64_t gid = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; gid < tcols;
-       gid += (int64_t)gridDim.x * blockDim.x) {
-    int lo = 0, hi = n_fields;  // field: wptr[lo] <= gid < wptr[lo+1]
-    while (hi - lo > 1) {
-      int mid = (lo + hi) >> 1;
-      if (wptr[mid] <= gid) lo = mid; else hi = mid;
-    }
-    const PackField F = pf[lo];
-    const int64_t c = gid - F.Wptr;
-    double a = 0, b = 0;
-    for (int64_t s = 0; s < F.S; ++s) {
-      a += pa[F.PO + s * F.W + c];
-      if (pb) b += pb[F.PO + s * F.W + c];
-    }
-    double* alpha = scal;
-    double* beta = scal + tcols;
-    double* rzp = scal + 2 * tcols;
-    double* bb = scal + 4 * tcols;
-    double* rr = scal + 5 * tcols;
-    if (mode == 0) {
-      rzp[gid] = a;
-      bb[gid] = b;
-      rr[gid] = b;
-      const int act = (c < F.nrows) && (b > 0);
-      active[gid] = act;
-      if (act) atomicAdd(n_active, 1);
-    } else if (mode == 1) {
-      double al = 0;
-      if (active[gid]) {
-        if (a > 0 && rzp[gid] > 0) al = rzp[gid] / a;
-        else if (rzp[gid] > 0) {
-          atomicOr(flags, kFlagNotSPD);
-          active[gid] = 0;
-        }
-      }
-      alpha[gid] = al;
-    } else {
-      rr[gid] = b;
-      double be = 0;
-      if (active[gid]) {
-        if (!isfinite(a) || !isfinite(b)) {
-          atomicOr(flags, kFlagNonFinite);
-          active[gid] = 0;
-        } else if (b <= tol2 * bb[gid]) {
-          active[gid] = 0;
-        } else {
-          be = rzp[gid] > 0 ? a / rzp[gid] : 0.0;
-          atomicAdd(n_active, 1);
-        }
-      }
-      beta[gid] = be;
-      rzp[gid] = a;
-    }
+// scalars (scal layout: alpha, beta, rz_prev, rz_new, bb, rr; each tcols).  A
+// block of warps per 32 columns (a field's width is a multiple of 32): warp w
+// takes segments w, w + W, ..., the first warp adds the W sums in order.
+constexpr int kPkRedWarps = 8;
+__global__ void __launch_bounds__(32 * kPkRedWarps) k_pk_reduce(
+    int mode, int64_t tcols, int n_fields, const int64_t* __restrict__ wptr,
+    const PackField* __restrict__ pf, double tol2, const double* __restrict__ pa,
+    const double* __restrict__ pb, double* __restrict__ scal, int* __restrict__ active,
+    int* __restrict__ n_active, unsigned* __restrict__ flags) {
+  __shared__ double sa[kPkRedWarps][32], sb[kPkRedWarps][32];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int64_t gid = (int64_t)blockIdx.x * 32 + lane;
+  int lo = 0, hi = n_fields;  // field: wptr[lo] <= gid < wptr[lo+1]
+  while (hi - lo > 1) {
+    int mid = (lo + hi) >> 1;
+    if (wptr[mid] <= gid) lo = mid; else hi = mid;
   }
+  const PackField F = pf[lo];
+  const int64_t c = gid - F.Wptr;
+  double a = 0, b = 0;
+  for (int64_t s = w; s < F.S; s += kPkRedWarps) {
+    a += pa[F.PO + s * F.W + c];
+    if (pb) b += pb[F.PO + s * F.W + c];
+  }
+  sa[w][lane] = a;
+  sb[w][lane] = b;
+  __syncthreads();
+  if (w != 0) return;
+#pragma unroll
+  for (int k = 1; k < kPkRedWarps; ++k) {
+    a += sa[k][lane];
+    b += sb[k][lane];
+  }
+  double* alpha = scal;
+  double* beta = scal + tcols;
+  double* rzp = scal + 2 * tcols;
+  double* bb = scal + 4 * tcols;
+  double* rr = scal + 5 * tcols;
+  int count = 0;
+  if (mode == 0) {
+    rzp[gid] = a;
+    bb[gid] = b;
+    rr[gid] = b;
+    const int act = (c < F.nrows) && (b > 0);
+    active[gid] = act;
+    count = act;
+  } else if (mode == 1) {
+    if (gid == 0) *n_active = 0;  // for the next mode 2
+    double al = 0;
+    if (active[gid]) {
+      if (a > 0 && rzp[gid] > 0) al = rzp[gid] / a;
+      else if (rzp[gid] > 0) {
+        atomicOr(flags, kFlagNotSPD);
+        active[gid] = 0;
+      }
+    }
+    alpha[gid] = al;
+  } else {
+    rr[gid] = b;
+    double be = 0;
+    if (active[gid]) {
+      if (!isfinite(a) || !isfinite(b)) {
+        atomicOr(flags, kFlagNonFinite);
+        active[gid] = 0;
+      } else if (b <= tol2 * bb[gid]) {
+        active[gid] = 0;
+      } else {
+        be = rzp[gid] > 0 ? a / rzp[gid] : 0.0;
+        count = 1;
+      }
+    }
+    beta[gid] = be;
+    rzp[gid] = a;
+  }
+  const unsigned above = __ballot_sync(0xffffffffu, count);
+  if (mode != 1 && lane == 0 && above) atomicAdd(n_active, __popc(above));
 }
 
 // Q = P + d o (K PD) for all fields: item = (row block b, group of WPB
@@ -456,11 +531,12 @@ static gm_status pack_setup(gm_ctx* c) {
   return GM_OK;
 }
 
-static void launch_spmm(gm_ctx* c, PackState& S, int wpb, cudaStream_t st, const float* dv) {
+static void launch_spmm(gm_ctx* c, PackState& S, int wpb, cudaStream_t st, const float* dv,
+                        bool planes_ready = false) {
   if (S.n_tc_items > 0) {
     panel_spmm_tc_packed(c, S.n_tc_items, S.tc_items, S.tc_base, S.tc_width, dv,
                          (const float*)S.Pp.p, (const float*)S.PD.p, (float*)S.Q.p,
-                         (int64_t)(S.PD.bytes / sizeof(float)), st, false);
+                         (int64_t)(S.PD.bytes / sizeof(float)), st, false, planes_ready);
     return;
   }
   const int sms = sm_count(c);
@@ -535,13 +611,18 @@ gm_status panels_fields(gm_ctx* c, const float* dv, const float* minv, const dou
   const double tol2 = tol * tol;
   const int wb = (int)std::min<int64_t>(ceil_div(n * 32, 256), 16 * sms);
   const int ib = (int)std::min<int64_t>(ceil_div(S.n_eitems * 32, 256), 16 * sms);
-  const int rb = (int)std::min<int64_t>(ceil_div(tc, 256), 8 * sms);
+  const unsigned rb = (unsigned)(tc / 32);
   const int nf = c->n_fields;
   const bool probe = c->probe_colour && c->probe_factor_done > 0;
   GM_CUDA_CHECK(c, cudaMemsetAsync(Rr, 0, (size_t)S.total_elems * sizeof(float), st));
   if (probe) {
     GM_PROF(c, "k_pk_rhs_probe");
-    k_pk_rhs_probe<<<(int)std::min<int64_t>(ceil_div(n, 256), 16 * sms), 256, 0, st>>>(
+    if (c->probe_factor_done >= 2.0)
+      k_pk_rhs_probe_w<<<wb, 256, 0, st>>>(n, c->field_of, S.pf, c->row_ptr, c->col,
+                                           (const float*)c->val, dv, c->tau, c->kdiag,
+                                           c->probe_colour, Rr);
+    else
+      k_pk_rhs_probe<<<(int)std::min<int64_t>(ceil_div(n, 256), 16 * sms), 256, 0, st>>>(
         n, c->field_of, S.pf, c->row_ptr, c->col, (const float*)c->val, dv, c->tau, c->kdiag,
         c->probe_colour, Rr);
   } else {
@@ -552,11 +633,11 @@ gm_status panels_fields(gm_ctx* c, const float* dv, const float* minv, const dou
   GM_LAUNCH_CHECK(c);
   GM_PROF(c, "k_pk_elem_init");
   k_pk_elem<kPkInit><<<ib, 256, 0, st>>>(S.n_eitems, S.eitems, S.pf, minv, dv, scal, tc, active,
-                                         X, Rr, P, PD, Q, pa, pb);
+                                         X, Rr, P, PD, Q, pa, pb, nullptr, 0);
   GM_LAUNCH_CHECK(c);
   GM_CUDA_CHECK(c, cudaMemsetAsync(n_active, 0, sizeof(int), st));
   GM_PROF(c, "k_pk_reduce");
-  k_pk_reduce<<<rb, 256, 0, st>>>(0, tc, nf, S.wptr, S.pf, tol2, pa, pb, scal, active, n_active,
+  k_pk_reduce<<<rb, 32 * kPkRedWarps, 0, st>>>(0, tc, nf, S.wptr, S.pf, tol2, pa, pb, scal, active, n_active,
                                   c->d_flags);
   GM_LAUNCH_CHECK(c);
   int* hn = (int*)c->h_pinned;
@@ -566,6 +647,15 @@ gm_status panels_fields(gm_ctx* c, const float* dv, const float* minv, const dou
   if (*hn > 0) {
     s = autotune(c, S, dv);
     if (s != GM_OK) return s;
+    // with the asynchronous tile product the direction update writes the BF16
+    // planes of PD itself; the first directions are split here
+    const bool planes = S.n_tc_items > 0 && c->tc_pf == 4;
+    const int64_t pe = (int64_t)(S.PD.bytes / sizeof(float));
+    if (planes) {
+      s = tc_split_planes(c, PD, pe);
+      if (s != GM_OK) return s;
+    }
+    uint16_t* pl = planes ? (uint16_t*)c->tc_planes.p : nullptr;
     // one CUDA graph = 8 CG iterations on the private stream
     const int chunk = 8;
     GM_CUDA_CHECK(c, cudaEventRecord(S.ev0, st));
@@ -574,18 +664,17 @@ gm_status panels_fields(gm_ctx* c, const float* dv, const float* minv, const dou
     cudaGraphExec_t exec = nullptr;
     GM_CUDA_CHECK(c, cudaStreamBeginCapture(S.gstream, cudaStreamCaptureModeThreadLocal));
     for (int k = 0; k < chunk; ++k) {
-      launch_spmm(c, S, S.wpb, S.gstream, dv);
+      launch_spmm(c, S, S.wpb, S.gstream, dv, planes);
       k_pk_elem<kPkPQ><<<ib, 256, 0, S.gstream>>>(S.n_eitems, S.eitems, S.pf, minv, dv, scal, tc,
-                                                  active, X, Rr, P, PD, Q, pa, pb);
-      k_pk_reduce<<<rb, 256, 0, S.gstream>>>(1, tc, nf, S.wptr, S.pf, tol2, pa, nullptr, scal,
+                                                  active, X, Rr, P, PD, Q, pa, pb, nullptr, 0);
+      k_pk_reduce<<<rb, 32 * kPkRedWarps, 0, S.gstream>>>(1, tc, nf, S.wptr, S.pf, tol2, pa, nullptr, scal,
                                              active, n_active, c->d_flags);
       k_pk_elem<kPkUpd1><<<ib, 256, 0, S.gstream>>>(S.n_eitems, S.eitems, S.pf, minv, dv, scal, tc,
-                                                    active, X, Rr, P, PD, Q, pa, pb);
-      cudaMemsetAsync(n_active, 0, sizeof(int), S.gstream);
-      k_pk_reduce<<<rb, 256, 0, S.gstream>>>(2, tc, nf, S.wptr, S.pf, tol2, pa, pb, scal, active,
+                                                    active, X, Rr, P, PD, Q, pa, pb, nullptr, 0);
+      k_pk_reduce<<<rb, 32 * kPkRedWarps, 0, S.gstream>>>(2, tc, nf, S.wptr, S.pf, tol2, pa, pb, scal, active,
                                              n_active, c->d_flags);
       k_pk_elem<kPkUpd2><<<ib, 256, 0, S.gstream>>>(S.n_eitems, S.eitems, S.pf, minv, dv, scal, tc,
-                                                    active, X, Rr, P, PD, Q, pa, pb);
+                                                    active, X, Rr, P, PD, Q, pa, pb, pl, pe);
     }
     cudaError_t ce = cudaStreamEndCapture(S.gstream, &graph);
     if (ce != cudaSuccess) return cuda_fail(c, ce, "graph capture");
@@ -595,7 +684,7 @@ gm_status panels_fields(gm_ctx* c, const float* dv, const float* minv, const dou
       c->prof_stream = S.gstream;
       GM_PROF(c, "graph_cg8");
       GM_CUDA_CHECK(c, cudaGraphLaunch(exec, S.gstream));
-      c->launches += 6 * chunk - 1;
+      c->launches += 6 * chunk - 1;  // kernels of the graph
       GM_LAUNCH_CHECK(c);
       c->prof_stream = nullptr;
       iters += chunk;

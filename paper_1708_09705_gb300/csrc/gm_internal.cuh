@@ -354,7 +354,9 @@ int tc_variant(gm_ctx* c, int R);
 gm_status panel_spmm_tc_packed(gm_ctx* c, int64_t n_items, const int2* items,
                                const int64_t* blk_base, const int32_t* blk_width, const float* dv,
                                const float* P, const float* PD, float* Q, int64_t pd_elems,
-                               cudaStream_t st, bool tune);
+                               cudaStream_t st, bool tune, bool planes_ready = false);
+// BF16 planes of PD into c->tc_planes (plane stride pd_elems), context stream
+gm_status tc_split_planes(gm_ctx* c, const float* PD, int64_t pd_elems);
 
 // Q = B P for an n x R FP32 panel with PD = d o P given (the variance panels'
 // product); part: max(tile blocks, ceil(n / 8)) x R doubles of scratch.

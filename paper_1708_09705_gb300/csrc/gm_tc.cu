@@ -1460,12 +1460,25 @@ int tc_variant(gm_ctx* c, int R) { return R <= kTcCols ? c->tc_pf_narrow : c->tc
 gm_status panel_spmm_tc_packed(gm_ctx* c, int64_t n_items, const int2* items,
                                const int64_t* blk_base, const int32_t* blk_width, const float* dv,
                                const float* P, const float* PD, float* Q, int64_t pd_elems,
-                               cudaStream_t st, bool tune) {
+                               cudaStream_t st, bool tune, bool planes_ready) {
   const TcPanels pk{blk_base, blk_width, (const int64_t*)c->tc_brow0.p, items,
                     c->tc_order ? (const int32_t*)c->tc_trow.p : nullptr};
   dim3 grid((unsigned)n_items);
   if (tune) return tc_tune(c, grid, c->n, 0, dv, P, PD, Q, nullptr, pk, pd_elems, c->tc_pf);
-  return launch_tc(c, c->tc_pf, grid, c->n, 0, dv, P, PD, Q, nullptr, pk, pd_elems, st);
+  return launch_tc(c, c->tc_pf, grid, c->n, 0, dv, P, PD, Q, nullptr, pk, pd_elems, st,
+                   planes_ready);
+}
+
+// The BF16 planes of PD (plane stride pd_elems) on the context stream.
+gm_status tc_split_planes(gm_ctx* c, const float* PD, int64_t pd_elems) {
+  if (!ensure(c, c->tc_planes, (size_t)std::max<int64_t>(pd_elems, 1) * 3 * sizeof(uint16_t)))
+    return set_error(c, GM_E_NOMEM, "BF16 planes of the panel");
+  const int sb = (int)std::min<int64_t>(std::max<int64_t>(ceil_div(pd_elems, 4 * 256), 1),
+                                        8 * sm_count(c));
+  GM_PROF(c, "k_split3_planes");
+  k_split3_planes<<<sb, 256, 0, c->stream>>>(pd_elems, PD, (uint16_t*)c->tc_planes.p);
+  GM_LAUNCH_CHECK(c);
+  return GM_OK;
 }
 
 }  // namespace gm
