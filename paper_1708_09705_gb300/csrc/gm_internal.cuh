@@ -130,6 +130,9 @@ struct gm_ctx {
   std::vector<int64_t> h_tc_boff;   // first tile block of each field (n_fields + 1)
   gm::Buffer tc_brow0, tc_boffd;    // first row of each block (+ end); device h_tc_boff
   gm::Buffer tc_trow, tc_tpos;      // tile order: row at tile position p, position of row i
+  gm::Buffer tc64_erow, tc64_ecol;  // FP64 form: exponents of K's rows and the panel's columns
+  int tc64_state = 0;               // FP64 tiles: 0 not asked for, 1 built, -1 do not fit
+  bool tc64_use = false;            // the current panels run on them
   bool tc_order = false;            // tc_trow / tc_tpos in use (else position = row)
   int tc_pf = 0;                    // tuned variant of the tile product (0: untuned) for
                                     // panels wider than one column group (and packed panels)
@@ -340,6 +343,18 @@ gm_status self_quadrature(gm_ctx* c, int64_t n_rows, const double* rs, double* k
 // Colour classes for probed variances when cfg.probe_factor > 0 (gm_probe.cu).
 gm_status probe_colouring(gm_ctx* c);
 
+// FP64 panel product on the tensor cores (gm_tc64.cu) over the tiles of gm_tc.cu:
+// tc64_prepare decides for a panel of n_cols right-hand sides (c->tc64_use) and
+// builds them on first use.
+// From kTc64MinWork products of stored entries and columns on: with its exponents
+// and digit planes the product takes 48 us at 400 stars x 416 columns (6e6), the
+// FP64 units 39; 232 against 1,306 us at 2,001 x 2,016 (7e8).
+constexpr double kTc64MinWork = 1.5e7;
+gm_status tc64_prepare(gm_ctx* c, int64_t n_cols);
+gm_status tc64_fill(gm_ctx* c, const int64_t* bptr, const int32_t* ucol);
+size_t tc64_kstep_bytes();
+gm_status panel_spmm_tc64(gm_ctx* c, int64_t n, int R, const double* dv, const double* P,
+                          const double* PD, double* Q, double* part_pq);
 // 128-row tiles and the tensor-core panel product (gm_tc.cu).
 bool tc_wanted(gm_ctx* c);
 gm_status tc_tiles_build(gm_ctx* c);

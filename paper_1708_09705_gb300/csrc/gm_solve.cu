@@ -1121,6 +1121,11 @@ static gm_status panel_product(gm_ctx* c, int64_t n, int64_t R, int nbx, dim3 gr
     return panel_spmm_tc(c, n, (int)R, (const float*)dv, (const float*)P, (const float*)PD,
                          (float*)Q, pa, planes_ready);
   }
+  if (sizeof(TV) == 8 && c->tc64_use) {
+    *nbx_used = (int)c->tc_nblk;
+    return panel_spmm_tc64(c, n, (int)R, (const double*)dv, (const double*)P, (const double*)PD,
+                           (double*)Q, pa);
+  }
   if (sizeof(TV) == 4 && c->t_nblk > 0)
     return panel_spmm_tiled(c, n, (int)R, nbx, (const float*)dv, (const float*)P,
                             (const float*)PD, (float*)Q, pa);
@@ -1157,6 +1162,10 @@ static gm_status panels(gm_ctx* c, int64_t n_rows, const int64_t* row_ptr, const
   const int64_t n = c->n;
   cudaStream_t st = c->stream;
   const int sms = sm_count(c);
+  if (sizeof(TV) == 8) {
+    const gm_status ts = tc64_prepare(c, n_cols_all);
+    if (ts != GM_OK) return ts;
+  }
   // panel width: all rows if they fit a memory budget, in multiples of 32
   int64_t R = c->cfg.rhs_panel > 0 ? c->cfg.rhs_panel : 0;
   if (R == 0) {
@@ -1167,9 +1176,9 @@ static gm_status panels(gm_ctx* c, int64_t n_rows, const int64_t* row_ptr, const
     // arrays already hold (they are reused or replaced), at most 160 GB: the
     // width then stays the same from one refresh to the next
     const size_t held = ws.P_X.bytes + ws.P_R.bytes + ws.P_P.bytes + ws.P_PD.bytes +
-                        ws.P_Q.bytes + (sizeof(TV) == 4 ? c->tc_planes.bytes : 0);
+                        ws.P_Q.bytes + c->tc_planes.bytes;
     double budget = std::min<double>(0.5 * ((double)free_b + (double)held), 160e9);
-    const double per = 5.0 * sizeof(TV) + (sizeof(TV) == 4 && c->tc_nblk > 0 ? 6.0 : 0.0);
+    const double per = 5.0 * sizeof(TV) + (sizeof(TV) == 4 ? (c->tc_nblk > 0 ? 6.0 : 0.0) : (c->tc64_use ? 16.0 : 0.0));
     R = (int64_t)(budget / (per * (double)n));
   }
   R = std::max<int64_t>(32, std::min<int64_t>(R, ceil_div(n_cols_all, 32) * 32));
@@ -1194,7 +1203,7 @@ static gm_status panels(gm_ctx* c, int64_t n_rows, const int64_t* row_ptr, const
   // tile), the tensor-core deflation step one per row chunk; then the rows
   // of the deflation term of r^T z (1, or 8 in the tensor-core form)
   const int64_t rows_a = std::max<int64_t>(std::max<int64_t>(std::max(nbx, nbe), nch),
-                                           sizeof(TV) == 4 ? c->tc_nblk : 0);
+                                           c->tc_nblk);
   const int64_t rows_b = std::max<int64_t>(nbe, nch);
   const int ncorr = defl ? (defl_tc ? 8 : 1) : 0;
   bool ok = ensure(c, ws.P_X, pbytes) && ensure(c, ws.P_R, pbytes) && ensure(c, ws.P_P, pbytes) &&

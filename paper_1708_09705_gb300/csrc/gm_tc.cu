@@ -1134,12 +1134,40 @@ bool tc_wanted(gm_ctx* c) {
   return !(e && e[0] == 's');
 }
 
+// FP64 contexts build their tiles when the first large enough panel product needs
+// them (a context that only assembles or runs PIC never does).
+gm_status tc64_prepare(gm_ctx* c, int64_t n_cols) {
+  c->tc64_use = false;
+  if (c->cfg.precision == GM_PREC_FP32 || c->n_fields > 1 || c->tc64_state < 0) return GM_OK;
+  const char* e = std::getenv("GM_SPMM");  // simt / tc pin the product
+  if (e && e[0] == 's') return GM_OK;
+  if ((double)c->nnz * (double)n_cols < kTc64MinWork && !(e && e[0] == 't')) return GM_OK;
+  if (c->tc64_state == 0) {
+    // the digit images take about 16 bytes per stored entry at a fill of one, a
+    // few times that on sparse tiles; leave them out where memory is short
+    size_t free_b = 0, tot_b = 0;
+    cudaMemGetInfo(&free_b, &tot_b);
+    if ((double)c->nnz * 64.0 > 0.2 * (double)free_b) {
+      c->tc64_state = -1;
+      return GM_OK;
+    }
+    const gm_status s = tc_tiles_build(c);
+    if (s != GM_OK) return s;
+    c->tc64_state = 1;
+  }
+  c->tc64_use = true;
+  return GM_OK;
+}
+
 gm_status tc_tiles_build(gm_ctx* c) {
   c->tc_nblk = 0;
   c->stats.tile_ksteps = 0;
   const int64_t n = c->n, nnz = c->nnz;
   cudaStream_t st = c->stream;
   const int sms = sm_count(c);
+  // operand images of a K-step: three BF16 pieces, or the FP64 form's digits
+  const bool f64 = c->cfg.precision != GM_PREC_FP32;
+  const size_t kbytes = f64 ? tc64_kstep_bytes() : (size_t)3 * kTcA;
   // field-aligned blocks of 128 rows
   const int nf = c->n_fields;
   c->h_tc_boff.assign(nf + 1, 0);
@@ -1239,7 +1267,7 @@ gm_status tc_tiles_build(gm_ctx* c) {
     if (!ucol) return set_error(c, GM_E_NOMEM, "tensor-core tile union");
     if (!ensure(c, c->tc_kbase, (nblk + 1) * sizeof(int64_t)) ||
         !ensure(c, c->tc_upad, std::max<int64_t>(nks, 1) * kTcK * sizeof(int32_t)) ||
-        !ensure(c, c->tc_img, std::max<int64_t>(nks, 1) * 3 * kTcA))
+        !ensure(c, c->tc_img, std::max<int64_t>(nks, 1) * kbytes))
       return set_error(c, GM_E_NOMEM, "tensor-core tiles");
     GM_CUDA_CHECK(c, cudaMemcpyAsync(bptr, hb.data(), (nblk + 1) * sizeof(int64_t),
                                      cudaMemcpyHostToDevice, st));
@@ -1290,7 +1318,7 @@ gm_status tc_tiles_build(gm_ctx* c) {
     nks = hk[nblk];
     if (!ensure(c, c->tc_kbase, (nblk + 1) * sizeof(int64_t)) ||
         !ensure(c, c->tc_upad, std::max<int64_t>(nks, 1) * kTcK * sizeof(int32_t)) ||
-        !ensure(c, c->tc_img, std::max<int64_t>(nks, 1) * 3 * kTcA))
+        !ensure(c, c->tc_img, std::max<int64_t>(nks, 1) * kbytes))
       return set_error(c, GM_E_NOMEM, "tensor-core tiles");
     GM_CUDA_CHECK(c, cudaMemcpyAsync(c->tc_kbase.p, hk.data(), (nblk + 1) * sizeof(int64_t),
                                      cudaMemcpyHostToDevice, st));
@@ -1301,12 +1329,17 @@ gm_status tc_tiles_build(gm_ctx* c) {
     GM_CUDA_CHECK(c, cudaStreamSynchronize(st));  // the scoped scratch is released here
   }
   int64_t* kbase = (int64_t*)c->tc_kbase.p;
-  GM_CUDA_CHECK(c, cudaMemsetAsync(c->tc_img.p, 0, (size_t)nks * 3 * kTcA, st));
+  GM_CUDA_CHECK(c, cudaMemsetAsync(c->tc_img.p, 0, (size_t)nks * kbytes, st));
+  if (f64) {
+    const gm_status fs = tc64_fill(c, bptr, ucol);
+    if (fs != GM_OK) return fs;
+  } else {
   GM_PROF(c, "k_tc_fill");
   k_tc_fill<<<wb, 256, 0, st>>>(n, c->row_ptr, c->col, (const float*)c->val, bptr, kbase, ucol,
                                 tb, tpos, (const int64_t*)c->tc_brow0.p,
                                 (unsigned char*)c->tc_img.p);
   GM_LAUNCH_CHECK(c);
+  }
   GM_CUDA_CHECK(c, cudaStreamSynchronize(st));
   dev_free_now(c, bptr, (nblk + 1) * sizeof(int64_t));
   dev_free_now(c, ucol, std::max<int64_t>(U, 1) * sizeof(int32_t));
