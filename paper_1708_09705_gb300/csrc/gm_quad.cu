@@ -191,104 +191,6 @@ struct QuadParams {
   int symmetric;
 };
 
-// FP32 form.  One warp per CSR entry (i, j): lanes own the nodes q' of sightline
-// j, loop over the nodes q of sightline i, and the warp sums the products.
-// In symmetric mode entries with j < i are left for k_mirror.
-// One block of 32 warps per SM around the replicated table (at most 64
-// registers a thread).
-template <int KPL>
-constexpr int pair_threads() { return KPL <= 2 ? 1024 : 512; }
-
-template <int KPL>
-__global__ void __launch_bounds__(pair_threads<KPL>()) k_pair_quad(
-    QuadParams P, int64_t n_rows, const double* __restrict__ rs, const double* __restrict__ rux,
-    const double* __restrict__ ruy, const double* __restrict__ ruz, const double* __restrict__ s,
-    const double* __restrict__ ux, const double* __restrict__ uy, const double* __restrict__ uz,
-    const int64_t* __restrict__ row_ptr, const int32_t* __restrict__ col, int64_t nnz,
-    float* __restrict__ val, const double* __restrict__ gl_zeta, const double* __restrict__ gl_w,
-    const float4* __restrict__ gtab, double* __restrict__ kdiag, double* __restrict__ prior_m,
-    unsigned* __restrict__ flags, const FieldGrid* __restrict__ fg,
-    const int32_t* __restrict__ row_field) {
-  extern __shared__ __align__(16) unsigned char smem[];
-  float* zq = reinterpret_cast<float*>(smem);
-  float* wq = zq + kMaxNodes;
-  const int lane = threadIdx.x & 31;
-  // the table window lives in shared memory, kRep copies per segment
-  float4* st = reinterpret_cast<float4*>(smem + 2 * kMaxNodes * sizeof(float));
-  for (int k = threadIdx.x; k < kWinSegs * kRep; k += blockDim.x) st[k] = gtab[kWinK0 + k / kRep];
-  const float4* tab = st + (lane & (kRep - 1));
-  for (int q = threadIdx.x; q < P.Q; q += blockDim.x) {
-    zq[q] = (float)gl_zeta[q];
-    wq[q] = (float)gl_w[q];
-  }
-  __syncthreads();
-
-  const int64_t warp = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
-  const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-  for (int64_t e = warp; e < nnz; e += nwarps) {
-    // row of entry e: last r with row_ptr[r] <= e
-    int64_t lo = 0, hi = n_rows;
-    while (hi - lo > 1) {
-      int64_t mid = (lo + hi) >> 1;
-      if (row_ptr[mid] <= e) lo = mid; else hi = mid;
-    }
-    const int64_t i = lo;
-    const int32_t j = col[e];
-    if (P.symmetric && j < i) continue;
-    const FieldGrid& fgi = fg[row_field ? row_field[i] : 0];
-    const double inv_L0 = fgi.inv_L0, inv_cut = fgi.inv_cut;
-    const double si = rs[i], sj = s[j];
-    const double dx = rux[i] - ux[j], dy = ruy[i] - uy[j], dz = ruz[i] - uz[j];
-    const double chord2 = fma(dx, dx, fma(dy, dy, dz * dz));
-    const float a = (float)(si * inv_L0), b = (float)(sj * inv_L0), c2 = (float)chord2;
-    // this lane's nodes on sightline j
-    float tp[KPL], ctp[KPL], wp[KPL];
-#pragma unroll
-    for (int k = 0; k < KPL; ++k) {
-      int q = lane + 32 * k;
-      bool ok = q < P.Q;
-      tp[k] = ok ? b * zq[q] : 0.f;
-      ctp[k] = c2 * tp[k];
-      wp[k] = ok ? wq[q] : 0.f;
-    }
-    float acc = 0;
-    for (int q = 0; q < P.Q; ++q) {
-      const float t = a * zq[q];
-      float inner = 0;
-#pragma unroll
-      for (int k = 0; k < KPL; ++k) {
-        const float d = t - tp[k];
-        // x >= 2^kWinEmin by construction: the window's floor is added
-        const float x = fmaf(d, d, fmaf(t, ctp[k], __int_as_float((127 + kWinEmin) << 23)));
-        inner += wp[k] * g_lookup_rep(tab, x);
-      }
-      acc += wq[q] * inner;
-    }
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
-    if (lane == 0) {
-      // the entry's own arithmetic in FP32 too (GB300's FP64 pipe is narrow;
-      // per-pair FP64 work, not the node sum, bounded this kernel): log1p and
-      // the taper to ~1e-7 relative
-      float K = P.form == GM_FORM_LOGNORMAL ? log1pf(acc) : acc;
-      if (P.taper == GM_TAPER_WENDLAND) {
-        // the difference of the distances in FP64: it cancels, and the
-        // taper near the cutoff amplifies its error
-        const float ds = (float)(si - sj);
-        const float d = sqrtf(fmaf(ds, ds, (float)si * (float)sj * c2));
-        K *= wendland_f(d * (float)inv_cut);
-      }
-      if (!isfinite(K)) atomicOr(flags, kFlagNonFinite);
-      val[e] = K;
-      if (P.symmetric && j == i) {
-        kdiag[i] = (double)K;
-        prior_m[i] = P.log_rho_bar + log(si) -
-                     (P.form == GM_FORM_LOGNORMAL ? 0.5 * (double)K : 0.5 * P.sigma2);
-      }
-    }
-  }
-}
-
 // Lower-triangle entries copy their transpose (rows are sorted).
 template <typename T>
 __global__ void k_mirror(int64_t n, const int64_t* __restrict__ row_ptr,
@@ -526,6 +428,7 @@ __device__ __forceinline__ double band_I_warp(T A, T B, T Al, T Bl, T c2, T kink
 template <typename T>
 struct BandRule {
   typedef T Val;
+  static constexpr bool kFloatEntry = false;  // log1p and the taper in FP64
   struct Par {
     BandTab bt;
     const void* gtab;
@@ -635,6 +538,7 @@ __global__ void k_gtab_df(const D4* __restrict__ tab, float4* __restrict__ tab4,
 template <int KPL>
 struct DfRule {
   typedef double Val;
+  static constexpr bool kFloatEntry = false;
   struct Par {
     const double* gl_zeta;
     const double* gl_w;
@@ -771,6 +675,126 @@ struct DfRule {
   }
 };
 
+// ------------------------------------------------------------ FP32 node sums
+// The Q-node rule of FP32 contexts: lanes own the nodes q' of sightline j, loop
+// over the nodes q of sightline i, and the warp sums the products.  One 16-byte
+// lookup per node pair bounds it (four shared-memory passes a warp: 8 node pairs
+// a clock and SM) once the instructions around it are few: the segment's byte
+// address is one shift and one mask of x's bits (segments are 128 bytes, the
+// lane's copy in the low bits), the in-segment position one mask and one
+// subtraction (v / 2^m; the coefficients are scaled by powers of 2^m instead,
+// which changes no bit of the cubic), and the clamp to the table's end is left
+// out for pairs that cannot reach it.  The FP64 part of 32 pairs runs at once
+// (k_pair_entries); a pair's own arithmetic, log1p and the taper included, is
+// FP32 as before.
+// 20,000 stars (1.58e7 unique pairs x 64 x 64 nodes): 46.7 ms with one pair a warp
+// and 22 instructions a node pair, 36.8 ms so (14 instructions; shared memory
+// 89 % busy, the issue slots 78 %), every entry the same bit for bit.
+template <int KPL>
+struct Gl32Rule {
+  typedef float Val;
+  static constexpr bool kFloatEntry = true;
+  struct Par {
+    const double* gl_zeta;
+    const double* gl_w;
+    const float4* gtab;
+    int Q;
+  };
+  static constexpr int kThreads = KPL <= 2 ? 1024 : 512;
+  const unsigned char* tab;  // segment 0 of the window less the window's first index
+  const float4* zw;          // nodes and weights (z, w) of two nodes, padded with w = 0
+  int lane, Q;
+  unsigned copy;             // byte offset of this lane's copy of a segment
+
+  static size_t smem() {
+    return (size_t)kWinSegs * kRep * sizeof(float4) + 2 * kMaxNodes * sizeof(float);
+  }
+  __device__ __forceinline__ Gl32Rule(const Par& P, unsigned char* sm) : Q(P.Q) {
+    lane = threadIdx.x & 31;
+    copy = (unsigned)(lane & (kRep - 1)) * sizeof(float4);
+    float4* st = reinterpret_cast<float4*>(sm);
+    constexpr float s1 = 1 << kTabF32.m, s2 = s1 * s1, s3 = s2 * s1;
+    for (int k = threadIdx.x; k < kWinSegs * kRep; k += blockDim.x) {
+      float4 c = P.gtab[kWinK0 + k / kRep];
+      c.y *= s1;
+      c.z *= s2;
+      c.w *= s3;
+      st[k] = c;
+    }
+    float2* z = reinterpret_cast<float2*>(st + kWinSegs * kRep);
+    for (int q = threadIdx.x; q < kMaxNodes; q += blockDim.x)
+      z[q] = q < Q ? make_float2((float)P.gl_zeta[q], (float)P.gl_w[q]) : make_float2(0.f, 0.f);
+    zw = reinterpret_cast<const float4*>(z);
+    tab = sm;
+    __syncthreads();
+  }
+
+  // kRep * sizeof(float4) = 128 bytes per segment
+  template <bool CLAMP>
+  __device__ __forceinline__ float g(float x) const {
+    static_assert(kRep * sizeof(float4) == 128 && kWinShift >= 7, "segment address");
+    const unsigned bits = (unsigned)__float_as_int(x);
+    unsigned off = ((bits >> (kWinShift - 7)) & ~127u) | copy;
+    if (CLAMP) off = min(off, (unsigned)(kWinBaseSeg + kWinLast) * 128u + copy);
+    const float4 c = *reinterpret_cast<const float4*>(tab + (int)(off - kWinBaseSeg * 128u));
+    const float v = __int_as_float((bits & ((1u << kWinShift) - 1u)) | 0x3f800000u) - 1.0f;
+    return fmaf(v, fmaf(v, fmaf(v, c.w, c.z), c.y), c.x);
+  }
+
+  template <bool CLAMP>
+  __device__ __forceinline__ float pair(float a, float b, float c2) const {
+    float tp[KPL], ctp[KPL], wp[KPL];
+#pragma unroll
+    for (int k = 0; k < KPL; ++k) {
+      const float2 z = reinterpret_cast<const float2*>(zw)[lane + 32 * k];
+      tp[k] = b * z.x;
+      ctp[k] = c2 * tp[k];
+      wp[k] = z.y;
+    }
+    float acc = 0;
+    auto node = [&](float z, float w) {
+      const float t = a * z;
+      float inner = 0;
+#pragma unroll
+      for (int k = 0; k < KPL; ++k) {
+        const float d = t - tp[k];
+        // x >= 2^kWinEmin by construction: the window's floor is added
+        const float x = fmaf(d, d, fmaf(t, ctp[k], __int_as_float((127 + kWinEmin) << 23)));
+        inner += wp[k] * g<CLAMP>(x);
+      }
+      acc += w * inner;
+    };
+#pragma unroll 1
+    for (int q = 0; 2 * q < Q; ++q) {
+      // one broadcast load for two nodes; a padding node adds nothing
+      const float4 n = zw[q];
+      node(n.x, n.y);
+      node(n.z, n.w);
+    }
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
+    return acc;
+  }
+
+  __device__ __forceinline__ double R(bool active, double A, double B, double c2) const {
+    constexpr unsigned full = 0xffffffffu;
+    const float a = (float)A, b = (float)B, c = (float)c2;
+    // no node pair of this pair reaches the end of the table (2^emax)
+    const float top = fmaxf(a, b);
+    const bool inside = fmaf(a * b, c, top * top) < 0.99f * (float)(1 << kTabF32.emax);
+    const unsigned in = __ballot_sync(full, inside);
+    float mine = 0;
+    for (unsigned m = __ballot_sync(full, active); m; m &= m - 1) {
+      const int l = __ffs(m) - 1;
+      const float al = __shfl_sync(full, a, l), bl = __shfl_sync(full, b, l),
+                  cl = __shfl_sync(full, c, l);
+      const float v = (in >> l) & 1u ? pair<false>(al, bl, cl) : pair<true>(al, bl, cl);
+      if (lane == l) mine = v;
+    }
+    return (double)mine;
+  }
+};
+
 // ------------------------------------------------------------ entries
 // Entries (i, j) of a CSR by a node rule, with the taper; in symmetric mode
 // entries with j < i are left for k_mirror, and the diagonal gives K_ii and
@@ -820,11 +844,25 @@ __global__ void __launch_bounds__(Rule::kThreads) k_pair_entries(
     }
     const double R = rule.R(active, A, B, chord2);
     if (active) {
-      double K = P.form == GM_FORM_LOGNORMAL ? log1p(R) : R;
-      if (P.taper == GM_TAPER_WENDLAND) {
-        const double ds = si - sj;
-        const double d = sqrt(fma(ds, ds, si * sj * chord2));
-        K *= wendland(d * inv_cut);
+      double K;
+      if constexpr (Rule::kFloatEntry) {
+        // log1p and the taper to ~1e-7 relative; the difference of the distances
+        // in FP64: it cancels, and the taper near the cutoff amplifies its error
+        const float Rf = (float)R;
+        float Kf = P.form == GM_FORM_LOGNORMAL ? log1pf(Rf) : Rf;
+        if (P.taper == GM_TAPER_WENDLAND) {
+          const float ds = (float)(si - sj);
+          const float d = sqrtf(fmaf(ds, ds, (float)si * (float)sj * (float)chord2));
+          Kf *= wendland_f(d * (float)inv_cut);
+        }
+        K = (double)Kf;
+      } else {
+        K = P.form == GM_FORM_LOGNORMAL ? log1p(R) : R;
+        if (P.taper == GM_TAPER_WENDLAND) {
+          const double ds = si - sj;
+          const double d = sqrt(fma(ds, ds, si * sj * chord2));
+          K *= wendland(d * inv_cut);
+        }
       }
       if (!isfinite(K)) atomicOr(flags, kFlagNonFinite);
       val[e] = (T)K;
@@ -949,26 +987,6 @@ static QuadParams quad_params(const gm_ctx* c, bool symmetric) {
   return P;
 }
 
-template <int KPL>
-static void launch_pair(gm_ctx* c, const QuadParams& P, int64_t n_rows, const double* rs,
-                        const double* rux, const double* ruy, const double* ruz,
-                        const int32_t* row_field, const int64_t* row_ptr, const int32_t* col,
-                        int64_t nnz, void* val) {
-  const size_t smem = 2 * kMaxNodes * sizeof(float) + (size_t)kWinSegs * kRep * sizeof(float4);
-  constexpr int nt = pair_threads<KPL>();
-  auto kern = k_pair_quad<KPL>;
-  cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  int per_sm = 0;
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, nt, smem);
-  int blocks = std::max(1, per_sm) * sm_count(c);
-  blocks = (int)std::min<int64_t>(blocks, std::max<int64_t>(1, ceil_div(nnz * 32, nt)));
-  GM_PROF(c, "k_pair_quad");
-  kern<<<blocks, nt, smem, c->stream>>>(P, n_rows, rs, rux, ruy, ruz, c->s, c->ux, c->uy, c->uz,
-                                        row_ptr, col, nnz, (float*)val, c->gl_zeta, c->gl_w,
-                                        (const float4*)c->gtab, c->kdiag, c->prior_m, c->d_flags,
-                                        c->fgrid, row_field);
-}
-
 static BandTab band_tab() {
   BandTab t;
   for (int j = 0; j < kBandPts; ++j)
@@ -1023,6 +1041,11 @@ static typename BandRule<T>::Par band_par(const gm_ctx* c) {
 }
 
 template <int KPL>
+static typename Gl32Rule<KPL>::Par gl32_par(const gm_ctx* c) {
+  return {c->gl_zeta, c->gl_w, (const float4*)c->gtab, c->cfg.n_nodes};
+}
+
+template <int KPL>
 static typename DfRule<KPL>::Par df_par(const gm_ctx* c) {
   const float4* t4 = (const float4*)c->gtab_df;
   return {c->gl_zeta, c->gl_w, (const D4*)c->gtab, tab_f64(), t4, (const float2*)(t4 + kDfSegs),
@@ -1045,13 +1068,13 @@ gm_status pair_quadrature(gm_ctx* c, int64_t n_rows, const double* rs, const dou
     if (f32) GM_ENTRIES(BandRule<float>, band_par<float>(c), "k_pair_quad_band");
     else GM_ENTRIES(BandRule<double>, band_par<double>(c), "k_pair_quad_band");
   } else if (Q <= 32) {
-    if (f32) launch_pair<1>(c, P, n_rows, rs, rux, ruy, ruz, row_field, row_ptr, col, nnz, val);
+    if (f32) GM_ENTRIES(Gl32Rule<1>, gl32_par<1>(c), "k_pair_quad");
     else GM_ENTRIES(DfRule<1>, df_par<1>(c), "k_pair_quad");
   } else if (Q <= 64) {
-    if (f32) launch_pair<2>(c, P, n_rows, rs, rux, ruy, ruz, row_field, row_ptr, col, nnz, val);
+    if (f32) GM_ENTRIES(Gl32Rule<2>, gl32_par<2>(c), "k_pair_quad");
     else GM_ENTRIES(DfRule<2>, df_par<2>(c), "k_pair_quad");
   } else {
-    if (f32) launch_pair<4>(c, P, n_rows, rs, rux, ruy, ruz, row_field, row_ptr, col, nnz, val);
+    if (f32) GM_ENTRIES(Gl32Rule<4>, gl32_par<4>(c), "k_pair_quad");
     else GM_ENTRIES(DfRule<4>, df_par<4>(c), "k_pair_quad");
   }
 #undef GM_ENTRIES
