@@ -1041,8 +1041,20 @@ static gm_status posterior_mean(gm_ctx* c, int64_t* iters, double* resid) {
     GM_PROF(c, "k_scale");
     k_scale<double><<<eb, 256, 0, st>>>(n, d64, w64, r64);  // rhs
     GM_LAUNCH_CHECK(c);
-    s = cg_single<TA, double>(c, r64, x64, tol, max_it, iters, resid);
-    if (s != GM_OK) return s;
+    if (small_cg_fits(c, 1)) {
+      double* part = (double*)ws.part.p;
+      double* hp = (double*)c->h_pinned;
+      s = small_cg(c, 1, 1, (const double*)ws.dv.p, (const double*)ws.minv.p, r64, x64, false, tol,
+                   part, part + 1, iters);
+      if (s != GM_OK) return s;
+      GM_CUDA_CHECK(c, cudaMemcpyAsync(hp, part, 2 * sizeof(double), cudaMemcpyDeviceToHost, st));
+      GM_CUDA_CHECK(c, cudaStreamSynchronize(st));
+      if (!std::isfinite(hp[1])) return set_error(c, GM_E_NONFINITE, "CG residual is not finite");
+      *resid = hp[0] > 0 ? std::sqrt(hp[1] / hp[0]) : 0.0;
+    } else {
+      s = cg_single<TA, double>(c, r64, x64, tol, max_it, iters, resid);
+      if (s != GM_OK) return s;
+    }
     GM_PROF(c, "k_alpha");
     k_alpha<double><<<eb, 256, 0, st>>>(n, b64, d64, x64, c->alpha);
   } else {
@@ -1162,7 +1174,8 @@ static gm_status panels(gm_ctx* c, int64_t n_rows, const int64_t* row_ptr, const
   const int64_t n = c->n;
   cudaStream_t st = c->stream;
   const int sms = sm_count(c);
-  if (sizeof(TV) == 8) {
+  const bool small = sizeof(TV) == 8 && small_cg_fits(c, n_cols_all);
+  if (sizeof(TV) == 8 && !small) {
     const gm_status ts = tc64_prepare(c, n_cols_all);
     if (ts != GM_OK) return ts;
   }
@@ -1259,6 +1272,14 @@ static gm_status panels(gm_ctx* c, int64_t n_rows, const int64_t* row_ptr, const
     GM_LAUNCH_CHECK(c);
     const bool use_warm = warm && c->cfg.warm_start && c->warm_R == R && n_cols_all <= R &&
                           c->warm_probe == (probe ? 1 : 0);
+    if (small) {  // whole columns per block, padded ones (zero) included
+      int64_t sit = 0;
+      const gm_status ss = small_cg(c, R, R, (const double*)dv, (const double*)minv,
+                                    (const double*)Rr, (double*)X, use_warm, tol, scal + 4 * R,
+                                    scal + 5 * R, &sit);
+      if (ss != GM_OK) return ss;
+      total_it += sit;
+    } else {
     if (use_warm) {
       GM_PROF(c, "k_panel_scale");
       k_panel_scale<TV><<<egrid, kBT, 0, st>>>(n, (int)R, dv, X, PD);
@@ -1367,6 +1388,7 @@ static gm_status panels(gm_ctx* c, int64_t n_rows, const int64_t* row_ptr, const
       }
     }
     total_it += std::min(it, max_it);
+    }  // !small
     if (probe) {
       GM_PROF(c, "k_panel_final_probe");
       k_panel_final_probe<TA, TV><<<(int)std::min<int64_t>(ceil_div(n * 32, 256), 16 * sms), 256,
