@@ -1346,7 +1346,10 @@ gm_status gm_pic_predict(gm_ctx* c, int64_t nq, const int32_t* q_block, const do
   }
   Buffer qcol;
   int64_t qnnz = 0;
-  st = neighbour_csr(c, nq, qs, ux, uy, uz, nullptr, false, qptr, qcol, &qnnz, nullptr);
+  // a query's own sub-catalogue only: the predictive reads no other star (at 6,000
+  // stars in 36 blocks a sixth of the neighbours' quadratures)
+  st = neighbour_csr(c, nq, qs, ux, uy, uz, nullptr, false, qptr, qcol, &qnnz, nullptr, qblk,
+                     pic_star_blocks(c));
   if (st != GM_OK) return st;
   ScopedDev bqc(c, qcol.p, qcol.bytes, ScopedDev::Adopt{});
   ScopedDev bqv(c, (size_t)std::max<int64_t>(qnnz, 1) * sizeof(double));

@@ -272,24 +272,22 @@ GM_HD inline void prec_task(int64_t e, int R, const double* Kinv, const double* 
   }
 }
 
-// Quadrature inputs of query-inducing pair p = q R + r.
+// Quadrature inputs (distances, chord) of query-inducing pair p = q R + r.
 GM_HD inline void qpair(int64_t p, int R, const double* qs, const double* qx, const double* qy,
                         const double* qz, const double* us, const double* ux, const double* uy,
                         const double* uz, double* si, double* sj, double* ch) {
   const int64_t q = p / R;
   const int r = (int)(p - q * R);
   const double dx = qx[q] - ux[r], dy = qy[q] - uy[r], dz = qz[q] - uz[r];
-  si[p] = qs[q];
-  sj[p] = us[r];
-  ch[p] = sqrt(dx * dx + dy * dy + dz * dz);
+  *si = qs[q];
+  *sj = us[r];
+  *ch = sqrt(dx * dx + dy * dy + dz * dz);
 }
 
-// K_su[p] (p = q R + r) from the pair's untapered value, tapered as K.
-GM_HD inline double ksu_entry(int64_t p, double inv_cut, int taper, const double* si,
-                              const double* sj, const double* ch, const double* kp) {
-  const double ds = si[p] - sj[p];
-  const double d = sqrt(ds * ds + si[p] * sj[p] * ch[p] * ch[p]);
-  return taper_weight(d, inv_cut, taper) * kp[p];
+// 3-D separation of a pair from its distances and chord.
+GM_HD inline double pair_distance(double si, double sj, double ch) {
+  const double ds = si - sj;
+  return sqrt(ds * ds + si * sj * ch * ch);
 }
 
 // Stored entry of star j in a query's CSR row [b, e) (columns sorted).

@@ -189,7 +189,9 @@ __global__ void k_neighbours(int64_t n_rows, const FieldGrid* __restrict__ fg,
                              const double* __restrict__ ux, const double* __restrict__ uy,
                              const double* __restrict__ uz, const int32_t* __restrict__ cell_start,
                              int64_t* __restrict__ count_or_ptr, int32_t* __restrict__ col,
-                             int64_t* __restrict__ diag_pos, bool self) {
+                             int64_t* __restrict__ diag_pos, bool self,
+                             const int32_t* __restrict__ row_tag,
+                             const int32_t* __restrict__ star_tag) {
   const int lane = threadIdx.x & 31;
   const int64_t warp = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
   const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
@@ -197,6 +199,7 @@ __global__ void k_neighbours(int64_t n_rows, const FieldGrid* __restrict__ fg,
     const double sr = rs[r], xr = rux[r], yr = ruy[r], zr = ruz[r];
     const FieldGrid g = fg[row_field ? row_field[r] : 0];
     const double cut2 = g.cut2;
+    const int32_t tag = row_tag ? row_tag[r] : 0;
     int cx, cy, cz;
     cell_coords(g, sr * xr, sr * yr, sr * zr, &cx, &cy, &cz);
     int64_t pos = kFill ? count_or_ptr[r] : 0;
@@ -215,7 +218,8 @@ __global__ void k_neighbours(int64_t n_rows, const FieldGrid* __restrict__ fg,
         for (int32_t jb = j0; jb < j1; jb += 32) {
           int32_t j = jb + lane;
           bool in = false;
-          if (j < j1) in = dist2(sr, xr, yr, zr, s[j], ux[j], uy[j], uz[j]) <= cut2;
+          if (j < j1 && (!row_tag || star_tag[j] == tag))
+            in = dist2(sr, xr, yr, zr, s[j], ux[j], uy[j], uz[j]) <= cut2;
           unsigned m = __ballot_sync(0xffffffffu, in);
           if (kFill) {
             if (in) {
@@ -444,7 +448,8 @@ gm_status unit_vectors(gm_ctx* c, int64_t n, const double* l, const double* b, d
 
 gm_status neighbour_csr(gm_ctx* c, int64_t n_rows, const double* rs, const double* rux,
                         const double* ruy, const double* ruz, const int32_t* row_field, bool self,
-                        int64_t* row_ptr, Buffer& col_buf, int64_t* nnz_out, int64_t* diag_pos) {
+                        int64_t* row_ptr, Buffer& col_buf, int64_t* nnz_out, int64_t* diag_pos,
+                        const int32_t* row_tag, const int32_t* star_tag) {
   cudaStream_t st = c->stream;
   const int sms = sm_count(c);
   int64_t* counts = (int64_t*)dev_alloc(c, (n_rows + 1) * sizeof(int64_t));
@@ -452,7 +457,8 @@ gm_status neighbour_csr(gm_ctx* c, int64_t n_rows, const double* rs, const doubl
   const int wb = (int)std::min<int64_t>(ceil_div(n_rows * 32, 256), 32 * sms);
   GM_PROF(c, "k_neighbours");
   k_neighbours<false><<<wb, 256, 0, st>>>(n_rows, c->fgrid, row_field, rs, rux, ruy, ruz, c->s, c->ux, c->uy,
-                                          c->uz, c->cell_start, counts, nullptr, nullptr, self);
+                                          c->uz, c->cell_start, counts, nullptr, nullptr, self,
+                                          row_tag, star_tag);
   GM_LAUNCH_CHECK(c);
   {
     gm_status sst = scan_i64(c, counts, row_ptr, n_rows);
@@ -468,7 +474,7 @@ gm_status neighbour_csr(gm_ctx* c, int64_t n_rows, const double* rs, const doubl
   GM_PROF(c, "k_neighbours");
   k_neighbours<true><<<wb, 256, 0, st>>>(n_rows, c->fgrid, row_field, rs, rux, ruy, ruz, c->s, c->ux, c->uy,
                                          c->uz, c->cell_start, row_ptr, (int32_t*)col_buf.p,
-                                         diag_pos, self);
+                                         diag_pos, self, row_tag, star_tag);
   GM_LAUNCH_CHECK(c);
   GM_CUDA_CHECK(c, cudaStreamSynchronize(st));
   dev_free_now(c, counts, (n_rows + 1) * sizeof(int64_t));

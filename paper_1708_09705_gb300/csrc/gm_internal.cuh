@@ -317,11 +317,13 @@ gm_status unit_vectors(gm_ctx* c, int64_t n, const double* l, const double* b, d
 // Counts neighbours within the cutoff of each row, scans to row_ptr (n_rows+1)
 // and fills sorted column indices.  `self` marks rows that are the stars
 // themselves (diag_pos is then filled).
-// row_field: field of each row (null: field 0).
+// row_field: field of each row (null: field 0).  row_tag (may be null): only the
+// stars j with star_tag[j] == row_tag[row].
 gm_status neighbour_csr(gm_ctx* c, int64_t n_rows, const double* rs,
                         const double* rux, const double* ruy, const double* ruz,
                         const int32_t* row_field, bool self, int64_t* row_ptr,
-                        Buffer& col_buf, int64_t* nnz_out, int64_t* diag_pos);
+                        Buffer& col_buf, int64_t* nnz_out, int64_t* diag_pos,
+                        const int32_t* row_tag = nullptr, const int32_t* star_tag = nullptr);
 gm_status phi_points_init(gm_ctx* c);
 gm_status gtab_update(gm_ctx* c);
 // Pair quadrature for CSR entries; symmetric mode computes j >= i and
@@ -477,6 +479,7 @@ gm_status pic_posterior(gm_ctx* c, int R, const double* us, const double* ux, co
                         const double* uz, const int32_t* h_block_int, int nb);
 bool pic_ready(gm_ctx* c);
 int pic_blocks(gm_ctx* c);
+const int32_t* pic_star_blocks(gm_ctx* c);  // sub-catalogue of each star (device)
 int pic_inducing(gm_ctx* c);
 const double* pic_mean(gm_ctx* c);
 const double* pic_cov(gm_ctx* c);

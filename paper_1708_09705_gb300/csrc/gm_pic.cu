@@ -177,12 +177,12 @@ struct PicState {
   int R = 0, nb = 0;
   int64_t n = 0;
   Buffer i64;  // boff (nb + 1), coff (nb + 1), bidx (n)
-  Buffer i32;  // dims (nb)
+  Buffer i32;  // dims (nb), block of each star (n)
   Buffer d;    // Lu (R^2), mean (R), cov (R^2), mu_u (R), us, ux, uy, uz (R),
                // A, Kku (n R), C factors (sum N_k^2)
   std::vector<int64_t> h_boff, h_coff;
   int64_t *boff = nullptr, *coff = nullptr, *bidx = nullptr;
-  int32_t* dims = nullptr;
+  int32_t *dims = nullptr, *blk = nullptr;
   double *Lu = nullptr, *mean = nullptr, *cov = nullptr, *mu_u = nullptr, *us = nullptr,
          *ux = nullptr, *uy = nullptr, *uz = nullptr, *A = nullptr, *Kku = nullptr, *C = nullptr;
   int max_block = 0;
@@ -202,6 +202,7 @@ bool pic_ready(gm_ctx* c) { return c->pic && c->pic->ready; }
 const double* pic_mean(gm_ctx* c) { return c->pic ? c->pic->mean : nullptr; }
 const double* pic_cov(gm_ctx* c) { return c->pic ? c->pic->cov : nullptr; }
 int pic_blocks(gm_ctx* c) { return c->pic ? c->pic->nb : 0; }
+const int32_t* pic_star_blocks(gm_ctx* c) { return c->pic ? c->pic->blk : nullptr; }
 int pic_inducing(gm_ctx* c) { return c->pic ? c->pic->R : 0; }
 
 gm_status pic_posterior(gm_ctx* c, int R, const double* us, const double* ux, const double* uy,
@@ -229,7 +230,7 @@ gm_status pic_posterior(gm_ctx* c, int R, const double* us, const double* ux, co
   const int64_t npair = (int64_t)R * (R + 1) / 2;
   const int64_t ncf = S->h_coff[nb];
   if (!ensure(c, S->i64, (size_t)(2 * (nb + 1) + n) * sizeof(int64_t)) ||
-      !ensure(c, S->i32, (size_t)std::max(nb, 1) * sizeof(int32_t)) ||
+      !ensure(c, S->i32, (size_t)(std::max(nb, 1) + n) * sizeof(int32_t)) ||
       !ensure(c, S->d, (size_t)(2 * RR + 7 * R + 2 * n * (int64_t)R + ncf) * sizeof(double))) {
     pic_free(c);
     return set_error(c, GM_E_NOMEM, "PIC state");
@@ -238,6 +239,7 @@ gm_status pic_posterior(gm_ctx* c, int R, const double* us, const double* ux, co
   S->coff = S->boff + nb + 1;
   S->bidx = S->coff + nb + 1;
   S->dims = (int32_t*)S->i32.p;
+  S->blk = S->dims + std::max(nb, 1);
   S->Lu = (double*)S->d.p;
   S->mean = S->Lu + RR;
   S->cov = S->mean + R;
@@ -272,6 +274,8 @@ gm_status pic_posterior(gm_ctx* c, int R, const double* us, const double* ux, co
   GM_CUDA_CHECK(c, cudaMemcpyAsync(d_rowpos, rowpos.data(), n * sizeof(int32_t),
                                    cudaMemcpyHostToDevice, st));
   GM_CUDA_CHECK(c, cudaMemcpyAsync(S->dims, dims.data(), nb * sizeof(int32_t),
+                                   cudaMemcpyHostToDevice, st));
+  GM_CUDA_CHECK(c, cudaMemcpyAsync(S->blk, h_block_int, n * sizeof(int32_t),
                                    cudaMemcpyHostToDevice, st));
   for (const double* src : {us, ux, uy, uz}) {
     double* dst = src == us ? S->us : src == ux ? S->ux : src == uy ? S->uy : S->uz;
@@ -370,23 +374,49 @@ gm_status pic_posterior(gm_ctx* c, int R, const double* us, const double* ux, co
 }
 
 // ---------------------------------------------------------------- prediction
-__global__ void k_pic_qpairs(int64_t np, int R, const double* __restrict__ qs,
-                             const double* __restrict__ qx, const double* __restrict__ qy,
-                             const double* __restrict__ qz, const double* __restrict__ us,
-                             const double* __restrict__ ux, const double* __restrict__ uy,
-                             const double* __restrict__ uz, double* __restrict__ si,
-                             double* __restrict__ sj, double* __restrict__ ch) {
-  for (int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; p < np;
-       p += (int64_t)gridDim.x * blockDim.x)
-    gmpic::qpair(p, R, qs, qx, qy, qz, us, ux, uy, uz, si, sj, ch);
+// Quadrature inputs of the query-inducing pairs p = q R + r within the cutoff: the
+// others' tapered covariance is zero, so they need none.  Compact (any order), with
+// p in idx and their number in count; K_su of all pairs is zeroed.
+__global__ void k_pic_qpairs(int64_t np, int R, double inv_cut, int taper,
+                             const double* __restrict__ qs, const double* __restrict__ qx,
+                             const double* __restrict__ qy, const double* __restrict__ qz,
+                             const double* __restrict__ us, const double* __restrict__ ux,
+                             const double* __restrict__ uy, const double* __restrict__ uz,
+                             double* __restrict__ si, double* __restrict__ sj,
+                             double* __restrict__ ch, int32_t* __restrict__ idx,
+                             unsigned long long* __restrict__ count, double* __restrict__ ksu) {
+  const int lane = threadIdx.x & 31;
+  for (int64_t p0 = blockIdx.x * (int64_t)blockDim.x; p0 < np; p0 += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t p = p0 + threadIdx.x;
+    double a = 0, b = 0, h = 0;
+    bool in = false;
+    if (p < np) {
+      gmpic::qpair(p, R, qs, qx, qy, qz, us, ux, uy, uz, &a, &b, &h);
+      in = gmpic::taper_weight(gmpic::pair_distance(a, b, h), inv_cut, taper) != 0.0;
+      ksu[p] = 0.0;
+    }
+    const unsigned m = __ballot_sync(0xffffffffu, in);
+    unsigned long long o = 0;
+    if (lane == 0 && m) o = atomicAdd(count, (unsigned long long)__popc(m));
+    o = __shfl_sync(0xffffffffu, o, 0) + __popc(m & ((1u << lane) - 1u));
+    if (in) {
+      si[o] = a;
+      sj[o] = b;
+      ch[o] = h;
+      idx[o] = (int32_t)p;
+    }
+  }
 }
 
-__global__ void k_pic_ksu(int64_t np, double inv_cut, int taper, const double* __restrict__ si,
+// Tapered K_su of the compact pairs.
+__global__ void k_pic_ksu(int64_t m, double inv_cut, int taper, const double* __restrict__ si,
                           const double* __restrict__ sj, const double* __restrict__ ch,
-                          double* __restrict__ kp) {
-  for (int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; p < np;
-       p += (int64_t)gridDim.x * blockDim.x)
-    kp[p] = gmpic::ksu_entry(p, inv_cut, taper, si, sj, ch, kp);
+                          const int32_t* __restrict__ idx, const double* __restrict__ kp,
+                          double* __restrict__ ksu) {
+  for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < m;
+       k += (int64_t)gridDim.x * blockDim.x)
+    ksu[idx[k]] =
+        gmpic::taper_weight(gmpic::pair_distance(si[k], sj[k], ch[k]), inv_cut, taper) * kp[k];
 }
 
 // One thread per query of the chunk [q0, q0 + nc).
@@ -418,28 +448,40 @@ gm_status pic_predict(gm_ctx* c, int64_t nq, const double* qs, const double* qx,
   PicState* S = c->pic;
   const int R = S->R;
   const int maxN = std::max(S->max_block, 1);
-  // queries per chunk: K_su pairs (4 R doubles each) and the scratch
-  // (3 R + 2 maxN doubles each) within about 1 GB
-  const int64_t per = 4 * (int64_t)R + 3 * (int64_t)R + 2 * (int64_t)maxN;
+  // queries per chunk: K_su and its pairs (6 R doubles each: K_su, distances, chord,
+  // value, index) and the scratch (3 R + 2 maxN doubles each) within about 1 GB
+  const int64_t per = 6 * (int64_t)R + 3 * (int64_t)R + 2 * (int64_t)maxN;
   const int64_t chunk = std::max<int64_t>(1, std::min<int64_t>(nq, (int64_t)(1 << 27) / per));
-  ScopedDev buf(c, (size_t)chunk * per * sizeof(double));
+  ScopedDev buf(c, (size_t)(chunk * per + 1) * sizeof(double));
   if (!buf.p) return set_error(c, GM_E_NOMEM, "PIC prediction scratch");
   double* si = (double*)buf.p;
-  double *sj = si + chunk * R, *ch = sj + chunk * R, *kp = ch + chunk * R, *w = kp + chunk * R;
+  double *sj = si + chunk * R, *ch = sj + chunk * R, *kc = ch + chunk * R, *kp = kc + chunk * R;
+  int32_t* idx = (int32_t*)(kp + chunk * R);
+  double* w = kp + 2 * chunk * R;
+  unsigned long long* count = (unsigned long long*)((double*)buf.p + chunk * per);
   cudaStream_t st = c->stream;
+  const double inv_cut = 1.0 / c->cfg.cutoff_pc;
+  const int taper = c->cfg.taper == GM_TAPER_WENDLAND ? 0 : 1;
   for (int64_t q0 = 0; q0 < nq; q0 += chunk) {
     const int64_t nc = std::min(chunk, nq - q0);
     const int64_t np = nc * R;
+    GM_CUDA_CHECK(c, cudaMemsetAsync(count, 0, sizeof(*count), st));
     GM_PROF(c, "k_pic_qpairs");
-    k_pic_qpairs<<<grid_for(c, np), 128, 0, st>>>(np, R, qs + q0, qx + q0, qy + q0, qz + q0,
-                                                  S->us, S->ux, S->uy, S->uz, si, sj, ch);
+    k_pic_qpairs<<<grid_for(c, np), 128, 0, st>>>(np, R, inv_cut, taper, qs + q0, qx + q0, qy + q0,
+                                                  qz + q0, S->us, S->ux, S->uy, S->uz, si, sj, ch,
+                                                  idx, count, kp);
     GM_LAUNCH_CHECK(c);
-    gm_status s = pairlist_quadrature(c, np, si, sj, ch, kp);
+    unsigned long long* hm = (unsigned long long*)c->h_pinned;
+    GM_CUDA_CHECK(c, cudaMemcpyAsync(hm, count, sizeof(*hm), cudaMemcpyDeviceToHost, st));
+    GM_CUDA_CHECK(c, cudaStreamSynchronize(st));
+    const int64_t m = (int64_t)*hm;
+    gm_status s = pairlist_quadrature(c, m, si, sj, ch, kc);
     if (s != GM_OK) return s;
-    GM_PROF(c, "k_pic_ksu");
-    k_pic_ksu<<<grid_for(c, np), 128, 0, st>>>(np, 1.0 / c->cfg.cutoff_pc, c->cfg.taper, si, sj,
-                                               ch, kp);
-    GM_LAUNCH_CHECK(c);
+    if (m > 0) {
+      GM_PROF(c, "k_pic_ksu");
+      k_pic_ksu<<<grid_for(c, m), 128, 0, st>>>(m, inv_cut, taper, si, sj, ch, idx, kc, kp);
+      GM_LAUNCH_CHECK(c);
+    }
     GM_PROF(c, "k_pic_point");
     k_pic_point<<<(unsigned)ceil_div(nc, 128), 128, 0, st>>>(
         q0, nc, R, maxN, qblk, S->boff, S->coff, S->bidx, S->Lu, S->C, S->A, S->Kku, S->mu_u,
