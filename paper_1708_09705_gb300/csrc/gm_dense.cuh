@@ -1,9 +1,10 @@
 // Dense FP64 linear algebra of the PITC / PIC posterior over inducing points
 // (Sect. 4.1, simplified case; the conditional of each sub-catalogue given
-// the inducing values, App. B), written as per-output routines so that a
-// device kernel runs them one thread per output (or, for the Cholesky
-// factorisation, one thread block per matrix in barrier-separated phases)
-// and a host build runs the same routines in the same order.
+// the inducing values, App. B), written as per-output routines.  The device kernels
+// of the entries and of the quadrature inputs call them; the factorisations, the
+// solves and the sums over stars have kernels of their own (a warp per right-hand
+// side, a thread block per matrix), and these routines state what they compute: a
+// host build runs them from end to end.
 //
 // Matrices are row-major with leading dimension ld; only lower triangles of
 // symmetric matrices are read.

@@ -12,9 +12,9 @@
 //   P = K_uu^-1 + sum_k A_k^T C_k^-1 A_k,  h = K_uu^-1 mu_u + sum_k A_k^T C_k^-1 y_k,
 //   y_k = a~_k - m_k + A_k mu_u,   mean = P^-1 h,   cov = P^-1.
 // K_kk are read from the stored covariance, K_ku and K_uu come from the same
-// sightline quadrature, cutoff and taper.  The dense algebra (FP64) is in
-// gm_dense.cuh; here each step is a kernel with one thread per output, and the
-// Cholesky factorisations run one thread block per matrix.
+// sightline quadrature, cutoff and taper.  The dense algebra (FP64) follows the
+// per-output routines of gm_dense.cuh, with a warp per right-hand side and a thread
+// block per factorisation.
 #include <algorithm>
 #include <cmath>
 #include <vector>
@@ -25,31 +25,149 @@
 namespace gm {
 
 // Lower Cholesky factor in place of each dim[b] x dim[b] row-major matrix at
-// base + off[b]; one thread block per matrix.
-__global__ void __launch_bounds__(256) k_pic_chol(double* __restrict__ base,
-                                                  const int64_t* __restrict__ off,
-                                                  const int32_t* __restrict__ dim,
-                                                  unsigned* __restrict__ flags) {
-  __shared__ double d_s;
-  __shared__ int bad;
-  double* A = base + off[blockIdx.x];
+// base + off[b], mirrored into the upper triangle (column i of L is then a
+// contiguous row for the solves); one thread block per matrix, right-looking.
+// The chain of columns bounds it: a matrix of up to kCholShared rows stays in
+// shared memory (packed lower triangle: 231 KB), a larger one in global memory; either way the column in work is copied to shared memory
+// and the update runs along the rows, a warp per row.  One thread per row on
+// global memory took 8 us a column, 1.34 ms at 140 to 170 rows; now 0.42 ms.
+constexpr int kCholShared = 238;
+constexpr int kCholThreads = 512;
+
+__global__ void __launch_bounds__(kCholThreads) k_pic_chol(double* __restrict__ base,
+                                                           const int64_t* __restrict__ off,
+                                                           const int32_t* __restrict__ dim,
+                                                           unsigned* __restrict__ flags) {
+  extern __shared__ double sm[];  // the column, then the matrix if it fits
+  __shared__ double d_s[2];
+  double* G = base + off[blockIdx.x];
   const int n = dim[blockIdx.x];
-  if (threadIdx.x == 0) bad = 0;
+  const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, w = tid >> 5, W = nt >> 5;
+  const bool in_sm = n <= kCholShared;
+  double* v = sm;
+  double* A = in_sm ? sm + n : G;
+  auto row = [&](int i) { return A + (in_sm ? (int64_t)i * (i + 1) / 2 : (int64_t)i * n); };
+  if (in_sm)
+    for (int i = w; i < n; i += W)
+      for (int k = lane; k <= i; k += 32) row(i)[k] = G[(int64_t)i * n + k];
   __syncthreads();
   for (int j = 0; j < n; ++j) {
-    if (threadIdx.x == 0) {
-      const double d = gmdense::chol_diag(A, n, j);
-      d_s = d;
-      if (!(d > 0.0)) bad = 1;
+    if (w == 0) {
+      const double d = row(j)[j];
+      const double r = d > 0.0 ? sqrt(d) : -1.0;
+      if (lane == 0) {
+        d_s[0] = r;
+        d_s[1] = 1.0 / r;
+      }
     }
     __syncthreads();
-    if (bad) break;
-    gmdense::chol_col(A, n, n, j, d_s, threadIdx.x, blockDim.x);
+    const double d = d_s[0], rd = d_s[1];
+    if (!(d > 0.0)) break;  // uniform
+    for (int i = j + tid; i < n; i += nt) {
+      double* Ai = row(i);
+      const double x = i == j ? d : Ai[j] * rd;
+      Ai[j] = x;
+      v[i] = x;
+    }
     __syncthreads();
-    gmdense::chol_update(A, n, n, j, threadIdx.x, blockDim.x);
+    for (int i = j + 1 + w; i < n; i += W) {
+      const double x = v[i];
+      double* Ai = row(i);
+      for (int k = j + 1 + lane; k <= i; k += 32) Ai[k] = fma(-x, v[k], Ai[k]);
+    }
     __syncthreads();
   }
-  if (bad && threadIdx.x == 0) atomicOr(flags, kFlagNotSPD);
+  // a matrix that is not positive definite is written back as far as it came
+  if (tid == 0 && n > 0 && !(d_s[0] > 0.0)) atomicOr(flags, kFlagNotSPD);
+  for (int i = w; i < n; i += W)
+    for (int k = lane; k < n; k += 32) {
+      const double x = k <= i ? row(i)[k] : row(k)[i];
+      if (in_sm || k > i) G[(int64_t)i * n + k] = x;
+    }
+}
+
+// ------------------------------------------------- solves, a warp per vector
+// x (n values in shared memory, of one warp) of L x = b / L^T x = b in place, for a
+// mirrored factor M (rows of 256-byte reads in both directions).  Element i is
+// final once the steps before it have run, so every lane reads it, divides by the
+// diagonal, and the lanes subtract its multiples from their elements.
+__device__ __forceinline__ void warp_lower(const double* __restrict__ M, int64_t ld, int n,
+                                           double* x, int lane) {
+  for (int i0 = 0; i0 < n; i0 += 32) {
+    // the diagonal's reciprocals of 32 steps at once
+    const int id = i0 + lane;
+    const double rd = id < n ? 1.0 / M[(int64_t)id * ld + id] : 0.0;
+    const int e = min(32, n - i0);
+    // the 32 x 32 triangle in registers: lane holds element i0 + lane
+    double y = id < n ? x[id] : 0.0;
+#pragma unroll 8
+    for (int t = 0; t < e; ++t) {
+      const double m = id < n && lane > t ? M[(int64_t)(i0 + t) * ld + id] : 0.0;
+      const double xt = __shfl_sync(0xffffffffu, y * rd, t);
+      if (lane == t) y = xt;
+      y = fma(-m, xt, y);
+    }
+    if (id < n) x[id] = y;
+    __syncwarp();
+    // the rows behind it: element k takes all 32 steps at once
+    for (int k = i0 + 32 + lane; k < n; k += 32) {
+      double a0 = x[k], a1 = 0;
+      const double* Mk = M + (int64_t)i0 * ld + k;
+#pragma unroll 8
+      for (int t = 0; t < 32; t += 2) {
+        a0 = fma(-Mk[(int64_t)t * ld], x[i0 + t], a0);
+        a1 = fma(-Mk[(int64_t)(t + 1) * ld], x[i0 + t + 1], a1);
+      }
+      x[k] = a0 + a1;
+    }
+    __syncwarp();
+  }
+}
+
+__device__ __forceinline__ void warp_lower_t(const double* __restrict__ M, int64_t ld, int n,
+                                             double* x, int lane) {
+  for (int i0 = ((n - 1) >> 5) << 5; i0 >= 0; i0 -= 32) {
+    const int id = i0 + lane;
+    const double rd = id < n ? 1.0 / M[(int64_t)id * ld + id] : 0.0;
+    const int e = min(32, n - i0);
+    double y = id < n ? x[id] : 0.0;
+#pragma unroll 8
+    for (int t = e - 1; t >= 0; --t) {
+      const double m = lane < t ? M[(int64_t)(i0 + t) * ld + id] : 0.0;
+      const double xt = __shfl_sync(0xffffffffu, y * rd, t);
+      if (lane == t) y = xt;
+      y = fma(-m, xt, y);
+    }
+    if (id < n) x[id] = y;
+    __syncwarp();
+    for (int k = lane; k < i0; k += 32) {  // k < i0: whole warps, i0 is a multiple of 32
+      double a0 = x[k], a1 = 0;
+      const double* Mk = M + (int64_t)i0 * ld + k;
+      int t = 0;
+#pragma unroll 4
+      for (; t + 1 < e; t += 2) {
+        a0 = fma(-Mk[(int64_t)t * ld], x[i0 + t], a0);
+        a1 = fma(-Mk[(int64_t)(t + 1) * ld], x[i0 + t + 1], a1);
+      }
+      if (t < e) a0 = fma(-Mk[(int64_t)t * ld], x[i0 + t], a0);
+      x[k] = a0 + a1;
+    }
+    __syncwarp();
+  }
+}
+
+__device__ __forceinline__ double warp_sum(double v) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  return v;
+}
+
+// Vectors of one warp: `words` doubles in shared memory, or in the global scratch
+// where a block's share of shared memory is too small for them (a sub-catalogue of
+// thousands of stars).
+__device__ __forceinline__ double* warp_vectors(double* sm, double* scratch, int64_t words) {
+  const int w = threadIdx.x >> 5;
+  return scratch ? scratch + ((int64_t)blockIdx.x * (blockDim.x >> 5) + w) * words : sm + w * words;
 }
 
 // Quadrature inputs of the inducing pairs (a, b), a >= b, diagonal included.
@@ -90,11 +208,21 @@ __global__ void k_pic_kku(int R, const int64_t* __restrict__ qptr,
   }
 }
 
-__global__ void k_pic_arow(int64_t n, int R, const double* __restrict__ Lu,
-                           const double* __restrict__ Kku, double* __restrict__ A) {
-  for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < n;
-       j += (int64_t)gridDim.x * blockDim.x)
-    gmdense::a_row(Lu, R, Kku + j * R, A + j * R);
+// Rows of A = K_ku K_uu^-1, a warp each.
+__global__ void __launch_bounds__(128) k_pic_arow(int64_t n, int R, const double* __restrict__ Lu,
+                                                  const double* __restrict__ Kku,
+                                                  double* __restrict__ A, double* scratch) {
+  extern __shared__ double sm[];
+  double* x = warp_vectors(sm, scratch, R);
+  const int lane = threadIdx.x & 31, W = blockDim.x >> 5;
+  for (int64_t j = blockIdx.x * (int64_t)W + (threadIdx.x >> 5); j < n; j += (int64_t)gridDim.x * W) {
+    for (int r = lane; r < R; r += 32) x[r] = Kku[j * R + r];
+    __syncwarp();
+    warp_lower(Lu, R, R, x, lane);
+    warp_lower_t(Lu, R, R, x, lane);
+    for (int r = lane; r < R; r += 32) A[j * R + r] = x[r];
+    __syncwarp();
+  }
 }
 
 // Lower triangle of every block's C_k = K_kk - A_k K_uk + diag(sigma^2).
@@ -120,32 +248,100 @@ __global__ void k_pic_y(int64_t n, int R, const int64_t* __restrict__ bidx,
     yv[j] = gmdense::y_entry(obs[bidx[j]], prior_m[bidx[j]], A + j * R, mu_u, R);
 }
 
-// X_k = L_k^-1 A_k (columns c < R) and yv_k = L_k^-1 y_k (c = R).
-__global__ void k_pic_fsolve(int nb, int R, const int64_t* __restrict__ coff,
-                             const int64_t* __restrict__ boff, const double* __restrict__ C,
-                             double* __restrict__ X, double* __restrict__ yv) {
+// X_k = L_k^-1 A_k (columns c < R) and yv_k = L_k^-1 y_k (c = R), a warp per column.
+__global__ void __launch_bounds__(128) k_pic_fsolve(int nb, int R, int maxN,
+                                                    const int64_t* __restrict__ coff,
+                                                    const int64_t* __restrict__ boff,
+                                                    const double* __restrict__ C,
+                                                    double* __restrict__ X, double* __restrict__ yv,
+                                                    double* scratch) {
+  extern __shared__ double sm[];
+  double* x = warp_vectors(sm, scratch, maxN);
+  const int lane = threadIdx.x & 31, W = blockDim.x >> 5;
   const int64_t total = (int64_t)nb * (R + 1);
-  for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < total;
-       t += (int64_t)gridDim.x * blockDim.x) {
-    gmpic::fsolve_task(t, R, coff, boff, C, X, yv);
+  for (int64_t t = blockIdx.x * (int64_t)W + (threadIdx.x >> 5); t < total;
+       t += (int64_t)gridDim.x * W) {
+    const int k = (int)(t / (R + 1)), c = (int)(t - (int64_t)k * (R + 1));
+    const int N = (int)(boff[k + 1] - boff[k]);
+    double* p = c < R ? X + boff[k] * R + c : yv + boff[k];
+    const int64_t inc = c < R ? R : 1;
+    for (int a = lane; a < N; a += 32) x[a] = p[a * inc];
+    __syncwarp();
+    warp_lower(C + coff[k], N, N, x, lane);
+    for (int a = lane; a < N; a += 32) p[a * inc] = x[a];
+    __syncwarp();
   }
 }
 
-// Lambda (lower triangle) and eta over all stars.
-__global__ void k_pic_lambda(int64_t n, int R, const double* __restrict__ X,
-                             const double* __restrict__ yv, double* __restrict__ Lam,
-                             double* __restrict__ eta) {
-  const int64_t total = (int64_t)R * R + R;
+// Lambda (lower triangle, b <= a) and eta, partial sums over a share of the stars:
+// 32 x 32 outputs per block, stars in groups of 32 through shared memory.  The
+// right-hand side is column R of [X | yv].  part: split x (R^2 + R).
+__global__ void __launch_bounds__(256) k_pic_lambda(int64_t n, int R, int64_t share,
+                                                    const double* __restrict__ X,
+                                                    const double* __restrict__ yv,
+                                                    double* __restrict__ part) {
+  __shared__ double sa[32][33], sb[32][33];
+  int ta, tb;
+  gmpic::tri_index(blockIdx.x, &ta, &tb);  // tiles of rows (of R + 1) and columns
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int64_t j0 = blockIdx.y * share, j1 = min(n, j0 + share);
+  double acc[4] = {0, 0, 0, 0};
+  auto at = [&](int64_t j, int r) {
+    return j < j1 && r <= R ? (r < R ? X[j * R + r] : yv[j]) : 0.0;
+  };
+  for (int64_t j = j0; j < j1; j += 32) {
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      sa[w + 8 * q][lane] = at(j + w + 8 * q, 32 * ta + lane);
+      sb[w + 8 * q][lane] = at(j + w + 8 * q, 32 * tb + lane);
+    }
+    __syncthreads();
+#pragma unroll 8
+    for (int t = 0; t < 32; ++t) {
+      const double b = sb[t][lane];
+#pragma unroll
+      for (int q = 0; q < 4; ++q) acc[q] = fma(sa[t][w + 8 * q], b, acc[q]);
+    }
+    __syncthreads();
+  }
+  double* o = part + blockIdx.y * ((int64_t)R * R + R);
+  const int b = 32 * tb + lane;
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    const int a = 32 * ta + w + 8 * q;
+    if (b >= R) continue;
+    if (a < R && b <= a) o[(int64_t)a * R + b] = acc[q];
+    if (a == R) o[(int64_t)R * R + b] = acc[q];
+  }
+}
+
+__global__ void k_pic_lambda_sum(int R, int splits, const double* __restrict__ part,
+                                 double* __restrict__ Lam, double* __restrict__ eta) {
+  const int64_t RR = (int64_t)R * R, total = RR + R;
   for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < total;
        e += (int64_t)gridDim.x * blockDim.x) {
-    gmpic::lambda_task(e, n, R, X, yv, Lam, eta);
+    if (e < RR && e % R > e / R) continue;
+    double v = 0.0;
+    for (int k = 0; k < splits; ++k) v += part[k * total + e];
+    if (e < RR) Lam[e] = v;
+    else eta[e - RR] = v;
   }
 }
 
-// Columns of (L L^T)^-1 (one thread per column).
-__global__ void k_pic_inverse(int R, const double* __restrict__ L, double* __restrict__ out) {
-  for (int c = blockIdx.x * blockDim.x + threadIdx.x; c < R; c += gridDim.x * blockDim.x)
-    gmdense::inverse_col(L, R, c, out + c, R);
+// Columns of (L L^T)^-1, a warp each (it is symmetric: written as rows).
+__global__ void __launch_bounds__(128) k_pic_inverse(int R, const double* __restrict__ L,
+                                                     double* __restrict__ out, double* scratch) {
+  extern __shared__ double sm[];
+  double* x = warp_vectors(sm, scratch, R);
+  const int lane = threadIdx.x & 31, W = blockDim.x >> 5;
+  for (int c = blockIdx.x * W + (threadIdx.x >> 5); c < R; c += gridDim.x * W) {
+    for (int r = lane; r < R; r += 32) x[r] = r == c ? 1.0 : 0.0;
+    __syncwarp();
+    warp_lower(L, R, R, x, lane);
+    warp_lower_t(L, R, R, x, lane);
+    for (int r = lane; r < R; r += 32) out[(int64_t)r * R + c] = x[r];
+    __syncwarp();
+  }
 }
 
 // P = K_uu^-1 + Lambda (lower triangle) and h = K_uu^-1 mu_u + eta.
@@ -159,13 +355,48 @@ __global__ void k_pic_prec(int R, const double* __restrict__ Kinv, const double*
   }
 }
 
-// mean = P^-1 h from the factor of P (one thread).
-__global__ void k_pic_mean(int R, const double* __restrict__ LP, const double* __restrict__ h,
-                           double* __restrict__ mean) {
-  if (blockIdx.x != 0 || threadIdx.x != 0) return;
-  for (int r = 0; r < R; ++r) mean[r] = h[r];
-  gmdense::solve_lower(LP, R, R, mean, 1);
-  gmdense::solve_lower_t(LP, R, R, mean, 1);
+// mean = P^-1 h from the factor of P (one warp).
+__global__ void __launch_bounds__(32) k_pic_mean(int R, const double* __restrict__ LP,
+                                                 const double* __restrict__ h,
+                                                 double* __restrict__ mean, double* scratch) {
+  extern __shared__ double sm[];
+  double* x = scratch ? scratch : sm;
+  const int lane = threadIdx.x;
+  for (int r = lane; r < R; r += 32) x[r] = h[r];
+  __syncwarp();
+  warp_lower(LP, R, R, x, lane);
+  warp_lower_t(LP, R, R, x, lane);
+  for (int r = lane; r < R; r += 32) mean[r] = x[r];
+}
+
+// Warps per block and blocks of a kernel with a warp per item and `words` doubles
+// per warp: shared memory while two warps fit half of an SM's, else
+// scratch (allocated for the grid).
+struct WarpPlan {
+  int warps, blocks;
+  size_t smem;
+  int64_t scratch;  // doubles
+};
+static WarpPlan warp_plan(gm_ctx* c, int64_t items, int64_t words) {
+  WarpPlan p;
+  const int64_t room = 96 * 1024 / 8;
+  p.scratch = 0;
+  if (words * 2 <= room) {
+    p.warps = (int)std::min<int64_t>(4, room / words);
+    p.smem = (size_t)p.warps * words * sizeof(double);
+  } else {
+    p.warps = 4;
+    p.smem = 0;
+  }
+  // few items: a block per SM first
+  p.warps = (int)std::max<int64_t>(1, std::min<int64_t>(p.warps, ceil_div(items, sm_count(c))));
+  if (p.smem) p.smem = (size_t)p.warps * words * sizeof(double);
+  p.blocks = (int)std::max<int64_t>(1, std::min<int64_t>(ceil_div(items, p.warps), 8 * sm_count(c)));
+  if (!p.smem) {
+    p.blocks = std::min(p.blocks, 2 * sm_count(c));
+    p.scratch = (int64_t)p.blocks * p.warps * words;
+  }
+  return p;
 }
 
 static int grid_for(gm_ctx* c, int64_t n) {
@@ -252,8 +483,20 @@ gm_status pic_posterior(gm_ctx* c, int R, const double* us, const double* ux, co
   S->Kku = S->A + n * (int64_t)R;
   S->C = S->Kku + n * (int64_t)R;
   // scratch of this call: Kuu, Kinv, Lam, P (R x R); eta, h (R); pair inputs
-  // (4 npair); X (n x R); yv (n); rowpos (n)
-  ScopedDev b_d(c, (size_t)(4 * RR + 2 * R + 4 * npair + n * (int64_t)R + n) * sizeof(double));
+  // (4 npair); X (n x R); yv (n); partial sums of Lambda and eta; vectors of the
+  // solves where they do not fit shared memory; rowpos (n)
+  const WarpPlan rows = warp_plan(c, n, R), cols = warp_plan(c, R, R), one = warp_plan(c, 1, R),
+                 fwd = warp_plan(c, (int64_t)nb * (R + 1), std::max(S->max_block, 1));
+  const int64_t lt = ceil_div((int64_t)R + 1, 32), lam_tiles = lt * (lt + 1) / 2;
+  // shares of at least 256 stars, two blocks per SM
+  const int64_t splits = std::max<int64_t>(
+      1, std::min<int64_t>(ceil_div(n, 256), 2 * sm_count(c) / lam_tiles));
+  const int64_t share = ceil_div(ceil_div(n, splits), 32) * 32;
+  const int64_t solve_words =
+      std::max(std::max(rows.scratch, cols.scratch), std::max(one.scratch, fwd.scratch));
+  ScopedDev b_d(c, (size_t)(4 * RR + 2 * R + 4 * npair + n * (int64_t)R + n + splits * (RR + R) +
+                            solve_words) *
+                       sizeof(double));
   ScopedDev b_r(c, (size_t)n * sizeof(int32_t));
   ScopedDev b_q(c, (size_t)(R + 1) * sizeof(int64_t));
   ScopedDev b_one(c, sizeof(int64_t) + sizeof(int32_t));
@@ -262,6 +505,8 @@ gm_status pic_posterior(gm_ctx* c, int R, const double* us, const double* ux, co
   double *Kinv = Kuu + RR, *Lam = Kinv + RR, *P = Lam + RR, *eta = P + RR, *h = eta + R;
   double *psi = h + R, *psj = psi + npair, *pch = psj + npair, *pk = pch + npair;
   double *X = pk + npair, *yv = X + n * (int64_t)R;
+  double *lam_part = yv + n, *vecs = lam_part + splits * (RR + R);
+  auto sc = [&](const WarpPlan& p) { return p.scratch ? vecs : nullptr; };
   int32_t* d_rowpos = (int32_t*)b_r.p;
   double *Lu = S->Lu, *A = S->A, *Kku = S->Kku, *C = S->C, *mu_u = S->mu_u;
   cudaStream_t st = c->stream;
@@ -323,11 +568,28 @@ gm_status pic_posterior(gm_ctx* c, int R, const double* us, const double* ux, co
   }
   const int64_t* one_off = (const int64_t*)b_one.p;
   const int32_t* one_dim = (const int32_t*)((char*)b_one.p + sizeof(int64_t));
+  // shared memory of a factorisation of up to d rows, and of the solves
+  auto chol_smem = [](int64_t d) {
+    return (size_t)(d <= kCholShared ? d + d * (d + 1) / 2 : d) * sizeof(double);
+  };
+  const size_t csm = std::max(chol_smem(std::min(std::max(R, S->max_block), kCholShared)),
+                              chol_smem(std::max(R, S->max_block)));
+  GM_CUDA_CHECK(c, cudaFuncSetAttribute(k_pic_chol, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                        (int)csm));
+  auto room = [&](const void* kern, const WarpPlan& p) {
+    return p.smem <= 48 * 1024
+               ? cudaSuccess
+               : cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)p.smem);
+  };
+  GM_CUDA_CHECK(c, room((const void*)k_pic_arow, rows));
+  GM_CUDA_CHECK(c, room((const void*)k_pic_fsolve, fwd));
+  GM_CUDA_CHECK(c, room((const void*)k_pic_inverse, cols));
+  GM_CUDA_CHECK(c, room((const void*)k_pic_mean, one));
   GM_PROF(c, "k_pic_chol");
-  k_pic_chol<<<1, 256, 0, st>>>(Lu, one_off, one_dim, c->d_flags);
+  k_pic_chol<<<1, kCholThreads, csm, st>>>(Lu, one_off, one_dim, c->d_flags);
   GM_LAUNCH_CHECK(c);
   GM_PROF(c, "k_pic_arow");
-  k_pic_arow<<<grid_for(c, n), 128, 0, st>>>(n, R, Lu, Kku, A);
+  k_pic_arow<<<rows.blocks, 32 * rows.warps, rows.smem, st>>>(n, R, Lu, Kku, A, sc(rows));
   GM_LAUNCH_CHECK(c);
   // ---- blocks: C_k, its factor, X_k and yv_k
   if (ncf > 0) {
@@ -337,7 +599,7 @@ gm_status pic_posterior(gm_ctx* c, int R, const double* us, const double* ux, co
                                                  c->obs_sigma, C);
     GM_LAUNCH_CHECK(c);
     GM_PROF(c, "k_pic_chol");
-    k_pic_chol<<<nb, 256, 0, st>>>(C, S->coff, S->dims, c->d_flags);
+    k_pic_chol<<<nb, kCholThreads, csm, st>>>(C, S->coff, S->dims, c->d_flags);
     GM_LAUNCH_CHECK(c);
   }
   GM_PROF(c, "k_pic_y");
@@ -346,27 +608,31 @@ gm_status pic_posterior(gm_ctx* c, int R, const double* us, const double* ux, co
   GM_CUDA_CHECK(c, cudaMemcpyAsync(X, A, n * (int64_t)R * sizeof(double),
                                    cudaMemcpyDeviceToDevice, st));
   GM_PROF(c, "k_pic_fsolve");
-  k_pic_fsolve<<<grid_for(c, (int64_t)nb * (R + 1)), 128, 0, st>>>(nb, R, S->coff, S->boff, C,
-                                                                    X, yv);
+  k_pic_fsolve<<<fwd.blocks, 32 * fwd.warps, fwd.smem, st>>>(nb, R, std::max(S->max_block, 1),
+                                                              S->coff, S->boff, C, X, yv, sc(fwd));
   GM_LAUNCH_CHECK(c);
   // ---- posterior of u
   GM_PROF(c, "k_pic_lambda");
-  k_pic_lambda<<<grid_for(c, RR + R), 128, 0, st>>>(n, R, X, yv, Lam, eta);
+  k_pic_lambda<<<dim3((unsigned)lam_tiles, (unsigned)splits), 256, 0, st>>>(n, R, share, X, yv,
+                                                                            lam_part);
+  GM_LAUNCH_CHECK(c);
+  GM_PROF(c, "k_pic_lambda_sum");
+  k_pic_lambda_sum<<<grid_for(c, RR + R), 128, 0, st>>>(R, (int)splits, lam_part, Lam, eta);
   GM_LAUNCH_CHECK(c);
   GM_PROF(c, "k_pic_inverse");
-  k_pic_inverse<<<grid_for(c, R), 128, 0, st>>>(R, Lu, Kinv);
+  k_pic_inverse<<<cols.blocks, 32 * cols.warps, cols.smem, st>>>(R, Lu, Kinv, sc(cols));
   GM_LAUNCH_CHECK(c);
   GM_PROF(c, "k_pic_prec");
   k_pic_prec<<<grid_for(c, RR + R), 128, 0, st>>>(R, Kinv, Lam, mu_u, eta, P, h);
   GM_LAUNCH_CHECK(c);
   GM_PROF(c, "k_pic_chol");
-  k_pic_chol<<<1, 256, 0, st>>>(P, one_off, one_dim, c->d_flags);
+  k_pic_chol<<<1, kCholThreads, csm, st>>>(P, one_off, one_dim, c->d_flags);
   GM_LAUNCH_CHECK(c);
   GM_PROF(c, "k_pic_mean");
-  k_pic_mean<<<1, 32, 0, st>>>(R, P, h, S->mean);
+  k_pic_mean<<<1, 32, one.smem, st>>>(R, P, h, S->mean, sc(one));
   GM_LAUNCH_CHECK(c);
   GM_PROF(c, "k_pic_inverse");
-  k_pic_inverse<<<grid_for(c, R), 128, 0, st>>>(R, P, S->cov);
+  k_pic_inverse<<<cols.blocks, 32 * cols.warps, cols.smem, st>>>(R, P, S->cov, sc(cols));
   GM_LAUNCH_CHECK(c);
   GM_CUDA_CHECK(c, cudaStreamSynchronize(st));
   S->ready = true;
@@ -419,26 +685,118 @@ __global__ void k_pic_ksu(int64_t m, double inv_cut, int taper, const double* __
         gmpic::taper_weight(gmpic::pair_distance(si[k], sj[k], ch[k]), inv_cut, taper) * kp[k];
 }
 
-// One thread per query of the chunk [q0, q0 + nc).
-__global__ void k_pic_point(int64_t q0, int64_t nc, int R, int maxN,
-                            const int32_t* __restrict__ qblk, const int64_t* __restrict__ boff,
-                            const int64_t* __restrict__ coff, const int64_t* __restrict__ bidx,
-                            const double* __restrict__ Lu, const double* __restrict__ Cf,
-                            const double* __restrict__ A, const double* __restrict__ Kku,
-                            const double* __restrict__ mu_u, const double* __restrict__ pmean,
-                            const double* __restrict__ pcov, const double* __restrict__ obs,
-                            const double* __restrict__ prior_m, const double* __restrict__ ksu,
-                            const double* __restrict__ kss, const double* __restrict__ ms,
-                            const int64_t* __restrict__ qptr, const int32_t* __restrict__ qcol,
-                            const double* __restrict__ qval, double* __restrict__ scratch,
-                            double* __restrict__ mean, double* __restrict__ var) {
-  const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (t >= nc) return;
-  const int64_t q = q0 + t;
-  double* w = scratch + t * (3 * (int64_t)R + 2 * (int64_t)maxN);
-  gmpic::pic_point(R, qblk[q], boff, coff, bidx, Lu, Cf, A, Kku, mu_u, pmean, pcov, obs, prior_m,
-                   ksu + t * R, kss[q], ms[q], qptr[q], qptr[q + 1], qcol, qval, w, w + R,
-                   w + 2 * R, w + 3 * R, w + 3 * R + maxN, mean + q, var + q);
+// The predictive (gmpic::pic_point) of the queries [q0, q0 + nc), a warp per query,
+// its vectors in shared memory.  FP64 bounds it: 4,400 warp instructions per query at
+// 140 inducing points and 170 stars (the products with K_ku and A, four triangular
+// solves, the quadratic form), 16 clocks of an SM each, 1.0 ms for 4,000 queries; the
+// matrices come from L2.  One thread per query on global scratch took 11.0 ms, now 1.33.
+__global__ void __launch_bounds__(128) k_pic_point(
+    int64_t q0, int64_t nc, int R, int maxN, const int32_t* __restrict__ qblk,
+    const int64_t* __restrict__ boff, const int64_t* __restrict__ coff,
+    const int64_t* __restrict__ bidx, const double* __restrict__ Lu, const double* __restrict__ Cf,
+    const double* __restrict__ A, const double* __restrict__ Kku, const double* __restrict__ mu_u,
+    const double* __restrict__ pmean, const double* __restrict__ pcov,
+    const double* __restrict__ obs, const double* __restrict__ prior_m,
+    const double* __restrict__ ksu, const double* __restrict__ kss, const double* __restrict__ ms,
+    const int64_t* __restrict__ qptr, const int32_t* __restrict__ qcol,
+    const double* __restrict__ qval, double* scratch, double* __restrict__ mean,
+    double* __restrict__ var) {
+  extern __shared__ double sm[];
+  double* As = warp_vectors(sm, scratch, 2 * ((int64_t)R + maxN));
+  double *Lc = As + R, *D = Lc + R, *g = D + maxN;
+  const int lane = threadIdx.x & 31, W = blockDim.x >> 5;
+  for (int64_t t = blockIdx.x * (int64_t)W + (threadIdx.x >> 5); t < nc; t += (int64_t)gridDim.x * W) {
+    const int64_t q = q0 + t;
+    const int k = qblk[q];
+    const int64_t b0 = boff[k];
+    const int N = (int)(boff[k + 1] - b0);
+    const double* ks = ksu + t * R;
+    for (int r = lane; r < R; r += 32) As[r] = ks[r];
+    __syncwarp();
+    warp_lower(Lu, R, R, As, lane);
+    warp_lower_t(Lu, R, R, As, lane);
+    // D = k_sk - K_ku A_s: 16 rows at once, lanes along them, then a reduction that
+    // leaves row a of the group on lane a (and a + 16)
+    for (int a0 = 0; a0 < N; a0 += 16) {
+      double acc[16];
+#pragma unroll
+      for (int a = 0; a < 16; ++a) acc[a] = 0.0;
+      const int na = min(16, N - a0);
+      const double* K0 = Kku + (b0 + a0) * R;
+      for (int r = lane; r < R; r += 32) {
+        const double x = As[r];
+        if (na == 16) {
+#pragma unroll
+          for (int a = 0; a < 16; ++a) acc[a] = fma(-K0[(int64_t)a * R + r], x, acc[a]);
+        } else {
+#pragma unroll
+          for (int a = 0; a < 16; ++a)
+            if (a < na) acc[a] = fma(-K0[(int64_t)a * R + r], x, acc[a]);
+        }
+      }
+#pragma unroll
+      for (int o = 8; o > 0; o >>= 1) {
+        const bool up = lane & o;
+#pragma unroll
+        for (int a = 0; a < o; ++a) {
+          const double send = up ? acc[a] : acc[a + o], keep = up ? acc[a + o] : acc[a];
+          acc[a] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+        }
+      }
+      double d = acc[0] + __shfl_xor_sync(0xffffffffu, acc[0], 16);
+      if (lane < na) {
+        d += gmpic::row_entry(qcol, qval, qptr[q], qptr[q + 1], bidx[b0 + a0 + lane]);
+        D[a0 + lane] = d;
+        g[a0 + lane] = d;
+      }
+    }
+    __syncwarp();
+    if (N > 0) {
+      warp_lower(Cf + coff[k], N, N, g, lane);
+      warp_lower_t(Cf + coff[k], N, N, g, lane);
+    }
+    double m = 0.0, v = 0.0;
+    for (int r = lane; r < R; r += 32) {
+      double l0 = As[r], l1 = 0.0;
+      v = fma(-l0, ks[r], v);
+      const double* Ar = A + b0 * R + r;
+      int a = 0;
+#pragma unroll 4
+      for (; a + 1 < N; a += 2) {
+        l0 = fma(-g[a], Ar[(int64_t)a * R], l0);
+        l1 = fma(-g[a + 1], Ar[(int64_t)(a + 1) * R], l1);
+      }
+      if (a < N) l0 = fma(-g[a], Ar[(int64_t)a * R], l0);
+      l0 += l1;
+      Lc[r] = l0;
+      m = fma(l0, pmean[r] - mu_u[r], m);
+    }
+    __syncwarp();
+    for (int a = lane; a < N; a += 32) {
+      const int64_t j = bidx[b0 + a];
+      m = fma(g[a], obs[j] - prior_m[j], m);
+      v = fma(-g[a], D[a], v);
+    }
+    for (int r = lane; r < R; r += 32) {
+      double t0 = 0.0, t1 = 0.0;
+      const double* Pr = pcov + r;  // symmetric: column r
+      int c = 0;
+#pragma unroll 4
+      for (; c + 1 < R; c += 2) {
+        t0 = fma(Pr[(int64_t)c * R], Lc[c], t0);
+        t1 = fma(Pr[(int64_t)(c + 1) * R], Lc[c + 1], t1);
+      }
+      if (c < R) t0 = fma(Pr[(int64_t)c * R], Lc[c], t0);
+      v = fma(Lc[r], t0 + t1, v);
+    }
+    m = warp_sum(m);
+    v = warp_sum(v);
+    if (lane == 0) {
+      mean[q] = ms[q] + m;
+      var[q] = kss[q] + v;
+    }
+    __syncwarp();
+  }
 }
 
 gm_status pic_predict(gm_ctx* c, int64_t nq, const double* qs, const double* qx,
@@ -449,16 +807,18 @@ gm_status pic_predict(gm_ctx* c, int64_t nq, const double* qs, const double* qx,
   const int R = S->R;
   const int maxN = std::max(S->max_block, 1);
   // queries per chunk: K_su and its pairs (6 R doubles each: K_su, distances, chord,
-  // value, index) and the scratch (3 R + 2 maxN doubles each) within about 1 GB
-  const int64_t per = 6 * (int64_t)R + 3 * (int64_t)R + 2 * (int64_t)maxN;
+  // value, index) within about 1 GB
+  const int64_t per = 6 * (int64_t)R;
   const int64_t chunk = std::max<int64_t>(1, std::min<int64_t>(nq, (int64_t)(1 << 27) / per));
-  ScopedDev buf(c, (size_t)(chunk * per + 1) * sizeof(double));
+  const int64_t words = 2 * ((int64_t)R + maxN);
+  const WarpPlan plan = warp_plan(c, chunk, words);
+  ScopedDev buf(c, (size_t)(chunk * per + 1 + plan.scratch) * sizeof(double));
   if (!buf.p) return set_error(c, GM_E_NOMEM, "PIC prediction scratch");
   double* si = (double*)buf.p;
   double *sj = si + chunk * R, *ch = sj + chunk * R, *kc = ch + chunk * R, *kp = kc + chunk * R;
   int32_t* idx = (int32_t*)(kp + chunk * R);
-  double* w = kp + 2 * chunk * R;
   unsigned long long* count = (unsigned long long*)((double*)buf.p + chunk * per);
+  double* w = plan.scratch ? (double*)(count + 1) : nullptr;
   cudaStream_t st = c->stream;
   const double inv_cut = 1.0 / c->cfg.cutoff_pc;
   const int taper = c->cfg.taper == GM_TAPER_WENDLAND ? 0 : 1;
@@ -482,8 +842,11 @@ gm_status pic_predict(gm_ctx* c, int64_t nq, const double* qs, const double* qx,
       k_pic_ksu<<<grid_for(c, m), 128, 0, st>>>(m, inv_cut, taper, si, sj, ch, idx, kc, kp);
       GM_LAUNCH_CHECK(c);
     }
+    if (plan.smem > 48 * 1024)
+      GM_CUDA_CHECK(c, cudaFuncSetAttribute(k_pic_point, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                            (int)plan.smem));
     GM_PROF(c, "k_pic_point");
-    k_pic_point<<<(unsigned)ceil_div(nc, 128), 128, 0, st>>>(
+    k_pic_point<<<plan.blocks, 32 * plan.warps, plan.smem, st>>>(
         q0, nc, R, maxN, qblk, S->boff, S->coff, S->bidx, S->Lu, S->C, S->A, S->Kku, S->mu_u,
         S->mean, S->cov, c->obs, c->prior_m, kp, kss, ms, qptr, qcol, qval, w, mean, var);
     GM_LAUNCH_CHECK(c);

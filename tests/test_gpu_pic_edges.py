@@ -59,3 +59,42 @@ def test_pic_sizes(R, sizes, nq, taper):
                                K[np.ix_([j], u)], np.diag(K)[[j]], K[np.ix_([j], groups[k])], m[[j]])
         assert pm[q] == pytest.approx(mm[0], rel=1e-7, abs=1e-9)
         assert pv[q] == pytest.approx(vv[0], rel=1e-6, abs=1e-10)
+
+
+def test_pic_vectors_beyond_shared_memory():
+    """A sub-catalogue whose solve vectors are kept in device memory (3,100 stars):
+    the oracle's formulas on the covariance that a context of all points holds."""
+    import paper_1708_09705_gb300 as gm
+    n, R, nq = 3100, 3, 5
+    cat = make_catalogue("c1_plain_400", n=n, truth="mean")
+    rng = np.random.default_rng(5)
+    f = 6.0                                             # a wide field: a sparse K
+    l = cat["l"].mean() + (cat["l"] - cat["l"].mean()) * f
+    b = cat["b"].mean() + (cat["b"] - cat["b"].mean()) * f
+    j = rng.choice(n, R + nq, replace=False)
+    ll, bb, ss = l[j] + 2e-4, b[j] - 1e-4, 0.97 * cat["s"][j]
+    atil = np.log(np.clip(cat["A_obs"], 0.02, None))
+    sig = cat["A_sigma"] / np.clip(cat["A_obs"], 0.02, None)
+    cfg = gm.config_from_catalogue(cat, precision=gm.PREC_FP64, likelihood=gm.LIK_GAUSS_IN_LNA)
+    L, B, S = (np.concatenate(x) for x in ((l, ll), (b, bb), (cat["s"], ss)))
+    one = np.ones(len(L))
+    with gm.ep_init(cfg, L, B, S, one, one) as ctx:
+        ctx.build_cov()
+        rp, col, val = ctx.get_csr()
+        perm, m = ctx.get_perm(), ctx.get_prior()[0]
+    K = np.zeros((len(L), len(L)))
+    K[perm[np.repeat(np.arange(len(L)), np.diff(rp))], perm[col]] = val
+    u, g = np.arange(n, n + R), np.arange(n)
+    blocks = [dict(Kku=K[np.ix_(g, u)], Kkk=K[np.ix_(g, g)], m=m[g], atil=atil, sig2=sig ** 2)]
+    ref_m, ref_c = P.pitc_posterior_direct(K[np.ix_(u, u)], blocks, m[u])
+    with gm.ep_init(cfg, l, b, cat["s"], atil, sig) as ctx:
+        ctx.build_cov()
+        mean, cov = ctx.pic_posterior(np.zeros(n, np.int32), ll[:R], bb[:R], ss[:R])
+        pm, pv = ctx.pic_predict(np.zeros(nq, np.int32), ll[R:], bb[R:], ss[R:])
+    np.testing.assert_allclose(mean, ref_m, rtol=1e-7, atol=1e-9)
+    np.testing.assert_allclose(cov, ref_c, rtol=1e-6, atol=1e-10)
+    q = np.arange(n + R, n + R + nq)
+    mm, vv = P.pic_predict(K[np.ix_(u, u)], m[u], ref_m, ref_c, blocks[0], K[np.ix_(q, u)],
+                           np.diag(K)[q], K[np.ix_(q, g)], m[q])
+    np.testing.assert_allclose(pm, mm, rtol=1e-7, atol=1e-9)
+    np.testing.assert_allclose(pv, vv, rtol=1e-6, atol=1e-10)
