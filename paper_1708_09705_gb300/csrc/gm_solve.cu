@@ -15,6 +15,8 @@
 // reruns are bit-identical.
 #include <algorithm>
 #include <cmath>
+#include <cstdlib>
+#include <cstring>
 #include <vector>
 
 #include "gm_internal.cuh"
@@ -27,6 +29,7 @@ struct Workspace {
   Buffer r32;                                          // FP32 refinement residual
   Buffer x, r, p, pd, q, dv, minv;                    // solver-precision vectors
   Buffer part;                                        // block partials (single RHS)
+  Buffer cg_sync;                                     // hand-overs of k_cg_run, info
   Buffer P_X, P_R, P_P, P_PD, P_Q;                    // panels n x R
   Buffer P_part, P_scal, P_active;                    // panel partials / scalars
 };
@@ -117,20 +120,20 @@ template <> struct Vec16<float> { using V = float4; using C = int4; };
 template <> struct Vec16<double> { using V = double2; using C = int2; };
 
 template <typename TAcc, typename TX>
-__device__ __forceinline__ TAcc vdot(const float4 v, const int4 c, const TX* __restrict__ x) {
+__device__ __forceinline__ TAcc vdot(const float4 v, const int4 c, const TX* x) {
   return (TAcc)v.x * (TAcc)x[c.x] + (TAcc)v.y * (TAcc)x[c.y] + (TAcc)v.z * (TAcc)x[c.z] +
          (TAcc)v.w * (TAcc)x[c.w];
 }
 template <typename TAcc, typename TX>
-__device__ __forceinline__ TAcc vdot(const double2 v, const int2 c, const TX* __restrict__ x) {
+__device__ __forceinline__ TAcc vdot(const double2 v, const int2 c, const TX* x) {
   return (TAcc)v.x * (TAcc)x[c.x] + (TAcc)v.y * (TAcc)x[c.y];
 }
 
-// This lane's share of sum_{e in [b, e1)} val[e] x[col[e]].
+// This lane's share of sum_{e in [b, e1)} val[e] x[col[e]].  (x is not restrict: the
+// kernel that runs a whole solve writes it between products.)
 template <typename TAcc, typename TA, typename TX>
 __device__ __forceinline__ TAcc row_dot_lane(int64_t b, int64_t e1, const int32_t* __restrict__ col,
-                                             const TA* __restrict__ val,
-                                             const TX* __restrict__ x, int lane) {
+                                             const TA* __restrict__ val, const TX* x, int lane) {
   constexpr int V = 16 / sizeof(TA);
   using VA = typename Vec16<TA>::V;
   using VC = typename Vec16<TA>::C;
@@ -232,6 +235,16 @@ __global__ void __launch_bounds__(kBT) k_cg_init(int64_t n, const TV* __restrict
   }
 }
 
+// The steps of one element, alike in the kernels of a step and of a whole solve.
+template <typename TV>
+__device__ __forceinline__ TV cg_r_step(TV r, TV a, TV q) {
+  return r - a * q;
+}
+template <typename TV>
+__device__ __forceinline__ TV cg_p_step(TV m, TV r, TV beta, TV p) {
+  return m * r + beta * p;
+}
+
 // Iteration it (1-based): alpha = rz_prev / pq; x += alpha p; r -= alpha q;
 // rz_new = r . M^-1 r into the other parity slot, rr = r . r.
 template <typename TV>
@@ -256,7 +269,7 @@ __global__ void __launch_bounds__(kBT) k_cg_update1(int64_t n, int it, const TV*
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
        i += (int64_t)G * blockDim.x) {
     x[i] += a * p[i];
-    TV ri = r[i] - a * q[i];
+    TV ri = cg_r_step(r[i], a, q[i]);
     r[i] = ri;
     rz += (double)ri * (double)(minv[i] * ri);
     rr += (double)ri * (double)ri;
@@ -283,9 +296,232 @@ __global__ void __launch_bounds__(kBT) k_cg_update2(int64_t n, int it, const TV*
   const TV beta = (TV)(rzp > 0 ? rzn / rzp : 0.0);
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
        i += (int64_t)G * blockDim.x) {
-    TV pi = minv[i] * r[i] + beta * p[i];
+    TV pi = cg_p_step(minv[i], r[i], beta, p[i]);
     p[i] = pi;
     pd[i] = dv[i] * pi;
+  }
+}
+
+// ---------------------------------------------------------------- whole solve
+// Blocks of a cooperative launch (every block resident) hand each other one value per
+// step through 16-byte slots {value, step}: written and read as one 128-bit access, so
+// that the value arrives with the signal.  What the writing block wrote before is
+// visible behind the wait to plain loads of the whole reading block.
+constexpr int kSlotSpins = 1 << 22;  // some seconds
+constexpr int kSlotMax = 1024;       // blocks at most
+
+__device__ __forceinline__ void slot_put(ulonglong2* slot, double v, unsigned long long step) {
+  asm volatile(
+      "{\n\t.reg .b128 t;\n\tmov.b128 t, {%1, %2};\n\t"
+      "fence.acq_rel.gpu;\n\tst.relaxed.gpu.global.b128 [%0], t;\n\t}"
+      :
+      : "l"(slot), "l"(__double_as_longlong(v)), "l"(step)
+      : "memory");
+}
+
+// Waits for slots [0, m) to reach `step` and leaves their values in v; false for the
+// whole block when a wait gave up.
+__device__ __forceinline__ bool slots_get(const ulonglong2* slots, int m, unsigned long long step,
+                                          double* v) {
+  int good = 1;
+  for (int k = threadIdx.x; k < m; k += blockDim.x) {
+    unsigned long long a = 0, b = 0;
+    int spins = 0;
+    do {
+      asm volatile(
+          "{\n\t.reg .b128 t;\n\tld.relaxed.gpu.global.b128 t, [%2];\n\t"
+          "mov.b128 {%0, %1}, t;\n\t}"
+          : "=l"(a), "=l"(b)
+          : "l"(slots + k)
+          : "memory");
+    } while (b != step && ++spins < kSlotSpins);
+    if (b != step) good = 0;
+    v[k] = __longlong_as_double((long long)a);
+    asm volatile("fence.acq_rel.gpu;" ::: "memory");
+  }
+  return __syncthreads_and(good) != 0;
+}
+
+// f(sum of m values in shared memory) in every thread: the sum by kBT threads in the
+// order of sum_partials2 in a block of that size, f by the first warp.  The FP64 unit
+// takes 16 clocks of an SM per warp instruction, so no other warp adds or divides.
+template <typename F>
+__device__ __forceinline__ double sum_values(const double* v, int m, double* sh, F f) {
+  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  if (w < kBT / 32) {
+    double a = 0;
+    if (w * 32 < m) {
+      for (int k = threadIdx.x; k < m; k += kBT) a += v[k];
+      a = warp_sum(a);
+    }
+    if (lane == 0) sh[w] = a;
+  }
+  __syncthreads();
+  if (w == 0) {
+    const double t = f(warp_sum(lane < kBT / 32 ? sh[lane] : 0.0));
+    if (lane == 0) sh[32] = t;
+  }
+  __syncthreads();
+  return sh[32];
+}
+
+// p . q of a warp's rows in the order of its rows.  FP32: 32 rows' products (exact in
+// FP64) take one conversion and multiplication on their lanes, then an addition each;
+// with one lane at work a row cost four FP64 instructions.
+struct RowDotsF32 {
+  float p = 0, q = 0;
+  int k = 0;
+  double sum = 0;
+  __device__ __forceinline__ void add(float pi, float qi, int lane) {
+    if (lane == k) {
+      p = pi;
+      q = qi;
+    }
+    if (++k == 32) flush();
+  }
+  __device__ __forceinline__ double flush() {
+    const double v = (double)p * (double)q;
+    for (int t = 0; t < k; ++t) sum += __shfl_sync(0xffffffffu, v, t);
+    k = 0;
+    return sum;
+  }
+};
+struct RowDotsF64 {
+  double sum = 0;
+  __device__ __forceinline__ void add(double pi, double qi, int) { sum += pi * qi; }
+  __device__ __forceinline__ double flush() { return sum; }
+};
+template <typename TV> struct RowDots { using T = RowDotsF64; };
+template <> struct RowDots<float> { using T = RowDotsF32; };
+
+// All iterations of a single-RHS CG behind k_cg_init in one cooperative launch:
+// k_apply_B, k_cg_update1 and k_cg_update2, element for element and sum for sum (the
+// vector steps by the first kBT threads of a block), so the bits are those of the
+// launches.  Three hand-overs an iteration: p . q of all blocks to those that hold
+// vector elements (the first n / kBT), r . z among these, D o p (and the end) from
+// these to all.  Latency bounds it: three launches took 33 to 36 us an iteration at
+// 4,000 to 16,000 stars; a grid barrier per step (atomic count, partial sums read
+// behind it) 24 to 27 us; this 21 to 25.  What is left, in thousands of clocks at
+// 16,000 stars: rows 10, FP64 sums and divisions (some 50 dependent operations) 15,
+// the hand-overs 2 to 4 each.
+// slots: 3 x G, zeroed.  info: iterations (max_it + 1 at the cap), 1 if a wait gave up.
+template <typename TA, typename TV>
+__global__ void __launch_bounds__(kBTB, 2) k_cg_run(
+    int64_t n, const int64_t* __restrict__ row_ptr, const int32_t* __restrict__ col,
+    const TA* __restrict__ val, const TV* __restrict__ dv, const TV* __restrict__ minv, TV* x,
+    TV* r, TV* p, TV* pd, TV* q, double* part, double tol2, int max_it, int check,
+    ulonglong2* slots, int* info, unsigned* flags) {
+  __shared__ double sh[40], v[kSlotMax];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int G = gridDim.x;
+  const int nv = (int)min((int64_t)G, (n + kBT - 1) / kBT);  // blocks with vector elements
+  const bool vec = blockIdx.x < nv;
+  ulonglong2 *s_pq = slots, *s_rz = slots + G, *s_pd = slots + 2 * G;
+  const int64_t warp = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
+  const int64_t nw = ((int64_t)G * blockDim.x) >> 5;
+  const int64_t i0 = threadIdx.x < kBT ? blockIdx.x * (int64_t)kBT + threadIdx.x : n;
+  const int64_t di = (int64_t)G * kBT;
+  const int64_t b0 = warp < n ? row_ptr[warp] : 0, e0 = warp < n ? row_ptr[warp + 1] : 0;
+  bool up = true;
+  double bb = 0, rzp = 0;  // b . b, and r . z of the last iteration (warp 0 of vec blocks)
+  auto same = [](double t) { return t; };
+  if (vec) {
+    for (int k = threadIdx.x; k < nv; k += blockDim.x) v[k] = part[4 * G + k];
+    __syncthreads();
+    bb = sum_values(v, nv, sh, same);
+    __syncthreads();
+    for (int k = threadIdx.x; k < nv; k += blockDim.x) v[k] = part[G + k];
+    __syncthreads();
+    rzp = sum_values(v, nv, sh, same);
+    __syncthreads();
+  }
+  int it = 1;
+  for (; it <= max_it; ++it) {
+    typename RowDots<TV>::T dots;
+    int64_t b = b0, e = e0;
+    for (int64_t i = warp; i < n; i += nw) {
+      const TV pi = __ldcg(p + i), dvi = dv[i];
+      TV acc = row_dot_lane<TV>(b, e, col, val, pd, lane);
+      const int64_t j = min(i + nw, n - 1);  // the next row's range, ahead of the sum
+      b = row_ptr[j];
+      e = row_ptr[j + 1];
+      acc = warp_sum(acc);  // the same in all lanes
+      const TV qi = pi + dvi * acc;
+      if (lane == 0) q[i] = qi;
+      dots.add(pi, qi, lane);
+    }
+    const double pq_w = dots.flush();
+    if (lane == 0) sh[w] = pq_w;
+    __syncthreads();
+    if (w == 0) {
+      const double t = warp_sum(lane < kBTB / 32 ? sh[lane] : 0.0);
+      if (lane == 0) slot_put(s_pq + blockIdx.x, t, it);
+    }
+    bool stop = false;
+    if (vec) {
+      if (!(up = slots_get(s_pq, G, it, v))) break;
+      const TV a = (TV)sum_values(v, G, sh, [&](double pq) {
+        if (!(rzp > 0)) return 0.0;
+        if (pq > 0) return rzp / pq;
+        if (blockIdx.x == 0 && lane == 0) atomicOr(flags, kFlagNotSPD);
+        return 0.0;
+      });
+      if (w < kBT / 32) {
+        double rz = 0, rr = 0;
+        for (int64_t i = i0; i < n; i += di) {
+          x[i] += a * p[i];
+          TV ri = cg_r_step(r[i], a, __ldcg(q + i));
+          r[i] = ri;
+          rz += (double)ri * (double)(minv[i] * ri);
+          rr += (double)ri * (double)ri;
+        }
+        rz = warp_sum(rz);
+        rr = warp_sum(rr);
+        if (lane == 0) {
+          sh[w] = rz;
+          sh[16 + w] = rr;
+        }
+      }
+      __syncthreads();
+      if (w == 1) {
+        const double t = warp_sum(lane < kBT / 32 ? sh[16 + lane] : 0.0);
+        if (lane == 0) part[3 * G + blockIdx.x] = t;
+      }
+      const double t = w == 0 ? warp_sum(lane < kBT / 32 ? sh[lane] : 0.0) : 0.0;
+      __syncthreads();  // ||r||^2 is written before the signal
+      if (threadIdx.x == 0) slot_put(s_rz + blockIdx.x, t, it);
+      if (!(up = slots_get(s_rz, nv, it, v))) break;
+      const TV beta = (TV)sum_values(v, nv, sh, [&](double rzn) {
+        const double t = rzp > 0 ? rzn / rzp : 0.0;
+        rzp = rzn;
+        return t;
+      });
+      if (it % check == 0 || it == max_it) {
+        __syncthreads();
+        for (int k = threadIdx.x; k < nv; k += blockDim.x) v[k] = __ldcg(part + 3 * G + k);
+        __syncthreads();
+        const double rr = sum_values(v, nv, sh, same);
+        stop = !isfinite(rr) || rr <= tol2 * bb;
+      }
+      if (!stop) {
+        for (int64_t i = i0; i < n; i += di) {
+          TV pi = cg_p_step(minv[i], r[i], beta, p[i]);
+          p[i] = pi;
+          pd[i] = dv[i] * pi;
+        }
+      }
+      __syncthreads();
+      if (threadIdx.x == 0) slot_put(s_pd + blockIdx.x, stop ? 1.0 : 0.0, it);
+    }
+    if (!(up = slots_get(s_pd, nv, it, v))) break;
+    stop = v[0] != 0.0;
+    __syncthreads();
+    if (stop) break;
+  }
+  if (threadIdx.x == 0 && blockIdx.x == 0) info[0] = it;
+  if (threadIdx.x == 0 && !up) {
+    info[1] = 1;
+    atomicOr(flags, kFlagTimeout);
   }
 }
 
@@ -932,6 +1168,60 @@ __global__ void k_panel_final_probe(int64_t n, int64_t c0, int64_t n_cols, int R
 // ---------------------------------------------------------------- host
 static int vec_grid(gm_ctx* c) { return 2 * sm_count(c); }
 
+// GM_CG=launches (read per solve): a launch per step, as the deflated solves run.
+static bool cg_in_one_launch() {
+  const char* e = std::getenv("GM_CG");
+  return !e || std::strcmp(e, "launches") != 0;
+}
+
+// The iterations behind k_cg_init in one launch; the partials of ||r||^2 are left in
+// c->h_pinned (G doubles).  *it: iterations, -1 where the grid cannot be resident at
+// once (nothing has run).  Synchronises.
+template <typename TA, typename TV>
+static gm_status cg_run(gm_ctx* c, int G, TV* x, double tol, int max_it, int check, int* it) {
+  Workspace& ws = W(c);
+  cudaStream_t st = c->stream;
+  if (G > kSlotMax) {
+    *it = -1;
+    return GM_OK;
+  }
+  const size_t sync_bytes = (3 * (size_t)G + 1) * sizeof(ulonglong2);
+  if (!ensure(c, ws.cg_sync, sync_bytes)) return set_error(c, GM_E_NOMEM, "CG hand-overs");
+  GM_CUDA_CHECK(c, cudaMemsetAsync(ws.cg_sync.p, 0, sync_bytes, st));
+  int64_t n = c->n;
+  const int64_t* row_ptr = c->row_ptr;
+  const int32_t* col = c->col;
+  const TA* val = (const TA*)c->val;
+  const TV *dv = (const TV*)ws.dv.p, *minv = (const TV*)ws.minv.p;
+  TV *r = (TV*)ws.r.p, *p = (TV*)ws.p.p, *pd = (TV*)ws.pd.p, *q = (TV*)ws.q.p;
+  double* part = (double*)ws.part.p;
+  double tol2 = tol * tol;
+  ulonglong2* slots = (ulonglong2*)ws.cg_sync.p;
+  int* info = (int*)(slots + 3 * G);
+  unsigned* flags = c->d_flags;
+  void* args[] = {&n, &row_ptr, &col, &val, &dv, &minv, &x, &r, &p, &pd,
+                  &q, &part, &tol2, &max_it, &check, &slots, &info, &flags};
+  GM_PROF(c, "k_cg_run");
+  const cudaError_t le = cudaLaunchCooperativeKernel((const void*)k_cg_run<TA, TV>, dim3(G),
+                                                     dim3(kBTB), args, 0, st);
+  if (le == cudaErrorCooperativeLaunchTooLarge || le == cudaErrorNotSupported) {
+    cudaGetLastError();  // fewer SMs for this process than the device has
+    *it = -1;
+  } else {
+    GM_CUDA_CHECK(c, le);
+  }
+  GM_LAUNCH_CHECK(c);
+  if (*it < 0) return GM_OK;
+  double* hp = (double*)c->h_pinned;
+  GM_CUDA_CHECK(c, cudaMemcpyAsync(hp, part + 3 * G, G * sizeof(double), cudaMemcpyDeviceToHost, st));
+  GM_CUDA_CHECK(c, cudaMemcpyAsync(hp + G, info, 2 * sizeof(int), cudaMemcpyDeviceToHost, st));
+  GM_CUDA_CHECK(c, cudaStreamSynchronize(st));
+  const int* hi = (const int*)(hp + G);
+  if (hi[1]) return set_error(c, GM_E_TIMEOUT, "bounded device wait expired");
+  *it = hi[0];
+  return GM_OK;
+}
+
 template <typename TA, typename TV>
 static gm_status cg_single(gm_ctx* c, const TV* rhs, TV* x, double tol, int max_it,
                            int64_t* iters, double* rel_resid) {
@@ -967,6 +1257,19 @@ static gm_status cg_single(gm_ctx* c, const TV* rhs, TV* x, double tol, int max_
   const int check = 8;
   double rr = bb;
   int it = 1;
+  if (!defl && cg_in_one_launch()) {
+    const gm_status rs = cg_run<TA, TV>(c, G, x, tol, max_it, check, &it);
+    if (rs != GM_OK) return rs;
+    if (it >= 0) {
+      rr = 0;
+      for (int k = 0; k < G; ++k) rr += hp[k];
+      if (!std::isfinite(rr)) return set_error(c, GM_E_NONFINITE, "CG residual is not finite");
+      *iters = std::min(it, max_it);
+      *rel_resid = std::sqrt(rr / bb);
+      return GM_OK;
+    }
+    it = 1;
+  }
   for (; it <= max_it; ++it) {
     GM_PROF(c, "k_apply_B");
     k_apply_B<TA, TV><<<G, kBTB, 0, st>>>(n, c->row_ptr, c->col, (const TA*)c->val, dv, p, pd, q, part);
