@@ -731,19 +731,19 @@ bool deflate_tc(gm_ctx* c) { return c->defl && c->defl->ready && c->defl->tc; }
 int deflate_tc_chunks(gm_ctx* c, int R) { return dtc_chunks(c, c->n, R); }
 
 gm_status deflate_step_tc(gm_ctx* c, int R, int nch, const double* alpha, const float* minv,
-                          float* X, float* Rr, const float* P, const float* Q, double* part_rz,
-                          double* part_rr, double* corr8) {
+                          float* Rr, const float* Q, double* part_rz, double* part_rr,
+                          double* corr8) {
   Deflation& F = D(c);
   if (!ensure(c, F.Cp2, (size_t)2 * nch * kDefK * R * sizeof(float)) ||
       !ensure(c, F.cimg, dtc_cimg_bytes(R)))
     return set_error(c, GM_E_NOMEM, "deflation projections");
-  return dtc_step(c, c->n, R, nch, F.yimg.p, alpha, minv, X, Rr, P, Q, part_rz, part_rr,
+  return dtc_step(c, c->n, R, nch, F.yimg.p, alpha, minv, Rr, Q, part_rz, part_rr,
                   (float*)F.Cp2.p, (const float*)F.wv.p, F.cimg.p, corr8);
 }
 
 gm_status deflate_update_tc(gm_ctx* c, int R, const float* minv, const float* dv,
-                            const double* beta, const int* active, const float* Rr, float* P,
-                            float* PD, bool planes) {
+                            const double* alpha, const double* beta, const int* active, float* X,
+                            const float* Rr, float* P, float* PD, bool planes) {
   Deflation& F = D(c);
   uint16_t* pl = nullptr;
   if (planes) {
@@ -751,7 +751,8 @@ gm_status deflate_update_tc(gm_ctx* c, int R, const float* minv, const float* dv
       return set_error(c, GM_E_NOMEM, "BF16 planes of the panel");
     pl = (uint16_t*)c->tc_planes.p;
   }
-  return dtc_update(c, c->n, R, F.ywimg.p, F.cimg.p, minv, dv, beta, active, Rr, P, PD, pl);
+  return dtc_update(c, c->n, R, F.ywimg.p, F.cimg.p, minv, dv, alpha, beta, active, X, Rr,
+                    P, PD, pl);
 }
 
 // Single right-hand side: c = Y^T r, add sum_j w_j c_j^2 to rz_slot[0]

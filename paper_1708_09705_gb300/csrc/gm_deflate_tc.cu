@@ -12,8 +12,7 @@
 //
 // k_dtc_step fuses the CG update of the panel with C's partial sums.  CTA =
 // (128 panel columns, a chunk of 16-row K-steps).  Per K-step the four
-// producer warps load X, P, R and Q of their rows, write X + alpha P and
-// R' = R - alpha Q, accumulate r'^T M^-1 r' and r'^T r' per column, and store
+// producer warps load R and Q of their rows, write R' = R - alpha Q, accumulate r'^T M^-1 r' and r'^T r' per column, and store
 // the three BF16 pieces of R' into a 128-byte-swizzled MN-major B tile; thread
 // 0 bulk-copies the K-step's image of the pieces of Y^T; one thread of the
 // fifth warp issues four MMAs (M = 128, N = 128, K = 16) with the pieces of Y^T
@@ -26,7 +25,7 @@
 // images of C's pieces.
 // k_dtc_update: CTA = (128 rows, 128 columns); bulk copies of the 128 x 64
 // images of Yw's pieces and the 128 x 64 images of C^T's pieces, 24 MMAs (six
-// products x four K-steps of 16), epilogue P = M^-1 R' + acc + beta P on
+// products x four K-steps of 16), epilogue X + alpha P and P = M^-1 R' + acc + beta P on
 // active columns (frozen columns keep P) and D P, either in FP32 or directly
 // as the three BF16 planes the tile product copies its B operand from.  The
 // accumulator rows go through shared memory first, so that every global
@@ -135,19 +134,22 @@ __global__ void k_dtc_img_rows(int64_t n, int64_t nblk, const float* __restrict_
 // ---------------------------------------------------------------- step
 // One producer thread's loads of a K-step.
 struct StepRegs {
-  float4 r[4], x[4], p[4], q[4];
+  float4 r[4], q[4];
   float m[4];
   int v;  // bit h: row h of the K-step is a row of the panel
 };
 
-// alpha null: C's partial rows of R only (X, R untouched, no rz / rr).
-// Three CTAs per SM (registers and shared memory); a second K-step of loads
-// in flight per producer needed ~230 registers (one CTA per SM) or spilled
-// at two CTAs per SM, and was slower either way.
+// alpha null: C's partial rows of R only (R untouched, no rz / rr).
+// Three CTAs per SM (registers and shared memory), the next K-step's loads in flight
+// while one is worked off.  X += alpha P is in k_dtc_update, which reads P anyway:
+// 9.5 panel arrays an iteration through the two kernels instead of 10.5, and the
+// registers of X and P hold the second K-step (with all four arrays it needed ~230
+// registers or spilled).  At 20,000 x 4,640: 482 -> 274 us (4.1 TB/s), and
+// k_dtc_update 361 -> 512 us (4.7 TB/s): 843 -> 786 us an iteration.
 __global__ void __launch_bounds__(kS1Threads, 3) k_dtc_step(
     int64_t n, int R, int kpc, const unsigned char* __restrict__ yimg,
-    const double* __restrict__ alpha, const float* __restrict__ minv, float* __restrict__ X,
-    float* __restrict__ Rr, const float* __restrict__ P, const float* __restrict__ Q,
+    const double* __restrict__ alpha, const float* __restrict__ minv, float* __restrict__ Rr,
+    const float* __restrict__ Q,
     double* __restrict__ part_rz, double* __restrict__ part_rr, float* __restrict__ Cp,
     unsigned* __restrict__ flags) {
   extern __shared__ __align__(1024) unsigned char smem_raw[];
@@ -203,8 +205,8 @@ __global__ void __launch_bounds__(kS1Threads, 3) k_dtc_step(
 #pragma unroll
     for (int e = 0; e < 4; ++e) a[e] = (upd && vcol) ? (float)alpha[col + e] : 0.f;
     int64_t issued = 0;
-    // the loads of one K-step: the thread's four row segments of R (and X,
-    // P, Q when updating)
+    // the loads of one K-step: the thread's four row segments of R (and Q when
+    // updating)
     auto load = [&](int64_t ks, StepRegs& S) {
       S.v = 0;
 #pragma unroll
@@ -213,13 +215,11 @@ __global__ void __launch_bounds__(kS1Threads, 3) k_dtc_step(
         const bool vh = vcol && i < n;
         S.v |= vh ? 1 << h : 0;
         S.m[h] = 0.f;
-        S.r[h] = S.x[h] = S.p[h] = S.q[h] = make_float4(0.f, 0.f, 0.f, 0.f);
+        S.r[h] = S.q[h] = make_float4(0.f, 0.f, 0.f, 0.f);
         if (vh) {
           const int64_t at = i * R + col;
           S.r[h] = *reinterpret_cast<const float4*>(Rr + at);
           if (upd) {
-            S.x[h] = *reinterpret_cast<const float4*>(X + at);
-            S.p[h] = __ldcs(reinterpret_cast<const float4*>(P + at));
             S.q[h] = __ldcs(reinterpret_cast<const float4*>(Q + at));
             S.m[h] = minv[i];
           }
@@ -248,18 +248,13 @@ __global__ void __launch_bounds__(kS1Threads, 3) k_dtc_step(
         float rv[4] = {S.r[h].x, S.r[h].y, S.r[h].z, S.r[h].w};
         if (upd && (S.v >> h & 1)) {
           const int64_t at = (16 * (ks0 + ks) + kr) * R + col;
-          const float xv[4] = {S.x[h].x, S.x[h].y, S.x[h].z, S.x[h].w};
-          const float pv[4] = {S.p[h].x, S.p[h].y, S.p[h].z, S.p[h].w};
           const float qv[4] = {S.q[h].x, S.q[h].y, S.q[h].z, S.q[h].w};
-          float xn[4];
 #pragma unroll
           for (int e = 0; e < 4; ++e) {
-            xn[e] = xv[e] + a[e] * pv[e];
             rv[e] = rv[e] - a[e] * qv[e];
             rz[e].add(rv[e] * (S.m[h] * rv[e]));
             rr[e].add(rv[e] * rv[e]);
           }
-          *reinterpret_cast<float4*>(X + at) = make_float4(xn[0], xn[1], xn[2], xn[3]);
           *reinterpret_cast<float4*>(Rr + at) = make_float4(rv[0], rv[1], rv[2], rv[3]);
         }
         uint2 p1, p2, p3;
@@ -275,10 +270,15 @@ __global__ void __launch_bounds__(kS1Threads, 3) k_dtc_step(
       tg::arrive(tg::smem(&fullB[s]));
       return true;
     };
-    StepRegs A;
-    for (int64_t ks = 0; ks < nks; ++ks) {
-      load(ks, A);
+    // the loads of the next K-step are in flight while one is worked off
+    StepRegs A, B;
+    if (nks > 0) load(0, A);
+    for (int64_t ks = 0; ks < nks; ks += 2) {
+      if (ks + 1 < nks) load(ks + 1, B);
       if (!produce(ks, A)) break;
+      if (ks + 1 >= nks) break;
+      if (ks + 2 < nks) load(ks + 2, A);
+      if (!produce(ks + 1, B)) break;
     }
     if (t == 0 && *abort_v) {  // bounded waits for the bulk copies still in flight
       for (int qq = 0; qq < kS1Ring; ++qq) {
@@ -408,26 +408,27 @@ __global__ void k_dtc_sum(int R, int ncg, int nparts, const float* __restrict__ 
 // ---------------------------------------------------------------- update
 // One lane's loads of two row pairs of the update's epilogue.
 struct EpiRegs {
-  float4 r[2], p[2];
+  float4 r[2], p[2], x[2];
   float m[2], d[2];
   int64_t at[2];
   int v;  // bit u: row pair u is a row of the panel
 };
 
-// beta null: P = M^-1 R' + Yw C on every column (the first residuals).
+// beta null: P = M^-1 R' + Yw C on every column (the first residuals; X untouched).
 // planes null: PD = d o P in FP32, else its three BF16 pieces, piece p at
 // planes + p * plane_elems (row-major like PD).
 __global__ void __launch_bounds__(256, 2) k_dtc_update(
     int64_t n, int R, const unsigned char* __restrict__ ywimg,
     const unsigned char* __restrict__ cimg, const float* __restrict__ minv,
-    const float* __restrict__ dv, const double* __restrict__ beta, const int* __restrict__ active,
+    const float* __restrict__ dv, const double* __restrict__ alpha,
+    const double* __restrict__ beta, const int* __restrict__ active, float* __restrict__ X,
     const float* __restrict__ Rr, float* __restrict__ P, float* __restrict__ PD,
     uint16_t* __restrict__ planes, int64_t plane_elems, unsigned* __restrict__ flags) {
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   __shared__ uint64_t full, done;
   __shared__ uint32_t tmem_base;
   __shared__ int abort_flag;
-  __shared__ float sh_be[128];
+  __shared__ float sh_be[128], sh_al[128];
   __shared__ int sh_act[128];
   volatile int* abort_v = &abort_flag;
   const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
@@ -446,6 +447,7 @@ __global__ void __launch_bounds__(256, 2) k_dtc_update(
     const int act = c < R && (!active || active[c] != 0);
     sh_act[t] = act;
     sh_be[t] = (beta && act) ? (float)beta[c] : 0.f;
+    sh_al[t] = (beta && c < R) ? (float)alpha[c] : 0.f;
   }
   if (warp == 0) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 128;" ::"r"(
@@ -505,12 +507,15 @@ __global__ void __launch_bounds__(256, 2) k_dtc_update(
       const int rl = 4 * bt + 2 * u + sub;
       const int64_t i = r0 + 32 * quad + rl;
       E.at[u] = i * R + c0 + cl;
-      E.r[u] = E.p[u] = make_float4(0.f, 0.f, 0.f, 0.f);
+      E.r[u] = E.p[u] = E.x[u] = make_float4(0.f, 0.f, 0.f, 0.f);
       E.m[u] = E.d[u] = 0.f;
       if (i < n) {
         E.v |= 1 << u;
         E.r[u] = __ldcs(reinterpret_cast<const float4*>(Rr + E.at[u]));
-        if (beta) E.p[u] = *reinterpret_cast<const float4*>(P + E.at[u]);
+        if (beta) {
+          E.p[u] = *reinterpret_cast<const float4*>(P + E.at[u]);
+          E.x[u] = __ldcs(reinterpret_cast<const float4*>(X + E.at[u]));
+        }
         E.m[u] = minv[i];
         E.d[u] = dv[i];
       }
@@ -525,6 +530,12 @@ __global__ void __launch_bounds__(256, 2) k_dtc_update(
       const float z4[4] = {zv.x, zv.y, zv.z, zv.w};
       const float r4[4] = {E.r[u].x, E.r[u].y, E.r[u].z, E.r[u].w};
       float p4[4] = {E.p[u].x, E.p[u].y, E.p[u].z, E.p[u].w};
+      if (beta) {
+        float x4[4] = {E.x[u].x, E.x[u].y, E.x[u].z, E.x[u].w};
+#pragma unroll
+        for (int e = 0; e < 4; ++e) x4[e] = x4[e] + sh_al[cl + e] * p4[e];
+        __stcs(reinterpret_cast<float4*>(X + E.at[u]), make_float4(x4[0], x4[1], x4[2], x4[3]));
+      }
 #pragma unroll
       for (int e = 0; e < 4; ++e) {
         const float pn = fmaf(sh_be[cl + e], p4[e], fmaf(E.m[u], r4[e], z4[e]));
@@ -639,9 +650,8 @@ int dtc_chunks(gm_ctx* c, int64_t n, int R) {
 }
 
 gm_status dtc_step(gm_ctx* c, int64_t n, int R, int nch, const void* yimg, const double* alpha,
-                   const float* minv, float* X, float* Rr, const float* P, const float* Q,
-                   double* part_rz, double* part_rr, float* Cp, const float* w, void* cimg,
-                   double* corr8) {
+                   const float* minv, float* Rr, const float* Q, double* part_rz,
+                   double* part_rr, float* Cp, const float* w, void* cimg, double* corr8) {
   gm_status a = dtc_attributes(c);
   if (a != GM_OK) return a;
   const int64_t nks = ceil_div(n, 16);
@@ -649,7 +659,7 @@ gm_status dtc_step(gm_ctx* c, int64_t n, int R, int nch, const void* yimg, const
   const int ncg = (int)ceil_div(R, kS1Cols);
   GM_PROF(c, "k_dtc_step");
   k_dtc_step<<<dim3((unsigned)ncg, (unsigned)nch), kS1Threads, kS1Smem, c->stream>>>(
-      n, R, kpc, (const unsigned char*)yimg, alpha, minv, X, Rr, P, Q, part_rz, part_rr, Cp,
+      n, R, kpc, (const unsigned char*)yimg, alpha, minv, Rr, Q, part_rz, part_rr, Cp,
       c->d_flags);
   GM_LAUNCH_CHECK(c);
   GM_PROF(c, "k_dtc_sum");
@@ -660,14 +670,16 @@ gm_status dtc_step(gm_ctx* c, int64_t n, int R, int nch, const void* yimg, const
 }
 
 gm_status dtc_update(gm_ctx* c, int64_t n, int R, const void* ywimg, const void* cimg,
-                     const float* minv, const float* dv, const double* beta, const int* active,
-                     const float* Rr, float* P, float* PD, uint16_t* planes) {
+                     const float* minv, const float* dv, const double* alpha,
+                     const double* beta, const int* active, float* X, const float* Rr, float* P,
+                     float* PD, uint16_t* planes) {
   gm_status a = dtc_attributes(c);
   if (a != GM_OK) return a;
   GM_PROF(c, "k_dtc_update");
   k_dtc_update<<<dim3((unsigned)ceil_div(R, 128), (unsigned)ceil_div(n, 128)), 256, kU2Smem,
                  c->stream>>>(n, R, (const unsigned char*)ywimg, (const unsigned char*)cimg, minv,
-                              dv, beta, active, Rr, P, PD, planes, n * (int64_t)R, c->d_flags);
+                              dv, alpha, beta, active, X, Rr, P, PD, planes, n * (int64_t)R,
+                              c->d_flags);
   GM_LAUNCH_CHECK(c);
   return GM_OK;
 }

@@ -408,18 +408,19 @@ void deflate_free(gm_ctx* c);
 bool deflate_tc(gm_ctx* c);
 // row chunks of deflate_step_tc for a panel of R columns (its partial rows)
 int deflate_tc_chunks(gm_ctx* c, int R);
-// alpha non-null: X += alpha P, Rr -= alpha Q and the per-chunk partial sums
+// alpha non-null: Rr -= alpha Q and the per-chunk partial sums
 // of r^T M^-1 r / r^T r (part_rz / part_rr, nch rows of R); alpha null: Rr
 // only.  Then C = Y^T Rr for deflate_update_tc and corr8 (8 rows of R) with
 // sum over rows = sum_j w_j C_jc^2.
 gm_status deflate_step_tc(gm_ctx* c, int R, int nch, const double* alpha, const float* minv,
-                          float* X, float* Rr, const float* P, const float* Q, double* part_rz,
-                          double* part_rr, double* corr8);
-// P = M^-1 Rr + Yw C + beta P on active columns (all, beta 0 when null); PD =
-// d o P in FP32, or (planes) its three BF16 pieces in c->tc_planes.
+                          float* Rr, const float* Q, double* part_rz, double* part_rr,
+                          double* corr8);
+// X += alpha P (beta non-null), then P = M^-1 Rr + Yw C + beta P on active columns
+// (all, beta 0 when null); PD = d o P in FP32, or (planes) its three BF16 pieces in
+// c->tc_planes.
 gm_status deflate_update_tc(gm_ctx* c, int R, const float* minv, const float* dv,
-                            const double* beta, const int* active, const float* Rr, float* P,
-                            float* PD, bool planes);
+                            const double* alpha, const double* beta, const int* active, float* X,
+                            const float* Rr, float* P, float* PD, bool planes);
 // kernels of the tensor-core form (gm_deflate_tc.cu)
 size_t dtc_yimg_bytes(int64_t n);
 size_t dtc_rowimg_bytes(int64_t n);
@@ -428,12 +429,12 @@ gm_status dtc_images(gm_ctx* c, int64_t n, const float* Y, const float* Yw, void
                      void* ywimg);
 int dtc_chunks(gm_ctx* c, int64_t n, int R);
 gm_status dtc_step(gm_ctx* c, int64_t n, int R, int nch, const void* yimg, const double* alpha,
-                   const float* minv, float* X, float* Rr, const float* P, const float* Q,
-                   double* part_rz, double* part_rr, float* Cp, const float* w, void* cimg,
-                   double* corr8);
+                   const float* minv, float* Rr, const float* Q, double* part_rz,
+                   double* part_rr, float* Cp, const float* w, void* cimg, double* corr8);
 gm_status dtc_update(gm_ctx* c, int64_t n, int R, const void* ywimg, const void* cimg,
-                     const float* minv, const float* dv, const double* beta, const int* active,
-                     const float* Rr, float* P, float* PD, uint16_t* planes);
+                     const float* minv, const float* dv, const double* alpha,
+                     const double* beta, const int* active, float* X, const float* Rr, float* P,
+                     float* PD, uint16_t* planes);
 
 // Row-block tiles of K for the FP32 variance panels (gm_tiles.cu).
 gm_status tiles_build(gm_ctx* c);

@@ -921,31 +921,31 @@ __global__ void __launch_bounds__(32 * kRedWarps) k_panel_reduce(
   if (mode != 1 && lane == 0 && above) atomicAdd(n_active, __popc(above));
 }
 
-// X += alpha P, Rr -= alpha Q, partial rz (with M^-1) and rr.
+// Rr -= alpha Q, partial rz (with M^-1) and rr.  (X += alpha P is in k_panel_update2,
+// which reads P anyway: nine panel arrays an iteration through the two passes instead
+// of ten.)  Blocks: column groups of 32 fastest.
 template <typename TV>
 __global__ void __launch_bounds__(kBT) k_panel_update1(int64_t n, int R, const TV* __restrict__ minv,
                                                        const double* __restrict__ scal,
-                                                       TV* __restrict__ X, TV* __restrict__ Rr,
-                                                       const TV* __restrict__ P,
+                                                       TV* __restrict__ Rr,
                                                        const TV* __restrict__ Q,
                                                        double* __restrict__ part_rz,
                                                        double* __restrict__ part_rr) {
   __shared__ double sh_a[8][32], sh_b[8][32];
   const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
-  const int c = blockIdx.y * 32 + lane;
-  const int64_t w = (int64_t)blockIdx.x * (blockDim.x >> 5) + wib;
-  const int64_t nw = (int64_t)gridDim.x * (blockDim.x >> 5);
+  const int nc = R >> 5, rb = blockIdx.x / nc, nrb = gridDim.x / nc;
+  const int c = (blockIdx.x - rb * nc) * 32 + lane;
+  const int64_t w = (int64_t)rb * (blockDim.x >> 5) + wib;
+  const int64_t nw = (int64_t)nrb * (blockDim.x >> 5);
   const TV a = (TV)scal[c];
   PartialSum<TV> rz, rr;
   // four rows per pass with all loads issued first (memory-level parallelism)
   int64_t i = w;
   for (; i + 3 * nw < n; i += 4 * nw) {
-    TV x[4], p[4], r[4], q[4], m[4];
+    TV r[4], q[4], m[4];
 #pragma unroll
     for (int u = 0; u < 4; ++u) {
       const int64_t k = (i + u * nw) * R + c;
-      x[u] = X[k];
-      p[u] = P[k];
       r[u] = Rr[k];
       q[u] = Q[k];
       m[u] = minv[i + u * nw];
@@ -953,7 +953,6 @@ __global__ void __launch_bounds__(kBT) k_panel_update1(int64_t n, int R, const T
 #pragma unroll
     for (int u = 0; u < 4; ++u) {
       const int64_t k = (i + u * nw) * R + c;
-      X[k] = x[u] + a * p[u];
       const TV ri = r[u] - a * q[u];
       Rr[k] = ri;
       rz.add(ri * (m[u] * ri));
@@ -962,7 +961,6 @@ __global__ void __launch_bounds__(kBT) k_panel_update1(int64_t n, int R, const T
   }
   for (; i < n; i += nw) {
     int64_t k = i * R + c;
-    X[k] += a * P[k];
     TV ri = Rr[k] - a * Q[k];
     Rr[k] = ri;
     rz.add(ri * (minv[i] * ri));
@@ -977,30 +975,124 @@ __global__ void __launch_bounds__(kBT) k_panel_update1(int64_t n, int R, const T
       s1 += sh_a[k][lane];
       s2 += sh_b[k][lane];
     }
-    part_rz[(int64_t)blockIdx.x * R + c] = s1;
-    part_rr[(int64_t)blockIdx.x * R + c] = s2;
+    part_rz[(int64_t)rb * R + c] = s1;
+    part_rr[(int64_t)rb * R + c] = s2;
   }
 }
 
-// P = M^-1 Rr + beta P (active columns), PD = d o P: in the panel's precision,
-// or (planes) as its three BF16 pieces, piece p at planes + p * plane_elems,
-// which the asynchronous tile product reads (the split of k_split3_planes,
-// without a pass of its own over PD).
+// The same for FP32 panels, whose single-precision alpha and beta flip with the
+// grouping of the compensated sums: nvb row groups of eight warps, as the panel
+// product's grid has them, four groups to a block.  The sums are added in pairs of
+// floats (hi, lo: 2^-48), a warp per group and sum, and converted once per block: with
+// FP64 conversions and additions, 16 clocks of an SM each, they were half of the pass
+// (60 -> 47 us at 4,000 x 4,000, 33 -> 31 at 8,000 x 1,024).
+// SHORT (at most two rows a warp and group): the loads of all groups first.
+constexpr int kUpdGroups = 4;
+template <bool XUP, bool SHORT>
+__global__ void __launch_bounds__(kBT) k_panel_update1_f32(
+    int64_t n, int R, int nvb, const float* __restrict__ minv, const double* __restrict__ scal,
+    float* __restrict__ X, float* __restrict__ Rr, const float* __restrict__ P,
+    const float* __restrict__ Q, double* __restrict__ part_rz, double* __restrict__ part_rr) {
+  __shared__ float2 sh[2][kUpdGroups][8][32];
+  constexpr int U = SHORT ? 2 : 4, V = SHORT ? kUpdGroups : 1;
+  const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
+  const int nc = R >> 5, B = blockIdx.x / nc;
+  const int c = (blockIdx.x - B * nc) * 32 + lane;
+  const int64_t nw = (int64_t)nvb * 8;
+  const float a = (float)scal[c];
+#pragma unroll
+  for (int v0 = 0; v0 < kUpdGroups; v0 += V) {
+    PartialSum<float> rz[V], rr[V];
+    // row group v0 + v starts at row i0 + 8 v
+    const int64_t i0 = (int64_t)(kUpdGroups * B + v0) * 8 + wib;
+    const int nv = min(V, nvb - (kUpdGroups * B + v0));  // groups there are
+    for (int64_t i = i0; nv > 0 && i < n; i += U * nw) {
+      float x[V][U], p[V][U], r[V][U], q[V][U], m[V][U];
+#pragma unroll
+      for (int v = 0; v < V; ++v)
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+          const int64_t j = i + 8 * v + u * nw, k = j * R + c;
+          const bool in = v < nv && j < n;
+          if (XUP) {
+            x[v][u] = in ? X[k] : 0.f;
+            p[v][u] = in ? P[k] : 0.f;
+          }
+          r[v][u] = in ? Rr[k] : 0.f;
+          q[v][u] = in ? Q[k] : 0.f;
+          m[v][u] = in ? minv[j] : 0.f;
+        }
+#pragma unroll
+      for (int v = 0; v < V; ++v)
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+          const int64_t j = i + 8 * v + u * nw, k = j * R + c;
+          if (v < nv && j < n) {
+            if (XUP) X[k] = x[v][u] + a * p[v][u];
+            const float ri = r[v][u] - a * q[v][u];
+            Rr[k] = ri;
+            rz[v].add(ri * (m[v][u] * ri));
+            rr[v].add(ri * ri);
+          }
+        }
+    }
+#pragma unroll
+    for (int v = 0; v < V; ++v) {
+      sh[0][v0 + v][wib][lane] = make_float2(rz[v].s, rz[v].c);
+      sh[1][v0 + v][wib][lane] = make_float2(rr[v].s, rr[v].c);
+    }
+  }
+  __syncthreads();
+  static_assert(2 * kUpdGroups == kBT / 32, "a warp per group and sum");
+  const int v = wib >> 1, which = wib & 1;
+  float hi = 0.f, lo = 0.f;
+  auto add = [&](float th, float tl) {  // + th + tl
+    const float t = hi + th, b = t - hi;
+    lo += ((hi - (t - b)) + (th - b)) + tl;
+    hi = t;
+  };
+#pragma unroll
+  for (int k = 0; k < 8; ++k) {
+    const float2 t = sh[which][v][k][lane];  // the value is t.x - t.y
+    add(t.x, -t.y);
+  }
+  __syncthreads();
+  sh[which][v][0][lane] = make_float2(hi, lo);
+  __syncthreads();
+  if (v != 0) return;
+#pragma unroll
+  for (int k = 1; k < kUpdGroups; ++k) {
+    const float2 t = sh[which][k][0][lane];
+    add(t.x, t.y);
+  }
+  (which ? part_rr : part_rz)[(int64_t)B * R + c] = (double)hi + (double)lo;
+}
+
+// X += alpha P; P = M^-1 Rr + beta P (active columns), PD = d o P: in the panel's
+// precision, or (planes) as its three BF16 pieces, piece p at planes + p *
+// plane_elems, which the asynchronous tile product reads (the split of
+// k_split3_planes, without a pass of its own over PD).
 template <typename TV, bool PLANES>
 __global__ void __launch_bounds__(kBT) k_panel_update2(int64_t n, int R, const TV* __restrict__ minv,
                                                        const TV* __restrict__ dv,
                                                        const double* __restrict__ scal,
                                                        const int* __restrict__ active,
+                                                       TV* __restrict__ X,
                                                        const TV* __restrict__ Rr,
                                                        TV* __restrict__ P, TV* __restrict__ PD,
                                                        uint16_t* __restrict__ planes,
                                                        int64_t plane_elems) {
   const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
-  const int c = blockIdx.y * 32 + lane;
-  if (!active[c]) return;  // frozen column: P is never read with alpha != 0
-  const int64_t w = (int64_t)blockIdx.x * (blockDim.x >> 5) + wib;
-  const int64_t nw = (int64_t)gridDim.x * (blockDim.x >> 5);
-  const TV be = (TV)scal[R + c];
+  const int nc = R >> 5, rb = blockIdx.x / nc, nrb = gridDim.x / nc;
+  const int c = (blockIdx.x - rb * nc) * 32 + lane;
+  const TV al = (TV)scal[c], be = (TV)scal[R + c];
+  const int64_t w = (int64_t)rb * (blockDim.x >> 5) + wib;
+  const int64_t nw = (int64_t)nrb * (blockDim.x >> 5);
+  if (!active[c]) {  // frozen column: P is never read with alpha != 0
+    if (al != (TV)0)   // frozen by this iteration: its last step
+      for (int64_t i = w; i < n; i += nw) X[i * R + c] += al * P[i * R + c];
+    return;
+  }
   auto put = [&](int64_t k, TV v) {
     if constexpr (PLANES) {
       uint32_t a, b, d;
@@ -1014,10 +1106,11 @@ __global__ void __launch_bounds__(kBT) k_panel_update2(int64_t n, int R, const T
   };
   int64_t i = w;
   for (; i + 3 * nw < n; i += 4 * nw) {
-    TV r[4], p[4], m[4], d[4];
+    TV x[4], r[4], p[4], m[4], d[4];
 #pragma unroll
     for (int u = 0; u < 4; ++u) {
       const int64_t k = (i + u * nw) * R + c;
+      x[u] = X[k];
       r[u] = Rr[k];
       p[u] = P[k];
       m[u] = minv[i + u * nw];
@@ -1026,6 +1119,7 @@ __global__ void __launch_bounds__(kBT) k_panel_update2(int64_t n, int R, const T
 #pragma unroll
     for (int u = 0; u < 4; ++u) {
       const int64_t k = (i + u * nw) * R + c;
+      X[k] = x[u] + al * p[u];
       const TV pi = m[u] * r[u] + be * p[u];
       P[k] = pi;
       put(k, d[u] * pi);
@@ -1033,6 +1127,7 @@ __global__ void __launch_bounds__(kBT) k_panel_update2(int64_t n, int R, const T
   }
   for (; i < n; i += nw) {
     int64_t k = i * R + c;
+    X[k] += al * P[k];
     TV pi = minv[i] * Rr[k] + be * P[k];
     P[k] = pi;
     put(k, dv[i] * pi);
@@ -1505,8 +1600,11 @@ static gm_status panels(gm_ctx* c, int64_t n_rows, const int64_t* row_ptr, const
   // flight), eight where that still leaves a dozen warps per scheduler.  (The
   // product's grid gave them two to three rows a warp, one after another:
   // 143 us for update1 at 4,000 x 4,000, 2.7 TB/s.)
-  const int rpw = n * (R / 32) / 8 >= 48ll * sms ? 8 : 4;
-  const int nbe = (int)ceil_div(n, 8 * rpw);
+  // FP32 sums keep the product's groups of rows (k_panel_update1_f32).
+  const int64_t panel_rows = n * (R / 32) / 8;
+  const int rpw = panel_rows >= 48ll * sms ? 8 : 4;
+  const int nbw = (int)ceil_div(n, 8 * rpw);      // blocks of the element-wise passes
+  const int nbe = sizeof(TV) == 4 ? nbx : nbw;    // partial rows of their sums
   const size_t pbytes = (size_t)n * R * sizeof(TV);
   // spectral deflation of the preconditioner (FP32 star panels of one field;
   // the vectors are prepared per refresh, before the mean solve), in its
@@ -1548,6 +1646,10 @@ static gm_status panels(gm_ctx* c, int64_t n_rows, const int64_t* row_ptr, const
   const int max_it = c->cfg.cg_max_iter;
   int* hn = (int*)c->h_pinned;
   dim3 grid(nbx, (unsigned)(R / 32)), egrid(nbe, (unsigned)(R / 32));
+  // the iteration's passes: column groups fastest, so that what runs at once reads
+  // neighbouring parts of the same rows
+  const unsigned ugrid = (unsigned)(nbw * (R / 32));
+  const unsigned u1grid = (unsigned)(ceil_div(nbe, kUpdGroups) * (R / 32));
   const int rb = (int)std::min<int64_t>(ceil_div(n_rows * 32, 256), 16 * sms);
   const int redb = (int)(R / 32);
   // warps of a reduction over `rows` partial rows: four rows each
@@ -1606,11 +1708,11 @@ static gm_status panels(gm_ctx* c, int64_t n_rows, const int64_t* row_ptr, const
       gm_status ds;
       if (defl_tc) {
         planes = tc_variant(c, (int)R) == 4;
-        ds = deflate_step_tc(c, (int)R, nch, nullptr, (const float*)minv, (float*)X, (float*)Rr,
-                             (const float*)P, (const float*)Q, nullptr, nullptr, corr);
+        ds = deflate_step_tc(c, (int)R, nch, nullptr, (const float*)minv, (float*)Rr,
+                             (const float*)Q, nullptr, nullptr, corr);
         if (ds == GM_OK)
-          ds = deflate_update_tc(c, (int)R, (const float*)minv, (const float*)dv, nullptr,
-                                 nullptr, (const float*)Rr, (float*)P, (float*)PD, planes);
+          ds = deflate_update_tc(c, (int)R, (const float*)minv, (const float*)dv, nullptr, nullptr,
+                                 nullptr, nullptr, (const float*)Rr, (float*)P, (float*)PD, planes);
       } else {
         ds = deflate_rhs(c, (int)R, (const float*)Rr, corr);
         if (ds == GM_OK)
@@ -1640,16 +1742,25 @@ static gm_status panels(gm_ctx* c, int64_t n_rows, const int64_t* row_ptr, const
                                                  pa, nullptr, nullptr, 0, scal, active, n_active,
                                                  c->d_flags);
       GM_LAUNCH_CHECK(c);
-      int nbr = nbe;  // partial rows of rz / rr
+      // partial rows of rz / rr
+      int nbr = sizeof(TV) == 4 ? (int)ceil_div(nbe, kUpdGroups) : nbe;
       if (defl_tc) {
-        // X, Rr update fused with C = Y^T Rr and the deflation rows
-        gm_status ds = deflate_step_tc(c, (int)R, nch, scal, (const float*)minv, (float*)X,
-                                       (float*)Rr, (const float*)P, (const float*)Q, pa, pb, corr);
+        // Rr update fused with C = Y^T Rr and the deflation rows
+        gm_status ds = deflate_step_tc(c, (int)R, nch, scal, (const float*)minv, (float*)Rr,
+                                       (const float*)Q, pa, pb, corr);
         if (ds != GM_OK) return ds;
         nbr = nch;
       } else {
         GM_PROF(c, "k_panel_update1");
-        k_panel_update1<TV><<<egrid, kBT, 0, st>>>(n, (int)R, minv, scal, X, Rr, P, Q, pa, pb);
+        // X with P in k_panel_update2, but the CUDA-core deflation update has no X
+        if constexpr (sizeof(TV) == 4) {
+          const bool brief = n <= 16ll * nbe;  // two rows a warp at most
+          auto kern = defl ? (brief ? k_panel_update1_f32<true, true> : k_panel_update1_f32<true, false>)
+                           : (brief ? k_panel_update1_f32<false, true> : k_panel_update1_f32<false, false>);
+          kern<<<u1grid, kBT, 0, st>>>(n, (int)R, nbe, minv, scal, X, Rr, P, Q, pa, pb);
+        } else {
+          k_panel_update1<TV><<<ugrid, kBT, 0, st>>>(n, (int)R, minv, scal, Rr, Q, pa, pb);
+        }
         GM_LAUNCH_CHECK(c);
         if (defl) {
           gm_status ds = deflate_rhs(c, (int)R, (const float*)Rr, corr);
@@ -1665,8 +1776,8 @@ static gm_status panels(gm_ctx* c, int64_t n_rows, const int64_t* row_ptr, const
       if (defl_tc) {
         planes = tc_variant(c, (int)R) == 4;
         gm_status ds = deflate_update_tc(c, (int)R, (const float*)minv, (const float*)dv,
-                                         scal + R, active, (const float*)Rr, (float*)P,
-                                         (float*)PD, planes);
+                                         scal, scal + R, active, (float*)X, (const float*)Rr,
+                                         (float*)P, (float*)PD, planes);
         if (ds != GM_OK) return ds;
       } else if (defl) {
         gm_status ds = deflate_update(c, (int)R, nbx, (const float*)minv, (const float*)dv,
@@ -1676,12 +1787,12 @@ static gm_status panels(gm_ctx* c, int64_t n_rows, const int64_t* row_ptr, const
         GM_PROF(c, "k_panel_update2");
         planes = sizeof(TV) == 4 && c->tc_nblk > 0 && tc_variant(c, (int)R) == 4;
         if (planes)
-          k_panel_update2<TV, true><<<egrid, kBT, 0, st>>>(n, (int)R, minv, dv, scal, active, Rr,
+          k_panel_update2<TV, true><<<ugrid, kBT, 0, st>>>(n, (int)R, minv, dv, scal, active, X, Rr,
                                                            P, PD, (uint16_t*)c->tc_planes.p,
                                                            n * (int64_t)R);
         else
-          k_panel_update2<TV, false><<<egrid, kBT, 0, st>>>(n, (int)R, minv, dv, scal, active, Rr,
-                                                            P, PD, nullptr, 0);
+          k_panel_update2<TV, false><<<ugrid, kBT, 0, st>>>(n, (int)R, minv, dv, scal, active, X,
+                                                            Rr, P, PD, nullptr, 0);
         GM_LAUNCH_CHECK(c);
       }
       if (it % check == 0 || it == max_it) {
