@@ -4,6 +4,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <cstdlib>
+#include <cstring>
 #include <string>
 #include <vector>
 
@@ -294,6 +296,13 @@ inline int sm_count(gm_ctx* c) {
 }
 
 inline int64_t ceil_div(int64_t a, int64_t b) { return (a + b - 1) / b; }
+
+// GM_WAIT_EXPIRES=<where>: one thread group of that kernel takes a wait that has
+// completed for one that ran out, so that tests reach the way out of it.
+inline bool wait_expires(const char* where) {
+  const char* e = std::getenv("GM_WAIT_EXPIRES");
+  return e && std::strcmp(e, where) == 0;
+}
 
 // ---------------------------------------------------------------- host rules
 // Gauss-Legendre on [-1,1] and Gauss-Hermite (weight exp(-x^2)) by Newton
