@@ -480,10 +480,13 @@ struct BandRule {
 // re-expanded about the middle of each segment, leading coefficients in two
 // floats; its error (2e-12 of g(0)) stays the rule's largest.  It covers
 // 2^kDfEmin <= x < 2^11 in shared memory; smaller separations (nodes that
-// coincide: the diagonal) use the FP64 table.
+// coincide: the diagonal) use the FP64 table.  Nodes of the same index are s_i - s_j
+// times the node apart, taken from the FP64 difference: from the two products, of
+// which 48 bits are kept, stars at nearly equal distances lost the separation.
 // PIC workload at 6,000 stars (cross-covariances of 4,140 points): 152 ms with
-// FP64 instructions, 19.2 ms so; entries differ by 1e-13 (against FP64 Bessel
-// functions both are 1.3e-10 off, on the diagonal).
+// FP64 instructions, 19.2 ms so.  Against FP64 Bessel functions entries between
+// different stars are 1.0e-12 off (largest 3.6e-12) in both forms, the diagonal
+// 1.4e-10 (the table ends at x = 2^-100).
 struct F2 {
   float h, l;
 };
@@ -607,9 +610,9 @@ struct DfRule {
     return {r.h, __fadd_rn(r.l, __fadd_rn(e, c.y))};
   }
 
-  // sum over the nodes of both sightlines
-  __device__ __forceinline__ double pair(F2 A, F2 B, F2 c2) const {
-    F2 tp[KPL], ct[KPL], acc[KPL];
+  // sum over the nodes of both sightlines; D = A - B
+  __device__ __forceinline__ double pair(F2 A, F2 B, F2 D, F2 c2) const {
+    F2 tp[KPL], ct[KPL], acc[KPL], dq[KPL];
     __syncwarp();
 #pragma unroll
     for (int k = 0; k < KPL; ++k) {
@@ -617,6 +620,7 @@ struct DfRule {
       const float4 z = q < Q ? zw[q] : make_float4(0.f, 0.f, 0.f, 0.f);
       const F2 zn = {z.x, z.y};
       tp[k] = f2_mul(B, zn);
+      dq[k] = f2_mul(D, zn);
       ct[k] = f2_mul(c2, tp[k]);
       acc[k] = {0.f, 0.f};
       const F2 t = f2_mul(A, zn);
@@ -630,10 +634,12 @@ struct DfRule {
       const F2 w = {z.z, z.w};
 #pragma unroll
       for (int k = 0; k < KPL; ++k) {
-        const F2 d = f2_sum(t.x, -tp[k].h);
-        const float dl = __fadd_rn(d.l, __fsub_rn(t.y, tp[k].l));
+        F2 d = f2_sum(t.x, -tp[k].h);
+        // where the high parts (nearly) cancel the low ones are all that is left
+        d = f2_fast(d.h, __fadd_rn(d.l, __fsub_rn(t.y, tp[k].l)));
+        if (q == lane + 32 * k) d = dq[k];
         const float p = __fmul_rn(d.h, d.h);
-        const float pe = __fmaf_rn(2.f * d.h, dl, __fmaf_rn(d.h, d.h, -p));
+        const float pe = __fmaf_rn(2.f * d.h, d.l, __fmaf_rn(d.h, d.h, -p));
         const float c = __fmul_rn(t.x, ct[k].h);
         const float ce = __fmaf_rn(t.y, ct[k].h,
                                    __fmaf_rn(t.x, ct[k].l, __fmaf_rn(t.x, ct[k].h, -c)));
@@ -661,14 +667,15 @@ struct DfRule {
 
   __device__ __forceinline__ double R(bool active, double A, double B, double c2) const {
     constexpr unsigned full = 0xffffffffu;
-    const F2 a = f2_of(A), b = f2_of(B), c = f2_of(c2);
+    const F2 a = f2_of(A), b = f2_of(B), e = f2_of(A - B), c = f2_of(c2);
     double mine = 0;
     for (unsigned m = __ballot_sync(full, active); m; m &= m - 1) {
       const int l = __ffs(m) - 1;
       const F2 al = {__shfl_sync(full, a.h, l), __shfl_sync(full, a.l, l)};
       const F2 bl = {__shfl_sync(full, b.h, l), __shfl_sync(full, b.l, l)};
+      const F2 el = {__shfl_sync(full, e.h, l), __shfl_sync(full, e.l, l)};
       const F2 cl = {__shfl_sync(full, c.h, l), __shfl_sync(full, c.l, l)};
-      const double v = pair(al, bl, cl);
+      const double v = pair(al, bl, el, cl);
       if (lane == l) mine = v;
     }
     return mine;
