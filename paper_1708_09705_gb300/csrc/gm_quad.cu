@@ -682,6 +682,73 @@ struct DfRule {
   }
 };
 
+// The same rule with FP64 instructions: contexts whose g leaves the range in which
+// two floats carry its 48 bits (df_fits), and GM_QUAD=fp64.
+template <int KPL>
+struct Gl64Rule {
+  typedef double Val;
+  static constexpr bool kFloatEntry = false;
+  struct Par {
+    const double* gl_zeta;
+    const double* gl_w;
+    const D4* gtab;
+    TabF64 td;
+    int Q;
+  };
+  static constexpr int kThreads = 256;
+  const double *z, *w;  // shared memory, padded with zeros
+  const D4* gtab;
+  TabF64 td;
+  int lane, Q;
+
+  static size_t smem() { return 2 * kMaxNodes * sizeof(double); }
+  __device__ __forceinline__ Gl64Rule(const Par& P, unsigned char* sm)
+      : gtab(P.gtab), td(P.td), Q(P.Q) {
+    lane = threadIdx.x & 31;
+    double* zs = reinterpret_cast<double*>(sm);
+    double* ws = zs + kMaxNodes;
+    for (int q = threadIdx.x; q < kMaxNodes; q += blockDim.x) {
+      zs[q] = q < Q ? P.gl_zeta[q] : 0.0;
+      ws[q] = q < Q ? P.gl_w[q] : 0.0;
+    }
+    z = zs;
+    w = ws;
+    __syncthreads();
+  }
+
+  __device__ __forceinline__ double pair(double A, double B, double c2) const {
+    double acc = 0;
+#pragma unroll 1
+    for (int q = 0; q < Q; ++q) {
+      const double t = A * z[q];
+      double inner = 0;
+#pragma unroll
+      for (int k = 0; k < KPL; ++k) {
+        const int p = lane + 32 * k;
+        const double tp = B * z[p];
+        const double d = p == q ? (A - B) * z[q] : t - tp;
+        inner += w[p] * g_lookup(gtab, td, d * d + t * (c2 * tp));
+      }
+      acc += w[q] * inner;
+    }
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
+    return acc;
+  }
+
+  __device__ __forceinline__ double R(bool active, double A, double B, double c2) const {
+    constexpr unsigned full = 0xffffffffu;
+    double mine = 0;
+    for (unsigned m = __ballot_sync(full, active); m; m &= m - 1) {
+      const int l = __ffs(m) - 1;
+      const double v = pair(__shfl_sync(full, A, l), __shfl_sync(full, B, l),
+                            __shfl_sync(full, c2, l));
+      if (lane == l) mine = v;
+    }
+    return mine;
+  }
+};
+
 // ------------------------------------------------------------ FP32 node sums
 // The Q-node rule of FP32 contexts: lanes own the nodes q' of sightline j, loop
 // over the nodes q of sightline i, and the warp sums the products.  One 16-byte
@@ -1059,6 +1126,23 @@ static typename DfRule<KPL>::Par df_par(const gm_ctx* c) {
           c->cfg.n_nodes};
 }
 
+template <int KPL>
+static typename Gl64Rule<KPL>::Par gl64_par(const gm_ctx* c) {
+  return {c->gl_zeta, c->gl_w, (const D4*)c->gtab, tab_f64(), c->cfg.n_nodes};
+}
+
+// Whether the node sums of an FP64 context run in pairs of floats: g(0), its largest
+// value, between 2^-30 (what it adds to a sum down to 2^-53 of that still has both
+// parts above the smallest float) and 2^100 (sums and coefficients below the largest).
+// For the lognormal form that is sigma2 up to 69; the FP64 form goes on to 520, where
+// its table, g over the cube of a segment, overflows.
+static bool df_fits(const gm_ctx* c) {
+  const char* e = std::getenv("GM_QUAD");
+  if (e && std::strcmp(e, "fp64") == 0) return false;
+  const double g0 = c->cfg.form == GM_FORM_LOGNORMAL ? std::expm1(c->cfg.sigma2) : c->cfg.sigma2;
+  return g0 >= 0x1p-30 && g0 <= 0x1p100;
+}
+
 gm_status pair_quadrature(gm_ctx* c, int64_t n_rows, const double* rs, const double* rux,
                           const double* ruy, const double* ruz, const int32_t* row_field,
                           const int64_t* row_ptr, const int32_t* col, int64_t nnz, void* val,
@@ -1069,6 +1153,7 @@ gm_status pair_quadrature(gm_ctx* c, int64_t n_rows, const double* rs, const dou
   QuadParams P = quad_params(c, symmetric);
   const int Q = c->cfg.n_nodes;
   const bool f32 = c->cfg.precision == GM_PREC_FP32;
+  const bool df = !f32 && df_fits(c);
 #define GM_ENTRIES(RULE, PAR, NAME) \
   launch_entries<RULE>(c, P, PAR, n_rows, rs, rux, ruy, ruz, row_field, row_ptr, col, nnz, val, NAME)
   if (c->cfg.quad_rule == GM_QUAD_BAND) {
@@ -1076,13 +1161,16 @@ gm_status pair_quadrature(gm_ctx* c, int64_t n_rows, const double* rs, const dou
     else GM_ENTRIES(BandRule<double>, band_par<double>(c), "k_pair_quad_band");
   } else if (Q <= 32) {
     if (f32) GM_ENTRIES(Gl32Rule<1>, gl32_par<1>(c), "k_pair_quad");
-    else GM_ENTRIES(DfRule<1>, df_par<1>(c), "k_pair_quad");
+    else if (df) GM_ENTRIES(DfRule<1>, df_par<1>(c), "k_pair_quad");
+    else GM_ENTRIES(Gl64Rule<1>, gl64_par<1>(c), "k_pair_quad_fp64");
   } else if (Q <= 64) {
     if (f32) GM_ENTRIES(Gl32Rule<2>, gl32_par<2>(c), "k_pair_quad");
-    else GM_ENTRIES(DfRule<2>, df_par<2>(c), "k_pair_quad");
+    else if (df) GM_ENTRIES(DfRule<2>, df_par<2>(c), "k_pair_quad");
+    else GM_ENTRIES(Gl64Rule<2>, gl64_par<2>(c), "k_pair_quad_fp64");
   } else {
     if (f32) GM_ENTRIES(Gl32Rule<4>, gl32_par<4>(c), "k_pair_quad");
-    else GM_ENTRIES(DfRule<4>, df_par<4>(c), "k_pair_quad");
+    else if (df) GM_ENTRIES(DfRule<4>, df_par<4>(c), "k_pair_quad");
+    else GM_ENTRIES(Gl64Rule<4>, gl64_par<4>(c), "k_pair_quad_fp64");
   }
 #undef GM_ENTRIES
   GM_LAUNCH_CHECK(c);
@@ -1120,8 +1208,14 @@ gm_status self_quadrature(gm_ctx* c, int64_t n_rows, const double* rs, double* k
 #define GM_SELF32(K)                                                                      \
   k_self_quad<K><<<blocks, 256, 0, c->stream>>>(P, n_rows, rs, c->gl_zeta, c->gl_w, c->gtab, \
                                                 tab_f32(), kss)
-#define GM_SELF64(K) \
-  launch_list<DfRule<K>>(c, P, df_par<K>(c), n_rows, rs, nullptr, nullptr, kss, "k_self_quad")
+#define GM_SELF64(K)                                                                             \
+  do {                                                                                           \
+    if (df_fits(c))                                                                              \
+      launch_list<DfRule<K>>(c, P, df_par<K>(c), n_rows, rs, nullptr, nullptr, kss, "k_self_quad"); \
+    else                                                                                         \
+      launch_list<Gl64Rule<K>>(c, P, gl64_par<K>(c), n_rows, rs, nullptr, nullptr, kss,          \
+                               "k_self_quad_fp64");                                              \
+  } while (0)
   if (c->cfg.quad_rule == GM_QUAD_BAND) {
     if (f32)
       launch_list<BandRule<float>>(c, P, band_par<float>(c), n_rows, rs, nullptr, nullptr, kss,
@@ -1227,19 +1321,23 @@ gm_status pairlist_quadrature(gm_ctx* c, int64_t n, const double* si, const doub
   QuadParams P = quad_params(c, false);
   const int Q = c->cfg.n_nodes;
   const bool f32 = c->cfg.precision == GM_PREC_FP32;
+  const bool df = !f32 && df_fits(c);
 #define GM_LIST(RULE, PAR, NAME) launch_list<RULE>(c, P, PAR, n, si, sj, chord, out, NAME)
   if (c->cfg.quad_rule == GM_QUAD_BAND) {
     if (f32) GM_LIST(BandRule<float>, band_par<float>(c), "k_pairlist_quad_band");
     else GM_LIST(BandRule<double>, band_par<double>(c), "k_pairlist_quad_band");
   } else if (Q <= 32) {
     if (f32) launch_pairlist<1>(c, P, n, si, sj, chord, out);
-    else GM_LIST(DfRule<1>, df_par<1>(c), "k_pairlist_quad");
+    else if (df) GM_LIST(DfRule<1>, df_par<1>(c), "k_pairlist_quad");
+    else GM_LIST(Gl64Rule<1>, gl64_par<1>(c), "k_pairlist_quad_fp64");
   } else if (Q <= 64) {
     if (f32) launch_pairlist<2>(c, P, n, si, sj, chord, out);
-    else GM_LIST(DfRule<2>, df_par<2>(c), "k_pairlist_quad");
+    else if (df) GM_LIST(DfRule<2>, df_par<2>(c), "k_pairlist_quad");
+    else GM_LIST(Gl64Rule<2>, gl64_par<2>(c), "k_pairlist_quad_fp64");
   } else {
     if (f32) launch_pairlist<4>(c, P, n, si, sj, chord, out);
-    else GM_LIST(DfRule<4>, df_par<4>(c), "k_pairlist_quad");
+    else if (df) GM_LIST(DfRule<4>, df_par<4>(c), "k_pairlist_quad");
+    else GM_LIST(Gl64Rule<4>, gl64_par<4>(c), "k_pairlist_quad_fp64");
   }
 #undef GM_LIST
   GM_LAUNCH_CHECK(c);
