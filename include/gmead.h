@@ -449,7 +449,8 @@ gm_status gm_surrogate_train(gm_ctx* ctx, int64_t n_pairs, int32_t steps, int32_
 gm_status gm_surrogate_grad(gm_ctx* ctx, int64_t n, const float* X, const float* Y, double lam,
                             float* grad_out, double* loss_out);
 /* Evaluates the surrogate for n pairs given by distances si, sj (pc) and
- * chord |u_i - u_j| (host or device arrays), at sigma2 and L0 (pc).
+ * chord |u_i - u_j| (host or device arrays; those of the context's own device are
+ * read where they are, and done with when the call returns), at sigma2 and L0 (pc).
  * Outputs y and e (FP32, length n).  GM_E_STATE without parameters. */
 gm_status gm_surrogate_eval(gm_ctx* ctx, int64_t n, const double* si, const double* sj,
                             const double* chord, double sigma2, double L0, float* y_out,

@@ -28,6 +28,7 @@
 #include <cmath>
 #include <vector>
 
+#include "gm_inputs.h"
 #include "gm_internal.cuh"
 
 namespace gm {
@@ -418,6 +419,16 @@ static bool mlp_is_dev(const void* p) {
   return a.type == cudaMemoryTypeDevice || a.type == cudaMemoryTypeManaged;
 }
 
+// Device of a pointer to device memory, -1 for any other memory.
+static int device_of(const void* p) {
+  cudaPointerAttributes a;
+  if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
+    cudaGetLastError();
+    return -1;
+  }
+  return a.type == cudaMemoryTypeDevice ? a.device : -1;
+}
+
 gm_status mlp_ensure(gm_ctx* c) {
   if (c->mlp_params) return GM_OK;
   c->mlp_params = (float*)dev_alloc(c, kMlpParams * sizeof(float));
@@ -465,12 +476,14 @@ extern "C" gm_status gm_surrogate_eval(gm_ctx* c, int64_t n, const double* si, c
   ScopedDev staging(c, total);
   double* buf = (double*)staging.p;
   if (!buf) return set_error(c, GM_E_NOMEM, "surrogate eval staging");
-  // host arrays are staged; device arrays are read in place (the call returns
-  // after the stream has drained)
+  // arrays in the context's device's own memory are read in place (the call returns
+  // after the stream has drained); all others are copied: host and managed ones,
+  // another GPU's, which the kernel could not read, and misaligned ones
   const double* src[3] = {si, sj, chord};
   for (int k = 0; k < 3; ++k) {
-    if (mlp_is_dev(src[k])) continue;
-    GM_CUDA_CHECK(c, cudaMemcpyAsync(buf + k * n, src[k], nb, cudaMemcpyHostToDevice, c->stream));
+    if (read_in_place(device_of(src[k]), c->device, src[k], sizeof(double))) continue;
+    const cudaMemcpyKind kind = mlp_is_dev(src[k]) ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice;
+    GM_CUDA_CHECK(c, cudaMemcpyAsync(buf + k * n, src[k], nb, kind, c->stream));
     src[k] = buf + k * n;
   }
   float* y = (float*)(buf + 3 * n);
