@@ -363,13 +363,16 @@ gm_status small_cg(gm_ctx* c, int64_t n_cols, int64_t ld, const double* dv, cons
                    const double* rhs, double* x, bool warm, double tol, double* bb, double* rr,
                    int64_t* iters);
 // FP64 panel product on the tensor cores (gm_tc64.cu) over the tiles of gm_tc.cu:
-// tc64_prepare decides for a panel of n_cols right-hand sides (c->tc64_use) and
-// builds them on first use.
+// tc64_prepare decides for a panel of that width (c->tc64_use) and builds them on
+// first use; where they are not worth it or do not fit, the FP64 units stay in use.
 // From kTc64MinWork products of stored entries and columns on: with its exponents
 // and digit planes the product takes 48 us at 400 stars x 416 columns (6e6), the
 // FP64 units 39; 232 against 1,306 us at 2,001 x 2,016 (7e8).
 constexpr double kTc64MinWork = 1.5e7;
-gm_status tc64_prepare(gm_ctx* c, int64_t n_cols);
+gm_status tc64_prepare(gm_ctx* c, int64_t width);
+void tc64_release(gm_ctx* c);  // gives the tiles back and goes without them
+// Digit planes and exponents of an n x R panel; false when they do not fit.
+bool tc64_panel_room(gm_ctx* c, int64_t n, int64_t R);
 gm_status tc64_fill(gm_ctx* c, const int64_t* bptr, const int32_t* ucol);
 size_t tc64_kstep_bytes();
 gm_status panel_spmm_tc64(gm_ctx* c, int64_t n, int R, const double* dv, const double* P,

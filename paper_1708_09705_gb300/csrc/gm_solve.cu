@@ -1574,7 +1574,8 @@ static gm_status panels(gm_ctx* c, int64_t n_rows, const int64_t* row_ptr, const
   const int sms = sm_count(c);
   const bool small = sizeof(TV) == 8 && small_cg_fits(c, n_cols_all);
   if (sizeof(TV) == 8 && !small) {
-    const gm_status ts = tc64_prepare(c, n_cols_all);
+    const gm_status ts = tc64_prepare(
+        c, c->cfg.rhs_panel > 0 ? std::min<int64_t>(c->cfg.rhs_panel, n_cols_all) : n_cols_all);
     if (ts != GM_OK) return ts;
   }
   // panel width: all rows if they fit a memory budget, in multiples of 32
@@ -1620,12 +1621,20 @@ static gm_status panels(gm_ctx* c, int64_t n_rows, const int64_t* row_ptr, const
                                            c->tc_nblk);
   const int64_t rows_b = std::max<int64_t>(nbe, nch);
   const int ncorr = defl ? (defl_tc ? 8 : 1) : 0;
-  bool ok = ensure(c, ws.P_X, pbytes) && ensure(c, ws.P_R, pbytes) && ensure(c, ws.P_P, pbytes) &&
-            ensure(c, ws.P_PD, pbytes) && ensure(c, ws.P_Q, pbytes) &&
-            ensure(c, ws.P_part, (size_t)(rows_a + rows_b + std::max(ncorr, 1)) * R *
-                                     sizeof(double)) &&
-            ensure(c, ws.P_scal, 6 * (size_t)R * sizeof(double)) &&
-            ensure(c, ws.P_active, (size_t)(R + 32) * sizeof(int));
+  auto room = [&]() {
+    return ensure(c, ws.P_X, pbytes) && ensure(c, ws.P_R, pbytes) && ensure(c, ws.P_P, pbytes) &&
+           ensure(c, ws.P_PD, pbytes) && ensure(c, ws.P_Q, pbytes) &&
+           ensure(c, ws.P_part, (size_t)(rows_a + rows_b + std::max(ncorr, 1)) * R *
+                                    sizeof(double)) &&
+           ensure(c, ws.P_scal, 6 * (size_t)R * sizeof(double)) &&
+           ensure(c, ws.P_active, (size_t)(R + 32) * sizeof(int));
+  };
+  bool ok = room();
+  if (sizeof(TV) == 8 && c->tc64_state > 0 && (!ok || (c->tc64_use && !tc64_panel_room(c, n, R)))) {
+    // the tensor-core product's tiles or digit planes do not fit beside the panels
+    tc64_release(c);
+    ok = room();
+  }
   if (!ok) return set_error(c, GM_E_NOMEM, "variance panels");
   TV *X = (TV*)ws.P_X.p, *Rr = (TV*)ws.P_R.p, *P = (TV*)ws.P_P.p, *PD = (TV*)ws.P_PD.p,
      *Q = (TV*)ws.P_Q.p;

@@ -31,6 +31,8 @@
 // partial sums of P^T Q for the CG step length (fixed order).
 #include <algorithm>
 #include <cstdlib>
+#include <optional>
+#include <string>
 #include <vector>
 
 #include "gm_internal.cuh"
@@ -1134,25 +1136,57 @@ bool tc_wanted(gm_ctx* c) {
   return !(e && e[0] == 's');
 }
 
+// Whether the FP64 tiles of nks K-steps are worth their time and memory.  A K-step
+// costs the tensor cores the same whatever it holds (2,048 entries at a fill of one),
+// the FP64 units pay per stored entry: the product with its exponents and digit planes
+// against the FP64 units took 180 / 125 us at a fill of 0.074 (2,001 stars and as many
+// columns), 404 / 481 at 0.116 (3,000), 534 / 425 at 0.069 (12,000 x 1,024), 217 / 288
+// at 0.19, 230 / 1,224 at 0.55.  The images may take a fifth of the free memory.
+constexpr double kTc64MinFill = 0.1;
+static bool tc64_worth(gm_ctx* c, int64_t nks) {
+  size_t free_b = 0, tot_b = 0;
+  cudaMemGetInfo(&free_b, &tot_b);
+  if ((double)nks * (double)tc64_kstep_bytes() > 0.2 * ((double)free_b + (double)c->tc_img.bytes))
+    return false;
+  const char* e = std::getenv("GM_SPMM");
+  return (e && e[0] == 't') || (double)c->nnz >= kTc64MinFill * (kTcRows * kTcK) * (double)nks;
+}
+
 // FP64 contexts build their tiles when the first large enough panel product needs
 // them (a context that only assembles or runs PIC never does).
-gm_status tc64_prepare(gm_ctx* c, int64_t n_cols) {
+void tc64_release(gm_ctx* c) {
+  for (Buffer* b : {&c->tc_img, &c->tc_planes, &c->tc_upad, &c->tc_kbase}) {
+    if (b->p) dev_free_now(c, b->p, b->bytes);
+    *b = Buffer{};
+  }
+  c->tc_nblk = c->tc_nks = 0;
+  c->stats.tile_ksteps = 0;
+  c->tc64_state = -1;
+  c->tc64_use = false;
+}
+
+gm_status tc64_prepare(gm_ctx* c, int64_t width) {
   c->tc64_use = false;
   if (c->cfg.precision == GM_PREC_FP32 || c->n_fields > 1 || c->tc64_state < 0) return GM_OK;
   const char* e = std::getenv("GM_SPMM");  // simt / tc pin the product
   if (e && e[0] == 's') return GM_OK;
-  if ((double)c->nnz * (double)n_cols < kTc64MinWork && !(e && e[0] == 't')) return GM_OK;
+  if ((double)c->nnz * (double)width < kTc64MinWork && !(e && e[0] == 't')) return GM_OK;
   if (c->tc64_state == 0) {
-    // the digit images take about 16 bytes per stored entry at a fill of one, a
-    // few times that on sparse tiles; leave them out where memory is short
-    size_t free_b = 0, tot_b = 0;
-    cudaMemGetInfo(&free_b, &tot_b);
-    if ((double)c->nnz * 64.0 > 0.2 * (double)free_b) {
+    // a block's union holds its 128 diagonal columns at least: rows this short cannot
+    // reach the fill that tc64_worth asks for
+    if ((double)c->nnz < kTc64MinFill * kTcRows * (double)c->n && !(e && e[0] == 't')) {
       c->tc64_state = -1;
       return GM_OK;
     }
+    const std::string before = c->last_error;
     const gm_status s = tc_tiles_build(c);
-    if (s != GM_OK) return s;
+    if (s != GM_OK && s != GM_E_NOMEM) return s;
+    if (s == GM_E_NOMEM || c->tc_nblk == 0) {
+      // no memory for them, or not worth it: the FP64 units need none of this
+      tc64_release(c);
+      c->last_error = before;
+      return GM_OK;
+    }
     c->tc64_state = 1;
   }
   c->tc64_use = true;
@@ -1240,7 +1274,9 @@ gm_status tc_tiles_build(gm_ctx* c) {
   std::vector<int64_t> hb(nblk + 1, 0), hk(nblk + 1, 0);
   int64_t U = 0, nks = 0;
   int32_t* ucol = nullptr;
-  int64_t* bptr = (int64_t*)dev_alloc(c, (nblk + 1) * sizeof(int64_t));
+  ScopedDev b_bptr(c, (nblk + 1) * sizeof(int64_t));
+  std::optional<ScopedDev> b_ucol;
+  int64_t* bptr = (int64_t*)b_bptr.p;
   if (!bptr) return set_error(c, GM_E_NOMEM, "tensor-core tile union");
   const int32_t* trow = c->tc_order ? (const int32_t*)c->tc_trow.p : nullptr;
   const size_t bm_smem = (size_t)nwords * sizeof(uint32_t);
@@ -1263,7 +1299,9 @@ gm_status tc_tiles_build(gm_ctx* c) {
     }
     U = hb[nblk];
     nks = hk[nblk];
-    ucol = (int32_t*)dev_alloc(c, std::max<int64_t>(U, 1) * sizeof(int32_t));
+    if (f64 && !tc64_worth(c, nks)) return GM_OK;
+    b_ucol.emplace(c, std::max<int64_t>(U, 1) * sizeof(int32_t));
+    ucol = (int32_t*)b_ucol->p;
     if (!ucol) return set_error(c, GM_E_NOMEM, "tensor-core tile union");
     if (!ensure(c, c->tc_kbase, (nblk + 1) * sizeof(int64_t)) ||
         !ensure(c, c->tc_upad, std::max<int64_t>(nks, 1) * kTcK * sizeof(int32_t)) ||
@@ -1300,7 +1338,8 @@ gm_status tc_tiles_build(gm_ctx* c) {
     if (s != GM_OK) return s;
     GM_CUDA_CHECK(c, cudaMemcpyAsync(&U, pos + nnz, sizeof(int64_t), cudaMemcpyDeviceToHost, st));
     GM_CUDA_CHECK(c, cudaStreamSynchronize(st));
-    ucol = (int32_t*)dev_alloc(c, std::max<int64_t>(U, 1) * sizeof(int32_t));
+    b_ucol.emplace(c, std::max<int64_t>(U, 1) * sizeof(int32_t));
+    ucol = (int32_t*)b_ucol->p;
     ScopedDev ub(c, std::max<int64_t>(U, 1) * sizeof(int32_t));
     if (!ucol || !ub.p) return set_error(c, GM_E_NOMEM, "tensor-core tile union");
     int32_t* ublk = (int32_t*)ub.p;
@@ -1316,6 +1355,7 @@ gm_status tc_tiles_build(gm_ctx* c) {
     GM_CUDA_CHECK(c, cudaStreamSynchronize(st));
     for (int64_t b = 0; b < nblk; ++b) hk[b + 1] = hk[b] + ceil_div(hb[b + 1] - hb[b], kTcK);
     nks = hk[nblk];
+    if (f64 && !tc64_worth(c, nks)) return GM_OK;
     if (!ensure(c, c->tc_kbase, (nblk + 1) * sizeof(int64_t)) ||
         !ensure(c, c->tc_upad, std::max<int64_t>(nks, 1) * kTcK * sizeof(int32_t)) ||
         !ensure(c, c->tc_img, std::max<int64_t>(nks, 1) * kbytes))
@@ -1334,15 +1374,13 @@ gm_status tc_tiles_build(gm_ctx* c) {
     const gm_status fs = tc64_fill(c, bptr, ucol);
     if (fs != GM_OK) return fs;
   } else {
-  GM_PROF(c, "k_tc_fill");
-  k_tc_fill<<<wb, 256, 0, st>>>(n, c->row_ptr, c->col, (const float*)c->val, bptr, kbase, ucol,
-                                tb, tpos, (const int64_t*)c->tc_brow0.p,
-                                (unsigned char*)c->tc_img.p);
-  GM_LAUNCH_CHECK(c);
+    GM_PROF(c, "k_tc_fill");
+    k_tc_fill<<<wb, 256, 0, st>>>(n, c->row_ptr, c->col, (const float*)c->val, bptr, kbase, ucol,
+                                  tb, tpos, (const int64_t*)c->tc_brow0.p,
+                                  (unsigned char*)c->tc_img.p);
+    GM_LAUNCH_CHECK(c);
   }
   GM_CUDA_CHECK(c, cudaStreamSynchronize(st));
-  dev_free_now(c, bptr, (nblk + 1) * sizeof(int64_t));
-  dev_free_now(c, ucol, std::max<int64_t>(U, 1) * sizeof(int32_t));
   c->tc_nblk = nblk;
   c->tc_nks = nks;
   c->stats.tile_ksteps = nks;

@@ -517,12 +517,15 @@ static gm_status launch_oz(gm_ctx* c, int64_t n, int R, const int* ecol, const d
   return GM_OK;
 }
 
+bool tc64_panel_room(gm_ctx* c, int64_t n, int64_t R) {
+  return ensure(c, c->tc_planes, (size_t)(n * R) * kOzDigits * sizeof(uint16_t)) &&
+         ensure(c, c->tc64_ecol, (size_t)R * sizeof(int));
+}
+
 gm_status panel_spmm_tc64(gm_ctx* c, int64_t n, int R, const double* dv, const double* P,
                           const double* PD, double* Q, double* part_pq) {
   const int64_t pe = n * (int64_t)R;
-  if (!ensure(c, c->tc_planes, (size_t)pe * kOzDigits * sizeof(uint16_t)) ||
-      !ensure(c, c->tc64_ecol, (size_t)R * sizeof(int)))
-    return set_error(c, GM_E_NOMEM, "digit planes of the panel");
+  if (!tc64_panel_room(c, n, R)) return set_error(c, GM_E_NOMEM, "digit planes of the panel");
   int* ecol = (int*)c->tc64_ecol.p;
   uint16_t* planes = (uint16_t*)c->tc_planes.p;
   const int sms = sm_count(c);
