@@ -475,7 +475,7 @@ gm_status gm_build_cov(gm_ctx* c, int64_t* nnz_out) {
   c->t_nblk = 0;
   c->tc_nblk = 0;
   c->tc64_state = 0;
-  c->ell_ready = false;
+  c->ell_state = 0;
   c->warm_R = 0;
   pack_invalidate(c);
   st = tc_wanted(c) ? tc_tiles_build(c) : tiles_build(c);

@@ -134,7 +134,7 @@ struct gm_ctx {
   gm::Buffer tc_trow, tc_tpos;      // tile order: row at tile position p, position of row i
   gm::Buffer tc64_erow, tc64_ecol;  // FP64 form: exponents of K's rows and the panel's columns
   gm::Buffer ell_off, ell_row, ell_col, ell_val, ell_iters;  // sliced rows of small FP64 problems
-  bool ell_ready = false;
+  int ell_state = 0;                // sliced rows: 0 not asked for, 1 built, -1 do not fit
   int tc64_state = 0;               // FP64 tiles: 0 not asked for, 1 built, -1 do not fit
   bool tc64_use = false;            // the current panels run on them
   bool tc_order = false;            // tc_trow / tc_tpos in use (else position = row)
@@ -359,6 +359,7 @@ gm_status probe_colouring(gm_ctx* c);
 // Small FP64 solves, one block per right-hand side (gm_small.cu): x of B x = rhs
 // for n_cols columns of leading dimension ld, ||b||^2 and ||r||^2 per column.
 bool small_cg_fits(gm_ctx* c, int64_t n_cols);
+void small_release(gm_ctx* c);  // gives the sliced rows back and goes without them
 gm_status small_cg(gm_ctx* c, int64_t n_cols, int64_t ld, const double* dv, const double* minv,
                    const double* rhs, double* x, bool warm, double tol, double* bb, double* rr,
                    int64_t* iters);

@@ -16,6 +16,7 @@
 // Padding entries point at their own row with value zero.
 #include <algorithm>
 #include <cstdlib>
+#include <string>
 
 #include "gm_internal.cuh"
 
@@ -247,27 +248,7 @@ __global__ void __launch_bounds__(T, T == 512 ? 3 : 1) k_cg_columns(SmallCg A) {
 }
 
 // ---------------------------------------------------------------- host
-// Whether a solve of n_cols FP64 right-hand sides runs here: the rows fit a block
-// and an SM's share of the columns is short.  Both forms' time per call, stored
-// entries x columns per SM beside it (a mean solve is in each):
-//   300 stars, own columns   14,460:  6.8 ms in panels,  2.5 ms here
-//   1,000, 5 query columns   85,404:  7.6 ms,            5.1 ms
-//   600, own columns        110,464: 11.6 ms,            8.1 ms
-//                           122,968: 11.8 ms,            9.9 ms
-//   1,000, 300 columns      170,808: 10.6 ms,           10.2 ms
-//   1,500, 5 columns        199,970: 12.0 ms,           11.3 ms
-//   1,500, 300 columns      399,940: 15.0 ms,           23.4 ms
-//   1,000, own columns      537,432: 15.0 ms,           22.6 ms
-bool small_cg_fits(gm_ctx* c, int64_t n_cols) {
-  if (c->cfg.precision == GM_PREC_FP32 || c->n_fields > 1 || c->n > kSmallMax) return false;
-  const char* e = std::getenv("GM_SPMM");  // a pinned product keeps the panels
-  if (e) return false;
-  const double waves = (double)ceil_div(n_cols, (int64_t)sm_count(c));
-  return (double)c->nnz * waves < kSmallWork;
-}
-
-gm_status small_prepare(gm_ctx* c) {
-  if (c->ell_ready) return GM_OK;
+static gm_status small_prepare(gm_ctx* c) {
   const int64_t n = c->n, ns = ceil_div(n, 32);
   cudaStream_t st = c->stream;
   ScopedDev cnt(c, ns * sizeof(int64_t)), slot(c, n * sizeof(int32_t));
@@ -293,23 +274,60 @@ gm_status small_prepare(gm_ctx* c) {
       (const int32_t*)c->ell_row.p, (const int64_t*)c->ell_off.p, (int32_t*)c->ell_col.p,
       (double*)c->ell_val.p);
   GM_LAUNCH_CHECK(c);
-  c->ell_ready = true;
+  if (!ensure(c, c->ell_iters, sizeof(int))) return set_error(c, GM_E_NOMEM, "iteration count");
   return GM_OK;
 }
 
-// Solves B x = rhs for n_cols columns (leading dimension ld); scal: 2 x ld doubles
+void small_release(gm_ctx* c) {
+  for (Buffer* b : {&c->ell_off, &c->ell_row, &c->ell_col, &c->ell_val, &c->ell_iters}) {
+    if (b->p) dev_free_now(c, b->p, b->bytes);
+    *b = Buffer{};
+  }
+  c->ell_state = -1;
+}
+
+// Whether a solve of n_cols FP64 right-hand sides runs here: the rows fit a block
+// an SM's share of the columns is short and the sliced rows fit.  Both forms' time per call, stored
+// entries x columns per SM beside it (a mean solve is in each):
+//   300 stars, own columns   14,460:  6.8 ms in panels,  2.5 ms here
+//   1,000, 5 query columns   85,404:  7.6 ms,            5.1 ms
+//   600, own columns        110,464: 11.6 ms,            8.1 ms
+//                           122,968: 11.8 ms,            9.9 ms
+//   1,000, 300 columns      170,808: 10.6 ms,           10.2 ms
+//   1,500, 5 columns        199,970: 12.0 ms,           11.3 ms
+//   1,500, 300 columns      399,940: 15.0 ms,           23.4 ms
+//   1,000, own columns      537,432: 15.0 ms,           22.6 ms
+bool small_cg_fits(gm_ctx* c, int64_t n_cols) {
+  if (c->cfg.precision == GM_PREC_FP32 || c->n_fields > 1 || c->n > kSmallMax ||
+      c->ell_state < 0)
+    return false;
+  const char* e = std::getenv("GM_SPMM");  // a pinned product keeps the panels
+  if (e) return false;
+  const double waves = (double)ceil_div(n_cols, (int64_t)sm_count(c));
+  if (!((double)c->nnz * waves < kSmallWork)) return false;
+  if (c->ell_state == 0) {
+    const std::string before = c->last_error;
+    if (small_prepare(c) != GM_OK) {
+      small_release(c);
+      c->last_error = before;
+      return false;
+    }
+    c->ell_state = 1;
+  }
+  return true;
+}
+
+// Behind small_cg_fits: solves B x = rhs for n_cols columns (leading dimension ld); scal: 2 x ld doubles
 // for ||b||^2 and ||r||^2 of the columns.  Synchronises.
 gm_status small_cg(gm_ctx* c, int64_t n_cols, int64_t ld, const double* dv, const double* minv,
                    const double* rhs, double* x, bool warm, double tol, double* bb, double* rr,
                    int64_t* iters) {
-  gm_status s = small_prepare(c);
-  if (s != GM_OK) return s;
   cudaStream_t st = c->stream;
-  if (!ensure(c, c->ell_iters, sizeof(int))) return set_error(c, GM_E_NOMEM, "iteration count");
   int* d_it = (int*)c->ell_iters.p;
   GM_CUDA_CHECK(c, cudaMemsetAsync(d_it, 0, sizeof(int), st));
-  // a column goes on to 1e-2 of the tolerance, as a panel's columns do while others
-  // need it: one iteration in ten, and the stopping error stays out of the results
+  // a column goes on to 1e-2 of the tolerance: one iteration in ten, and the stopping
+  // error stays out of the results (a panel's columns go on too, to 1e-3 of it, while
+  // others need it)
   SmallCg A{(int)c->n, (const int64_t*)c->ell_off.p, (const int32_t*)c->ell_row.p,
             (const int32_t*)c->ell_col.p, (const double*)c->ell_val.p, dv, minv, rhs, x, ld, 1e-4 * tol * tol,
             warm ? 1 : 0, c->cfg.cg_max_iter, bb, rr, d_it, c->d_flags};

@@ -1572,7 +1572,7 @@ static gm_status panels(gm_ctx* c, int64_t n_rows, const int64_t* row_ptr, const
   const int64_t n = c->n;
   cudaStream_t st = c->stream;
   const int sms = sm_count(c);
-  const bool small = sizeof(TV) == 8 && small_cg_fits(c, n_cols_all);
+  bool small = sizeof(TV) == 8 && small_cg_fits(c, n_cols_all);
   if (sizeof(TV) == 8 && !small) {
     const gm_status ts = tc64_prepare(
         c, c->cfg.rhs_panel > 0 ? std::min<int64_t>(c->cfg.rhs_panel, n_cols_all) : n_cols_all);
@@ -1630,9 +1630,15 @@ static gm_status panels(gm_ctx* c, int64_t n_rows, const int64_t* row_ptr, const
            ensure(c, ws.P_active, (size_t)(R + 32) * sizeof(int));
   };
   bool ok = room();
-  if (sizeof(TV) == 8 && c->tc64_state > 0 && (!ok || (c->tc64_use && !tc64_panel_room(c, n, R)))) {
+  if (sizeof(TV) == 8 && !small && c->tc64_state > 0 &&
+      (!ok || (c->tc64_use && !tc64_panel_room(c, n, R)))) {
     // the tensor-core product's tiles or digit planes do not fit beside the panels
     tc64_release(c);
+    ok = room();
+  }
+  if (sizeof(TV) == 8 && !ok && c->ell_state > 0) {  // nor do the sliced rows
+    small_release(c);
+    small = c->tc64_use = false;
     ok = room();
   }
   if (!ok) return set_error(c, GM_E_NOMEM, "variance panels");

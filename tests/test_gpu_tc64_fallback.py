@@ -89,7 +89,7 @@ def test_no_memory_for_the_tiles(what, monkeypatch):
     _same(got, want)
 
 
-@pytest.mark.parametrize("n,side,L0,panel,used", [(2001, 20.0, 5.0, 0, False),
+@pytest.mark.parametrize("n,side,L0,panel,used", [(2100, 20.0, 5.0, 0, False),
                                                   (12000, 30.0, 5.0, 1024, False),
                                                   (3000, 20.0, 8.0, 0, True)])
 def test_sparse_rows_keep_the_fp64_units(n, side, L0, panel, used, monkeypatch):
