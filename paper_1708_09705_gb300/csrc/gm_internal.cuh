@@ -360,6 +360,7 @@ gm_status probe_colouring(gm_ctx* c);
 // for n_cols columns of leading dimension ld, ||b||^2 and ||r||^2 per column.
 bool small_cg_fits(gm_ctx* c, int64_t n_cols);
 void small_release(gm_ctx* c);  // gives the sliced rows back and goes without them
+bool small_cg_mean_fits(gm_ctx* c);  // the one column of a mean solve
 gm_status small_cg(gm_ctx* c, int64_t n_cols, int64_t ld, const double* dv, const double* minv,
                    const double* rhs, double* x, bool warm, double tol, double* bb, double* rr,
                    int64_t* iters);

@@ -111,7 +111,8 @@ __device__ __forceinline__ void small_sum(double (&v)[NV], double* sh) {
   for (int k = 0; k < NV; ++k) v[k] = sh[NV * 1024 + k];
 }
 
-constexpr double kSmallWork = 1.3e5;      // stored entries x columns per SM
+constexpr double kSmallWork = 2.0e5;      // stored entries x columns per SM
+constexpr double kSmallMean = 1.6e4;      // stored entries of a mean solve
 
 // T: threads at most; three blocks of 512 share an SM (a warp's chain of loads and
 // additions is long, the FP64 unit wants the other columns meanwhile)
@@ -286,23 +287,24 @@ void small_release(gm_ctx* c) {
   c->ell_state = -1;
 }
 
-// Whether a solve of n_cols FP64 right-hand sides runs here: the rows fit a block
-// an SM's share of the columns is short and the sliced rows fit.  Both forms' time per call, stored
-// entries x columns per SM beside it (a mean solve is in each):
-//   300 stars, own columns   14,460:  6.8 ms in panels,  2.5 ms here
-//   1,000, 5 query columns   85,404:  7.6 ms,            5.1 ms
-//   600, own columns        110,464: 11.6 ms,            8.1 ms
-//                           122,968: 11.8 ms,            9.9 ms
-//   1,000, 300 columns      170,808: 10.6 ms,           10.2 ms
-//   1,500, 5 columns        199,970: 12.0 ms,           11.3 ms
-//   1,500, 300 columns      399,940: 15.0 ms,           23.4 ms
-//   1,000, own columns      537,432: 15.0 ms,           22.6 ms
+// Whether a solve of n_cols FP64 right-hand sides runs here: the rows fit a block,
+// an SM's share of the columns is short and the sliced rows fit the memory.  Times of
+// a call without its mean solve, stored entries x columns per SM beside it:
+//   400 stars, own columns    39,330:  4.4 ms in panels,  2.0 ms here
+//   600                      131,448:  7.6,               6.6
+//   640                      192,020:  7.4,               7.0
+//   700                      211,590:  8.4,               8.4
+//   760                      254,280:  8.2,               9.1
+//   1,300, 100 queries       144,496: 12.4,               7.9
+//   1,500, 100 queries       176,962: 10.3,               9.0
+//   1,700, 100 queries       228,742: 11.8,              11.2
+//   2,000, 100 queries       297,812: 12.8,              14.5
 bool small_cg_fits(gm_ctx* c, int64_t n_cols) {
   if (c->cfg.precision == GM_PREC_FP32 || c->n_fields > 1 || c->n > kSmallMax ||
       c->ell_state < 0)
     return false;
-  const char* e = std::getenv("GM_SPMM");  // a pinned product keeps the panels
-  if (e) return false;
+  const char* e = std::getenv("GM_SPMM");  // a pinned product (simt, tc) keeps the panels
+  if (e && (e[0] == 's' || e[0] == 't')) return false;
   const double waves = (double)ceil_div(n_cols, (int64_t)sm_count(c));
   if (!((double)c->nnz * waves < kSmallWork)) return false;
   if (c->ell_state == 0) {
@@ -315,6 +317,13 @@ bool small_cg_fits(gm_ctx* c, int64_t n_cols) {
     c->ell_state = 1;
   }
   return true;
+}
+
+// A mean solve has one column: a block on one SM, against k_cg_run over the chip
+// (about 15 us an iteration): 1.1 / 1.2 ms at 14,600 stored entries, 2.5 / 1.3 at
+// 43,000, 3.8 / 1.6 at 86,600.
+bool small_cg_mean_fits(gm_ctx* c) {
+  return (double)c->nnz < kSmallMean && small_cg_fits(c, 1);
 }
 
 // Behind small_cg_fits: solves B x = rhs for n_cols columns (leading dimension ld); scal: 2 x ld doubles

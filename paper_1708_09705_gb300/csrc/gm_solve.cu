@@ -1439,7 +1439,7 @@ static gm_status posterior_mean(gm_ctx* c, int64_t* iters, double* resid) {
     GM_PROF(c, "k_scale");
     k_scale<double><<<eb, 256, 0, st>>>(n, d64, w64, r64);  // rhs
     GM_LAUNCH_CHECK(c);
-    if (small_cg_fits(c, 1)) {
+    if (small_cg_mean_fits(c)) {
       double* part = (double*)ws.part.p;
       double* hp = (double*)c->h_pinned;
       s = small_cg(c, 1, 1, (const double*)ws.dv.p, (const double*)ws.minv.p, r64, x64, false, tol,
