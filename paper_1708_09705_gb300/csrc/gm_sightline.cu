@@ -301,9 +301,14 @@ __global__ void __launch_bounds__(32)
       float u = bf < 0.f ? fmaxf(cp, 0.f) / (s - bf) : (bf + s) / -cm;
       // grazing within the estimate's own error: the motion turns at -b / cm
       if (fabsf(disc) <= fuzz) u = fmaxf(0.98f * fminf(u, -bf / cm), 0.f);
-      const bool met = live && j + 1 < m && disc > -fuzz && u >= 0.f && u <= U &&
-                       !(bf < 0.f && cp < -1e-9f);
-      ue[k] = met ? u : INFINITY;
+      bool met = disc > -fuzz && u >= 0.f && u <= U && !(bf < 0.f && cp < -1e-9f);
+      // values whose squares leave the range of floats: timed, whatever they estimate
+      const float big = fmaxf(fabsf(bf), fmaxf(fabsf(cp), fabsf(cm)));
+      if (!(big > 1e-15f && big < 1e15f)) {
+        met = true;
+        u = 0.f;
+      }
+      ue[k] = met && live && j + 1 < m ? u : INFINITY;
     }
     double th = 0.0;
     int bj = M;
