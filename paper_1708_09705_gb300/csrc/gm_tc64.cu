@@ -16,9 +16,12 @@
 //     every sum is an integer up to 2^24: exact, in any order;
 //   * each read-out adds the eight accumulators into two 64-bit integers per
 //     element; the result is rounded once, at the end.
-// What is left out (i + j >= 8) and the rounding of v are below 2^-60 of the
-// largest entry of the row times the largest of the column, where an FP64 sum of
-// the same length rounds every partial sum at 2^-53 of it.
+// What is left out (i + j >= 8: seven products of up to 2^14 at 2^-76) and the rounding
+// of v are below 2^-57 of the row's largest entry times the column's largest, per stored
+// entry of the row, where an FP64 sum rounds every partial sum at 2^-53.  The bound is of
+// the two maxima, not of each term: an entry keeps 53 bits down to 2^-9 of its column's
+// largest, and fewer below that.  Errors of the posteriors against 64-bit references
+// did not grow (3.3e-10 at 2,001 stars in both forms).
 //
 // Layout.  128-row tiles with unions of columns as in the FP32 product, K-steps
 // of 16 union columns, eight 4 KB images per K-step.  The panel's digits are
