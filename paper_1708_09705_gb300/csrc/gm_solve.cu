@@ -1271,7 +1271,7 @@ static bool cg_in_one_launch() {
 
 // The iterations behind k_cg_init in one launch; the partials of ||r||^2 are left in
 // c->h_pinned (G doubles).  *it: iterations, -1 where the grid cannot be resident at
-// once (nothing has run).  Synchronises.
+// once or its slots find no memory (nothing has run).  Synchronises.
 template <typename TA, typename TV>
 static gm_status cg_run(gm_ctx* c, int G, TV* x, double tol, int max_it, int check, int* it) {
   Workspace& ws = W(c);
@@ -1281,7 +1281,10 @@ static gm_status cg_run(gm_ctx* c, int G, TV* x, double tol, int max_it, int che
     return GM_OK;
   }
   const size_t sync_bytes = (3 * (size_t)G + 1) * sizeof(ulonglong2);
-  if (!ensure(c, ws.cg_sync, sync_bytes)) return set_error(c, GM_E_NOMEM, "CG hand-overs");
+  if (!ensure(c, ws.cg_sync, sync_bytes)) {  // the launches per step need none
+    *it = -1;
+    return GM_OK;
+  }
   GM_CUDA_CHECK(c, cudaMemsetAsync(ws.cg_sync.p, 0, sync_bytes, st));
   int64_t n = c->n;
   const int64_t* row_ptr = c->row_ptr;
