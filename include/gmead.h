@@ -63,7 +63,11 @@ typedef enum {
 } gm_status;
 
 /* Arithmetic of the covariance values, quadrature and CG inner iterations.
- * Site updates and the moments they use are always FP64. */
+ * Site updates and the moments they use are always FP64.  GM_PREC_FP64 sums the
+ * Gauss-Legendre nodes as pairs of floats (about 47 bits a term; entries within 1e-12
+ * of FP64 sums) and, on large problems, multiplies K by panels in 62-bit fixed point
+ * under the largest entry of each row and column; log1p, taper, vectors and all other
+ * sums are FP64. */
 enum { GM_PREC_FP64 = 0, GM_PREC_FP32 = 1 };
 /* Log-extinction moments from the density moments: lognormal moment match
  * (K = log1p(I/(s_i s_j)), m = ln(rho_bar s) - K_ii/2) or first order. */

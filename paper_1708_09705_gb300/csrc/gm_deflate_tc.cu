@@ -12,9 +12,9 @@
 //
 // k_dtc_step fuses the CG update of the panel with C's partial sums.  CTA =
 // (128 panel columns, a chunk of 16-row K-steps).  Per K-step the four
-// producer warps load R and Q of their rows, write R' = R - alpha Q, accumulate r'^T M^-1 r' and r'^T r' per column, and store
-// the three BF16 pieces of R' into a 128-byte-swizzled MN-major B tile; thread
-// 0 bulk-copies the K-step's image of the pieces of Y^T; one thread of the
+// producer warps load R and Q of their rows, write R' = R - alpha Q, accumulate
+// r'^T M^-1 r' and r'^T r' per column, and store the three BF16 pieces
+// of R' into a 128-byte-swizzled MN-major B tile; thread 0 bulk-copies the K-step's image of the pieces of Y^T; one thread of the
 // fifth warp issues four MMAs (M = 128, N = 128, K = 16) with the pieces of Y^T
 // stacked in M: [Y1; Y2] R'3, [Y1; Y2] R'2, [Y1; Y2] R'1 and [Y3; 0] R'1.  The
 // accumulator's two 64-row halves then hold Y1 R' + Y3 R'1 and Y2 R' (seven

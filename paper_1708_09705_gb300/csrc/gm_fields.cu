@@ -623,8 +623,8 @@ gm_status panels_fields(gm_ctx* c, const float* dv, const float* minv, const dou
                                            c->probe_colour, Rr);
     else
       k_pk_rhs_probe<<<(int)std::min<int64_t>(ceil_div(n, 256), 16 * sms), 256, 0, st>>>(
-        n, c->field_of, S.pf, c->row_ptr, c->col, (const float*)c->val, dv, c->tau, c->kdiag,
-        c->probe_colour, Rr);
+          n, c->field_of, S.pf, c->row_ptr, c->col, (const float*)c->val, dv, c->tau, c->kdiag,
+          c->probe_colour, Rr);
   } else {
     GM_PROF(c, "k_pk_rhs");
     k_pk_rhs<<<wb, 256, 0, st>>>(n, c->field_of, S.pf, c->row_ptr, c->col, (const float*)c->val,
@@ -637,8 +637,8 @@ gm_status panels_fields(gm_ctx* c, const float* dv, const float* minv, const dou
   GM_LAUNCH_CHECK(c);
   GM_CUDA_CHECK(c, cudaMemsetAsync(n_active, 0, sizeof(int), st));
   GM_PROF(c, "k_pk_reduce");
-  k_pk_reduce<<<rb, 32 * kPkRedWarps, 0, st>>>(0, tc, nf, S.wptr, S.pf, tol2, pa, pb, scal, active, n_active,
-                                  c->d_flags);
+  k_pk_reduce<<<rb, 32 * kPkRedWarps, 0, st>>>(0, tc, nf, S.wptr, S.pf, tol2, pa, pb, scal, active,
+                                               n_active, c->d_flags);
   GM_LAUNCH_CHECK(c);
   int* hn = (int*)c->h_pinned;
   GM_CUDA_CHECK(c, cudaMemcpyAsync(hn, n_active, sizeof(int), cudaMemcpyDeviceToHost, st));
@@ -667,12 +667,12 @@ gm_status panels_fields(gm_ctx* c, const float* dv, const float* minv, const dou
       launch_spmm(c, S, S.wpb, S.gstream, dv, planes);
       k_pk_elem<kPkPQ><<<ib, 256, 0, S.gstream>>>(S.n_eitems, S.eitems, S.pf, minv, dv, scal, tc,
                                                   active, X, Rr, P, PD, Q, pa, pb, nullptr, 0);
-      k_pk_reduce<<<rb, 32 * kPkRedWarps, 0, S.gstream>>>(1, tc, nf, S.wptr, S.pf, tol2, pa, nullptr, scal,
-                                             active, n_active, c->d_flags);
+      k_pk_reduce<<<rb, 32 * kPkRedWarps, 0, S.gstream>>>(
+          1, tc, nf, S.wptr, S.pf, tol2, pa, nullptr, scal, active, n_active, c->d_flags);
       k_pk_elem<kPkUpd1><<<ib, 256, 0, S.gstream>>>(S.n_eitems, S.eitems, S.pf, minv, dv, scal, tc,
                                                     active, X, Rr, P, PD, Q, pa, pb, nullptr, 0);
-      k_pk_reduce<<<rb, 32 * kPkRedWarps, 0, S.gstream>>>(2, tc, nf, S.wptr, S.pf, tol2, pa, pb, scal, active,
-                                             n_active, c->d_flags);
+      k_pk_reduce<<<rb, 32 * kPkRedWarps, 0, S.gstream>>>(
+          2, tc, nf, S.wptr, S.pf, tol2, pa, pb, scal, active, n_active, c->d_flags);
       k_pk_elem<kPkUpd2><<<ib, 256, 0, S.gstream>>>(S.n_eitems, S.eitems, S.pf, minv, dv, scal, tc,
                                                     active, X, Rr, P, PD, Q, pa, pb, pl, pe);
     }

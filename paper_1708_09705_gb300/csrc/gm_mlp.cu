@@ -482,7 +482,8 @@ extern "C" gm_status gm_surrogate_eval(gm_ctx* c, int64_t n, const double* si, c
   const double* src[3] = {si, sj, chord};
   for (int k = 0; k < 3; ++k) {
     if (read_in_place(device_of(src[k]), c->device, src[k], sizeof(double))) continue;
-    const cudaMemcpyKind kind = mlp_is_dev(src[k]) ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice;
+    const cudaMemcpyKind kind =
+        mlp_is_dev(src[k]) ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice;
     GM_CUDA_CHECK(c, cudaMemcpyAsync(buf + k * n, src[k], nb, kind, c->stream));
     src[k] = buf + k * n;
   }

@@ -28,7 +28,8 @@ namespace gm {
 // base + off[b], mirrored into the upper triangle (column i of L is then a
 // contiguous row for the solves); one thread block per matrix, right-looking.
 // The chain of columns bounds it: a matrix of up to kCholShared rows stays in
-// shared memory (packed lower triangle: 231 KB), a larger one in global memory; either way the column in work is copied to shared memory
+// shared memory (packed lower triangle and the column in work: 229,432 bytes), a larger
+// one in global memory; either way the column in work is copied to shared memory
 // and the update runs along the rows, a warp per row.  One thread per row on
 // global memory took 8 us a column, 1.34 ms at 140 to 170 rows; now 0.42 ms.
 constexpr int kCholShared = 238;

@@ -261,7 +261,7 @@ __global__ void k_self_quad(QuadParams P, int64_t n_rows, const double* __restri
 //     log1p, taper) is done for a batch of up to 32 pairs at once, a lane per
 //     pair, and the batch's pairs are then integrated one after another by
 //     the whole warp (band_batch);
-//   * the graded breakpoints come from a 16-entry table (no pow / log), their
+//   * the graded breakpoints come from a 12-entry table (no pow / log), their
 //     clipping, merging with the kink and counting from ballots and shuffles;
 //   * the FP32 form places nodes and panels in FP32 (the partition it sums
 //     over is a partition whatever its rounding), and reads g from the

@@ -1,5 +1,6 @@
 // Sightline sampler of the dA/ds >= 0 conditioning (Sect. 5): exact HMC for
-// each sightline's truncated Gaussian predictive, one thread per sightline.
+// each sightline's truncated Gaussian predictive: a few lanes per sightline up to 32
+// points, one thread beyond that.
 // The per-sightline arithmetic is in gm_hmc.cuh.
 #include <algorithm>
 #include <cstdlib>
@@ -138,8 +139,8 @@ __global__ void __launch_bounds__(64)
 // until none can be earlier.  The outward root is t = phi + acos(-c / r) unless
 // the hit grazes, where the sign of the derivative is evaluated as before.
 // The sightlines of a warp do not wait for each other's steps.
-// 4,096 sightlines x 16 points x 120 steps: 172 ms with one thread per sightline
-// timing every wall, 18 ms so (bit for bit the same samples).
+// A call of 4,096 sightlines x 16 points x 120 steps: 193 ms with one thread per
+// sightline timing every wall, 19.0 ms so (bit for bit the same samples).
 constexpr float kHgMargin = 1.02f;    // of the estimate (relative) ...
 constexpr float kHgFloor = 4e-6f;     // ... and of u near zero (absolute)
 

@@ -267,7 +267,8 @@ static gm_status small_prepare(gm_ctx* c) {
                                    cudaMemcpyDeviceToHost, st));
   GM_CUDA_CHECK(c, cudaStreamSynchronize(st));
   const int64_t total = std::max<int64_t>(*h, 1);
-  if (!ensure(c, c->ell_col, total * sizeof(int32_t)) || !ensure(c, c->ell_val, total * sizeof(double)))
+  if (!ensure(c, c->ell_col, total * sizeof(int32_t)) ||
+      !ensure(c, c->ell_val, total * sizeof(double)))
     return set_error(c, GM_E_NOMEM, "sliced rows");
   GM_PROF(c, "k_ell_fill");
   k_ell_fill<<<(unsigned)ns, 128, 0, st>>>(
@@ -326,8 +327,8 @@ bool small_cg_mean_fits(gm_ctx* c) {
   return (double)c->nnz < kSmallMean && small_cg_fits(c, 1);
 }
 
-// Behind small_cg_fits: solves B x = rhs for n_cols columns (leading dimension ld); scal: 2 x ld doubles
-// for ||b||^2 and ||r||^2 of the columns.  Synchronises.
+// Behind small_cg_fits: solves B x = rhs for n_cols columns (leading dimension ld); bb
+// and rr: ||b||^2 and ||r||^2 of the columns.  Synchronises.
 gm_status small_cg(gm_ctx* c, int64_t n_cols, int64_t ld, const double* dv, const double* minv,
                    const double* rhs, double* x, bool warm, double tol, double* bb, double* rr,
                    int64_t* iters) {
@@ -338,13 +339,15 @@ gm_status small_cg(gm_ctx* c, int64_t n_cols, int64_t ld, const double* dv, cons
   // error stays out of the results (a panel's columns go on too, to 1e-3 of it, while
   // others need it)
   SmallCg A{(int)c->n, (const int64_t*)c->ell_off.p, (const int32_t*)c->ell_row.p,
-            (const int32_t*)c->ell_col.p, (const double*)c->ell_val.p, dv, minv, rhs, x, ld, 1e-4 * tol * tol,
+            (const int32_t*)c->ell_col.p, (const double*)c->ell_val.p, dv, minv, rhs, x, ld,
+            1e-4 * tol * tol,
             warm ? 1 : 0, c->cfg.cg_max_iter, bb, rr, d_it, c->d_flags};
   const int rpt = c->n > 1024 ? 2 : 1;
   const int T = (int)(ceil_div(ceil_div(c->n, rpt), 128) * 128);  // groups of four warps
   const size_t smem = (((c->n + 31) & ~31ll) + 2 * 1024 + 8) * sizeof(double);
   GM_PROF(c, "k_cg_columns");
-  auto kern = rpt == 2 ? k_cg_columns<2, 1024> : T > 512 ? k_cg_columns<1, 1024> : k_cg_columns<1, 512>;
+  auto kern = rpt == 2 ? k_cg_columns<2, 1024>
+                       : T > 512 ? k_cg_columns<1, 1024> : k_cg_columns<1, 512>;
   GM_CUDA_CHECK(c, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   kern<<<(unsigned)n_cols, T, smem, st>>>(A);
   GM_LAUNCH_CHECK(c);

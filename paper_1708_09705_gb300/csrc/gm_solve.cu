@@ -1593,7 +1593,9 @@ static gm_status panels(gm_ctx* c, int64_t n_rows, const int64_t* row_ptr, const
     const size_t held = ws.P_X.bytes + ws.P_R.bytes + ws.P_P.bytes + ws.P_PD.bytes +
                         ws.P_Q.bytes + c->tc_planes.bytes;
     double budget = std::min<double>(0.5 * ((double)free_b + (double)held), 160e9);
-    const double per = 5.0 * sizeof(TV) + (sizeof(TV) == 4 ? (c->tc_nblk > 0 ? 6.0 : 0.0) : (c->tc64_use ? 16.0 : 0.0));
+    const double planes = sizeof(TV) == 4 ? (c->tc_nblk > 0 ? 6.0 : 0.0)  // of the tile products
+                                          : (c->tc64_use ? 16.0 : 0.0);
+    const double per = 5.0 * sizeof(TV) + planes;
     R = (int64_t)(budget / (per * (double)n));
   }
   R = std::max<int64_t>(32, std::min<int64_t>(R, ceil_div(n_cols_all, 32) * 32));
@@ -1703,123 +1705,123 @@ static gm_status panels(gm_ctx* c, int64_t n_rows, const int64_t* row_ptr, const
       if (ss != GM_OK) return ss;
       total_it += sit;
     } else {
-    if (use_warm) {
-      GM_PROF(c, "k_panel_scale");
-      k_panel_scale<TV><<<egrid, kBT, 0, st>>>(n, (int)R, dv, X, PD);
-      GM_LAUNCH_CHECK(c);
-      int nbu = nbx;
-      gm_status ss = panel_product<TA, TV>(c, n, R, nbx, grid, dv, X, PD, Q, pa, &nbu);
-      if (ss != GM_OK) return ss;
-      GM_PROF(c, "k_panel_init_warm");
-      k_panel_init_warm<TV><<<egrid, kBT, 0, st>>>(n, (int)R, minv, dv, Rr, Q, P, PD, pa, pb);
-      GM_LAUNCH_CHECK(c);
-    } else {
-      GM_PROF(c, "k_panel_init");
-      k_panel_init<TV><<<egrid, kBT, 0, st>>>(n, (int)R, minv, dv, X, Rr, P, PD, pa, pb);
-      GM_LAUNCH_CHECK(c);
-    }
-    // the BF16 planes of PD were written by the deflation update (the
-    // asynchronous tile product then skips its split)
-    bool planes = false;
-    if (defl) {
-      // z = M_d^-1 r for the initial residuals: P, PD and the rz rows
-      gm_status ds;
-      if (defl_tc) {
-        planes = tc_variant(c, (int)R) == 4;
-        ds = deflate_step_tc(c, (int)R, nch, nullptr, (const float*)minv, (float*)Rr,
-                             (const float*)Q, nullptr, nullptr, corr);
-        if (ds == GM_OK)
-          ds = deflate_update_tc(c, (int)R, (const float*)minv, (const float*)dv, nullptr, nullptr,
-                                 nullptr, nullptr, (const float*)Rr, (float*)P, (float*)PD, planes);
-      } else {
-        ds = deflate_rhs(c, (int)R, (const float*)Rr, corr);
-        if (ds == GM_OK)
-          ds = deflate_update(c, (int)R, nbx, (const float*)minv, (const float*)dv, nullptr,
-                              nullptr, (const float*)Rr, (float*)P, (float*)PD);
-      }
-      if (ds != GM_OK) return ds;
-    }
-    GM_CUDA_CHECK(c, cudaMemsetAsync(n_active, 0, sizeof(int), st));
-    GM_PROF(c, "k_panel_reduce");
-    k_panel_reduce<<<redb, redt(nbe), 0, st>>>(0, nbe, (int)R, ncols, tol2, frozen2, 0, max_it, pa,
-                                               pb, corr, ncorr, scal, active, n_active,
-                                               c->d_flags);
-    GM_LAUNCH_CHECK(c);
-    const int check = 8;
-    GM_CUDA_CHECK(c, cudaMemcpyAsync(hn, n_active, sizeof(int), cudaMemcpyDeviceToHost, st));
-    GM_CUDA_CHECK(c, cudaStreamSynchronize(st));
-    int it = *hn == 0 ? 0 : 1;  // no active column (all right-hand sides zero): no iteration
-    for (; it >= 1 && it <= max_it; ++it) {
-      int nbu = nbx;
-      {
-        gm_status ss = panel_product<TA, TV>(c, n, R, nbx, grid, dv, P, PD, Q, pa, &nbu, planes);
+      if (use_warm) {
+        GM_PROF(c, "k_panel_scale");
+        k_panel_scale<TV><<<egrid, kBT, 0, st>>>(n, (int)R, dv, X, PD);
+        GM_LAUNCH_CHECK(c);
+        int nbu = nbx;
+        gm_status ss = panel_product<TA, TV>(c, n, R, nbx, grid, dv, X, PD, Q, pa, &nbu);
         if (ss != GM_OK) return ss;
-      }
-      GM_PROF(c, "k_panel_reduce");
-      k_panel_reduce<<<redb, redt(nbu), 0, st>>>(1, nbu, (int)R, ncols, tol2, frozen2, it, max_it,
-                                                 pa, nullptr, nullptr, 0, scal, active, n_active,
-                                                 c->d_flags);
-      GM_LAUNCH_CHECK(c);
-      // partial rows of rz / rr
-      int nbr = sizeof(TV) == 4 ? (int)ceil_div(nbe, kUpdGroups) : nbe;
-      if (defl_tc) {
-        // Rr update fused with C = Y^T Rr and the deflation rows
-        gm_status ds = deflate_step_tc(c, (int)R, nch, scal, (const float*)minv, (float*)Rr,
-                                       (const float*)Q, pa, pb, corr);
-        if (ds != GM_OK) return ds;
-        nbr = nch;
+        GM_PROF(c, "k_panel_init_warm");
+        k_panel_init_warm<TV><<<egrid, kBT, 0, st>>>(n, (int)R, minv, dv, Rr, Q, P, PD, pa, pb);
+        GM_LAUNCH_CHECK(c);
       } else {
-        GM_PROF(c, "k_panel_update1");
-        // X with P in k_panel_update2, but the CUDA-core deflation update has no X
-        if constexpr (sizeof(TV) == 4) {
-          const bool brief = n <= 16ll * nbe;  // two rows a warp at most
-          auto kern = defl ? (brief ? k_panel_update1_f32<true, true> : k_panel_update1_f32<true, false>)
-                           : (brief ? k_panel_update1_f32<false, true> : k_panel_update1_f32<false, false>);
-          kern<<<u1grid, kBT, 0, st>>>(n, (int)R, nbe, minv, scal, X, Rr, P, Q, pa, pb);
+        GM_PROF(c, "k_panel_init");
+        k_panel_init<TV><<<egrid, kBT, 0, st>>>(n, (int)R, minv, dv, X, Rr, P, PD, pa, pb);
+        GM_LAUNCH_CHECK(c);
+      }
+      // the BF16 planes of PD were written by the deflation update (the
+      // asynchronous tile product then skips its split)
+      bool planes = false;
+      if (defl) {
+        // z = M_d^-1 r for the initial residuals: P, PD and the rz rows
+        gm_status ds;
+        if (defl_tc) {
+          planes = tc_variant(c, (int)R) == 4;
+          ds = deflate_step_tc(c, (int)R, nch, nullptr, (const float*)minv, (float*)Rr,
+                               (const float*)Q, nullptr, nullptr, corr);
+          if (ds == GM_OK)
+            ds = deflate_update_tc(c, (int)R, (const float*)minv, (const float*)dv, nullptr, nullptr,
+                                   nullptr, nullptr, (const float*)Rr, (float*)P, (float*)PD, planes);
         } else {
-          k_panel_update1<TV><<<ugrid, kBT, 0, st>>>(n, (int)R, minv, scal, Rr, Q, pa, pb);
+          ds = deflate_rhs(c, (int)R, (const float*)Rr, corr);
+          if (ds == GM_OK)
+            ds = deflate_update(c, (int)R, nbx, (const float*)minv, (const float*)dv, nullptr,
+                                nullptr, (const float*)Rr, (float*)P, (float*)PD);
         }
-        GM_LAUNCH_CHECK(c);
-        if (defl) {
-          gm_status ds = deflate_rhs(c, (int)R, (const float*)Rr, corr);
-          if (ds != GM_OK) return ds;
-        }
+        if (ds != GM_OK) return ds;
       }
+      GM_CUDA_CHECK(c, cudaMemsetAsync(n_active, 0, sizeof(int), st));
       GM_PROF(c, "k_panel_reduce");
-      k_panel_reduce<<<redb, redt(nbr), 0, st>>>(2, nbr, (int)R, ncols, tol2, frozen2, it, max_it,
-                                                 pa, pb, corr, ncorr, scal, active, n_active,
+      k_panel_reduce<<<redb, redt(nbe), 0, st>>>(0, nbe, (int)R, ncols, tol2, frozen2, 0, max_it, pa,
+                                                 pb, corr, ncorr, scal, active, n_active,
                                                  c->d_flags);
       GM_LAUNCH_CHECK(c);
-      planes = false;
-      if (defl_tc) {
-        planes = tc_variant(c, (int)R) == 4;
-        gm_status ds = deflate_update_tc(c, (int)R, (const float*)minv, (const float*)dv,
-                                         scal, scal + R, active, (float*)X, (const float*)Rr,
-                                         (float*)P, (float*)PD, planes);
-        if (ds != GM_OK) return ds;
-      } else if (defl) {
-        gm_status ds = deflate_update(c, (int)R, nbx, (const float*)minv, (const float*)dv,
-                                      scal + R, active, (const float*)Rr, (float*)P, (float*)PD);
-        if (ds != GM_OK) return ds;
-      } else {
-        GM_PROF(c, "k_panel_update2");
-        planes = sizeof(TV) == 4 && c->tc_nblk > 0 && tc_variant(c, (int)R) == 4;
-        if (planes)
-          k_panel_update2<TV, true><<<ugrid, kBT, 0, st>>>(n, (int)R, minv, dv, scal, active, X, Rr,
-                                                           P, PD, (uint16_t*)c->tc_planes.p,
-                                                           n * (int64_t)R);
-        else
-          k_panel_update2<TV, false><<<ugrid, kBT, 0, st>>>(n, (int)R, minv, dv, scal, active, X,
-                                                            Rr, P, PD, nullptr, 0);
+      const int check = 8;
+      GM_CUDA_CHECK(c, cudaMemcpyAsync(hn, n_active, sizeof(int), cudaMemcpyDeviceToHost, st));
+      GM_CUDA_CHECK(c, cudaStreamSynchronize(st));
+      int it = *hn == 0 ? 0 : 1;  // no active column (all right-hand sides zero): no iteration
+      for (; it >= 1 && it <= max_it; ++it) {
+        int nbu = nbx;
+        {
+          gm_status ss = panel_product<TA, TV>(c, n, R, nbx, grid, dv, P, PD, Q, pa, &nbu, planes);
+          if (ss != GM_OK) return ss;
+        }
+        GM_PROF(c, "k_panel_reduce");
+        k_panel_reduce<<<redb, redt(nbu), 0, st>>>(1, nbu, (int)R, ncols, tol2, frozen2, it, max_it,
+                                                   pa, nullptr, nullptr, 0, scal, active, n_active,
+                                                   c->d_flags);
         GM_LAUNCH_CHECK(c);
+        // partial rows of rz / rr
+        int nbr = sizeof(TV) == 4 ? (int)ceil_div(nbe, kUpdGroups) : nbe;
+        if (defl_tc) {
+          // Rr update fused with C = Y^T Rr and the deflation rows
+          gm_status ds = deflate_step_tc(c, (int)R, nch, scal, (const float*)minv, (float*)Rr,
+                                         (const float*)Q, pa, pb, corr);
+          if (ds != GM_OK) return ds;
+          nbr = nch;
+        } else {
+          GM_PROF(c, "k_panel_update1");
+          // X with P in k_panel_update2, but the CUDA-core deflation update has no X
+          if constexpr (sizeof(TV) == 4) {
+            const bool brief = n <= 16ll * nbe;  // two rows a warp at most
+            auto kern = defl ? (brief ? k_panel_update1_f32<true, true> : k_panel_update1_f32<true, false>)
+                             : (brief ? k_panel_update1_f32<false, true> : k_panel_update1_f32<false, false>);
+            kern<<<u1grid, kBT, 0, st>>>(n, (int)R, nbe, minv, scal, X, Rr, P, Q, pa, pb);
+          } else {
+            k_panel_update1<TV><<<ugrid, kBT, 0, st>>>(n, (int)R, minv, scal, Rr, Q, pa, pb);
+          }
+          GM_LAUNCH_CHECK(c);
+          if (defl) {
+            gm_status ds = deflate_rhs(c, (int)R, (const float*)Rr, corr);
+            if (ds != GM_OK) return ds;
+          }
+        }
+        GM_PROF(c, "k_panel_reduce");
+        k_panel_reduce<<<redb, redt(nbr), 0, st>>>(2, nbr, (int)R, ncols, tol2, frozen2, it, max_it,
+                                                   pa, pb, corr, ncorr, scal, active, n_active,
+                                                   c->d_flags);
+        GM_LAUNCH_CHECK(c);
+        planes = false;
+        if (defl_tc) {
+          planes = tc_variant(c, (int)R) == 4;
+          gm_status ds = deflate_update_tc(c, (int)R, (const float*)minv, (const float*)dv,
+                                           scal, scal + R, active, (float*)X, (const float*)Rr,
+                                           (float*)P, (float*)PD, planes);
+          if (ds != GM_OK) return ds;
+        } else if (defl) {
+          gm_status ds = deflate_update(c, (int)R, nbx, (const float*)minv, (const float*)dv,
+                                        scal + R, active, (const float*)Rr, (float*)P, (float*)PD);
+          if (ds != GM_OK) return ds;
+        } else {
+          GM_PROF(c, "k_panel_update2");
+          planes = sizeof(TV) == 4 && c->tc_nblk > 0 && tc_variant(c, (int)R) == 4;
+          if (planes)
+            k_panel_update2<TV, true><<<ugrid, kBT, 0, st>>>(n, (int)R, minv, dv, scal, active, X, Rr,
+                                                             P, PD, (uint16_t*)c->tc_planes.p,
+                                                             n * (int64_t)R);
+          else
+            k_panel_update2<TV, false><<<ugrid, kBT, 0, st>>>(n, (int)R, minv, dv, scal, active, X,
+                                                              Rr, P, PD, nullptr, 0);
+          GM_LAUNCH_CHECK(c);
+        }
+        if (it % check == 0 || it == max_it) {
+          GM_CUDA_CHECK(c, cudaMemcpyAsync(hn, n_active, sizeof(int), cudaMemcpyDeviceToHost, st));
+          GM_CUDA_CHECK(c, cudaStreamSynchronize(st));
+          if (*hn == 0) break;
+        }
       }
-      if (it % check == 0 || it == max_it) {
-        GM_CUDA_CHECK(c, cudaMemcpyAsync(hn, n_active, sizeof(int), cudaMemcpyDeviceToHost, st));
-        GM_CUDA_CHECK(c, cudaStreamSynchronize(st));
-        if (*hn == 0) break;
-      }
-    }
-    total_it += std::min(it, max_it);
+      total_it += std::min(it, max_it);
     }  // !small
     if (probe) {
       GM_PROF(c, "k_panel_final_probe");

@@ -381,7 +381,8 @@ __global__ void __launch_bounds__(Oz<NC>::kThreads, 1) k_panel_spmm_tc64(
     const uint32_t ta = tmem + ((uint32_t)(32 * quad) << 16) + 16u * sub;
     for (int64_t per = 0; per < nper; ++per) {
       bool up = tg::wait(tg::smem(&accfull), (uint32_t)(per & 1), abort_v);
-      if (expire && per == nper - 1 && b == 0 && blockIdx.x == 0 && warp == 5 && lane == 7) up = false;
+      if (expire && per == nper - 1 && b == 0 && blockIdx.x == 0 && warp == 5 && lane == 7)
+        up = false;
       // the warp's lanes leave together: the loads below are for whole warps
       if (!__all_sync(0xffffffffu, up)) {
         abort_flag = 1;
