@@ -435,7 +435,7 @@ struct BandRule {
     TabF64 td;
   };
   // FP32: one block of 32 warps per SM around the replicated table window
-  static constexpr int kThreads = sizeof(T) == 4 ? 1024 : 256;
+  static constexpr int kThreads = sizeof(T) == 4 ? 1024 : 256, kBound = kThreads;
   GLook<T> g;
   BandLane<T> L;
   int lane;
@@ -483,10 +483,10 @@ struct BandRule {
 // coincide: the diagonal) use the FP64 table.  Nodes of the same index are s_i - s_j
 // times the node apart, taken from the FP64 difference: from the two products, of
 // which 48 bits are kept, stars at nearly equal distances lost the separation.
-// PIC workload at 6,000 stars (cross-covariances of 4,140 points): 152 ms with
-// FP64 instructions, 19.2 ms so.  Against FP64 Bessel functions entries between
-// different stars are 1.0e-12 off (largest 3.6e-12) in both forms, the diagonal
-// 1.4e-10 (the table ends at x = 2^-100).
+// 2,001 stars, 64 nodes (161,494 unique pairs): 18.5 ms with FP64 instructions
+// (Gl64Rule), 3.2 ms so; 4.9 and 0.88 ms at 32 nodes.  Against FP64 Bessel functions
+// entries between different stars are 1.0e-12 off (largest 3.6e-12) in both forms, the
+// diagonal 1.4e-10 (the table ends at x = 2^-100).
 struct F2 {
   float h, l;
 };
@@ -551,7 +551,9 @@ struct DfRule {
     const float2* tab2;
     int Q;
   };
-  static constexpr int kThreads = 512;
+  // launched with 512; up to 64 nodes within the registers of 1,024 (64 a thread), so
+  // that two blocks share an SM
+  static constexpr int kThreads = 512, kBound = KPL <= 2 ? 1024 : 512;
   static constexpr int kWarps = kThreads / 32;
   const float4* t4;
   const float2* t2;
@@ -695,7 +697,7 @@ struct Gl64Rule {
     TabF64 td;
     int Q;
   };
-  static constexpr int kThreads = 256;
+  static constexpr int kThreads = 256, kBound = kThreads;
   const double *z, *w;  // shared memory, padded with zeros
   const D4* gtab;
   TabF64 td;
@@ -774,7 +776,7 @@ struct Gl32Rule {
     const float4* gtab;
     int Q;
   };
-  static constexpr int kThreads = KPL <= 2 ? 1024 : 512;
+  static constexpr int kThreads = KPL <= 2 ? 1024 : 512, kBound = kThreads;
   const unsigned char* tab;  // segment 0 of the window less the window's first index
   const float4* zw;          // nodes and weights (z, w) of two nodes, padded with w = 0
   int lane, Q;
@@ -876,7 +878,7 @@ struct Gl32Rule {
 // to 32): the FP64 part of a pair (distances, chord, log1p, taper) runs a lane
 // per pair, the node sums a warp per pair.
 template <typename Rule>
-__global__ void __launch_bounds__(Rule::kThreads) k_pair_entries(
+__global__ void __launch_bounds__(Rule::kBound) k_pair_entries(
     QuadParams P, typename Rule::Par rp, int batch, int64_t n_rows, const double* __restrict__ rs,
     const double* __restrict__ rux, const double* __restrict__ ruy, const double* __restrict__ ruz,
     const double* __restrict__ s, const double* __restrict__ ux, const double* __restrict__ uy,
@@ -953,7 +955,7 @@ __global__ void __launch_bounds__(Rule::kThreads) k_pair_entries(
 // u_j|): K = log1p(R) (or R) without the taper; sj null: the self-covariance of
 // the points si, at the precision of the stored entries.
 template <typename Rule>
-__global__ void __launch_bounds__(Rule::kThreads) k_pair_list(
+__global__ void __launch_bounds__(Rule::kBound) k_pair_list(
     QuadParams P, typename Rule::Par rp, int batch, int64_t n, const double* __restrict__ si,
     const double* __restrict__ sj, const double* __restrict__ chord, double* __restrict__ out) {
   extern __shared__ __align__(16) unsigned char smem[];
