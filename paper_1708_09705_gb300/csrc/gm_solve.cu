@@ -1453,7 +1453,11 @@ static gm_status posterior_mean(gm_ctx* c, int64_t* iters, double* resid) {
       if (!std::isfinite(hp[1])) return set_error(c, GM_E_NONFINITE, "CG residual is not finite");
       *resid = hp[0] > 0 ? std::sqrt(hp[1] / hp[0]) : 0.0;
     } else {
-      s = cg_single<TA, double>(c, r64, x64, tol, max_it, iters, resid);
+      // to 1e-2 of the tolerance, as the blocks per column go: where a residual just
+      // meets the tolerance, the last bit of an entry or site decides whether the solve
+      // goes on, and means at 2,001 stars were 1e-11 to 1.1e-9 off (24 catalogues at
+      // 1e-12; 0.8e-11 to 2.5e-11 so, the table's share).  Some 16 iterations of 24 us.
+      s = cg_single<TA, double>(c, r64, x64, 1e-2 * tol, max_it, iters, resid);
       if (s != GM_OK) return s;
     }
     GM_PROF(c, "k_alpha");
