@@ -501,7 +501,7 @@ gm_status gm_cov_rows(gm_ctx* ctx, int64_t row0, int64_t nrows, int32_t source,
  *                largest relative site change and the number of skipped stars
  * All arrays must be DEVICE pointers of the current device (or managed
  * memory), length n; host pointers and memory of another GPU: GM_E_INVAL.
- * The scratch is a file-scope device array of about 66 KB that every GPU
+ * The scratch is a file-scope device array of about 1 KB that every GPU
  * loading the library keeps until the process exits.  The first call on a
  * device (and the first after a device reset) uploads the Gauss-Hermite rule
  * with a synchronous copy and a device synchronisation, so make that first

@@ -23,7 +23,6 @@ namespace gm {
 struct SiteParams {
   double damping;
   double vc_floor;
-  int lik;
 };
 
 // Work split.  A group of G lanes (a power of two up to 32) owns a star: every
@@ -136,29 +135,29 @@ __device__ __forceinline__ void tilted_in_order(double mc, double vc, double obs
 
 constexpr int kSiteThreads = 128;
 
-// Shared by the context's update and the allocation-free one: `last` (null:
-// the caller reduces part_delta) makes the last block to finish reduce the
-// block maxima and put the three results to last.out.
-struct SiteLast {
-  unsigned long long* ticket;   // blocks finished
-  unsigned long long* out;      // skip count, flags, maximum (bits of a double)
-};
+// What an instantiation computes: the tilted moments split over the group's lanes, or
+// in order (Gaussian in A), or the closed form (Gaussian in ln A).  The closed form is
+// bound by its FP64 divisions, eleven a star: 1,000,000 stars 267 us a call, 315 as a
+// branch of the split form, which took two of them twice and ended in a last block's
+// reduction (279 before there was a split form).
+enum SiteForm { kSplit, kInOrder, kClosed };
 
-template <int G, bool IN_ORDER>
+template <int G, SiteForm FORM>
 __global__ void __launch_bounds__(kSiteThreads) k_site_update(
     int64_t n, SiteParams P, const double* __restrict__ mu, const double* __restrict__ var,
     const double* __restrict__ obs, const double* __restrict__ sig, double* __restrict__ tau,
     double* __restrict__ nu, const double* __restrict__ gh_x, const double* __restrict__ gh_w,
-    double* __restrict__ part_delta, unsigned long long* __restrict__ skipped,
-    unsigned* __restrict__ flags, SiteLast last) {
+    double* __restrict__ part_delta, unsigned long long* __restrict__ max_delta,
+    unsigned long long* __restrict__ skipped, unsigned* __restrict__ flags) {
   __shared__ double ghx[kGH], ghw[kGH];
   __shared__ double sh[kSiteThreads / 32];
-  __shared__ int is_last;
-  for (int k = threadIdx.x; k < kGH; k += blockDim.x) {
-    ghx[k] = gh_x[k];
-    ghw[k] = gh_w[k];
+  if (FORM != kClosed) {
+    for (int k = threadIdx.x; k < kGH; k += blockDim.x) {
+      ghx[k] = gh_x[k];
+      ghw[k] = gh_w[k];
+    }
+    __syncthreads();
   }
-  __syncthreads();
   constexpr int kPerBlock = kSiteThreads / G;
   const int sub = threadIdx.x & (G - 1);
   double dmax = 0;
@@ -183,10 +182,10 @@ __global__ void __launch_bounds__(kSiteThreads) k_site_update(
       s2 = sg * sg;
     }
     double mh = 0, vh = 1;
-    if (P.lik == GM_LIK_GAUSS_IN_LNA) {
-      vh = 1.0 / (1.0 / vc + 1.0 / s2);
-      mh = vh * (mc / vc + ob / s2);
-    } else if (IN_ORDER) {
+    if (FORM == kClosed) {
+      vh = 1.0 / (tc + 1.0 / s2);  // tc = 1 / vc, ncv = mc / vc by now
+      mh = vh * (ncv + ob / s2);
+    } else if (FORM == kInOrder) {
       if (!skip) tilted_in_order(mc, vc, ob, s2, ghx, ghw, &mh, &vh);
     } else {
       double S0 = 0, S1 = 0, S2 = 0;
@@ -238,28 +237,10 @@ __global__ void __launch_bounds__(kSiteThreads) k_site_update(
     double v = 0;
     for (int w = 0; w < kSiteThreads / 32; ++w) v = fmax(v, sh[w]);
     if (!isfinite(v)) atomicOr(flags, kFlagNonFinite);
-    part_delta[blockIdx.x] = v;
-    is_last = 0;
-    if (last.ticket) {
-      __threadfence();
-      is_last = atomicAdd(last.ticket, 1ull) == gridDim.x - 1;
-    }
-  }
-  __syncthreads();
-  if (!is_last) return;
-  __threadfence();
-  double v = 0;
-  for (int k = threadIdx.x; k < (int)gridDim.x; k += blockDim.x)
-    v = fmax(v, *(volatile double*)(part_delta + k));
-  for (int off = 16; off > 0; off >>= 1) v = fmax(v, __shfl_xor_sync(0xffffffffu, v, off));
-  if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = v;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double mx = 0;
-    for (int w = 0; w < kSiteThreads / 32; ++w) mx = fmax(mx, sh[w]);
-    last.out[0] = *(volatile unsigned long long*)skipped;
-    last.out[1] = *(volatile unsigned*)flags;
-    last.out[2] = (unsigned long long)__double_as_longlong(mx);
+    // the blocks' maxima for the caller to reduce, or their maximum (non-negative
+    // doubles have their bits in the same order)
+    if (part_delta) part_delta[blockIdx.x] = v;
+    else atomicMax(max_delta, (unsigned long long)__double_as_longlong(v));
   }
 }
 
@@ -281,29 +262,24 @@ static int site_blocks(int64_t n, int group, int64_t max_blocks) {
   return (int)std::min<int64_t>(ceil_div(n * group, kSiteThreads), max_blocks);
 }
 
-// group 0: the in-order update
-static void launch_site(int group, int blocks, cudaStream_t st, int64_t n, const SiteParams& P,
-                        const double* mu, const double* var, const double* obs, const double* sig,
-                        double* tau, double* nu, const double* gh_x, const double* gh_w,
-                        double* part, unsigned long long* skipped, unsigned* flags,
-                        SiteLast last) {
-#define GM_SITE(G)                                                                            \
-  case G:                                                                                     \
-    k_site_update<G, false><<<blocks, kSiteThreads, 0, st>>>(                                 \
-        n, P, mu, var, obs, sig, tau, nu, gh_x, gh_w, part, skipped, flags, last);            \
-    break
-  switch (group) {
-    GM_SITE(32);
-    GM_SITE(16);
-    GM_SITE(8);
-    GM_SITE(4);
-    GM_SITE(2);
-    GM_SITE(1);
-    default:
-      k_site_update<1, true><<<blocks, kSiteThreads, 0, st>>>(n, P, mu, var, obs, sig, tau, nu,
-                                                              gh_x, gh_w, part, skipped, flags,
-                                                              last);
-  }
+// group: lanes per star of the split form (the others have one)
+static void launch_site(SiteForm form, int group, int blocks, cudaStream_t st, int64_t n,
+                        const SiteParams& P, const double* mu, const double* var,
+                        const double* obs, const double* sig, double* tau, double* nu,
+                        const double* gh_x, const double* gh_w, double* part,
+                        unsigned long long* max_delta, unsigned long long* skipped,
+                        unsigned* flags) {
+#define GM_SITE(G, FORM)                                   \
+  k_site_update<G, FORM><<<blocks, kSiteThreads, 0, st>>>( \
+      n, P, mu, var, obs, sig, tau, nu, gh_x, gh_w, part, max_delta, skipped, flags)
+  if (form == kClosed) GM_SITE(1, kClosed);
+  else if (form == kInOrder) GM_SITE(1, kInOrder);
+  else if (group == 32) GM_SITE(32, kSplit);
+  else if (group == 16) GM_SITE(16, kSplit);
+  else if (group == 8) GM_SITE(8, kSplit);
+  else if (group == 4) GM_SITE(4, kSplit);
+  else if (group == 2) GM_SITE(2, kSplit);
+  else GM_SITE(1, kSplit);
 #undef GM_SITE
 }
 
@@ -311,16 +287,19 @@ gm_status site_update(gm_ctx* c, double* max_delta, int64_t* skipped) {
   const int64_t n = c->n;
   cudaStream_t st = c->stream;
   const int sms = sm_count(c);
-  const int group = c->cfg.precision == GM_PREC_FP32 ? 0 : site_group(n, sms);
-  const int G = site_blocks(n, std::max(group, 1), 4 * sms);
+  const SiteForm form = c->cfg.likelihood == GM_LIK_GAUSS_IN_LNA ? kClosed
+                        : c->cfg.precision == GM_PREC_FP32       ? kInOrder
+                                                                 : kSplit;
+  const int group = form == kSplit ? site_group(n, sms) : 1;
+  const int G = site_blocks(n, group, 4 * sms);
   double* part = (double*)dev_alloc(c, (G + 1) * sizeof(double) + sizeof(unsigned long long));
   if (!part) return set_error(c, GM_E_NOMEM, "site partials");
   unsigned long long* cnt = (unsigned long long*)(part + G);
   GM_CUDA_CHECK(c, cudaMemsetAsync(cnt, 0, sizeof(unsigned long long), st));
-  SiteParams P{c->cfg.damping, c->cfg.vc_floor, c->cfg.likelihood};
+  SiteParams P{c->cfg.damping, c->cfg.vc_floor};
   GM_PROF(c, "k_site_update");
-  launch_site(group, G, st, n, P, c->mu, c->var, c->obs, c->obs_sigma, c->tau, c->nu, c->gh_x,
-              c->gh_wx, part, cnt, c->d_flags, SiteLast{nullptr, nullptr});
+  launch_site(form, group, G, st, n, P, c->mu, c->var, c->obs, c->obs_sigma, c->tau, c->nu, c->gh_x,
+              c->gh_wx, part, nullptr, cnt, c->d_flags);
   GM_LAUNCH_CHECK(c);
   double* hp = (double*)c->h_pinned;
   GM_CUDA_CHECK(c, cudaMemcpyAsync(hp, part, (G + 1) * sizeof(double), cudaMemcpyDeviceToHost, st));
@@ -343,22 +322,20 @@ gm_status site_update(gm_ctx* c, double* max_delta, int64_t* skipped) {
 // running inside a memory-capped or pre-reserved budget, or a service loop
 // that must not call cudaMalloc/cudaFree on its latency path.  For them the
 // EP site update runs on caller-owned arrays, with its scratch (Gauss-Hermite
-// table, per-block maxima, skip counter, flags) in the file-scope array
-// below.  It is sized for one block per 128 stars up to kNaMaxBlocks blocks,
-// so n <= kNaMaxStars.  Every GPU that loads the library holds the array
+// table, skip counter, flags, maximum) in the file-scope array below.  A block
+// takes 128 stars or fewer, up to kNaMaxBlocks blocks: n <= kNaMaxStars.  Every GPU that loads the library holds the array
 // until the process exits.  All calls share it: concurrent calls on the GPU
 // race with one another and must be serialised by the caller.
 // ---------------------------------------------------------------------------
 constexpr int kNaMaxBlocks = 8192;
 constexpr int64_t kNaMaxStars = 128ll * kNaMaxBlocks;  // 1,048,576
-constexpr int kNaSlots = 2 * kGH + kNaMaxBlocks + 6;   // doubles
+constexpr int kNaSlots = 2 * kGH + 3;                  // doubles
 constexpr int kNaMaxDevices = 64;
 
 static __device__ __align__(256) double g_na_scratch[kNaSlots];
 
 // Scratch layout (doubles): [0, kGH) nodes, [kGH, 2 kGH) weights * exp(x^2),
-// [2 kGH, 2 kGH + kNaMaxBlocks) per-block maxima, then 64-bit words: the skip
-// counter, the flags, the count of finished blocks and the three results.
+// then 64-bit words: the skip counter, the flags, the maximum (bits of a double).
 // Per device, the scratch address at which the rule was last uploaded.  The
 // address is resolved again on every call, so a module reloaded after a
 // device reset (new address) gets its rule uploaded again instead of a stale
@@ -433,12 +410,9 @@ extern "C" gm_status gm_site_update_noalloc(int64_t n, const double* mu, const d
   cudaStream_t s = (cudaStream_t)stream;
   double* gh_x = base;
   double* gh_w = base + kGH;
-  double* part = base + 2 * kGH;
-  unsigned long long* skipped = (unsigned long long*)(part + kNaMaxBlocks);
+  unsigned long long* skipped = (unsigned long long*)(base + 2 * kGH);
   unsigned* flags = (unsigned*)(skipped + 1);
-  unsigned long long* ticket = skipped + 2;
-  unsigned long long* res = skipped + 3;
-  // the counters keep the previous call's values: clear them
+  // the words keep the previous call's values: clear them
   if (cudaMemsetAsync(skipped, 0, 3 * sizeof(double), s) != cudaSuccess) {
     cudaGetLastError();
     return GM_E_CUDA;
@@ -448,13 +422,14 @@ extern "C" gm_status gm_site_update_noalloc(int64_t n, const double* mu, const d
     cudaGetLastError();
     return GM_E_CUDA;
   }
-  const int group = site_group(n, sms > 0 ? sms : 1);
-  SiteParams P{damping, vc_floor, likelihood};
-  launch_site(group, site_blocks(n, group, kNaMaxBlocks), s, n, P, mu, var, obs, obs_sigma, tau,
-              nu, gh_x, gh_w, part, skipped, flags, SiteLast{ticket, res});
+  const SiteForm form = likelihood == GM_LIK_GAUSS_IN_LNA ? kClosed : kSplit;
+  const int group = form == kSplit ? site_group(n, sms > 0 ? sms : 1) : 1;
+  SiteParams P{damping, vc_floor};
+  launch_site(form, group, site_blocks(n, group, kNaMaxBlocks), s, n, P, mu, var, obs, obs_sigma, tau,
+              nu, gh_x, gh_w, nullptr, skipped + 2, skipped, flags);
   if (cudaGetLastError() != cudaSuccess) return GM_E_CUDA;
   unsigned long long h[3];
-  if (cudaMemcpyAsync(h, res, 3 * sizeof(double), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
+  if (cudaMemcpyAsync(h, skipped, 3 * sizeof(double), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
       cudaStreamSynchronize(s) != cudaSuccess) {
     cudaGetLastError();
     return GM_E_CUDA;
