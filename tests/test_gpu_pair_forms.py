@@ -44,6 +44,28 @@ def test_forms_agree(Q, form, monkeypatch):
     np.testing.assert_allclose(v, v64, rtol=1e-12)
 
 
+@pytest.mark.parametrize("n", [700, 1300])
+def test_forms_agree_in_batches(n, monkeypatch):
+    """Lists long enough for several entries a warp (44,000 and 160,000; the forms take
+    batches of different sizes), every entry once: no gaps, no doubles, symmetric."""
+    import paper_1708_09705_gb300 as gm
+    cat = make_catalogue("c1_plain_400", n=n, truth="mean")
+    out = []
+    for mode in ("", "fp64"):
+        monkeypatch.setenv("GM_QUAD", mode)
+        cfg = gm.config_from_catalogue(cat, precision=gm.PREC_FP64, n_nodes=8)
+        with gm.ep_init(cfg, cat["l"], cat["b"], cat["s"], cat["A_obs"], cat["A_sigma"]) as ctx:
+            ctx.build_cov()
+            out.append(ctx.get_csr() + ctx.get_prior())
+    for a, b in zip(*out):
+        np.testing.assert_allclose(a, b, rtol=1e-12)
+    rp, col, val = out[0][:3]
+    K = np.zeros((n, n))
+    K[np.repeat(np.arange(n), np.diff(rp)), col] = val
+    np.testing.assert_array_equal(K, K.T)
+    assert np.all(val > 0) and np.all(np.diag(K) > 0)
+
+
 @pytest.mark.parametrize("sigma2", [1e-12, 1e-8, 60.0, 75.0, 100.0, 500.0])
 def test_range_of_sigma2(sigma2):
     """One star: R = sum over both nodes of w w' g, g = expm1(sigma2 phi), from the
