@@ -267,7 +267,7 @@ __global__ void k_self_quad(QuadParams P, int64_t n_rows, const double* __restri
 //     over is a partition whatever its rounding), and reads g from the
 //     replicated table window of the 64-node kernel.
 // 6,000 stars of the 5-degree field (3.0e6 stored entries, FP32): 199 ms with
-// every lane finding its panels by FP64 pow / log, 2.6 ms so (5.8e8 unique
+// every lane finding its panels by FP64 pow / log, 2.2 ms so (6.7e8 unique
 // pairs/s); the carried sums cost 0.2 ms of it and lower the entries' error
 // against FP64 from 4.8e-8 to 3.3e-8.
 constexpr int kBandPts = 12;  // breakpoints h0 (q^j - 1) / (q - 1), j < 12: 0 .. 88.6 >= kK
@@ -483,8 +483,8 @@ struct BandRule {
 // coincide: the diagonal) use the FP64 table.  Nodes of the same index are s_i - s_j
 // times the node apart, taken from the FP64 difference: from the two products, of
 // which 48 bits are kept, stars at nearly equal distances lost the separation.
-// 2,001 stars, 64 nodes (161,494 unique pairs): 18.5 ms with FP64 instructions
-// (Gl64Rule), 3.2 ms so; 4.9 and 0.88 ms at 32 nodes.  Against FP64 Bessel functions
+// 2,001 stars, 64 nodes (161,494 unique pairs): 14.2 ms with FP64 instructions
+// (Gl64Rule), 2.3 ms so; 4.1 and 0.65 ms at 32 nodes.  Against FP64 Bessel functions
 // entries between different stars are 1.0e-12 off (largest 3.6e-12) in both forms, the
 // diagonal 1.4e-10 (the table ends at x = 2^-100).
 struct F2 {
@@ -764,8 +764,8 @@ struct Gl64Rule {
 // (k_pair_entries); a pair's own arithmetic, log1p and the taper included, is
 // FP32 as before.
 // 20,000 stars (1.58e7 unique pairs x 64 x 64 nodes): 46.7 ms with one pair a warp
-// and 22 instructions a node pair, 36.8 ms so (14 instructions; shared memory
-// 89 % busy, the issue slots 78 %), every entry the same bit for bit.
+// and 22 instructions a node pair, 32.9 ms so (14 instructions; shared memory 88 %
+// busy over all SMs, the issue slots 75 %), every entry the same bit for bit.
 template <int KPL>
 struct Gl32Rule {
   typedef float Val;
